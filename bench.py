@@ -29,11 +29,11 @@ sys.path.insert(0, ROOT)
 # ncu summaries of the kernels' DRAM traffic (profiles/traffic_<kernel>_<workload>.txt): used only while the
 # kernel's sources hash to the value recorded with the counters
 KERNEL_SOURCES = {
-    'k_validate_warp': ['kernels_walk.cu', 'warpwalk.cuh', 'device.cuh', 'packs.cuh'],
-    'k_forward_gs': ['region_forward.cu', 'gscols.cuh', 'skeleton.cuh', 'walk.cuh', 'device.cuh', 'seqpack.cuh'],
-    'k_forward': ['region_forward.cu', 'warpwalk.cuh', 'device.cuh', 'seqpack.cuh'],
-    'k_good': ['region_good.cu', 'gscols.cuh', 'device.cuh', 'seqpack.cuh'],
-    'k_check': ['region_check.cuh', 'region_check_sm.cu', 'region_check_global.cu', 'warpwalk.cuh', 'device.cuh'],
+    'k_validate_warp': ['kernels_walk.cu', 'warpwalk.cuh', 'rows.cuh', 'device.cuh', 'packs.cuh'],
+    'k_forward_gs': ['region_forward.cu', 'gscols.cuh', 'rows.cuh', 'skeleton.cuh', 'walk.cuh', 'device.cuh',
+                     'seqpack.cuh'],
+    'k_good': ['region_good.cu', 'rows.cuh', 'device.cuh', 'seqpack.cuh'],
+    'k_check': ['region_check.cu', 'warpwalk.cuh', 'rows.cuh', 'device.cuh'],
 }
 
 
@@ -448,7 +448,7 @@ def main():
     peak_ops, peak_ms = epic.measure_int_peak()
     peak_t = peak_ops / 1e12
     work = None
-    if cen and dom in ('k_forward_gs', 'k_forward', 'k_good') and 'forward_pairs' in cen:
+    if cen and dom in ('k_forward_gs', 'k_good') and 'forward_pairs' in cen:
         work = 3.0 * cen['forward_pairs'] * cen['words']
         work_note = 'forward charts of x: %.0f (node, origin) pairs x %d words x 3 (oracle census, %s)' % (
             cen['forward_pairs'], cen['words'], cen['forward_sample'])
@@ -464,7 +464,7 @@ def main():
     by_kernel = {}
     if cen and 'forward_pairs' in cen:
         fwork = 3.0 * cen['forward_pairs'] * cen['words']
-        for kname in ('k_forward_gs', 'k_forward', 'k_good'):
+        for kname in ('k_forward_gs', 'k_good'):
             if kname in kms and kms[kname] > 0:
                 a_t = fwork / (kms[kname] / 1e3) / 1e12
                 by_kernel[kname] = {'achieved': a_t, 'frac': a_t / peak_t, 'kernel_ms': kms[kname]}

@@ -24,27 +24,26 @@ class CoverCols {
   const DevGrammar& g;
   Workspace ws;
   WsDims dims;
-  WalkShared& sh;
   int W, FW;
-  __device__ CoverCols(const DevGrammar& g_, Workspace w, WsDims d, WalkShared& shared)
-      : g(g_), ws(w), dims(d), sh(shared), W(g_.W), FW(g_.FW) {}
+  __device__ CoverCols(const DevGrammar& g_, Workspace w, WsDims d)
+      : g(g_), ws(w), dims(d), W(g_.W), FW(g_.FW) {}
 
   __device__ void reset() {
     if (threadIdx.x == 0) {
-      sh.ncols = 0;
-      sh.status = kWalkOk;
+      walk_sh().ncols = 0;
+      walk_sh().status = kWalkOk;
     }
     __syncthreads();
   }
   __device__ void cleanup() {}
   __device__ int open_column() {
-    int c = sh.ncols;
+    int c = walk_sh().ncols;
     if (c >= dims.nmax || c >= kMaxCols) {
-      if (threadIdx.x == 0) sh.status = kWalkOverflow;
+      if (threadIdx.x == 0) walk_sh().status = kWalkOverflow;
       return -1;
     }
     for (int w = threadIdx.x; w < FW; w += blockDim.x) ws.cov[(size_t)c * FW + w] = 0;
-    if (threadIdx.x == 0) sh.scratch_i[0] = c;
+    if (threadIdx.x == 0) walk_sh().scratch_i[0] = c;
     __syncthreads();
     return c;
   }
@@ -54,21 +53,21 @@ class CoverCols {
   }
   // dst |= src (epsilon) or dst |= shift(src & lbl) over the item words
   __device__ void arrive_labels(int src, bool eps) {
-    int c = sh.scratch_i[0];
+    int c = walk_sh().scratch_i[0];
     const uint32_t* s = ws.cov + (size_t)src * FW;
     uint32_t* d = ws.cov + (size_t)c * FW;
     if (eps) {
       for (int w = threadIdx.x; w < FW; w += blockDim.x) d[w] |= s[w];
     } else {
       for (int w = threadIdx.x; w < W; w += blockDim.x) {
-        uint32_t v = s[w] & sh.lbl[w];
-        uint32_t p = w > 0 ? (s[w - 1] & sh.lbl[w - 1]) : 0u;
+        uint32_t v = s[w] & walk_sh().lbl[w];
+        uint32_t p = w > 0 ? (s[w - 1] & walk_sh().lbl[w - 1]) : 0u;
         d[w] |= (v << 1) | (p >> 31);
       }
     }
     __syncthreads();
   }
-  __device__ void close_column(int c, bool gap) {
+  __device__ __noinline__ void close_column(int c, bool gap) {
     __shared__ uint32_t R[kMaxFW];
     const uint32_t* rows = gap ? g.cov_all_close : g.cov_eps_close;
     uint32_t* S = ws.cov + (size_t)c * FW;
@@ -76,17 +75,23 @@ class CoverCols {
     __syncthreads();
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nwarps = blockDim.x >> 5;
-    // each warp takes every nwarps-th set state and ORs its closure row
-    int seen = 0;
-    for (int w = 0; w < FW; ++w) {
+    // the warps share out the set words; a state already in R is in the closure
+    // of one whose row was added, and adds nothing (a row added meanwhile is
+    // added twice at worst)
+    for (int w = warp; w < FW; w += nwarps) {
       uint32_t m = S[w];
-      while (m) {
-        int b = __ffs(m) - 1;
+      for (;;) {
+        m &= ~*(volatile uint32_t*)&R[w];
+        m = __shfl_sync(0xffffffffu, m, 0);
+        if (!m) break;
+        const int b = __ffs(m) - 1;
         m &= m - 1;
-        if ((seen++ % nwarps) != warp) continue;
         const uint32_t* r = rows + (size_t)((w << 5) + b) * FW;
-        for (int v = lane; v < FW; v += 32)
-          if (r[v]) atomicOr(&R[v], r[v]);
+        for (int v = lane; v < FW; v += 32) {
+          const uint32_t x = r[v];
+          if (x & ~*(volatile uint32_t*)&R[v]) atomicOr(&R[v], x);
+        }
+        __syncwarp();
       }
     }
     __syncthreads();
@@ -102,7 +107,7 @@ class CoverCols {
     __syncthreads();
     if (threadIdx.x == 0) {
       ws.col_off[c] = nz;
-      sh.ncols = c + 1;
+      walk_sh().ncols = c + 1;
     }
     __syncthreads();
   }

@@ -2,6 +2,8 @@
 #pragma once
 #include <cstdint>
 
+#include <vector_types.h>
+
 namespace epic {
 
 // One lex-table entry (Sec. 4.1 / Alg. 2 memoization restated as a table):
@@ -66,7 +68,14 @@ struct DevGrammar {
   const int32_t* nt_comp;
   const int32_t* ny_off;          // [V+1]
   const int32_t* ny;
-  int gs_par;                     // CTA walks: warp-parallel origin sweep (gscols.cuh)
+  // items by nonterminal as (word, mask) pairs (CSR over V): the complete
+  // items with that left side, and the items waiting on it
+  const int32_t* cpl_off;         // [V+1]
+  const uint2* cpl;               // [n_cpl]
+  const int32_t* wait_off;        // [V+1]
+  const uint2* wait;
+  int n_cpl, n_wait;
+  int any_nullable;               // some item's next symbol is a nullable nonterminal
 };
 
 // The greedy transducer of one token from lexer state q (Sec. 4.1): at state
@@ -160,8 +169,8 @@ __device__ inline LexEntry lex_at(const DevGrammar& g, const LexEntry* table, in
 
 // Per-CTA workspace of the Earley walk (global memory).
 struct Workspace {
-  uint32_t* stage;   // [nmax][W] dense rows of the column under construction (zero when idle)
-  uint32_t* bdone;   // [nmax][VW] nonterminals already completed per origin (current column)
+  uint32_t* stage;   // [nmax][W] rows of the open column without a shared-memory slot (zero when idle)
+  uint32_t* bdone;   // [nmax][VW] nonterminals already completed per origin (current column), the same
   int32_t* col_off;  // [nmax + 1] entry range of each finished column
   int32_t* org;      // [emax] origin column of each entry
   uint32_t* bits;    // [emax][W]

@@ -213,12 +213,12 @@ epic_status ensure_workspace(epic_lexer_table* t, int want_ctas, int n, cudaStre
 // total fits EPIC_WARP_WORKSPACE_MB (default a quarter of the GPU).
 epic_status ensure_wworkspace(epic_lexer_table* t, long long checks, int n, cudaStream_t st) {
   const epic_grammar* g = t->g;
-  int W = g->dg.W, VW = g->dg.VW;
+  int W = g->dg.W;
   int nmax = std::min(kWCols, 8 * n + 256);
   long long emax = 256ll * std::max(1, n);
   if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) emax = atoll(e);
   const size_t budget = workspace_budget("EPIC_WARP_WORKSPACE_MB", 0.25, t->d_wws ? t->wws_bytes : 0);
-  size_t per = wbytes_per_warp(nmax, emax, W, VW);
+  size_t per = wbytes_per_warp(nmax, emax, W);
   long long warps = std::min<long long>(checks, (long long)sm_count() * 2 * kWarpsPerCta);
   warps = std::max<long long>(kWarpsPerCta, (warps + kWarpsPerCta - 1) / kWarpsPerCta * kWarpsPerCta);
   while (warps > kWarpsPerCta && per * (size_t)warps > budget) warps -= kWarpsPerCta;
@@ -250,8 +250,7 @@ WPack wpack_of(const epic_lexer_table* t) {
   p.nmax = t->wnmax;
   p.emax = t->wemax;
   p.W = t->g->dg.W;
-  p.VW = t->g->dg.VW;
-  p.per_warp = wbytes_per_warp(p.nmax, p.emax, p.W, p.VW);
+  p.per_warp = wbytes_per_warp(p.nmax, p.emax, p.W);
   return p;
 }
 
@@ -296,33 +295,14 @@ epic_status region_prepare(const epic_grammar* g, epic_lexer_table* t, const int
   if (s != EPIC_OK) return s;
   sp.base = t->d_seq;
   t->last = st;
-  const size_t smem_cap = 190 * 1024;
-  const int rmax = 256;
-  bool sm = dg.W <= 32;
   // 1. forward charts
   {
-    int wpc = kWarpsPerCta;
-    size_t per = smem_per_warp(sp.nmax, rmax, dg.W, dg.VW);
-    if (sm) wpc = (int)std::min<size_t>(kWarpsPerCta, smem_cap / per);
-    // wide item sets: one CTA per sequence (Gauss-Seidel columns); narrow
-    // ones: one warp per sequence.  EPIC_FORWARD_CTA=0/1 overrides.
-    bool cta_walk = dg.W > 32;
-    if (const char* e = getenv("EPIC_FORWARD_CTA")) cta_walk = atoi(e) != 0;
     t->nk = 3;
-    t->kname[0] = cta_walk ? "k_forward_gs" : "k_forward";
+    t->kname[0] = "k_forward_gs";
     t->kname[1] = "k_good";
     t->kname[2] = "k_check";
     mark(t, 0, st);
-    if (cta_walk) {
-      launch_forward_gs(std::min(B, 4 * sm_count()), st, dg, t->d_table, t->vocab, d_x, B, n, sp, t->d_stats);
-    } else if (sm && wpc >= 1) {
-      size_t dyn = per * wpc;
-      launch_forward(true, (B + wpc - 1) / wpc, 32 * wpc, dyn, st, dg, t->d_table, t->vocab, d_x, B, n, sp, rmax,
-                     t->d_stats);
-    } else {
-      launch_forward(false, (B + kWarpsPerCta - 1) / kWarpsPerCta, 32 * kWarpsPerCta, 0, st, dg, t->d_table,
-                     t->vocab, d_x, B, n, sp, 0, t->d_stats);
-    }
+    launch_forward_gs(std::min(B, 4 * sm_count()), st, dg, t->d_table, t->vocab, d_x, B, n, sp, t->d_stats);
   }
   // 2. good masks
   mark(t, 1, st);
@@ -343,8 +323,7 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
   wp.emax = std::max(8192ll, 64ll * n);
   if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) wp.emax = atoll(e);
   wp.W = dg.W;
-  wp.VW = dg.VW;
-  wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, wp.W, wp.VW);
+  wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, wp.W);
   const size_t wbudget = workspace_budget("EPIC_WARP_WORKSPACE_MB", 0.25, t->d_wws ? t->wws_bytes : 0);
   long long warps = std::min<long long>(total, (long long)sm_count() * 2 * kWarpsPerCta);
   warps = std::max<long long>(1, warps);
@@ -370,9 +349,6 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
   epic_status s = grow(t, (char**)&t->d_regs, &t->regs_bytes, (size_t)warps * 3 * wp.nmax * 4);
   if (s != EPIC_OK) return s;
   t->last = st;
-  const size_t smem_cap = 190 * 1024;
-  const int rmax = 256;
-  bool sm = dg.W <= 32;
   // 1-2. forward charts and good masks
   SeqPack sp;
   s = region_prepare(g, t, d_x, B, n, sp, st);
@@ -381,20 +357,9 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
   t->n_vkernels += 3;
   // 3. checks
   cudaMemsetAsync(t->d_counter, 0, 8, st);
-  size_t per = smem_per_warp(wp.nmax, rmax, dg.W, dg.VW);
-  int wpc = sm ? (int)std::min<size_t>(kWarpsPerCta, smem_cap / per) : 0;
-  wpc = (int)std::min<long long>(wpc, warps);  // every launched warp owns an allocated workspace
-  if (wpc >= 1) {
-    int blocks = (int)std::max<long long>(1, warps / wpc);
-    size_t dyn = per * wpc;
-    launch_check_sm(blocks, 32 * wpc, dyn, st, dg, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand, K, total, d_valid,
-                    sp, wp, t->d_regs, rmax, t->d_counter, t->d_stats);
-  } else {
-    int per_cta = (int)std::min<long long>(kWarpsPerCta, warps);
-    int blocks = (int)std::max<long long>(1, warps / per_cta);
-    launch_check_global(blocks, 32 * per_cta, 0, st, dg, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand, K, total,
-                        d_valid, sp, wp, t->d_regs, 0, t->d_counter, t->d_stats);
-  }
+  const int per_cta = (int)std::min<long long>(kWarpsPerCta, warps);  // every warp owns an allocated workspace
+  launch_check((int)std::max<long long>(1, warps / per_cta), 32 * per_cta, st, dg, t->d_table, t->vocab, d_x, n, d_pos,
+               k, d_cand, K, total, d_valid, sp, wp, t->d_regs, t->d_counter, t->d_stats);
   mark(t, 3, st);
   return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
@@ -421,7 +386,7 @@ int epic_debug_phase_read(unsigned long long* out16, int reset) {
   if (cudaDeviceSynchronize() != cudaSuccess) return -1;
   for (int i = 0; i < 16; ++i) out16[i] = 0;
   if (phase_read_walk(out16, reset) != 0 || phase_read_forward(out16, reset) != 0 ||
-      phase_read_check_sm(out16, reset) != 0 || phase_read_check_global(out16, reset) != 0)
+      phase_read_check(out16, reset) != 0)
     return -1;
   for (int i = 0; i < 16; ++i) out16[16 + i] = 0;
   if (phase_read_good(out16 + 16, reset) != 0) return -1;
@@ -540,6 +505,36 @@ epic_status epic_grammar_create(const epic_grammar_desc* desc, epic_grammar** ou
       if (g->dfa.next[(size_t)q * 256 + c] >= 0) ext[q] = 1;
   up(ext, &d.dfa_ext);
   up(G.skip, &d.skip);
+  {
+    // complete / waiting items by nonterminal as (word, mask) pairs
+    auto lists = [&](auto member, std::vector<int32_t>& off, std::vector<uint2>& lst) {
+      std::vector<std::vector<uint2>> by((size_t)G.V);
+      for (int i = 0; i < G.D; ++i) {
+        const int A = member(i);
+        if (A < 0) continue;
+        auto& l = by[(size_t)A];
+        if (l.empty() || l.back().x != (uint32_t)(i >> 5)) l.push_back(uint2{(uint32_t)(i >> 5), 0u});
+        l.back().y |= 1u << (i & 31);
+      }
+      off.assign(1, 0);
+      for (auto& l : by) {
+        lst.insert(lst.end(), l.begin(), l.end());
+        off.push_back((int32_t)lst.size());
+      }
+    };
+    std::vector<int32_t> coff, woff;
+    std::vector<uint2> cl, wl;
+    lists([&](int i) { return G.item_next[i] < 0 && i != G.accept_item ? G.item_lhs[i] : -1; }, coff, cl);
+    lists([&](int i) { return G.item_next[i] >= G.T ? G.item_next[i] - G.T : -1; }, woff, wl);
+    d.n_cpl = (int)cl.size();
+    d.n_wait = (int)wl.size();
+    up(coff, &d.cpl_off);
+    up(cl, &d.cpl);
+    up(woff, &d.wait_off);
+    up(wl, &d.wait);
+    d.any_nullable = 0;
+    for (uint32_t m : G.nullable_next) d.any_nullable |= m != 0;
+  }
   {
     // runs of advanceable items for the doubling closure (see device.cuh)
     int maxlen = 0;
@@ -824,36 +819,15 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   if (s != EPIC_OK) return s;
   t->last = st;
   cudaMemsetAsync(t->d_counter, 0, 8, st);
-  // rows of the open column in shared memory (512 slots per warp, as many
-  // warps per CTA as fit) when the item set is narrow, else the global stage
-  WPack wp = wpack_of(t);
-  const size_t smem_cap = 190 * 1024;  // + 27 KB static per CTA <= 227 KB
-  const int rmax = 256;
-  size_t per = smem_per_warp(wp.nmax, rmax, wp.W, wp.VW);
-  const DevGrammar& dg = t->dgl;
-  size_t gt = gtab_bytes(dg.T, dg.V, dg.W, dg.D, dg.Q);
-  int gsm = (gt + 4 * per <= smem_cap) ? 1 : 0;  // tables in shared memory if 4 warps still fit
-  int wpc = (int)std::min<size_t>(kWarpsPerCta, (smem_cap - (gsm ? gt : 0)) / per);
-  if (const char* e = getenv("EPIC_GLOBAL_STAGE"))
-    if (atoi(e)) wpc = 0;
-  if (wp.W > 32) wpc = 0;
   // spread the walks over every SM: no more warps per CTA than walks per SM
-  int per_sm = (int)((t->wwarps + sm_count() - 1) / sm_count());
-  if (wpc > per_sm) wpc = std::max(2, per_sm);
+  const int per_sm = (t->wwarps + sm_count() - 1) / sm_count();
+  const int wpc = std::max(1, std::min(kWarpsPerCta, per_sm));
   t->n_vkernels += 1;
   t->nk = 1;
   t->kname[0] = "k_validate_warp";
   mark(t, 0, st);
-  if (wpc >= 2) {
-    size_t dyn = per * wpc + (gsm ? gt : 0);
-    int blocks = (t->wwarps + wpc - 1) / wpc;
-    if ((size_t)blocks * wpc > (size_t)t->wwarps) blocks = t->wwarps / wpc;
-    launch_validate_warp(true, blocks, 32 * wpc, dyn, st, t->dgl, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand, K,
-                         total, d_valid, wp, rmax, gsm, t->d_counter, t->d_stats);
-  } else {
-    launch_validate_warp(false, t->wwarps / kWarpsPerCta, 32 * kWarpsPerCta, 0, st, t->dgl, t->d_table, t->vocab, d_x,
-                         n, d_pos, k, d_cand, K, total, d_valid, wp, 0, 0, t->d_counter, t->d_stats);
-  }
+  launch_validate_warp(t->wwarps / wpc, 32 * wpc, st, t->dgl, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand, K, total,
+                       d_valid, wpack_of(t), 0, t->d_counter, t->d_stats);
   mark(t, 1, st);
   return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
@@ -921,7 +895,7 @@ epic_status epic_validate_batch_noalloc(const epic_grammar* g, const epic_lexer_
     }
     base = (char*)g_noalloc_ptr[dev];
   }
-  const int W = g->dg.W, VW = g->dg.VW;
+  const int W = g->dg.W;
   // Wide item sets walk the whole graph per check with rows in the global
   // stage, which takes seconds per check on long rows of large grammars; the
   // fixed array holds too few walks for that to finish in reasonable time,
@@ -932,36 +906,21 @@ epic_status epic_validate_batch_noalloc(const epic_grammar* g, const epic_lexer_
   wp.nmax = std::min(kWCols, 8 * n + 256);
   wp.emax = 256ll * n;
   wp.W = W;
-  wp.VW = VW;
-  wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, W, VW);
+  wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, W);
   long long fit = (long long)((kNoAllocBytes - 256) / wp.per_warp);
   if (fit < 1) return EPIC_ERR_CAPACITY;  // one walk's workspace does not fit the array
-  const size_t smem_cap = 190 * 1024;
-  const int rmax = 256;
-  size_t sper = smem_per_warp(wp.nmax, rmax, W, VW);
-  int wpc = (W > 32) ? 0 : (int)std::min<size_t>(kWarpsPerCta, smem_cap / sper);
   unsigned long long* counter = (unsigned long long*)base;
   // the kernel reads the table's lex entries and adds into its counters:
   // epic_get_stats and epic_lexer_table_destroy synchronize this stream
   t->last = st;
   if (cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st) != cudaSuccess) return EPIC_ERR_CUDA;
   t->n_vkernels += 1;
-  if (wpc >= 2) {
-    long long warps = std::min<long long>({total, fit, (long long)sm_count() * 2 * kWarpsPerCta});
-    int per_cta = (int)std::min<long long>(wpc, warps);
-    int blocks = (int)(warps / per_cta);
-    size_t dyn = sper * per_cta;
-    launch_validate_warp(true, blocks, 32 * per_cta, dyn, st, t->dgl, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand,
-                         K, total, d_valid, wp, rmax, 0, counter, t->d_stats);
-  } else {
-    // the global stage and its completed-NT sets must start at zero
-    long long warps = std::min<long long>({total, fit, (long long)sm_count() * 2 * kWarpsPerCta});
-    int per_cta = (int)std::min<long long>(kWarpsPerCta, warps);
-    int blocks = (int)(warps / per_cta);
-    if (cudaMemsetAsync(wp.base, 0, wp.per_warp * (size_t)blocks * per_cta, st) != cudaSuccess) return EPIC_ERR_CUDA;
-    launch_validate_warp(false, blocks, 32 * per_cta, 0, st, t->dgl, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand,
-                         K, total, d_valid, wp, 0, 0, counter, t->d_stats);
-  }
+  const long long warps = std::min<long long>({total, fit, (long long)sm_count() * 2 * kWarpsPerCta});
+  // as many warps per CTA as walks per SM
+  const int per_cta = (int)std::max<long long>(
+      1, std::min<long long>(kWarpsPerCta, (warps + sm_count() - 1) / sm_count()));
+  launch_validate_warp((int)(warps / per_cta), 32 * per_cta, st, t->dgl, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand, K,
+                       total, d_valid, wp, 1, counter, t->d_stats);
   return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
 

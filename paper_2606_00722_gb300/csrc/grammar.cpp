@@ -369,7 +369,7 @@ GrammarTables build_tables(int T, const std::vector<uint8_t>& skip, int V, int s
     D += G.rhs_off[p + 1] - G.rhs_off[p] + 1;
   }
   G.D = D;
-  G.W = (D + 31) / 32;
+  G.W = ((D + 31) / 32 + 3) / 4 * 4;  // whole 16-byte pieces
   int W = G.W;
   G.item_next.assign(D, -1);
   G.item_lhs.assign(D, -1);

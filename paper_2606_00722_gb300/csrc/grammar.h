@@ -36,7 +36,7 @@ struct GrammarTables {
   std::vector<int32_t> rhs_off, rhs;    // CSR
   int aug = -1;
   // dotted items: item(p, d) = item_base[p] + d, d in 0..|rhs_p|
-  int D = 0, W = 0;                     // items and 32-bit words per item bitset
+  int D = 0, W = 0;                     // items and 32-bit words per item bitset (a multiple of 4)
   std::vector<int32_t> item_base;       // [P']
   std::vector<int32_t> item_next;       // [D] symbol after the dot, -1 if complete
   std::vector<int32_t> item_lhs;        // [D] lhs of the item's production (-1 for S')

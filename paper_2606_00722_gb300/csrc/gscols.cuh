@@ -1,72 +1,68 @@
-// Earley columns for wide grammars: one CTA closes each column with a
-// Gauss-Seidel sweep over its origins (Alg. 3's completion, highest origin
-// first), the whole CTA scattering each origin's completions.
+// Earley columns of the CTA walks: one CTA closes each column of a chart, its
+// warps working through the column's origins on their own (Alg. 3's
+// completion).
 //
-// Why a descending sweep visits every origin once: completing nonterminal A
-// from origin o at column c advances the items of column o that wait on A;
-// those items have origins o2 <= o.  So a row with origin o only receives
-// from origins >= o, and once every higher origin is closed, row o's only
-// remaining source is the entry of column o with origin o itself (the items
-// predicted at o).  That self-loop is closed on its own (one warp, row in
-// registers) before the completions are scattered, once, over the other
-// entries of column o by every warp (entries of one column have distinct
-// origins, so no two warps write one row).  Predictions at c only feed row c
-// (items predicted at c have origin c), and completions from c at c are the
-// nullable / gap advances of every row (Aycock & Horspool; inside a gap
-// every symbol derives some terminal string of the trimmed grammar), so
-// predictions are made once the lower origins are closed.
+// Completing nonterminal A from origin o at column c advances the items of
+// column o that wait on A; those items have origins o2 <= o, so a row with
+// origin o only receives from origins >= o.  The sweep therefore runs from
+// the highest origin down, asynchronously: each warp repeatedly claims the
+// highest dirty origin below c (clearing its bit), closes its row together
+// with the self-loop through the entry of column o with origin o (the items
+// predicted at o) in registers, and scatters the nonterminals that no earlier
+// visit completed over the other entries of column o with atomic ORs, marking
+// the rows it changes dirty again.  A row may be claimed while another warp
+// still writes into it; the writer sets the dirty bit after its writes
+// (fenced), so the row is visited again and nothing is lost.  The sweep ends
+// when no bit is dirty and no warp holds an origin.  The rules are monotone,
+// so the result is the least fixpoint whatever the order.
 //
-// Same graph, chart layout, recording and results as EarleyColsT
-// (walk.cuh); only the order of the closure differs (the least fixpoint is
-// the same).
+// What bounds it: the chain of dependent visits, each a few dependent
+// shared-memory steps long, and the loads of column o's entries.  Hence
+//  - the rows of the open column, their completed-nonterminal sets, the column
+//    offsets and the span step's tables live in shared memory (an origin gets
+//    a row slot on first touch; a column with more origins than slots puts the
+//    rest in the global stage).  A visit makes no global store, and its fences
+//    wait for shared memory only;
+//  - completed nonterminals are read off a row by one lane per nonterminal
+//    testing its (word, mask) pairs, 32 nonterminals per ballot, and the items
+//    waiting on new nonterminals are OR-ed from EXP_NT rows: no per-item loops
+//    and no shared-memory atomics;
+//  - a row takes LR lanes of KW consecutive words (rows are padded to a
+//    multiple of four words, so a lane moves 16 bytes at a time and a shift by
+//    one item costs one shuffle): 4 lanes x 4 words up to 16 words, 16 x 4 up
+//    to 64, 32 x 8 up to 256.  A warp scatters 32 / LR entries per step, and
+//    when it works on one row its lane groups hold copies and share out the
+//    EXP_NT rows.  (Instruction issue, at 36 % of the active cycles with one
+//    word per lane and 32-word steps, was the bound: clike-512 spent about 70
+//    instructions per scattered entry.)
+// Predictions at c only feed row c (items predicted at c have origin c), and
+// the prediction closures are closed under further predictions, so they are
+// made once, after the lower origins are closed; completions from c at c are
+// the nullable / gap advances of every row (Aycock & Horspool; inside a gap
+// every symbol derives some terminal string of the trimmed grammar).
 #pragma once
+#include "rows.cuh"
 #include "walk.cuh"
 #include "warpwalk.cuh"  // phase timers
 
 namespace epic {
 
 constexpr int kGsMaxWarps = 16;
-constexpr long long kGsMaxSteps = 1ll << 22;  // origin visits per column
-constexpr long long kGsMaxIdle = 1ll << 24;   // polls of an idle warp per column (warp-parallel sweep)
-
-// Per-warp scratch of the warp-parallel sweep (dynamic shared memory):
-// nonterminal words, then the warp's completion mask.
-constexpr int kGsWarpScratch = kMaxVW + kMaxW;
-__host__ __device__ inline size_t gs_warp_scratch_bytes() { return (size_t)kGsMaxWarps * kGsWarpScratch * 4; }
-
-// The origin sweep of the CTA walks: warp-parallel for item sets of at most
-// 64 words, whose columns are short enough for one warp to scatter (on
-// clike-512, W = 64: forward charts 22 % faster), the descending block sweep
-// for wider ones (random-stress-1024, W = 213: the warp-parallel sweep took
-// 20-45 % longer, one warp scattering columns of hundreds of entries);
-// EPIC_GS_PARALLEL=0/1 overrides.
-inline int gs_parallel_enabled(int W) {
-  const char* e = getenv("EPIC_GS_PARALLEL");
-  return e ? (atoi(e) != 0) : (W <= 64 ? 1 : 0);
-}
-
-// Shared memory of the Gauss-Seidel columns (beside WalkShared).
-struct GsShared {
-  uint32_t expn[kMaxW];               // items waiting on the current origin's completions
-  uint32_t nnew[kMaxVW];              // nonterminals newly completed from the current origin
-  uint32_t nstep[kMaxVW];             // of one self-closure round
-  uint32_t vset[kMaxVW];              // nonterminals waited on in this column
-  uint32_t vdone[kMaxVW];             // ... already predicted
-  uint32_t uni[kMaxW];                // union of the column's rows (waited nonterminals)
-  int32_t cur_o;
-  int32_t flag;
-  int32_t labelled;  // the open column has a labelled arrival (else only epsilon ones)
-  int32_t busy;      // warp-parallel sweep: warps holding an origin
-};
+// Threads of a CTA walk: eight warps for narrow rows, so that two CTAs share
+// an SM with 128 registers a thread, four for tiny grammars, whose columns hold
+// too few origins for more.
+inline int gs_threads(int W) { return W <= 4 ? 128 : (W <= 16 ? 256 : 32 * kGsMaxWarps); }
+template <class S>
+constexpr int kGsThreads = S::LR == 4 ? 256 : 32 * kGsMaxWarps;
+constexpr long long kGsMaxSteps = 1ll << 22;  // origin visits per column and warp
+constexpr long long kGsMaxIdle = 1ll << 24;   // polls of an idle warp per column
 
 // Grammar tables read by the per-item loops, staged in shared memory:
-// item -> next symbol / lhs (int16 [D]) and the W-word masks.
+// item -> next symbol (int16 [D]) and the W-word masks.
 struct GsTables {
   const int16_t* item_next;
-  const int16_t* item_lhs;
   const uint32_t* complete;
   const uint32_t* any_nt;
-  const uint32_t* any_term;
   const uint32_t* next_any;
   const uint32_t* nullable_next;
   const uint32_t* adv_pow;  // [2][steps][W] (DevGrammar::adv_pow)
@@ -74,7 +70,7 @@ struct GsTables {
 
 __host__ __device__ inline size_t gs_tables_bytes(int D, int W, int steps) {
   auto r = [](size_t b) { return (b + 15) & ~(size_t)15; };
-  return 2 * r((size_t)D * 2) + 5 * r((size_t)W * 4) + r((size_t)2 * steps * W * 4);
+  return r((size_t)D * 2) + 4 * r((size_t)W * 4) + r((size_t)2 * steps * W * 4);
 }
 
 // Block: copy the tables into smem (gs_tables_bytes) and point t at them.
@@ -89,425 +85,361 @@ __device__ inline void gs_stage_tables(const DevGrammar& g, unsigned char* smem,
     return dst;
   };
   t.item_next = (const int16_t*)put(g.item_next, (size_t)g.D * 2);
-  t.item_lhs = (const int16_t*)put(g.item_lhs, (size_t)g.D * 2);
   t.complete = (const uint32_t*)put(g.complete, (size_t)g.W * 4);
   t.any_nt = (const uint32_t*)put(g.any_nt, (size_t)g.W * 4);
-  t.any_term = (const uint32_t*)put(g.any_term, (size_t)g.W * 4);
   t.next_any = (const uint32_t*)put(g.next_any, (size_t)g.W * 4);
   t.nullable_next = (const uint32_t*)put(g.nullable_next, (size_t)g.W * 4);
   t.adv_pow = (const uint32_t*)put(g.adv_pow, (size_t)2 * g.adv_steps * g.W * 4);
   __syncthreads();
 }
 
-template <bool REC>
+// Dynamic shared memory of the CTA walks (byte offsets): WalkSmem, the tables
+// above, then the pieces below; `rows` row slots take what is left.
+struct GsPlan {
+  uint32_t o_off, o_list;  // complete items by nonterminal (CSR over V)
+  uint32_t o_scr;          // per-warp scratch, W words each
+  uint32_t o_col;          // column offsets [nmax + 1]
+  uint32_t o_slot;         // row slot of each origin [nmax] (uint16)
+  uint32_t o_self;         // bit o: column o has an entry with origin o
+  uint32_t o_exp;          // EXP_NT rows; 0: read from global memory
+  uint32_t o_walk;         // span step tables; 0: in the global workspace
+  uint32_t o_zero;         // a row of zeros, for origins without a slot
+  uint32_t o_rows, o_done; // row slots, completed nonterminals per slot
+  int rows;
+  uint32_t bytes;
+};
+
+constexpr uint32_t kSlotNone = 0xFFFFu, kSlotGlobal = 0xFFFEu;
+constexpr size_t kGsWalkBytesPerState = 7 * 4 + 16 + 32 + 16;  // WalkScratch per lexer state
+
+// limit: dynamic shared memory a CTA may take.  Narrow rows keep to what lets
+// two CTAs share an SM.
+inline GsPlan gs_plan(const DevGrammar& g, int nmax, size_t limit) {
+  auto r = [](size_t b) { return (b + 15) & ~(size_t)15; };
+  GsPlan p;
+  size_t o = kWalkSmemBytes + r(gs_tables_bytes(g.D, g.W, g.adv_steps));
+  auto put = [&](size_t bytes) {
+    const size_t at = o;
+    o += r(bytes);
+    return (uint32_t)at;
+  };
+  p.o_off = put((size_t)(g.V + 1) * 4);
+  p.o_list = put((size_t)g.n_cpl * 8);
+  p.o_scr = put((size_t)kGsMaxWarps * g.W * 4);
+  p.o_col = put((size_t)(nmax + 1) * 4);
+  p.o_slot = put((size_t)nmax * 2);
+  p.o_self = put((size_t)((nmax + 31) / 32) * 4);
+  p.o_zero = put((size_t)g.W * 4);
+  const size_t per_row = (size_t)(g.W + g.VW) * 4;
+  const size_t least = 64 * per_row;  // rows that always come first
+  const size_t walk = (size_t)g.Q * kGsWalkBytesPerState, ex = (size_t)g.V * g.W * 4;
+  p.o_walk = o + r(walk) + least <= limit ? put(walk) : 0;
+  p.o_exp = o + r(ex) + 2 * least <= limit ? put(ex) : 0;
+  const size_t left = limit > o + 32 ? limit - o - 32 : 0;
+  long long rows = (long long)(left / per_row);
+  rows = rows > nmax ? nmax : rows;
+  rows = rows > 1024 ? 1024 : rows;
+  p.rows = (int)rows;
+  p.o_rows = put((size_t)rows * g.W * 4);
+  p.o_done = put((size_t)rows * g.VW * 4);
+  p.bytes = (uint32_t)o;
+  return p;
+}
+// 227 KB per CTA less the static shared memory of the walk kernels (at most
+// 10 KB); half of an SM's 228 KB for the narrow rows
+inline size_t gs_limit(int W) { return W <= 16 ? (size_t)102 * 1024 : (size_t)216 * 1024; }
+
+// The steps of one column are calls (not inlined at each of the walk's many
+// uses): inlined, the selection kernels took six minutes to compile.
+template <bool REC, class S>
 class EarleyColsGS {
  public:
-  static constexpr int KW = kMaxW / 32;  // item words per lane
+  static constexpr int KW = S::KW, LR = S::LR, NG = S::NG;
+  using Row = RowRegs<S>;
+  static constexpr bool kRecord = REC;
   const DevGrammar& g;
   const GsTables& tb;
-  const LexEntry* table;
-  Workspace ws;
-  WalkScratch sc;
+  const GsPlan& plan;
+  Workspace ws;  // col_off is the shared-memory copy
   WsDims dims;
-  WalkShared& sh;
-  GsShared& gs;
-  int W, VW;
-  static constexpr bool kRecord = REC;
+  int W, VW, R;
   const BlockRec* rec = nullptr;
-  uint32_t* wnt = nullptr;  // recording walks: per-warp nonterminal sets [warps][kMaxVW] (shared memory)
-  // Warp-parallel sweep (set both): every warp claims dirty origins on its
-  // own and scatters their completions alone; ws.bdone keeps, per origin of
-  // the open column, the nonterminals whose completions were scattered.
-  bool par = false;
-  uint32_t* wscr = nullptr;  // [warps][kGsWarpScratch] (shared memory)
+  uint32_t *rows, *done, *selfb;
+  uint16_t* slot_of;
 
-  __device__ EarleyColsGS(const DevGrammar& g_, const GsTables& t_, const LexEntry* t, Workspace w, WalkScratch s,
-                          WsDims d, WalkShared& shared, GsShared& gss)
-      : g(g_), tb(t_), table(t), ws(w), sc(s), dims(d), sh(shared), gs(gss), W(g_.W), VW(g_.VW) {}
-
-  __device__ int nwarps() const { return blockDim.x >> 5; }
-  __device__ bool column_has_accept(int c, int start_col) { return accepts(c, start_col); }
-  __device__ void seed(int c) { arrive_item(c, g.start_item); }
-  __device__ void arrive_labels(int src, bool eps) { arrive(src, eps ? nullptr : sh.lbl, !eps); }
-
-  __device__ void reset() {
-    if (threadIdx.x == 0) {
-      sh.ncols = 0;
-      sh.nent = 0;
-      sh.status = kWalkOk;
-      sh.nedges = 0;
-      ws.col_off[0] = 0;
+  // What the visits and scatters of a column read at every step, copied to
+  // registers once per call: the object itself lies in local memory, and its
+  // members would be read again after every barrier and atomic.
+  struct Hot {
+    int W, VW, V, R, steps, nullable;
+    uint32_t s_rows, s_zero;      // shared addresses: row slots, the zero row
+    const uint32_t *adv, *complete, *selfb, *exp_nt;
+    uint32_t *scr, *rows, *done, *stage, *bdone;
+    uint16_t* slot_of;
+    const int32_t *c_off, *col, *org;
+    const uint2* c_lst;
+    const uint32_t* bits;
+    __device__ __forceinline__ uint32_t slot(int o) const { return *(const volatile uint16_t*)(slot_of + o); }
+    __device__ __forceinline__ uint32_t* done_of(uint32_t s, int o) const {
+      return s < (uint32_t)R ? done + (size_t)s * VW : bdone + (size_t)o * VW;
     }
-    clear_bitmap(sh.touched, kMaxCols);
-    clear_bitmap(sh.dirty, kMaxCols);
-    for (int v = threadIdx.x; v < kMaxVW; v += blockDim.x) {
-      gs.vset[v] = 0;
-      gs.vdone[v] = 0;
+  };
+  __device__ __forceinline__ Hot hot() const {
+    unsigned char* m = gs_smem();
+    Hot h;
+    h.W = W;
+    h.VW = VW;
+    h.V = g.V;
+    h.R = R;
+    h.steps = g.adv_steps;
+    h.nullable = g.any_nullable;
+    h.s_rows = gs_saddr(m + plan.o_rows);
+    h.s_zero = gs_saddr(m + plan.o_zero);
+    h.adv = tb.adv_pow;
+    h.complete = tb.complete;
+    h.selfb = (const uint32_t*)(m + plan.o_self);
+    h.exp_nt = plan.o_exp ? (const uint32_t*)(m + plan.o_exp) : g.exp_nt;
+    h.scr = (uint32_t*)(m + plan.o_scr) + (size_t)(threadIdx.x >> 5) * W;
+    h.rows = (uint32_t*)(m + plan.o_rows);
+    h.done = (uint32_t*)(m + plan.o_done);
+    h.stage = ws.stage;
+    h.bdone = ws.bdone;
+    h.slot_of = (uint16_t*)(m + plan.o_slot);
+    h.c_off = (const int32_t*)(m + plan.o_off);
+    h.c_lst = (const uint2*)(m + plan.o_list);
+    h.col = (const int32_t*)(m + plan.o_col);
+    h.org = ws.org;
+    h.bits = ws.bits;
+    return h;
+  }
+
+  __device__ EarleyColsGS(const DevGrammar& g_, const GsTables& t_, const GsPlan& p, unsigned char* smem, Workspace w,
+                          WsDims d)
+      : g(g_), tb(t_), plan(p), ws(w), dims(d), W(g_.W), VW(g_.VW), R(p.rows) {
+    ws.col_off = (int32_t*)(smem + p.o_col);
+    slot_of = (uint16_t*)(smem + p.o_slot);
+    selfb = (uint32_t*)(smem + p.o_self);
+    rows = (uint32_t*)(smem + p.o_rows);
+    done = (uint32_t*)(smem + p.o_done);
+  }
+
+  // The walk's span tables in shared memory when they fit.
+  __device__ static void place_scratch(const DevGrammar& g, const GsPlan& p, unsigned char* smem, WalkScratch& sc) {
+    if (!p.o_walk) return;
+    unsigned char* q = smem + p.o_walk;
+    const size_t Q = (size_t)g.Q;
+    sc.ent = (LexEntry*)q;
+    q += Q * 16;
+    sc.g_tail = (uint8_t*)q;
+    q += Q * 16;
+    sc.g_lbl = (uint32_t*)q;
+    q += Q * 32;
+    int32_t** a[7] = {&sc.g_src, &sc.g_end, &sc.g_len, &sc.g_last, &sc.f_q, &sc.f_c, &sc.key_q};
+    for (int i = 0; i < 7; ++i, q += Q * 4) *a[i] = (int32_t*)q;
+  }
+
+  // Block, once per kernel: the shared tables, empty slots, zero rows.
+  __device__ void init(unsigned char* smem) {
+    int32_t* off = (int32_t*)(smem + plan.o_off);
+    for (int v = threadIdx.x; v <= g.V; v += blockDim.x) off[v] = g.cpl_off[v];
+    uint2* lst = (uint2*)(smem + plan.o_list);
+    for (int i = threadIdx.x; i < g.n_cpl; i += blockDim.x) lst[i] = g.cpl[i];
+    if (plan.o_exp) {
+      uint32_t* ex = (uint32_t*)(smem + plan.o_exp);
+      for (int i = threadIdx.x; i < g.V * W; i += blockDim.x) ex[i] = g.exp_nt[i];
     }
-    if (threadIdx.x == 0) gs.labelled = 0;
+    for (int i = threadIdx.x; i < W; i += blockDim.x) ((uint32_t*)(smem + plan.o_zero))[i] = 0;
+    for (int i = threadIdx.x; i < R * W; i += blockDim.x) rows[i] = 0;
+    for (int i = threadIdx.x; i < R * VW; i += blockDim.x) done[i] = 0;
+    for (int i = threadIdx.x; i < dims.nmax; i += blockDim.x) slot_of[i] = (uint16_t)kSlotNone;
     __syncthreads();
   }
 
-  __device__ int ncols() const { return sh.ncols; }
+  __device__ int nwarps() const { return blockDim.x >> 5; }
+  __device__ bool column_has_accept(int c, int start_col) { return accepts(c, start_col); }
+  __device__ void arrive_labels(int src, bool eps) { arrive(src, !eps); }
+
+  __device__ void reset() {
+    if (threadIdx.x == 0) {
+      walk_sh().ncols = 0;
+      walk_sh().nent = 0;
+      walk_sh().status = kWalkOk;
+      walk_sh().nedges = 0;
+      ws.col_off[0] = 0;
+      walk_gs().labelled = 0;
+      walk_gs().nslots = 0;
+    }
+    clear_bitmap(walk_sh().touched, kMaxCols);
+    clear_bitmap(walk_sh().dirty, kMaxCols);
+    clear_bitmap(selfb, dims.nmax);
+    __syncthreads();
+  }
+
+  __device__ int ncols() const { return walk_sh().ncols; }
   __device__ int open_column() {
-    int c = sh.ncols;
+    int c = walk_sh().ncols;
     if (c >= dims.nmax || c >= kMaxCols) {
-      if (threadIdx.x == 0) sh.status = kWalkOverflow;
+      if (threadIdx.x == 0) walk_sh().status = kWalkOverflow;
       return -1;
     }
     return c;
   }
 
+  // ------------------------------------------------------------ row slots
+  __device__ __forceinline__ static uint32_t vld(const uint32_t* p) { return *(const volatile uint32_t*)p; }
+  __device__ __forceinline__ uint32_t slot(int o) const { return *(const volatile uint16_t*)(slot_of + o); }
+  __device__ __forceinline__ uint32_t* row_of(uint32_t s, int o) const {
+    return s < (uint32_t)R ? rows + (size_t)s * W : ws.stage + (size_t)o * W;
+  }
+  __device__ __forceinline__ uint32_t* done_of(uint32_t s, int o) const {
+    return s < (uint32_t)R ? done + (size_t)s * VW : ws.bdone + (size_t)o * VW;
+  }
+  // One thread: the slot of origin o, claimed on its first touch.  A claim
+  // that loses the race leaves its slot unused (zero) in this column.
+  __device__ __forceinline__ uint32_t claim(int o) { return claim(slot_of, R, o); }
+  __device__ static uint32_t claim(uint16_t* slot_of, int R, int o) {
+    uint32_t s = *(const volatile uint16_t*)(slot_of + o);
+    if (s != kSlotNone) return s;
+    const int t = atomicAdd(&walk_gs().nslots, 1);
+    const uint32_t want = t < R ? (uint32_t)t : kSlotGlobal;
+    const unsigned short old =
+        atomicCAS((unsigned short*)(slot_of + o), (unsigned short)kSlotNone, (unsigned short)want);
+    return old == (unsigned short)kSlotNone ? want : (uint32_t)old;
+  }
+  __device__ static __forceinline__ void mark(int o) {
+    atomicOr(&walk_sh().touched[o >> 5], 1u << (o & 31));
+    atomicOr(&walk_sh().dirty[o >> 5], 1u << (o & 31));
+  }
+
   // ------------------------------------------------------------ row kernels
-  // Warp: dst |= shift(src & M) (or src & M, or src when M is null), lanes over
-  // words; returns whether dst changed.  dst is owned by this warp.
-  __device__ bool warp_or_into(uint32_t* dst, const uint32_t* src, const uint32_t* M, bool shift) {
-    const int lane = threadIdx.x & 31;
-    uint32_t v[KW];
-#pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      v[i] = (w < W) ? (M ? (src[w] & M[w]) : src[w]) : 0u;
-    }
-    bool ch = false;
-    uint32_t carry = 0;
-#pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      if (32 * i >= W) break;
-      const int w = lane + 32 * i;
-      uint32_t add = v[i];
-      if (shift) {
-        uint32_t prev = __shfl_up_sync(0xffffffffu, v[i], 1);
-        if (lane == 0) prev = carry;
-        carry = __shfl_sync(0xffffffffu, v[i], 31);
-        add = (v[i] << 1) | (prev >> 31);
-      }
-      if (w < W && add) {
-        const uint32_t old = dst[w];
-        if ((old | add) != old) {
-          dst[w] = old | add;
-          ch = true;
-        }
-      }
-    }
-    return __any_sync(0xffffffffu, ch);
-  }
-
-  // Warp, row in registers (lane l holds words l, l+32, ...): the closure of r
-  // under item i -> i + 1 for i in the advance mask (mode 0: nullable_next,
-  // 1: next_any), by doubling: step s adds i + 2^s for every i in r that
-  // starts a run of 2^s advanceable items; steps in increasing order reach
-  // every i + d with d < 2^steps, which covers the longest production.
-  __device__ void reg_advance(uint32_t (&r)[KW], int mode) {
-    const int lane = threadIdx.x & 31;
-    for (int st = 0; st < g.adv_steps; ++st) {
-      const uint32_t* M = tb.adv_pow + ((size_t)mode * g.adv_steps + st) * W;
-      const int k = 1 << st;
-      if (k < 32) {
-        uint32_t carry = 0;
-#pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          if (32 * i >= W) break;
-          const int w = lane + 32 * i;
-          const uint32_t v = (w < W) ? (r[i] & M[w]) : 0u;
-          uint32_t prev = __shfl_up_sync(0xffffffffu, v, 1);
-          if (lane == 0) prev = carry;
-          carry = __shfl_sync(0xffffffffu, v, 31);
-          r[i] |= (v << k) | (prev >> (32 - k));
-        }
-      } else {  // whole words: word w takes word w - k/32 (never above 64: rhs <= 62)
-        const int dw = k >> 5;
-        uint32_t v[KW];
-#pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          const int w = lane + 32 * i;
-          v[i] = (w < W) ? (r[i] & M[w]) : 0u;
-        }
-#pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          if (32 * i >= W) break;
-          // source word lane + 32 i - dw, dw in {1, 2}
-          const int sl = (lane - dw) & 31;
-          const uint32_t same = __shfl_sync(0xffffffffu, v[i], sl);
-          const uint32_t prevw = (i > 0) ? __shfl_sync(0xffffffffu, v[i > 0 ? i - 1 : 0], sl) : 0u;
-          r[i] |= (lane >= dw) ? same : prevw;
-        }
-      }
-    }
-  }
-
-  // Arrivals: for every entry (o, y) of column src, stage[o] |= shift(y & M).
-  __device__ void arrive(int src, const uint32_t* M, bool shift) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = nwarps();
-    if (shift && threadIdx.x == 0) gs.labelled = 1;
-    if (REC && threadIdx.x == 0) {
-      if (sh.nedges >= rec->edge_cap) {
-        sh.status = kWalkOverflow;
-      } else {
-        const int e = sh.nedges++;
-        rec->e_dst[e] = sh.ncols;
-        rec->e_src[e] = src;
-        for (int w = 0; w < 8; ++w) rec->e_lbl[(size_t)e * 8 + w] = shift ? sh.lbl8[w] : 0u;
-      }
-    }
-    const int b = ws.col_off[src], e = ws.col_off[src + 1];
-    for (int k = b + warp; k < e; k += nw) {
-      const int o = ws.org[k];
-      const bool ch = warp_or_into(ws.stage + (size_t)o * W, ws.bits + (size_t)k * W, M, shift);
-      if (ch && lane == 0) {
-        atomicOr(&sh.touched[o >> 5], 1u << (o & 31));
-        atomicOr(&sh.dirty[o >> 5], 1u << (o & 31));
-      }
-    }
-    __syncthreads();
-  }
-
-  __device__ void arrive_item(int origin, int item) {
-    if (threadIdx.x == 0) {
-      ws.stage[(size_t)origin * W + (item >> 5)] |= 1u << (item & 31);
-      sh.touched[origin >> 5] |= 1u << (origin & 31);
-      sh.dirty[origin >> 5] |= 1u << (origin & 31);
-    }
-    __syncthreads();
-  }
-
-  // Warp: highest set bit of bm at or below `top`, or -1.
-  __device__ static int warp_highest_at_or_below(const uint32_t* bm, int top) {
-    const int lane = threadIdx.x & 31;
-    if (top < 0) return -1;
-    for (int wtop = top >> 5; wtop >= 0; wtop -= 32) {
-      const int w = wtop - lane;
-      uint32_t v = (w >= 0) ? bm[w] : 0u;
-      if (w == (top >> 5)) v &= (top & 31) == 31 ? 0xffffffffu : ((2u << (top & 31)) - 1u);
-      const unsigned any = __ballot_sync(0xffffffffu, v != 0);
-      if (any) {
-        const int l = __ffs(any) - 1;
-        const uint32_t vv = __shfl_sync(0xffffffffu, v, l);
-        return ((wtop - l) << 5) + (31 - __clz(vv));
-      }
-    }
-    return -1;
-  }
-
-  // Warp 0: close origin o's row on its own (the self-loop through the entry
-  // of column o with origin o); leaves the nonterminals newly completed from
-  // o in gs.nnew.  Returns whether there are any.
-  __device__ bool close_origin(int o, int mode) {
-    const int lane = threadIdx.x & 31;
-#ifdef EPIC_PHASE_TIMERS
-    if (lane == 0) atomicAdd(&g_phase[15], 1ull);
-#endif
-    uint32_t* row = ws.stage + (size_t)o * W;
-    uint32_t r[KW], e[KW];
-#pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      r[i] = (w < W) ? row[w] : 0u;
-      e[i] = 0u;
-    }
-    const int kb = ws.col_off[o], ke = ws.col_off[o + 1];
-    const bool self = ke > kb && ws.org[ke - 1] == o;  // entries are stored by ascending origin
-    if (self) {
-      const uint32_t* E = ws.bits + (size_t)(ke - 1) * W;
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        e[i] = (w < W) ? (E[w] & tb.any_nt[w]) : 0u;
-      }
-    }
-    uint32_t done = 0, tot = 0;  // lane v < VW: word v of the completed / new sets
-    uint32_t cseen[KW];          // complete items already counted
-#pragma unroll
-    for (int i = 0; i < KW; ++i) cseen[i] = 0u;
-    for (int round = 0; round < 64 * kMaxW; ++round) {
-#ifdef EPIC_PHASE_TIMERS
-      if (lane == 0) atomicAdd(&g_phase[14], 1ull);
-#endif
-      reg_advance(r, mode);
-      if (lane < VW) gs.nstep[lane] = 0;
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        uint32_t m = (w < W) ? (r[i] & tb.complete[w] & ~cseen[i]) : 0u;
-        cseen[i] |= m;
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1;
-          const int A = tb.item_lhs[(w << 5) + b];
-          atomicOr(&gs.nstep[A >> 5], 1u << (A & 31));
-        }
-      }
-      __syncwarp();
-      const uint32_t nw = (lane < VW) ? (gs.nstep[lane] & ~done) : 0u;
-      done |= nw;
-      tot |= nw;
-      if (!__any_sync(0xffffffffu, nw != 0) || !self) break;
-      if (lane < VW) gs.nstep[lane] = nw;
-      __syncwarp();
-      // the self entry's items waiting on a new nonterminal advance into r
-      bool ch = false;
-      uint32_t carry = 0;
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        if (32 * i >= W) break;
-        const int w = lane + 32 * i;
-        uint32_t x = 0, m = e[i];
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1;
-          const int B = tb.item_next[(w << 5) + b] - g.T;
-          if ((gs.nstep[B >> 5] >> (B & 31)) & 1u) x |= 1u << b;
-        }
-        uint32_t prev = __shfl_up_sync(0xffffffffu, x, 1);
-        if (lane == 0) prev = carry;
-        carry = __shfl_sync(0xffffffffu, x, 31);
-        const uint32_t add = ((x << 1) | (prev >> 31)) & ~r[i];
-        ch |= add != 0;
-        r[i] |= add;
-      }
-      __syncwarp();
-      if (!__any_sync(0xffffffffu, ch)) break;
-    }
-#pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      if (w < W) row[w] = r[i];
-    }
-    if (lane < VW) gs.nnew[lane] = tot;
-    __syncwarp();
-    return __any_sync(0xffffffffu, tot != 0);
-  }
-
-  // Block: gs.expn = items waiting on a member of gs.nnew (item test per word).
-  __device__ void build_expn() {
-    for (int w = threadIdx.x; w < W; w += blockDim.x) {
-      uint32_t acc = 0, m = tb.any_nt[w];
-      while (m) {
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        const int B = tb.item_next[(w << 5) + b] - g.T;
-        if ((gs.nnew[B >> 5] >> (B & 31)) & 1u) acc |= 1u << b;
-      }
-      gs.expn[w] = acc;
-    }
-  }
-
-  // Block: completions from origin o into the rows of the other entries of
-  // column o: stage[org] |= shift(bits & gs.expn).  One thread per (entry,
-  // word), consecutive threads on consecutive words (coalesced), four words
-  // in flight per thread; entries of one column have distinct origins, so
-  // every stage word has one writer.  Changed entries are flagged in
-  // gs.chg, then their origins marked touched and dirty.
-  __device__ void scatter_column(int o) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = nwarps();
-    const int kb = ws.col_off[o], ke = ws.col_off[o + 1];
+  // Warp: row(origin) |= bits & m, shifted to the next item when SHIFT, for
+  // entries of kb .. ke - 1; marks the origins whose rows change.  Entries go
+  // NG at a time, steps first, first + stride, ...; m: the mask words of this
+  // lane.  Origins and row addresses of 32 entries are looked up at once; the
+  // common case (the row already holds the items) is loads, a shuffle and a
+  // vote.
+  template <bool SHIFT>
+  __device__ static __forceinline__ void scatter(const Hot& h, int kb, int ke, const uint32_t (&m)[KW], int first, int stride) {
+    constexpr int U = LR == 16 ? 4 : 2;  // steps in flight
+    const int lane = threadIdx.x & 31, li = Row::li(), gi = Row::gi();
     const int ne = ke - kb;
-    const bool self = ne > 0 && ws.org[ke - 1] == o;
-    const int nsc = self ? ne - 1 : ne;  // the self entry is the last one
-#ifdef EPIC_PHASE_TIMERS
-    if (threadIdx.x == 0) atomicAdd(&g_phase[12], (unsigned long long)nsc * W);
-#endif
-    // the completion mask in registers: lane l holds words l, l + 32, ...
-    uint32_t ex[KW];
+    const int W = h.W, R = h.R;
+    const uint32_t* bits = h.bits + (size_t)kb * W;
+    const uint32_t s_rows = h.s_rows, s_zero = h.s_zero;
+    const unsigned group = LR == 32 ? 0xffffffffu : ((1u << LR) - 1u) << (gi * LR);
+    for (int c0 = 0; (c0 * stride + first) * NG < ne; c0 += LR) {
+      // lane t looks up entry t of the chunk: step c0 + t / NG, place t % NG
+      const int et = ((c0 + lane / NG) * stride + first) * NG + lane % NG;
+      const bool okt = et < ne;
+      const int o_t = okt ? h.org[kb + et] : 0;
+      const uint32_t s_t = okt ? h.slot(o_t) : kSlotNone;
+      const uint32_t a_t = s_t < (uint32_t)R ? s_rows + s_t * (uint32_t)(W * 4) : s_zero;
+      const int steps = min(LR, (ne - first * NG + stride * NG - 1) / (stride * NG) - c0);
+      for (int u0 = 0; u0 < steps; u0 += U) {
+        uint32_t v[U][KW];
 #pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      ex[i] = (w < W) ? gs.expn[w] : 0u;
-    }
-    const uint32_t* __restrict__ bits = ws.bits + (size_t)kb * W;
-    // one warp per entry, two entries in flight; entries of one column have
-    // distinct origins, so every stage row has one writer
-    for (int e0 = warp; e0 < nsc; e0 += 2 * nw) {
-      const int e1 = e0 + nw;
-      const bool has1 = e1 < nsc;
-      const uint32_t* s0 = bits + (size_t)e0 * W;
-      const uint32_t* s1 = bits + (size_t)(has1 ? e1 : e0) * W;
-      uint32_t v0[KW], v1[KW];
+        for (int u = 0; u < U; ++u) {
+          const int e = ((c0 + u0 + u) * stride + first) * NG + gi;
+          if (u0 + u < steps && e < ne) {
+            Row::load(bits + (size_t)e * W, W, v[u]);
+          } else {
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        v0[i] = ex[i] ? (__ldg(s0 + w) & ex[i]) : 0u;
-        v1[i] = (ex[i] && has1) ? (__ldg(s1 + w) & ex[i]) : 0u;
-      }
-      uint32_t* d0 = ws.stage + (size_t)ws.org[kb + e0] * W;
-      uint32_t* d1 = ws.stage + (size_t)ws.org[kb + (has1 ? e1 : e0)] * W;
-      // the shifted words (item (p, d) -> (p, d + 1)), then every destination
-      // word loaded before any store (no store may alias a pending load)
-      uint32_t a0[KW], a1[KW];
-      {
-        uint32_t c0 = 0, c1 = 0;
-#pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          uint32_t p0 = __shfl_up_sync(0xffffffffu, v0[i], 1);
-          uint32_t p1 = __shfl_up_sync(0xffffffffu, v1[i], 1);
-          if (lane == 0) {
-            p0 = c0;
-            p1 = c1;
+            for (int i = 0; i < KW; ++i) v[u][i] = 0u;
           }
-          c0 = __shfl_sync(0xffffffffu, v0[i], 31);
-          c1 = __shfl_sync(0xffffffffu, v1[i], 31);
-          a0[i] = (v0[i] << 1) | (p0 >> 31);
-          a1[i] = has1 ? ((v1[i] << 1) | (p1 >> 31)) : 0u;
         }
-      }
-      uint32_t q0[KW], q1[KW];
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        q0[i] = (w < W && a0[i]) ? d0[w] : 0u;
-        q1[i] = (w < W && a1[i]) ? d1[w] : 0u;
-      }
-      bool ch0 = false, ch1 = false;
+        for (int u = 0; u < U; ++u) {
+          const int t = ((u0 + u) * NG + gi) & 31;
+          const uint32_t addr = __shfl_sync(0xffffffffu, a_t, t);
+          uint32_t q[KW];
+          Row::load_shared(addr, W, q);
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        if (w < W && (a0[i] & ~q0[i])) {
-          d0[w] = q0[i] | a0[i];
-          ch0 = true;
-        }
-        if (w < W && (a1[i] & ~q1[i])) {
-          d1[w] = q1[i] | a1[i];
-          ch1 = true;
+          for (int i = 0; i < KW; ++i) v[u][i] &= m[i];
+          if (SHIFT) Row::shift_up(v[u]);
+          uint32_t nw = 0;
+#pragma unroll
+          for (int i = 0; i < KW; ++i) nw |= v[u][i] & ~q[i];
+          const unsigned bal = __ballot_sync(0xffffffffu, nw != 0);
+          if (bal) {
+            const bool mine = (bal & group) != 0;
+            const int o2 = __shfl_sync(0xffffffffu, o_t, t);
+            uint32_t s = __shfl_sync(0xffffffffu, s_t, t);
+            if (mine && li == 0 && s == kSlotNone) s = claim(h.slot_of, R, o2);
+            s = __shfl_sync(0xffffffffu, s, 0, LR);
+            bool ch = mine;
+            if (mine && s < (uint32_t)R) {
+              const uint32_t d = s_rows + s * (uint32_t)(W * 4) + (uint32_t)(li * KW) * 4u;
+#pragma unroll
+              for (int i = 0; i < KW; ++i)
+                if (v[u][i] & ~q[i]) gs_red_or(d + 4u * i, v[u][i]);
+            } else if (mine) {  // no slot left: the row is in the global stage
+              uint32_t* d = h.stage + (size_t)o2 * W + li * KW;
+              ch = false;
+#pragma unroll
+              for (int i = 0; i < KW; ++i)
+                if (v[u][i] && (v[u][i] & ~vld(d + i))) {
+                  atomicOr(d + i, v[u][i]);
+                  ch = true;
+                }
+            }
+            __threadfence_block();  // every lane's row writes before the dirty bit
+            const unsigned chm = __ballot_sync(0xffffffffu, ch);
+            if (li == 0 && (chm & group)) mark(o2);
+          }
         }
       }
-      ch0 = __any_sync(0xffffffffu, ch0);
-      ch1 = __any_sync(0xffffffffu, ch1);
-      if (lane == 0) {
-        if (ch0) {
-          const int o2 = ws.org[kb + e0];
-          atomicOr(&sh.touched[o2 >> 5], 1u << (o2 & 31));
-          atomicOr(&sh.dirty[o2 >> 5], 1u << (o2 & 31));
-        }
-        if (ch1 && has1) {
-          const int o2 = ws.org[kb + e1];
-          atomicOr(&sh.touched[o2 >> 5], 1u << (o2 & 31));
-          atomicOr(&sh.dirty[o2 >> 5], 1u << (o2 & 31));
-        }
+    }
+    __syncwarp();
+  }
+
+  // Arrivals: for every entry (o, y) of column src, row(o) |= shift(y & lbl)
+  // (labelled) or row(o) |= y (epsilon).
+  __device__ __noinline__ void arrive(int src, bool shift) {
+    const int warp = threadIdx.x >> 5, nw = nwarps();
+    if (shift && threadIdx.x == 0) walk_gs().labelled = 1;
+    if (REC && threadIdx.x == 0) {
+      if (walk_sh().nedges >= rec->edge_cap) {
+        walk_sh().status = kWalkOverflow;
+      } else {
+        const int e = walk_sh().nedges++;
+        rec->e_dst[e] = walk_sh().ncols;
+        rec->e_src[e] = src;
+        for (int w = 0; w < 8; ++w) rec->e_lbl[(size_t)e * 8 + w] = shift ? walk_sh().lbl8[w] : 0u;
       }
+    }
+    const Hot h = hot();
+    uint32_t m[KW];
+    if (shift) {
+      Row::load(walk_sh().lbl, h.W, m);
+    } else {
+#pragma unroll
+      for (int i = 0; i < KW; ++i) m[i] = 0xffffffffu;
+    }
+    if (shift)
+      scatter<true>(h, h.col[src], h.col[src + 1], m, warp, nw);
+    else
+      scatter<false>(h, h.col[src], h.col[src + 1], m, warp, nw);
+    __syncthreads();
+  }
+
+  __device__ void seed(int c) {
+    if (threadIdx.x == 0) {
+      const uint32_t s = claim(c);
+      row_of(s, c)[g.start_item >> 5] |= 1u << (g.start_item & 31);
+      mark(c);
     }
     __syncthreads();
   }
 
-  // ------------------------------------------------------ warp-parallel sweep
-  // The same least fixpoint as the descending sweep, reached without block
-  // barriers: each warp repeatedly claims the highest dirty origin below c
-  // (clearing its bit), closes its row with the self-loop, claims in
-  // ws.bdone the nonterminals it completes that no visit scattered yet, and
-  // scatters those over column o with atomic ORs, marking the rows it changes
-  // dirty again.  A row may be claimed while another warp still writes into
-  // it; the writer sets the dirty bit after its writes (fenced), so the row
-  // is visited again and nothing is lost.  The sweep ends when no bit is
-  // dirty and no warp holds an origin.  Rows are read through L2 (ld.cg):
-  // other warps' atomics do not update this SM's L1.
-
+  // ------------------------------------------------------------ the sweep
+  // Warp: highest set bit of bm at or below `top`, or -1 (bits may be set and
+  // cleared meanwhile).
   __device__ static int warp_highest_dirty(const uint32_t* bm, int top) {
     const int lane = threadIdx.x & 31;
     if (top < 0) return -1;
-    const volatile uint32_t* vb = bm;
     for (int wtop = top >> 5; wtop >= 0; wtop -= 32) {
       const int w = wtop - lane;
-      uint32_t v = (w >= 0) ? vb[w] : 0u;
+      uint32_t v = (w >= 0) ? vld(bm + w) : 0u;
       if (w == (top >> 5)) v &= (top & 31) == 31 ? 0xffffffffu : ((2u << (top & 31)) - 1u);
       const unsigned any = __ballot_sync(0xffffffffu, v != 0);
       if (any) {
@@ -519,210 +451,116 @@ class EarleyColsGS {
     return -1;
   }
 
-  // Warp: close row o with its self-loop (as close_origin), the nonterminals
-  // already scattered for o taken as done; returns, in lane v < VW, word v of
-  // the nonterminals this visit claimed (completed from o and not yet
-  // scattered by any visit).
-  __device__ uint32_t close_origin_claim(int o, int mode, uint32_t* nstep) {
-    const int lane = threadIdx.x & 31;
-    uint32_t* row = ws.stage + (size_t)o * W;
-    uint32_t* bd = ws.bdone + (size_t)o * VW;
-    // done before the row: a visit writes its row before it claims
-    uint32_t known = (lane < VW) ? __ldcg(bd + lane) : 0u;
+  // Warp: close row o with its self-loop and scatter the nonterminals that it
+  // newly completes over the other entries of column o.
+  __device__ static __forceinline__ void visit(const Hot& h, int o, int mode) {
+    const int W = h.W, VW = h.VW;
+    const int lane = threadIdx.x & 31, li = Row::li();
+    const uint32_t s = h.slot(o);
+    uint32_t* bd = h.done_of(s, o);
+    // done before the row: a visit writes its row before it records what it
+    // completed (those were scattered, and advanced in this row, already)
+    uint32_t known = (lane < VW) ? vld(bd + lane) : 0u;
     __threadfence_block();
-    uint32_t r[KW], r0[KW], e[KW];
+    // every lane group holds a copy of the row
+    uint32_t r[KW], r0[KW], e[KW], ex[KW];
+    const int kb = h.col[o], ke = h.col[o + 1];
+    const bool self = (h.selfb[o >> 5] >> (o & 31)) & 1u;  // the last entry: origins ascend
+    const uint32_t s_row = h.s_rows + s * (uint32_t)(W * 4);
+    const bool in_smem = s < (uint32_t)h.R;
+    if (in_smem) {
+      Row::load_shared(s_row, W, r);
+    } else {
+#pragma unroll
+      for (int i = 0; i < KW; ++i) r[i] = li * KW + i < W ? vld(h.stage + (size_t)o * W + li * KW + i) : 0u;
+    }
+    if (self) {
+      Row::load(h.bits + (size_t)(ke - 1) * W, W, e);
+    } else {
+#pragma unroll
+      for (int i = 0; i < KW; ++i) e[i] = 0u;
+    }
 #pragma unroll
     for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      r[i] = (w < W) ? __ldcg(row + w) : 0u;
       r0[i] = r[i];
-      e[i] = 0u;
+      ex[i] = 0u;
     }
-    const int kb = ws.col_off[o], ke = ws.col_off[o + 1];
-    const bool self = ke > kb && ws.org[ke - 1] == o;
-    if (self) {
-      const uint32_t* E = ws.bits + (size_t)(ke - 1) * W;
+    uint32_t tot = 0;  // lane v < VW: word v of the nonterminals new in this visit
+    uint32_t cs[KW];   // complete items looked at
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        e[i] = (w < W) ? (E[w] & tb.any_nt[w]) : 0u;
-      }
-    }
-    uint32_t tot = 0;
-    uint32_t cseen[KW];
-#pragma unroll
-    for (int i = 0; i < KW; ++i) cseen[i] = 0u;
+    for (int i = 0; i < KW; ++i) cs[i] = 0u;
     for (int round = 0; round < 64 * kMaxW; ++round) {
-      reg_advance(r, mode);
-      if (lane < VW) nstep[lane] = 0;
-      __syncwarp();
+      Row::advance(r, h.adv, mode, h.steps, h.nullable, W);
+      uint32_t cm[KW];
+      Row::load(h.complete, W, cm);
+      bool fresh = false;
 #pragma unroll
       for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        uint32_t m = (w < W) ? (r[i] & tb.complete[w] & ~cseen[i]) : 0u;
-        cseen[i] |= m;
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1;
-          const int A = tb.item_lhs[(w << 5) + b];
-          atomicOr(&nstep[A >> 5], 1u << (A & 31));
-        }
+        cm[i] &= r[i] & ~cs[i];
+        cs[i] |= cm[i];
+        fresh |= cm[i] != 0;
       }
+      if (!__any_sync(0xffffffffu, fresh)) break;
+      if (lane < LR) Row::store(h.scr, W, cm);
       __syncwarp();
-      const uint32_t nw = (lane < VW) ? (nstep[lane] & ~known) : 0u;
+      const uint32_t nw = warp_ntset(h.scr, h.c_off, h.c_lst, h.V, VW) & ~known;
+      __syncwarp();
+      if (!__any_sync(0xffffffffu, nw != 0)) break;
       known |= nw;
       tot |= nw;
-      if (!__any_sync(0xffffffffu, nw != 0) || !self) break;
-      if (lane < VW) nstep[lane] = nw;
-      __syncwarp();
+      uint32_t x[KW];
+      Row::waiting_on(nw, h.exp_nt, W, VW, x);
       bool ch = false;
-      uint32_t carry = 0;
 #pragma unroll
       for (int i = 0; i < KW; ++i) {
-        if (32 * i >= W) break;
-        const int w = lane + 32 * i;
-        uint32_t x = 0, m = e[i];
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1;
-          const int B = tb.item_next[(w << 5) + b] - g.T;
-          if ((nstep[B >> 5] >> (B & 31)) & 1u) x |= 1u << b;
-        }
-        uint32_t prev = __shfl_up_sync(0xffffffffu, x, 1);
-        if (lane == 0) prev = carry;
-        carry = __shfl_sync(0xffffffffu, x, 31);
-        const uint32_t add = ((x << 1) | (prev >> 31)) & ~r[i];
-        ch |= add != 0;
-        r[i] |= add;
+        ex[i] |= x[i];
+        x[i] &= e[i];  // the self entry's items waiting on a new nonterminal advance into r
       }
-      __syncwarp();
+      Row::shift_up(x);
+#pragma unroll
+      for (int i = 0; i < KW; ++i) {
+        ch |= (x[i] & ~r[i]) != 0;
+        r[i] |= x[i];
+      }
       if (!__any_sync(0xffffffffu, ch)) break;
     }
+    if (lane < LR) {
 #pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      if (w < W && (r[i] & ~r0[i])) atomicOr(row + w, r[i]);
+      for (int i = 0; i < KW; ++i)
+        if (r[i] & ~r0[i]) {
+          if (in_smem)
+            gs_red_or(s_row + (uint32_t)(li * KW + i) * 4u, r[i]);
+          else
+            atomicOr(h.stage + (size_t)o * W + li * KW + i, r[i]);
+        }
     }
+    if (!__any_sync(0xffffffffu, tot != 0)) return;
     __threadfence_block();
-    uint32_t mine = 0;
-    if (lane < VW && tot) mine = tot & ~atomicOr(bd + lane, tot);
-    return mine;
-  }
-
-  // Warp: completions of the nonterminals in nnew (nnew[v], v < VW) from
-  // origin o into the rows of the other entries of column o.
-  __device__ void scatter_warp(int o, const uint32_t* nnew, uint32_t* expn) {
-    const int lane = threadIdx.x & 31;
-    for (int w = lane; w < W; w += 32) {
-      uint32_t acc = 0, m = tb.any_nt[w];
-      while (m) {
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        const int B = tb.item_next[(w << 5) + b] - g.T;
-        if ((nnew[B >> 5] >> (B & 31)) & 1u) acc |= 1u << b;
-      }
-      expn[w] = acc;
-    }
     __syncwarp();
-    uint32_t ex[KW];
-#pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      ex[i] = (w < W) ? expn[w] : 0u;
-    }
-    const int kb = ws.col_off[o], ke = ws.col_off[o + 1];
-    const bool self = ke > kb && ws.org[ke - 1] == o;
-    const int nsc = (self ? ke - 1 : ke) - kb;
-    const uint32_t* __restrict__ bits = ws.bits + (size_t)kb * W;
-    for (int e0 = 0; e0 < nsc; e0 += 2) {
-      const bool has1 = e0 + 1 < nsc;
-      const uint32_t* s0 = bits + (size_t)e0 * W;
-      const uint32_t* s1 = bits + (size_t)(has1 ? e0 + 1 : e0) * W;
-      uint32_t v0[KW], v1[KW];
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        v0[i] = ex[i] ? (__ldg(s0 + w) & ex[i]) : 0u;
-        v1[i] = (ex[i] && has1) ? (__ldg(s1 + w) & ex[i]) : 0u;
-      }
-      const int o0 = ws.org[kb + e0], o1 = ws.org[kb + (has1 ? e0 + 1 : e0)];
-      uint32_t* d0 = ws.stage + (size_t)o0 * W;
-      uint32_t* d1 = ws.stage + (size_t)o1 * W;
-      uint32_t a0[KW], a1[KW];
-      {
-        uint32_t c0 = 0, c1 = 0;
-#pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          uint32_t p0 = __shfl_up_sync(0xffffffffu, v0[i], 1);
-          uint32_t p1 = __shfl_up_sync(0xffffffffu, v1[i], 1);
-          if (lane == 0) {
-            p0 = c0;
-            p1 = c1;
-          }
-          c0 = __shfl_sync(0xffffffffu, v0[i], 31);
-          c1 = __shfl_sync(0xffffffffu, v1[i], 31);
-          a0[i] = (v0[i] << 1) | (p0 >> 31);
-          a1[i] = has1 ? ((v1[i] << 1) | (p1 >> 31)) : 0u;
-        }
-      }
-      uint32_t q0[KW], q1[KW];
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        q0[i] = (w < W && a0[i]) ? __ldcg(d0 + w) : 0u;
-        q1[i] = (w < W && a1[i]) ? __ldcg(d1 + w) : 0u;
-      }
-      bool ch0 = false, ch1 = false;
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        if (w < W && (a0[i] & ~q0[i])) {
-          atomicOr(d0 + w, a0[i]);
-          ch0 = true;
-        }
-        if (w < W && (a1[i] & ~q1[i])) {
-          atomicOr(d1 + w, a1[i]);
-          ch1 = true;
-        }
-      }
-      __threadfence_block();  // every lane's row writes before the dirty bits
-      ch0 = __any_sync(0xffffffffu, ch0);
-      ch1 = __any_sync(0xffffffffu, ch1);
-      __syncwarp();
-      if (lane == 0) {
-        if (ch0) {
-          atomicOr(&sh.touched[o0 >> 5], 1u << (o0 & 31));
-          atomicOr(&sh.dirty[o0 >> 5], 1u << (o0 & 31));
-        }
-        if (ch1 && has1) {
-          atomicOr(&sh.touched[o1 >> 5], 1u << (o1 & 31));
-          atomicOr(&sh.dirty[o1 >> 5], 1u << (o1 & 31));
-        }
-      }
-      __syncwarp();
-    }
+    if (lane < VW && tot) atomicOr(bd + lane, tot);
+    scatter<true>(h, kb, self ? ke - 1 : ke, ex, 0, 1);
   }
 
-  // Block: the origins below c, closed warp-parallel (every warp returns
-  // when the sweep is done).
-  __device__ void close_origins_par(int c, int mode) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t* nstep = wscr + (size_t)warp * kGsWarpScratch;
-    uint32_t* expn = nstep + kMaxVW;
-    volatile int32_t* busy = &gs.busy;
+  // Block: close the origins below c (every warp returns when nothing is
+  // dirty and no warp holds an origin).
+  __device__ void close_origins(int c, int mode) {
+    const Hot h = hot();
+    const int lane = threadIdx.x & 31;
+    const volatile int32_t* busy = &walk_gs().busy;
     long long visits = 0, idle = 0;
     for (;;) {
-      // claim the highest dirty origin; a holder counts itself busy right
-      // after its claim (a warp that saw nothing dirty and no holder in that
-      // gap leaves early, and the holder finishes what its origin causes)
+      // claim the highest dirty origin; a holder counts itself busy before
+      // its claim clears the bit, so "no holder, then nothing dirty" means done
       int o = -1;
       for (int tries = 0; tries < 64; ++tries) {
-        const int h = warp_highest_dirty(sh.dirty, c - 1);
+        const int h = warp_highest_dirty(walk_sh().dirty, c - 1);
         if (h < 0) break;
         uint32_t old = 0;
         if (lane == 0) {
-          old = atomicAnd(&sh.dirty[h >> 5], ~(1u << (h & 31)));
-          if ((old >> (h & 31)) & 1u) atomicAdd(&gs.busy, 1);
+          atomicAdd(&walk_gs().busy, 1);
+          __threadfence_block();
+          old = atomicAnd(&walk_sh().dirty[h >> 5], ~(1u << (h & 31)));
+          if (!((old >> (h & 31)) & 1u)) atomicSub(&walk_gs().busy, 1);
         }
         old = __shfl_sync(0xffffffffu, old, 0);
         if ((old >> (h & 31)) & 1u) {
@@ -731,313 +569,240 @@ class EarleyColsGS {
         }
       }
       if (o < 0) {
-        // done when no warp holds an origin and, after that, nothing is dirty
         int b = 0;
         if (lane == 0) b = *busy;
         b = __shfl_sync(0xffffffffu, b, 0);
         __threadfence_block();
-        if (b == 0 && warp_highest_dirty(sh.dirty, c - 1) < 0) break;
+        if (b == 0 && warp_highest_dirty(walk_sh().dirty, c - 1) < 0) break;
         if (++idle > kGsMaxIdle) {
-          if (lane == 0) sh.status = kWalkOverflow;
+          if (lane == 0) walk_sh().status = kWalkOverflow;
           break;
         }
-        __nanosleep(64);
+        __nanosleep(40);
         continue;
       }
       __syncwarp();  // the claim (lane 0) before any lane reads the row
       __threadfence_block();
-      if (++visits > kGsMaxSteps) {
-        if (lane == 0) {
-          sh.status = kWalkOverflow;
-          atomicSub(&gs.busy, 1);
-        }
-        __syncwarp();
-        break;
+      if (++visits <= kGsMaxSteps) {
+        visit(h, o, mode);
+      } else if (lane == 0) {
+        walk_sh().status = kWalkOverflow;
       }
-      const uint32_t mine = close_origin_claim(o, mode, nstep);
-      if (lane < VW) nstep[lane] = mine;
-      __syncwarp();
-      if (__any_sync(0xffffffffu, mine != 0)) scatter_warp(o, nstep, expn);
       __threadfence_block();
       __syncwarp();
-      if (lane == 0) atomicSub(&gs.busy, 1);
+      if (lane == 0) atomicSub(&walk_gs().busy, 1);
       __syncwarp();
+      if (visits > kGsMaxSteps) break;
     }
   }
 
   // Closure of column c (gap: a node with a Sigma_lex* self-loop).
-  __device__ void close_column(int c, bool gap) {
+  __device__ __noinline__ void close_column(int c, bool gap) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = nwarps();
     if (REC && threadIdx.x == 0) rec->col_gap[c] = gap ? 1 : 0;
     const int mode = gap ? 1 : 0;  // the advance rule: next_any in a gap, nullable_next elsewhere
-    // 1. origins below c, highest first; warp 0 walks down the dirty origins
-    //    until one completes something new, then every warp scatters.
-    //    A node (not a gap) reached only by epsilon edges from finished
-    //    columns needs none of it: each of its rows is a union of rows that
-    //    are closed under completion and advance, and so is the union (what
-    //    an origin completes here, it completed in one of the sources, whose
-    //    rows below already hold the advanced items).
-    int top = (!gap && !gs.labelled) ? -1 : c - 1;
-    if (par) {
-      if (threadIdx.x == 0) gs.busy = 0;
+    // 1. origins below c.  A node (not a gap) reached only by epsilon edges
+    //    from finished columns needs no sweep: each of its rows is a union of
+    //    rows that are closed under completion and advance, and so is the
+    //    union (what an origin completes here, it completed in one of the
+    //    sources, whose rows below already hold the advanced items).
+    PH_BEGIN(t_or);
+    if (gap || walk_gs().labelled) {
+      if (threadIdx.x == 0) walk_gs().busy = 0;
       __syncthreads();
-      if (top >= 0) close_origins_par(c, mode);
-      __syncthreads();
-      if (sh.status == kWalkOverflow) return;
-      top = -1;  // the descending sweep below has nothing left
+      close_origins(c, mode);
     }
-    for (long long step = 0;; ++step) {
-      if (warp == 0) {
-        PH_BEGIN(t_or);
-        int o = -1;
-        for (long long guard = 0; guard <= kGsMaxSteps; ++guard) {
-          o = warp_highest_at_or_below(sh.dirty, top);
-          if (o < 0) break;
-          if (lane == 0) sh.dirty[o >> 5] &= ~(1u << (o & 31));
-          __syncwarp();
-          top = o - 1;
-          if (close_origin(o, mode)) break;
-          o = -1;
-        }
-        if (lane == 0) gs.cur_o = o;
-        PH_END(8, t_or);
-      }
-      __syncthreads();
-      const int o = gs.cur_o;
-      if (o < 0) break;
-      if (step > kGsMaxSteps) {
-        if (threadIdx.x == 0) sh.status = kWalkOverflow;
-        __syncthreads();
-        return;
-      }
-      PH_BEGIN(t_sc);
-      build_expn();
-      __syncthreads();
-      scatter_column(o);
-      PH_END(9, t_sc);
-    }
-    // 2. predictions: nonterminals waited on by any row of the column; row c
-    //    is closed with them (its completions at c are the advance rules)
+    for (int w = threadIdx.x; w < W; w += blockDim.x) walk_gs().uni[w] = 0;
+    __syncthreads();
+    PH_END(8, t_or);
+    if (walk_sh().status == kWalkOverflow) return;
+    // 2. predictions: nonterminals waited on by any row of the column
     PH_BEGIN(t_pr);
-    for (int w = threadIdx.x; w < W; w += blockDim.x) gs.uni[w] = 0;
-    __syncthreads();
-    bitmap_to_list(sh, sh.touched, c + 1);
-    const int nl = sh.list_n;
-    for (int i = warp; i < nl; i += nw) {
-      const uint32_t* row = ws.stage + (size_t)sh.list[i] * W;
-      for (int w = lane; w < W; w += 32) {
-        const uint32_t v = row[w] & tb.any_nt[w];
-        if (v) atomicOr(&gs.uni[w], v);
+    bitmap_to_list(walk_sh().touched, c + 1);
+    const int nl = walk_sh().list_n;
+    {
+      uint32_t acc[KW];
+#pragma unroll
+      for (int i = 0; i < KW; ++i) acc[i] = 0u;
+      for (int i = warp * NG + Row::gi(); i < nl; i += nw * NG) {
+        const int o = walk_sh().list[i];
+        uint32_t v[KW];
+        Row::load(row_of(slot(o), o), W, v);
+#pragma unroll
+        for (int j = 0; j < KW; ++j) acc[j] |= v[j];
       }
+      uint32_t an[KW];
+      Row::load(tb.any_nt, W, an);
+#pragma unroll
+      for (int j = 0; j < KW; ++j)
+        if (acc[j] & an[j]) atomicOr(&walk_gs().uni[Row::li() * KW + j], acc[j] & an[j]);
     }
     __syncthreads();
-    for (int round = 0; round < 4 * kMaxVW + 4; ++round) {
-      // vset |= nonterminals after the dot in uni
-      for (int w = threadIdx.x; w < W; w += blockDim.x) {
-        uint32_t m = gs.uni[w];
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1;
-          const int B = tb.item_next[(w << 5) + b] - g.T;
-          atomicOr(&gs.vset[B >> 5], 1u << (B & 31));
+    for (int v = warp; v < VW; v += nw) {  // one warp per word of the set
+      const int A = (v << 5) + lane;
+      bool hit = false;
+      if (A < g.V)
+        for (int q = g.wait_off[A], e = g.wait_off[A + 1]; q < e && !hit; ++q) {
+          const uint2 p = g.wait[q];
+          hit = (walk_gs().uni[p.x] & p.y) != 0;
         }
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        uint32_t any = 0;
-        for (int v = 0; v < VW; ++v) {
-          const uint32_t nw2 = gs.vset[v] & ~gs.vdone[v];
-          gs.nnew[v] = nw2;
-          any |= nw2;
-        }
-        gs.flag = any != 0;
-      }
-      __syncthreads();
-      if (!gs.flag) break;
+      const uint32_t b = __ballot_sync(0xffffffffu, hit);
+      if (lane == 0) walk_gs().vset[v] = b;
+    }
+    if (threadIdx.x == 0) claim(c);
+    __syncthreads();
+    uint32_t* crow = row_of(slot(c), c);
+    {
       const uint32_t* P = gap ? g.gap_pred : g.pred;
-      uint32_t* crow = ws.stage + (size_t)c * W;
-      for (int w = threadIdx.x; w < W; w += blockDim.x) {
-        uint32_t acc = 0;
-        for (int v = 0; v < VW; ++v) {
-          uint32_t m = gs.nnew[v];
-          while (m) {
-            const int b = __ffs(m) - 1;
-            m &= m - 1;
-            acc |= P[(size_t)((v << 5) + b) * W + w];
-          }
-        }
-        crow[w] |= acc;
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        for (int v = 0; v < VW; ++v) gs.vdone[v] |= gs.nnew[v];
-        sh.touched[c >> 5] |= 1u << (c & 31);
-      }
-      if (warp == 0) {  // advance row c, add its items to uni
-        uint32_t r[KW];
+      uint32_t acc[KW];
 #pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          const int w = lane + 32 * i;
-          r[i] = (w < W) ? crow[w] : 0u;
-        }
-        reg_advance(r, mode);
+      for (int i = 0; i < KW; ++i) acc[i] = 0u;
+      // the warps' lane groups share out the nonterminals
+      const int part = warp * NG + Row::gi(), parts = nw * NG;
+      int seen = 0;
+      for (int v = 0; v < VW; ++v) {
+        uint32_t m = walk_gs().vset[v];
+        while (m) {
+          const int b0 = __ffs(m) - 1;
+          m &= m - 1;
+          if (seen++ % parts != part) continue;
+          uint32_t x[KW];
+          Row::load(P + (size_t)((v << 5) + b0) * W, W, x);
 #pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          const int w = lane + 32 * i;
-          if (w < W) {
-            crow[w] = r[i];
-            gs.uni[w] |= r[i] & tb.any_nt[w];
-          }
+          for (int i = 0; i < KW; ++i) acc[i] |= x[i];
         }
       }
-      __syncthreads();
+      bool nz = false;
+#pragma unroll
+      for (int i = 0; i < KW; ++i)
+        if (acc[i]) {
+          atomicOr(crow + Row::li() * KW + i, acc[i]);
+          nz = true;
+        }
+      if (__any_sync(0xffffffffu, nz) && lane == 0) atomicOr(&walk_sh().touched[c >> 5], 1u << (c & 31));
     }
-    // a seeded row c (the walk's first column) is closed by the advance as well
-    if (warp == 0 && bit_get(sh.dirty, c)) {
-      uint32_t* crow = ws.stage + (size_t)c * W;
+    __syncthreads();
+    // a seeded row c (the walk's first column) is closed by the advance rule
+    if (warp == 0 && bit_get(walk_sh().dirty, c)) {
       uint32_t r[KW];
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        r[i] = (w < W) ? crow[w] : 0u;
-      }
-      reg_advance(r, mode);
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        if (w < W) crow[w] = r[i];
-      }
-      if (lane == 0) sh.dirty[c >> 5] &= ~(1u << (c & 31));
+      Row::load(crow, W, r);
+      Row::advance(r, tb.adv_pow, mode, g.adv_steps, g.any_nullable, W);
+      __syncwarp();
+      if (lane < LR) Row::store(crow, W, r);
     }
     __syncthreads();
     PH_END(10, t_pr);
   }
 
-  // Move the touched nonzero rows into the entry store as column c (origins
-  // ascending), recording completed nonterminals and summaries.
-  __device__ void finish_column(int c) {
+  // Move the rows of the open column into the entry store as column c
+  // (origins ascending), recording completed nonterminals and summaries.  A
+  // touched row is never empty.
+  __device__ __noinline__ void finish_column(int c) {
     PH_BEGIN(t_fi);
-    finish_inner(c);
-    PH_END(11, t_fi);
-  }
-  __device__ void finish_inner(int c) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = nwarps();
-    bitmap_to_list(sh, sh.touched, c + 1);
-    const int nl = sh.list_n;
-    for (int i = warp; i < nl; i += nw) {
-      const uint32_t* row = ws.stage + (size_t)sh.list[i] * W;
-      bool nz = false;
-      for (int w = lane; w < W; w += 32) nz |= row[w] != 0;
-      nz = __any_sync(0xffffffffu, nz);
-      if (lane == 0) sh.prefix[i] = nz ? 1 : 0;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int s = 0;
-      for (int i = 0; i < nl; ++i) {
-        const int f = sh.prefix[i];
-        sh.prefix[i] = f ? s : -1;
-        s += f;
-      }
-      const long long base = ws.col_off[c];
-      if (base + s > dims.emax) {
-        sh.status = kWalkOverflow;
-      } else {
-        ws.col_off[c + 1] = (int)(base + s);
-        sh.nent = base + s;
-      }
-      sh.ncols = c + 1;
-    }
-    __syncthreads();
-    const bool ok = sh.status != kWalkOverflow;
+    const int warp = threadIdx.x >> 5, nw = nwarps();
+    bitmap_to_list(walk_sh().touched, c + 1);
+    const int nl = walk_sh().list_n;
     const int base = ws.col_off[c];
-    for (int i = warp; i < nl; i += nw) {
-      const int o = sh.list[i];
-      uint32_t* row = ws.stage + (size_t)o * W;
-      const int slot = sh.prefix[i];
-      if (ok && slot >= 0) {
-        if (lane == 0) ws.org[base + slot] = o;
-        uint32_t* dst = ws.bits + (size_t)(base + slot) * W;
-        for (int w = lane; w < W; w += 32) dst[w] = row[w];
-        if constexpr (REC) record_entry(row, (long long)base + slot);
+    const bool ok = (long long)base + nl <= dims.emax;
+    if (threadIdx.x == 0) {
+      if (!ok) {
+        walk_sh().status = kWalkOverflow;
+      } else {
+        ws.col_off[c + 1] = base + nl;
+        walk_sh().nent = base + nl;
       }
-      __syncwarp();
-      for (int w = lane; w < W; w += 32) row[w] = 0;
-      if (par)
-        for (int v = lane; v < VW; v += 32) ws.bdone[(size_t)o * VW + v] = 0;
+      walk_sh().ncols = c + 1;
+      walk_gs().labelled = 0;
+      walk_gs().nslots = 0;
     }
-    clear_bitmap(sh.touched, c + 1);
-    clear_bitmap(sh.dirty, c + 1);
-    for (int v = threadIdx.x; v < kMaxVW; v += blockDim.x) {
-      gs.vset[v] = 0;
-      gs.vdone[v] = 0;
+    if constexpr (REC) {
+      if (ok)
+        for (int i = warp; i < nl; i += nw) {
+          const int o = walk_sh().list[i];
+          record_entry(row_of(slot(o), o), (size_t)base + i);
+        }
     }
-    if (threadIdx.x == 0) gs.labelled = 0;
+    if (REC) __syncthreads();  // rows are cleared below, by other warps than read them here
+    // one lane group per row
+    for (int i = warp * NG + Row::gi(); i < nl; i += nw * NG) {
+      const int o = walk_sh().list[i];
+      const uint32_t s = slot(o);
+      uint32_t* row = row_of(s, o);
+      uint32_t v[KW];
+      Row::load(row, W, v);
+      if (ok) {
+        const size_t k = (size_t)base + i;
+        Row::store(ws.bits + k * W, W, v);
+        if (Row::li() == 0) {
+          ws.org[k] = o;
+          if (o == c) selfb[c >> 5] |= 1u << (c & 31);  // one group holds origin c
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < KW; ++j) v[j] = 0u;
+      Row::store(row, W, v);
+      uint32_t* bd = done_of(s, o);
+      for (int w = Row::li(); w < VW; w += LR) bd[w] = 0;
+      if (Row::li() == 0) slot_of[o] = (uint16_t)kSlotNone;
+    }
     __syncthreads();
+    if (threadIdx.x == 0) slot_of[c] = (uint16_t)kSlotNone;  // claimed even if nothing was predicted
+    clear_bitmap(walk_sh().touched, c + 1);
+    clear_bitmap(walk_sh().dirty, c + 1);
+    __syncthreads();
+    PH_END(11, t_fi);
   }
 
   __device__ bool column_empty(int c) const { return ws.col_off[c + 1] == ws.col_off[c]; }
 
-  // Warp: completed nonterminals and folded summaries of stored entry k.
-  __device__ void record_entry(const uint32_t* row, long long k) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t* nts = wnt + (size_t)warp * kMaxVW;
-    for (int v = lane; v < VW; v += 32) nts[v] = 0;
-    __syncwarp();
+  // Warp: completed nonterminals and folded summaries of entry k, its row in
+  // memory.
+  __device__ void record_entry(const uint32_t* row, size_t k) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t cn = warp_ntset(row, (const int32_t*)(gs_smem() + plan.o_off), (const uint2*)(gs_smem() + plan.o_list),
+                                   g.V, VW);
+    if (lane < VW) rec->cnt[k * VW + lane] = cn;
     uint32_t fnt = 0, ft = 0;
     for (int w = lane; w < W; w += 32) {
-      const uint32_t r = row[w];
-      uint32_t m = r & tb.complete[w];
+      uint32_t m = row[w] & tb.next_any[w];
       while (m) {
         const int b = __ffs(m) - 1;
         m &= m - 1;
-        const int B = tb.item_lhs[(w << 5) + b];
-        atomicOr(&nts[B >> 5], 1u << (B & 31));
-      }
-      m = r & tb.any_nt[w];
-      while (m) {
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        fnt |= 1u << ((tb.item_next[(w << 5) + b] - g.T) & 31);
-      }
-      m = r & tb.any_term[w];
-      while (m) {
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        ft |= 1u << (tb.item_next[(w << 5) + b] & 31);
+        const int s = tb.item_next[(w << 5) + b];
+        if (s >= g.T)
+          fnt |= 1u << ((s - g.T) & 31);
+        else
+          ft |= 1u << (s & 31);
       }
     }
-    for (int off = 16; off; off >>= 1) {
-      fnt |= __shfl_xor_sync(0xffffffffu, fnt, off);
-      ft |= __shfl_xor_sync(0xffffffffu, ft, off);
-    }
-    __syncwarp();
-    for (int v = lane; v < VW; v += 32) rec->cnt[(size_t)k * VW + v] = nts[v];
+    fnt = __reduce_or_sync(0xffffffffu, fnt);
+    ft = __reduce_or_sync(0xffffffffu, ft);
     if (lane == 0) {
-      rec->esum[(size_t)k * 2] = fnt;
-      rec->esum[(size_t)k * 2 + 1] = ft;
+      rec->esum[k * 2] = fnt;
+      rec->esum[k * 2 + 1] = ft;
     }
-    __syncwarp();
   }
 
-  // After an aborted walk: return the staging rows of the open column to zero.
+  // After an aborted walk: return the rows of the open column to zero.
   __device__ void cleanup() {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = nwarps();
-    bitmap_to_list(sh, sh.touched, kMaxCols);
-    const int nl = sh.list_n;
-    for (int i = warp; i < nl; i += nw) {
-      const int o = sh.list[i];
-      for (int w = lane; w < W; w += 32) ws.stage[(size_t)o * W + w] = 0;
-      if (par)
-        for (int v = lane; v < VW; v += 32) ws.bdone[(size_t)o * VW + v] = 0;
+    __syncthreads();
+    for (int o = warp; o < dims.nmax; o += nw) {
+      const uint32_t s = slot(o);
+      if (s == kSlotNone) continue;
+      uint32_t* row = row_of(s, o);
+      for (int w = lane; w < W; w += 32) row[w] = 0;
+      uint32_t* bd = done_of(s, o);
+      for (int v = lane; v < VW; v += 32) bd[v] = 0;
+      __syncwarp();
+      if (lane == 0) slot_of[o] = (uint16_t)kSlotNone;
     }
-    clear_bitmap(sh.touched, kMaxCols);
-    clear_bitmap(sh.dirty, kMaxCols);
-    for (int v = threadIdx.x; v < kMaxVW; v += blockDim.x) {
-      gs.vset[v] = 0;
-      gs.vdone[v] = 0;
+    if (threadIdx.x == 0) {
+      walk_gs().labelled = 0;
+      walk_gs().nslots = 0;
     }
-    if (threadIdx.x == 0) gs.labelled = 0;
+    clear_bitmap(walk_sh().touched, kMaxCols);
+    clear_bitmap(walk_sh().dirty, kMaxCols);
     __syncthreads();
   }
 

@@ -27,21 +27,23 @@ struct SelFrame {
 // once, one CTA each per sequence, before the recursion; k_select reuses the
 // two answers when it asks for exactly these tests.  spec[b] = {cover,
 // exact}: 1 pass, 0 fail, -1 not available (overflow / bad input).
-__global__ void __launch_bounds__(kSelThreads) k_select_spec(DevGrammar g, const LexEntry* __restrict__ table, int vocab,
+template <class S>
+__global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1) k_select_spec(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table, int vocab,
                                                           const int32_t* __restrict__ x, int B, int n,
                                                           const int32_t* __restrict__ pos, int k,
                                                           const int32_t* __restrict__ tok, int8_t* __restrict__ spec,
                                                           WsPack wsp) {
-  __shared__ WalkShared sh;
-  __shared__ GsShared gss;
   __shared__ int s_pos[kMaxSel], s_tok[kMaxSel];
   __shared__ int ns;
   extern __shared__ __align__(16) unsigned char dyn[];
   GsTables tb;
-  gs_stage_tables(g, dyn, tb);
+  gs_stage_tables(g, dyn + kWalkSmemBytes, tb);
   Workspace ws;
   WalkScratch sc;
   wsp.carve(blockIdx.x, ws, sc);
+  EarleyColsGS<false, S>::place_scratch(g, plan, dyn, sc);
+  EarleyColsGS<false, S> ecols(g, tb, plan, dyn, ws, wsp.dims);
+  ecols.init(dyn);
   for (int job = blockIdx.x; job < 2 * B; job += gridDim.x) {
     int b = job >> 1;
     bool exact = job & 1;
@@ -61,14 +63,11 @@ __global__ void __launch_bounds__(kSelThreads) k_select_spec(DevGrammar g, const
     if (ns >= 2) {  // a set of at most one candidate is never tested
       Subst s{s_pos, s_tok, ns};
       if (exact) {
-        EarleyColsGS<false> cols(g, tb, table, ws, sc, wsp.dims, sh, gss);
-        cols.par = g.gs_par != 0;
-        cols.wscr = (uint32_t*)(dyn + gs_tables_bytes(g.D, g.W, g.adv_steps));
-        Walk<EarleyColsGS<false>> w(cols, g, table, sc, sh, vocab);
+        Walk<EarleyColsGS<false, S>> w(ecols, g, table, sc, vocab);
         r = w.run(x + (long long)b * n, n, s);
       } else {
-        CoverCols cols(g, ws, wsp.dims, sh);
-        Walk<CoverCols> w(cols, g, table, sc, sh, vocab);
+        CoverCols cols(g, ws, wsp.dims);
+        Walk<CoverCols> w(cols, g, table, sc, vocab);
         r = w.run(x + (long long)b * n, n, s);
       }
     }
@@ -77,17 +76,16 @@ __global__ void __launch_bounds__(kSelThreads) k_select_spec(DevGrammar g, const
   }
 }
 
-__global__ void __launch_bounds__(kSelThreads) k_select(DevGrammar g, const LexEntry* __restrict__ table, int vocab,
+template <class S>
+__global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1) k_select(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table, int vocab,
                                                      const int32_t* __restrict__ x, int B, int n,
                                                      const int32_t* __restrict__ pos, int k,
                                                      const int32_t* __restrict__ tok, const float* __restrict__ conf,
                                                      uint8_t* __restrict__ selected, WsPack wsp,
                                                      const int8_t* __restrict__ spec, unsigned long long* stats) {
-  __shared__ WalkShared sh;
-  __shared__ GsShared gss;
   extern __shared__ __align__(16) unsigned char dyn[];
   GsTables tb;
-  gs_stage_tables(g, dyn, tb);
+  gs_stage_tables(g, dyn + kWalkSmemBytes, tb);
   __shared__ int c_slot[kMaxSel], c_pos[kMaxSel], c_tok[kMaxSel];
   __shared__ int s_pos[kMaxSel], s_tok[kMaxSel];
   __shared__ SelFrame stack[2 * kMaxSel + 8];
@@ -96,12 +94,12 @@ __global__ void __launch_bounds__(kSelThreads) k_select(DevGrammar g, const LexE
   Workspace ws;
   WalkScratch sc;
   wsp.carve(blockIdx.x, ws, sc);
-  EarleyColsGS<false> ecols(g, tb, table, ws, sc, wsp.dims, sh, gss);
-  ecols.par = g.gs_par != 0;
-  ecols.wscr = (uint32_t*)(dyn + gs_tables_bytes(g.D, g.W, g.adv_steps));
-  CoverCols ccols(g, ws, wsp.dims, sh);
-  Walk<EarleyColsGS<false>> exact(ecols, g, table, sc, sh, vocab);
-  Walk<CoverCols> cover(ccols, g, table, sc, sh, vocab);
+  EarleyColsGS<false, S>::place_scratch(g, plan, dyn, sc);
+  EarleyColsGS<false, S> ecols(g, tb, plan, dyn, ws, wsp.dims);
+  ecols.init(dyn);
+  CoverCols ccols(g, ws, wsp.dims);
+  Walk<EarleyColsGS<false, S>> exact(ecols, g, table, sc, vocab);
+  Walk<CoverCols> cover(ccols, g, table, sc, vocab);
   for (int b = blockIdx.x; b < B; b += gridDim.x) {
     const int32_t* xb = x + (long long)b * n;
     if (threadIdx.x == 0) {
@@ -390,7 +388,8 @@ __device__ int fallback_best(int b, const int32_t* xb, const int32_t* pos, int k
 
 // One round: job (b, s) tests the s-th candidate of sequence b's order.
 // res[(b m + s) 2] = candidate (-1: none), [+1] = 1 pass, 0 fail, -1 capacity.
-__global__ void __launch_bounds__(kSelThreads) k_fallback_round(DevGrammar g, const LexEntry* __restrict__ table,
+template <class S>
+__global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1) k_fallback_round(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table,
                                                              int vocab, const int32_t* __restrict__ x, int B, int n,
                                                              const int32_t* __restrict__ pos, int k,
                                                              const int32_t* __restrict__ cand,
@@ -398,11 +397,9 @@ __global__ void __launch_bounds__(kSelThreads) k_fallback_round(DevGrammar g, co
                                                              const uint8_t* __restrict__ rej,
                                                              const int32_t* __restrict__ fb, int32_t* __restrict__ res,
                                                              WsPack wsp, unsigned long long* stats) {
-  __shared__ WalkShared sh;
-  __shared__ GsShared gss;
   extern __shared__ __align__(16) unsigned char dyn[];
   GsTables tb;
-  gs_stage_tables(g, dyn, tb);
+  gs_stage_tables(g, dyn + kWalkSmemBytes, tb);
   __shared__ float r_cf[kSelThreads / 32];
   __shared__ int r_q[kSelThreads / 32];
   __shared__ int excl[kMaxFallbackSpec];
@@ -410,10 +407,10 @@ __global__ void __launch_bounds__(kSelThreads) k_fallback_round(DevGrammar g, co
   Workspace ws;
   WalkScratch sc;
   wsp.carve(blockIdx.x, ws, sc);
-  EarleyColsGS<false> cols(g, tb, table, ws, sc, wsp.dims, sh, gss);
-  cols.par = g.gs_par != 0;
-  cols.wscr = (uint32_t*)(dyn + gs_tables_bytes(g.D, g.W, g.adv_steps));
-  Walk<EarleyColsGS<false>> walk(cols, g, table, sc, sh, vocab);
+  EarleyColsGS<false, S>::place_scratch(g, plan, dyn, sc);
+  EarleyColsGS<false, S> cols(g, tb, plan, dyn, ws, wsp.dims);
+  cols.init(dyn);
+  Walk<EarleyColsGS<false, S>> walk(cols, g, table, sc, vocab);
   unsigned long long n_chk = 0;
   for (long long job = blockIdx.x; job < (long long)B * m; job += gridDim.x) {
     const int b = (int)(job / m), sl = (int)(job % m);
@@ -502,21 +499,23 @@ namespace epic {
 void launch_select_spec(dim3 grid, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
                         const int32_t* x, int B, int n, const int32_t* pos, int k, const int32_t* tok, int8_t* spec,
                         const WsPack& wsp) {
-  const size_t dyn = gs_tables_bytes(g.D, g.W, g.adv_steps) + gs_warp_scratch_bytes();
-  DevGrammar gg = g;
-  gg.gs_par = gs_parallel_enabled(g.W);
-  cudaFuncSetAttribute(k_select_spec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  k_select_spec<<<grid, kSelThreads, dyn, st>>>(gg, table, vocab, x, B, n, pos, k, tok, spec, wsp);
+  const GsPlan p = gs_plan(g, wsp.dims.nmax, gs_limit(g.W));
+  auto go = [&](auto* kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
+    kernel<<<grid, gs_threads(g.W), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, tok, spec, wsp);
+  };
+  with_row_shape(g.W, [&](auto s) { go(k_select_spec<decltype(s)>); });
 }
 
 void launch_select(dim3 grid, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
                    const int32_t* x, int B, int n, const int32_t* pos, int k, const int32_t* tok, const float* conf,
                    uint8_t* selected, const WsPack& wsp, const int8_t* spec, unsigned long long* stats) {
-  const size_t dyn = gs_tables_bytes(g.D, g.W, g.adv_steps) + gs_warp_scratch_bytes();
-  DevGrammar gg = g;
-  gg.gs_par = gs_parallel_enabled(g.W);
-  cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  k_select<<<grid, kSelThreads, dyn, st>>>(gg, table, vocab, x, B, n, pos, k, tok, conf, selected, wsp, spec, stats);
+  const GsPlan p = gs_plan(g, wsp.dims.nmax, gs_limit(g.W));
+  auto go = [&](auto* kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
+    kernel<<<grid, gs_threads(g.W), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, tok, conf, selected, wsp, spec, stats);
+  };
+  with_row_shape(g.W, [&](auto s) { go(k_select<decltype(s)>); });
 }
 
 void launch_fallback_init(int B, cudaStream_t st, int n, const int32_t* pos, int k, const float* conf, int K,
@@ -530,12 +529,13 @@ void launch_fallback_round(dim3 grid, cudaStream_t st, const DevGrammar& g, cons
                            const int32_t* x, int B, int n, const int32_t* pos, int k, const int32_t* cand,
                            const float* conf, int K, int m, const uint8_t* rej, const int32_t* fb, int32_t* res,
                            const WsPack& wsp, unsigned long long* stats) {
-  const size_t dyn = gs_tables_bytes(g.D, g.W, g.adv_steps) + gs_warp_scratch_bytes();
-  DevGrammar gg = g;
-  gg.gs_par = gs_parallel_enabled(g.W);
-  cudaFuncSetAttribute(k_fallback_round, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  k_fallback_round<<<grid, kSelThreads, dyn, st>>>(gg, table, vocab, x, B, n, pos, k, cand, conf, K, m, rej, fb, res,
+  const GsPlan p = gs_plan(g, wsp.dims.nmax, gs_limit(g.W));
+  auto go = [&](auto* kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
+    kernel<<<grid, gs_threads(g.W), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, cand, conf, K, m, rej, fb, res,
                                                 wsp, stats);
+  };
+  with_row_shape(g.W, [&](auto s) { go(k_fallback_round<decltype(s)>); });
 }
 
 void launch_fallback_resolve(int B, cudaStream_t st, int32_t* x, int n, const int32_t* pos, int k,

@@ -1,6 +1,8 @@
 // Whole-graph walks: one warp per validity check (kernel and launcher).
 #include <cuda_runtime.h>
 
+#define EPIC_STEP __noinline__  // column steps as calls (compile time)
+
 #include "launch.h"
 
 using namespace epic;
@@ -8,78 +10,22 @@ using namespace epic;
 // K2-K4 (warp form): one warp per validity check; warps pull checks from a
 // counter.  Each check walks the lexeme graph of x (+) (pos, tok) and runs
 // bit-parallel Earley recognition over it.
-// Copy the walk's grammar tables into shared memory and point `out` at them.
-__device__ void stage_grammar(const DevGrammar& g, unsigned char* smem, DevGrammar& out) {
-  out = g;
-  unsigned char* p = smem;
-  auto put = [&](const void* src, size_t bytes) -> void* {
-    void* dst = p;
-    const uint32_t* s4 = (const uint32_t*)src;
-    uint32_t* d4 = (uint32_t*)dst;
-    size_t n4 = bytes / 4;
-    for (size_t i = threadIdx.x; i < n4; i += blockDim.x) d4[i] = s4[i];
-    for (size_t i = n4 * 4 + threadIdx.x; i < bytes; i += blockDim.x)
-      ((unsigned char*)dst)[i] = ((const unsigned char*)src)[i];
-    p += (bytes + 15) & ~(size_t)15;
-    return dst;
-  };
-  out.exp_term = (const uint32_t*)put(g.exp_term, (size_t)g.T * g.W * 4);
-  out.exp_nt = (const uint32_t*)put(g.exp_nt, (size_t)g.V * g.W * 4);
-  out.pred = (const uint32_t*)put(g.pred, (size_t)g.V * g.W * 4);
-  out.gap_pred = (const uint32_t*)put(g.gap_pred, (size_t)g.V * g.W * 4);
-  out.any_nt = (const uint32_t*)put(g.any_nt, (size_t)g.W * 4);
-  out.any_term = (const uint32_t*)put(g.any_term, (size_t)g.W * 4);
-  out.next_any = (const uint32_t*)put(g.next_any, (size_t)g.W * 4);
-  out.nullable_next = (const uint32_t*)put(g.nullable_next, (size_t)g.W * 4);
-  out.complete = (const uint32_t*)put(g.complete, (size_t)g.W * 4);
-  out.item_next = (const int16_t*)put(g.item_next, (size_t)g.D * 2);
-  out.item_lhs = (const int16_t*)put(g.item_lhs, (size_t)g.D * 2);
-  out.dfa_accept = (const int16_t*)put(g.dfa_accept, (size_t)g.Q * 2);
-  out.dfa_ext = (const uint8_t*)put(g.dfa_ext, (size_t)g.Q);
-  out.skip = (const uint8_t*)put(g.skip, (size_t)g.T);
-  __syncthreads();
-}
-
-template <bool SM>
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_validate_warp(
+// zero_stage: the workspace is a shared array with earlier contents, so each
+// warp clears its own stage first (walks leave it zero).
+template <class S>
+__global__ void __launch_bounds__(32 * kWarpsPerCta, 2) k_validate_warp(
     DevGrammar g, const LexEntry* __restrict__ table, int vocab, const int32_t* __restrict__ x, int n,
     const int32_t* __restrict__ pos, int k, const int32_t* __restrict__ cand, int K, long long total,
-    uint8_t* __restrict__ valid, WPack wp, int rmax, int gtab_smem, unsigned long long* counter,
-    unsigned long long* stats) {
+    uint8_t* __restrict__ valid, WPack wp, int zero_stage, unsigned long long* counter, unsigned long long* stats) {
   __shared__ WSh shm[kWarpsPerCta];
-  extern __shared__ __align__(16) unsigned char dyn[];
-  int warp = threadIdx.x >> 5;
-  WSh& sh = shm[warp];
-  for (int w = threadIdx.x & 31; w < kWCols / 32; w += 32) {
-    sh.touched[w] = 0;
-    sh.dirty[w] = 0;
+  const int warp = threadIdx.x >> 5;
+  WWs ws = wp.carve((long long)blockIdx.x * (blockDim.x >> 5) + warp);
+  if (zero_stage) {
+    uint4* p = reinterpret_cast<uint4*>(ws.stage);
+    for (int i = threadIdx.x & 31; i < wp.nmax * (g.W / 4); i += 32) p[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
   }
-  for (int v = threadIdx.x & 31; v < kWMaxVW; v += 32) {
-    sh.vset[v] = 0;
-    sh.vdone[v] = 0;
-  }
-  __syncwarp();
-  // the grammar tables in shared memory when they fit (gtab > 0)
-  DevGrammar gs = g;
-  size_t gt = 0;
-  if constexpr (SM) {
-    if (gtab_smem) {
-      stage_grammar(g, dyn, gs);
-      gt = gtab_bytes(g.T, g.V, g.W, g.D, g.Q);
-    }
-  }
-  WarpWalker<SM> walk(gs, table, wp.carve((long long)blockIdx.x * (blockDim.x >> 5) + warp), sh, wp.nmax, wp.emax,
-                      vocab);
-  if constexpr (SM) {
-    size_t per = smem_per_warp(wp.nmax, rmax, g.W, g.VW);
-    unsigned char* base = dyn + gt + per * warp;
-    uint32_t* rows = (uint32_t*)base;
-    uint32_t* bd = rows + (size_t)rmax * g.W;
-    int32_t* sorg = (int32_t*)(bd + (size_t)rmax * g.VW);
-    uint32_t* ssum = (uint32_t*)(sorg + rmax);
-    int16_t* so = (int16_t*)(ssum + 2 * rmax);
-    walk.set_smem(rows, bd, so, sorg, ssum, rmax);
-  }
+  WarpWalker<S, false> walk(g, table, ws, shm[warp], wp.nmax, wp.emax, vocab);
   unsigned long long n_checks = 0, n_valid = 0, n_ovf = 0, n_bad = 0, n_cols = 0, n_ent = 0;
   for (;;) {
     long long jb = 0;
@@ -110,18 +56,14 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) k_validate_warp(
 
 namespace epic {
 
-void launch_validate_warp(bool sm, dim3 grid, dim3 block, size_t dyn, cudaStream_t st, const DevGrammar& g,
-                          const LexEntry* table, int vocab, const int32_t* x, int n, const int32_t* pos, int k,
-                          const int32_t* cand, int K, long long total, uint8_t* valid, const WPack& wp, int rmax,
-                          int gsm, unsigned long long* counter, unsigned long long* stats) {
-  if (sm) {
-    cudaFuncSetAttribute(k_validate_warp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    k_validate_warp<true><<<grid, block, dyn, st>>>(g, table, vocab, x, n, pos, k, cand, K, total, valid, wp, rmax,
-                                                    gsm, counter, stats);
-  } else {
-    k_validate_warp<false><<<grid, block, dyn, st>>>(g, table, vocab, x, n, pos, k, cand, K, total, valid, wp, rmax,
-                                                     gsm, counter, stats);
-  }
+void launch_validate_warp(dim3 grid, dim3 block, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
+                          const int32_t* x, int n, const int32_t* pos, int k, const int32_t* cand, int K,
+                          long long total, uint8_t* valid, const WPack& wp, int zero_stage,
+                          unsigned long long* counter, unsigned long long* stats) {
+  with_row_shape(g.W, [&](auto shape) {
+    k_validate_warp<decltype(shape)><<<grid, block, 0, st>>>(g, table, vocab, x, n, pos, k, cand, K, total, valid, wp,
+                                                             zero_stage, counter, stats);
+  });
 }
 
 int phase_read_walk(unsigned long long* out16, int reset) {

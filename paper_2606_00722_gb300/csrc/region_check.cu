@@ -1,14 +1,21 @@
 // Checks by region, step 3: one warp per check walks only the candidate's
-// region over the sequence's forward chart (see region.cuh).
-#pragma once
+// region over the sequence's forward chart (see region.cuh), with its
+// launcher.
+#include <cuda_runtime.h>
+
+// the walk's column steps as calls: inlined at each use, this file took more
+// than two minutes to compile
+#define EPIC_STEP __noinline__
+
+#include "launch.h"
 #include "region.cuh"
 
 namespace epic {
 
 // ------------------------------------------------------------------ 3. checks by region
-template <bool SM>
+template <class S>
 struct RegionCheck {
-  WarpWalker<SM, true>& w;
+  WarpWalker<S, true>& w;
   SeqArena& a;
   int32_t* fmap;     // [nmax] F node -> own column with carried rows (-1)
   int32_t* act;      // [nmax] own columns whose rows wait on nonterminals
@@ -21,11 +28,9 @@ struct RegionCheck {
     const int NF = meta[M_NCOLS];
     // base chart
     w.base_cols = NF;
-    w.base_ent = a.ws.col_off[NF];
     w.b_col_off = a.ws.col_off;
     w.b_org = a.ws.org;
     w.b_bits = a.ws.bits;
-    w.b_esum = a.ws.esum;
     w.good = a.good;
     w.b_eidx = a.eidx;
     w.accept_node = meta[M_ACCEPT];
@@ -153,10 +158,10 @@ struct RegionCheck {
         bool eps = true;
         for (int lw = 0; lw < 8; ++lw) eps &= L[lw] == 0;
         if (eps) {
-          w.arrive(oc, nullptr, false);
+          w.arrive(oc, false);
         } else {
           w.label_set(L);
-          w.arrive(oc, w.sh.lbl, true);
+          w.arrive(oc, true);
         }
       }
       // nested constituents from an earlier carrying node u completing at j
@@ -164,16 +169,15 @@ struct RegionCheck {
         int u = act[ai], uf = act_f[ai];
         long long kc = w.find_base(j, uf);
         if (kc < 0) continue;
-        for (int v = lane; v < w.VW; v += 32) w.sh.nt[v] = a.rec.cnt[(size_t)kc * w.VW + v];
-        __syncwarp();
-        uint32_t fold = 0;
-        for (int v = 0; v < w.VW; ++v) fold |= w.sh.nt[v];
-        if (!fold) continue;
-        expn_of_set(w.g, w.sh.nt, w.sh.expn);
-        __syncwarp();
+        const uint32_t set = lane < w.VW ? a.rec.cnt[(size_t)kc * w.VW + lane] : 0u;
+        if (!__any_sync(0xffffffffu, set != 0)) continue;
+        uint32_t ex[S::KW];
+        RowRegs<S>::waiting_on(set, w.g.exp_nt, w.W, w.VW, ex);
         w.col_labelled = true;  // new items to close, not a copy of a closed column
-        w.scatter(u, w.sh.expn, true, 0, fold);
-        if (w.status) return -1;
+        const int32_t* org;
+        const uint32_t* bits;
+        const int ne = w.column(u, org, bits);
+        w.template scatter<true>(w.hot(), org, bits, ne, ex);
       }
       w.close_column(c, a.rec.col_gap[j] != 0);
       w.finish_column(c);
@@ -223,37 +227,16 @@ struct RegScratch {
   int32_t* act_f;
 };
 
-template <bool SM>
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_check(
+template <class S>
+__global__ void __launch_bounds__(32 * kWarpsPerCta, 2) k_check(
     DevGrammar g, const LexEntry* __restrict__ table, int vocab, const int32_t* __restrict__ x, int n,
     const int32_t* __restrict__ pos, int k, const int32_t* __restrict__ cand, int K, long long total,
-    uint8_t* __restrict__ valid, SeqPack sp, WPack wp, int32_t* __restrict__ regs, int rmax,
-    unsigned long long* counter, unsigned long long* stats) {
+    uint8_t* __restrict__ valid, SeqPack sp, WPack wp, int32_t* __restrict__ regs, unsigned long long* counter,
+    unsigned long long* stats) {
   __shared__ WSh shm[kWarpsPerCta];
-  extern __shared__ __align__(16) unsigned char dyn[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  WSh& sh = shm[warp];
-  for (int w = lane; w < kWCols / 32; w += 32) {
-    sh.touched[w] = 0;
-    sh.dirty[w] = 0;
-  }
-  for (int v = lane; v < kWMaxVW; v += 32) {
-    sh.vset[v] = 0;
-    sh.vdone[v] = 0;
-  }
-  __syncwarp();
   const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
-  WarpWalker<SM, true> walk(g, table, wp.carve(gw), sh, wp.nmax, wp.emax, vocab);
-  if constexpr (SM) {
-    size_t per = smem_per_warp(wp.nmax, rmax, g.W, g.VW);
-    unsigned char* base = dyn + per * warp;
-    uint32_t* rows = (uint32_t*)base;
-    uint32_t* bd = rows + (size_t)rmax * g.W;
-    int32_t* sorg = (int32_t*)(bd + (size_t)rmax * g.VW);
-    uint32_t* ssum = (uint32_t*)(sorg + rmax);
-    int16_t* so = (int16_t*)(ssum + 2 * rmax);
-    walk.set_smem(rows, bd, so, sorg, ssum, rmax);
-  }
+  WarpWalker<S, true> walk(g, table, wp.carve(gw), shm[warp], wp.nmax, wp.emax, vocab);
   RegScratch rs;
   rs.fmap = regs + (size_t)gw * 3 * wp.nmax;
   rs.act = rs.fmap + wp.nmax;
@@ -278,21 +261,19 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) k_check(
       if (fs == 0) {
         r = 0;  // x is not completable, so no update of it is
       } else if (fs == 1) {
-        RegionCheck<SM> rc{walk, a, rs.fmap, rs.act, rs.act_f};
+        RegionCheck<S> rc{walk, a, rs.fmap, rs.act, rs.act_f};
         r = rc.run(xb, n, i, t);
         if (r < 0) walk.cleanup();
         own_cols = walk.ncols - walk.base_cols;
         own_ent = walk.nent;
       } else {  // the sequence's forward chart did not fit: walk the whole check
         walk.base_cols = 0;
-        walk.base_ent = 0;
         walk.suffix_mode = false;
         r = walk.run(xb, n, i, t);
         own_cols = walk.ncols;
         own_ent = walk.nent;
       }
       walk.base_cols = 0;
-      walk.base_ent = 0;
       walk.suffix_mode = false;
     }
     if (lane == 0) valid[jb] = r == 1 ? 1 : (r == -1 ? 2 : 0);
@@ -311,6 +292,33 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) k_check(
     atomicAdd(&stats[4], n_cols);
     atomicAdd(&stats[5], n_ent);
   }
+}
+
+void launch_check(dim3 grid, dim3 block, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
+                  const int32_t* x, int n, const int32_t* pos, int k, const int32_t* cand, int K, long long total,
+                  uint8_t* valid, const SeqPack& sp, const WPack& wp, int32_t* regs, unsigned long long* counter,
+                  unsigned long long* stats) {
+  with_row_shape(g.W, [&](auto shape) {
+    k_check<decltype(shape)><<<grid, block, 0, st>>>(g, table, vocab, x, n, pos, k, cand, K, total, valid, sp, wp,
+                                                     regs, counter, stats);
+  });
+}
+
+// measurement builds: this translation unit's phase counters of the walk
+int phase_read_check(unsigned long long* out16, int reset) {
+#ifdef EPIC_PHASE_TIMERS
+  unsigned long long h[16];
+  if (cudaMemcpyFromSymbol(h, g_phase, sizeof(h)) != cudaSuccess) return -1;
+  for (int i = 0; i < 16; ++i) out16[i] += h[i];
+  if (reset) {
+    unsigned long long z[16] = {0};
+    if (cudaMemcpyToSymbol(g_phase, z, sizeof(z)) != cudaSuccess) return -1;
+  }
+#else
+  (void)out16;
+  (void)reset;
+#endif
+  return 0;
 }
 
 }  // namespace epic

@@ -7,37 +7,103 @@
 
 namespace epic {
 
-// ------------------------------------------------------------------ 2. good masks
-// warp: dst |= src >> 1 over W words ((item i+1 good) => candidate i)
-__device__ __forceinline__ uint32_t shr1_word(const uint32_t* src, int w, int W) {
-  uint32_t v = src[w] >> 1;
-  if (w + 1 < W) v |= src[w + 1] << 31;
-  return v;
+constexpr int kGoodWarps = 16;          // one CTA per sequence
+constexpr int kGoodEdges = 32;          // out-edges whose label masks are held at once
+constexpr int kGoodMaxRounds = 1 << 18; // in-column rounds (each makes at least one item good)
+
+// Dynamic shared memory of the good pass (byte offsets).
+struct GoodPlan {
+  uint32_t o_masks;              // next_any [W]
+  uint32_t o_cpl_off, o_cpl;     // complete items by nonterminal
+  uint32_t o_wait_off, o_wait;   // waiting items by nonterminal
+  uint32_t o_exp;                // EXP_NT rows; 0: read from global memory
+  uint32_t o_scr;                // per-warp scratch, W words each
+  uint32_t o_cmp;                // per-warp list of a batch's active lanes
+  uint32_t o_lbl;                // label masks of a chunk of out-edges
+  uint32_t o_loc;                // entry of each origin in the open column (uint16), 0xFFFF none
+  uint32_t o_chg, o_nxt, o_open; // bitmaps over the open column's entries
+  uint32_t o_fold;               // folded completions of each successor
+  uint32_t o_sux;                // items waiting on what completes at a successor; sux rows
+  uint32_t o_row, o_gnt;         // good masks and good nonterminals of the open column; rows rows
+  int sux, rows;
+  uint32_t bytes;
+};
+
+static GoodPlan good_plan(const DevGrammar& g, int nmax) {
+  auto r = [](size_t b) { return (b + 15) & ~(size_t)15; };
+  const size_t limit = g.W <= 16 ? (size_t)108 * 1024 : (size_t)220 * 1024;
+  GoodPlan p;
+  size_t o = 0;
+  auto put = [&](size_t bytes) {
+    const size_t at = o;
+    o += r(bytes);
+    return (uint32_t)at;
+  };
+  p.o_masks = put((size_t)g.W * 4);
+  p.o_cpl_off = put((size_t)(g.V + 1) * 4);
+  p.o_cpl = put((size_t)g.n_cpl * 8);
+  p.o_wait_off = put((size_t)(g.V + 1) * 4);
+  p.o_wait = put((size_t)g.n_wait * 8);
+  p.o_scr = put((size_t)kGoodWarps * g.W * 4);
+  p.o_cmp = put((size_t)kGoodWarps * 32 * 4);
+  p.o_lbl = put((size_t)kGoodEdges * g.W * 4);
+  p.o_loc = put((size_t)nmax * 2);
+  const size_t bm = (size_t)((nmax + 31) / 32) * 4;
+  p.o_chg = put(bm);
+  p.o_nxt = put(bm);
+  p.o_open = put(bm);
+  p.o_fold = put((size_t)nmax * 4);
+  const size_t ex = (size_t)g.V * g.W * 4, per_row = (size_t)(2 * g.W + g.VW) * 4;
+  p.o_exp = o + r(ex) + 64 * per_row <= limit ? put(ex) : 0;
+  const size_t left = limit > o + 64 ? limit - o - 64 : 0;
+  long long rows = (long long)(left / per_row);
+  rows = rows > nmax ? nmax : (rows > 1024 ? 1024 : rows);
+  p.sux = p.rows = (int)rows;
+  p.o_sux = put((size_t)rows * g.W * 4);
+  p.o_row = put((size_t)rows * g.W * 4);
+  p.o_gnt = put((size_t)rows * g.VW * 4);
+  p.bytes = (uint32_t)o;
+  return p;
 }
 
-constexpr int kGoodWarps = 16;  // one CTA per sequence
-
-// Warp, row in registers: r |= bits & M & shr1(r) until stable -- an item is
-// good when it may advance within its own row and the advanced item is good.
-template <int KW>
-__device__ __forceinline__ void good_in_row(uint32_t (&r)[KW], const uint32_t (&bits)[KW], const uint32_t (&M)[KW],
-                                            int W) {
-  const int lane = threadIdx.x & 31;
+// Row in registers (a copy in every lane group, or one per group):
+// r |= bits & M & (r shifted down) until stable -- an item is good when it may
+// advance within its own row and the advanced item is good.
+template <class S>
+__device__ __forceinline__ void good_in_row(uint32_t (&r)[S::KW], const uint32_t (&bits)[S::KW],
+                                            const uint32_t (&M)[S::KW]) {
+  bool some = false;
+#pragma unroll
+  for (int i = 0; i < S::KW; ++i) some |= (bits[i] & M[i] & ~r[i]) != 0;
+  if (!__any_sync(0xffffffffu, some)) return;
   for (int it = 0; it < 64; ++it) {
+    uint32_t s[S::KW];
+    RowRegs<S>::shift_down(r, s);
     bool ch = false;
 #pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      if (32 * i >= W) break;
-      // bit b of word w takes bit b+1 (bit 0 of word w+1 for b = 31)
-      uint32_t nxt = __shfl_down_sync(0xffffffffu, r[i], 1);
-      const uint32_t wrap = (i + 1 < KW) ? __shfl_sync(0xffffffffu, r[i + 1], 0) : 0u;
-      if (lane == 31) nxt = wrap;
-      const uint32_t s = (r[i] >> 1) | (nxt << 31);
-      const uint32_t add = bits[i] & M[i] & s & ~r[i];
+    for (int i = 0; i < S::KW; ++i) {
+      const uint32_t add = bits[i] & M[i] & s[i] & ~r[i];
       ch |= add != 0;
       r[i] |= add;
     }
     if (!__any_sync(0xffffffffu, ch)) break;
+  }
+}
+
+// Block, one warp per array: a[1 .. n] becomes its inclusive prefix sums
+// (a[0] = 0).
+__device__ inline void warp_prefix(int32_t* a, int n) {
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  for (int i0 = 1; i0 <= n; i0 += 32) {
+    const int i = i0 + lane;
+    int s = i <= n ? a[i] : 0;
+    for (int off = 1; off < 32; off <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, s, off);
+      if (lane >= off) s += t;
+    }
+    if (i <= n) a[i] = base + s;
+    base += __shfl_sync(0xffffffffu, s, 31);
   }
 }
 
@@ -52,399 +118,552 @@ __device__ __forceinline__ void good_in_row(uint32_t (&r)[KW], const uint32_t (&
 //  - it is complete with left side B, and some item of column o, origin o2,
 //    waiting on B has its advanced item good at (j, o2).
 // The first three read later columns only (final); the in-row ones (gap,
-// nullable) close each row on its own.  The last one reads entries (j, o2)
-// of this column with o2 <= o, so the entries holding complete items are
-// closed in ascending origin order, once each: the whole CTA gathers which
-// completed nonterminals of (j, o) some waiting item of column o turns good,
-// then one warp closes (j, o) with its own self-loop (the entry of column o
-// with origin o maps back to (j, o)).
-__global__ void __launch_bounds__(32 * kGoodWarps, 1) k_good(DevGrammar g, int B, SeqPack sp) {
+// nullable) close each row on its own.  The last one reads rows of this
+// column, and runs in rounds over the entries with complete items, all warps
+// at once: a round looks at the pairs (j, o), (o, o2) whose row (j, o2)
+// changed in the round before, so a pair is read again only when it can add
+// something, and an entry whose completed nonterminals are all good is done.
+// Rounds end when no row changes; there are as many as completions nest at
+// one end node.  (One entry at a time in ascending origin order, with four
+// block barriers each, left the CTA at barriers for most of the pass.)
+//
+// The open column's good masks, the items waiting on what completes at each
+// successor column and the grammar lists sit in shared memory; rows beyond
+// the slots stay in global memory.  What is left is bound by the loads of
+// other columns' rows (several in flight per warp) and the barriers per round.
+template <class S>
+__global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(DevGrammar g, int B, SeqPack sp, GoodPlan p) {
   extern __shared__ __align__(16) unsigned char dyn[];
-  GsTables tb;
-  gs_stage_tables(g, dyn, tb);
+  using Row = RowRegs<S>;
+  constexpr int KW = S::KW, LR = S::LR, NG = S::NG;
+  constexpr int U = KW == 4 ? 4 : 2;  // rows in flight per lane group
+  const int li = Row::li(), gi = Row::gi();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
-  const int W = g.W, VW = g.VW;
-  constexpr int KW = kWMaxW / 32;  // item words per lane
-  __shared__ int s_self;
-  __shared__ uint32_t s_cn[kWMaxVW], s_bset[kWMaxVW];
-  __shared__ uint32_t s_expn[kWMaxW];
-  __shared__ uint32_t s_xall[kWMaxW];
-  __shared__ uint32_t s_items[kWMaxW];  // good-advanceable waiting items of the gather
-  __shared__ int s_flag;
+  const int W = g.W, VW = g.VW, V = g.V;
+  uint32_t* next_any = (uint32_t*)(dyn + p.o_masks);
+  int32_t* c_off = (int32_t*)(dyn + p.o_cpl_off);
+  uint2* c_lst = (uint2*)(dyn + p.o_cpl);
+  int32_t* w_off = (int32_t*)(dyn + p.o_wait_off);
+  uint2* w_lst = (uint2*)(dyn + p.o_wait);
+  uint32_t* scr = (uint32_t*)(dyn + p.o_scr) + (size_t)warp * W;
+  uint32_t* cmp = (uint32_t*)(dyn + p.o_cmp) + warp * 32;
+  const uint32_t s_row = gs_saddr(dyn + p.o_row);
+  uint32_t* lbl = (uint32_t*)(dyn + p.o_lbl);
+  uint16_t* loc = (uint16_t*)(dyn + p.o_loc);
+  uint32_t* open = (uint32_t*)(dyn + p.o_open);
+  uint32_t* sfold = (uint32_t*)(dyn + p.o_fold);
+  const uint32_t* exp_nt = g.exp_nt;
+  __shared__ int s_self, s_more, s_next;
+  __shared__ __align__(16) uint32_t s_xall[kWMaxW];
+  // the grammar lists
+  for (int i = tid; i < W; i += nthr) next_any[i] = g.next_any[i];
+  for (int i = tid; i <= V; i += nthr) {
+    c_off[i] = g.cpl_off[i];
+    w_off[i] = g.wait_off[i];
+  }
+  for (int i = tid; i < g.n_cpl; i += nthr) c_lst[i] = g.cpl[i];
+  for (int i = tid; i < g.n_wait; i += nthr) w_lst[i] = g.wait[i];
+  if (p.o_exp) {
+    uint32_t* ex = (uint32_t*)(dyn + p.o_exp);
+    for (int i = tid; i < V * W; i += nthr) ex[i] = g.exp_nt[i];
+    exp_nt = ex;
+  }
+  for (int i = tid; i < sp.nmax; i += nthr) loc[i] = 0xFFFFu;
+  __syncthreads();
+  // ---- warp helpers
+  // the active lanes of a batch, in order, with a value each: cmp[t] =
+  // value << 5 | lane; returns how many
+  auto compact = [&](bool active, int value) -> int {
+    const unsigned m = __ballot_sync(0xffffffffu, active);
+    __syncwarp();
+    if (active) cmp[__popc(m & ((1u << lane) - 1u))] = ((uint32_t)value << 5) | (uint32_t)lane;
+    __syncwarp();
+    return __popc(m);
+  };
+  // the nonterminals that the items of row wait on
+  auto waited = [&](const uint32_t(&row)[KW]) -> uint32_t {
+    if (lane < LR) Row::store(scr, W, row);
+    __syncwarp();
+    uint32_t mine = 0;
+    for (int v = 0; v < VW; ++v) {
+      const int A = (v << 5) + lane;
+      bool hit = false;
+      if (A < V)
+        for (int q = w_off[A], e = w_off[A + 1]; q < e && !hit; ++q) hit = (scr[w_lst[q].x] & w_lst[q].y) != 0;
+      const uint32_t b = __ballot_sync(0xffffffffu, hit);
+      if (lane == v) mine = b;
+    }
+    __syncwarp();
+    return mine;
+  };
+  // the complete items whose left side is in the set
+  auto completes = [&](uint32_t set, uint32_t(&c)[KW]) {
+    for (int w = lane; w < W; w += 32) scr[w] = 0;
+    __syncwarp();
+    for (int v = 0; v < VW; ++v) {
+      const uint32_t m = __shfl_sync(0xffffffffu, set, v);
+      if ((m >> lane) & 1u) {
+        const int A = (v << 5) + lane;
+        for (int q = c_off[A]; q < c_off[A + 1]; ++q) atomicOr(&scr[c_lst[q].x], c_lst[q].y);
+      }
+    }
+    __syncwarp();
+    Row::load(scr, W, c);
+    __syncwarp();
+  };
   for (long long b = blockIdx.x; b < B; b += gridDim.x) {
-  PH_BEGIN(t_setup);
-  SeqArena a = sp.carve(b);
-  int32_t* meta = a.rec.meta;
-  if (meta[M_STATUS] != 1) continue;
-  const int N = meta[M_NCOLS], NE = meta[M_NEDGES];
-  const int32_t* col = a.ws.col_off;
-  const int32_t* org = a.ws.org;
-  const int start = meta[M_START], accept = meta[M_ACCEPT];
-  int32_t* cur_o = a.cursor;          // [N + 1]
-  int32_t* cur_s = a.cursor + N + 1;  // [N + 1]
-  // edges by source and entries by origin (CSR), entry index by (column, origin)
-  for (int j = tid; j <= N; j += nthr) {
-    a.in_off[j] = 0;
-    a.out_off[j] = 0;
-    a.succ_off[j] = 0;
-  }
-  for (int u = tid; u < N; u += nthr) a.last_col[u] = -1;
-  const size_t ntri = (size_t)N * (N + 1) / 2;
-  for (size_t q = tid; q < ntri; q += nthr) a.eidx[q] = -1;
-  __syncthreads();
-  for (int e = tid; e < NE; e += nthr) {
-    atomicAdd(&a.in_off[a.rec.e_dst[e] + 1], 1);
-    atomicAdd(&a.out_off[a.rec.e_src[e] + 1], 1);
-  }
-  for (int j = warp; j < N; j += kGoodWarps)
-    for (long long k = col[j] + lane; k < col[j + 1]; k += 32) {
-      const int o = org[k];
-      a.eidx[tri_index(j, o)] = (int32_t)k;
-      a.gnz[k] = 0;
-      atomicAdd(&a.succ_off[o + 1], 1);
-      atomicMax(&a.last_col[o], j);
+    PH_BEGIN(t_setup);
+    SeqArena a = sp.carve(b);
+    int32_t* meta = a.rec.meta;
+    if (meta[M_STATUS] != 1) continue;
+    const int N = meta[M_NCOLS], NE = meta[M_NEDGES];
+    const int32_t* col = a.ws.col_off;
+    const int32_t* org = a.ws.org;
+    const uint32_t* bits_g = a.ws.bits;
+    const int start = meta[M_START], accept = meta[M_ACCEPT];
+    int32_t* cur_o = a.cursor;          // [N + 1]
+    int32_t* cur_s = a.cursor + N + 1;  // [N + 1]
+    // edges by source and entries by origin (CSR), entry index by (column, origin)
+    for (int j = tid; j <= N; j += nthr) {
+      a.in_off[j] = 0;
+      a.out_off[j] = 0;
+      a.succ_off[j] = 0;
     }
-  __syncthreads();
-  if (tid == 0)
-    for (int j = 0; j < N; ++j) {
-      a.in_off[j + 1] += a.in_off[j];
-      a.out_off[j + 1] += a.out_off[j];
-      a.succ_off[j + 1] += a.succ_off[j];
+    for (int u = tid; u < N; u += nthr) a.last_col[u] = -1;
+    const size_t ntri = (size_t)N * (N + 1) / 2;
+    for (size_t q = tid; q < ntri; q += nthr) a.eidx[q] = -1;
+    __syncthreads();
+    for (int e = tid; e < NE; e += nthr) {
+      atomicAdd(&a.in_off[a.rec.e_dst[e] + 1], 1);
+      atomicAdd(&a.out_off[a.rec.e_src[e] + 1], 1);
     }
-  __syncthreads();
-  for (int j = tid; j < N; j += nthr) {
-    cur_o[j] = a.out_off[j];
-    cur_s[j] = a.succ_off[j];
-  }
-  __syncthreads();
-  for (int e = tid; e < NE; e += nthr) a.out_idx[atomicAdd(&cur_o[a.rec.e_src[e]], 1)] = e;
-  for (int j = warp; j < N; j += kGoodWarps)
-    for (long long k = col[j] + lane; k < col[j + 1]; k += 32) a.succ_idx[atomicAdd(&cur_s[org[k]], 1)] = j;
-  __syncthreads();
-
-  PH_END(0, t_setup);
-  uint32_t* G = a.good;
-  uint32_t* sfold = (uint32_t*)a.cursor;  // per successor of the column (the cursors are free now)
-  for (int w = tid; w < kWMaxW; w += nthr) s_items[w] = 0;
-  __syncthreads();
-  for (int j = N - 1; j >= 0; --j) {
-    const int s0 = a.succ_off[j], s1 = a.succ_off[j + 1];
-    const bool gap = a.rec.col_gap[j] != 0;
-    const long long k0 = col[j], k1 = col[j + 1];
-    if (k0 == k1) continue;
-    // EXPN of what completes from origin j at each column j2 (j2 = j included)
-    PH_BEGIN(t_succ);
-    if (tid == 0) s_self = -1;
-    __syncthreads();
-    for (int si = s0 + tid; si < s1; si += nthr)
-      if (a.succ_idx[si] == j) s_self = si - s0;
-    __syncthreads();
-    const int self_si = s_self;
-    for (int si = s0 + warp; si < s1; si += kGoodWarps) {
-      const int j2 = a.succ_idx[si];
-      const uint32_t* cn = a.rec.cnt + (size_t)a.eidx[tri_index(j2, j)] * VW;
-      uint32_t f = 0;
-      for (int v = 0; v < VW; ++v) f |= cn[v];
-      if (f) expn_of_set(g, cn, a.expn + (size_t)(si - s0) * W);
-      if (lane == 0) sfold[si - s0] = f;  // folded (bit C mod 32): 0 = nothing completes
-    }
-    __syncthreads();
-    // union of the completion masks of the successors after j
-    for (int w = tid; w < W; w += nthr) {
-      uint32_t u = 0;
-      for (int si = s0; si < s1; ++si)
-        if (si - s0 != self_si && sfold[si - s0]) u |= a.expn[(size_t)(si - s0) * W + w];
-      s_xall[w] = u;
-    }
-    __syncthreads();
-    PH_END(1, t_succ);
-    // in-row rules of this column: the gap self-loop and nullable completions
-    PH_BEGIN(t_a);
-    uint32_t inrow[KW];
-#pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      const int w = lane + 32 * i;
-      uint32_t m = 0;
-      if (w < W) {
-        if (gap) m |= tb.next_any[w];
-        if (self_si >= 0 && sfold[self_si]) m |= a.expn[(size_t)self_si * W + w];
+    for (int j = warp; j < N; j += kGoodWarps)
+      for (long long k = col[j] + lane; k < col[j + 1]; k += 32) {
+        const int o = org[k];
+        a.eidx[tri_index(j, o)] = (int32_t)k;
+        a.gnz[k] = 0;
+        atomicAdd(&a.succ_off[o + 1], 1);
+        atomicMax(&a.last_col[o], j);
       }
-      inrow[i] = m;
+    __syncthreads();
+    if (warp < 3) warp_prefix(warp == 0 ? a.in_off : (warp == 1 ? a.out_off : a.succ_off), N);
+    __syncthreads();
+    for (int j = tid; j < N; j += nthr) {
+      cur_o[j] = a.out_off[j];
+      cur_s[j] = a.succ_off[j];
     }
-    // A. the rules that read later columns, then the in-row closure (one warp
-    //    per entry)
-    for (long long k = k0 + warp; k < k1; k += kGoodWarps) {
-      const int o = org[k];
-      const uint32_t* bp = a.ws.bits + (size_t)k * W;
-      uint32_t acc[KW], bits[KW];
+    __syncthreads();
+    for (int e = tid; e < NE; e += nthr) a.out_idx[atomicAdd(&cur_o[a.rec.e_src[e]], 1)] = e;
+    for (int j = warp; j < N; j += kGoodWarps)
+      for (long long k = col[j] + lane; k < col[j + 1]; k += 32) a.succ_idx[atomicAdd(&cur_s[org[k]], 1)] = j;
+    __syncthreads();
+    PH_END(0, t_setup);
+    uint32_t* G = a.good;
+    for (int j = N - 1; j >= 0; --j) {
+      const int s0 = a.succ_off[j], s1 = a.succ_off[j + 1];
+      const bool gap = a.rec.col_gap[j] != 0;
+      const int k0 = col[j], ne = col[j + 1] - k0;
+      if (ne == 0) continue;
+      uint32_t* chg = (uint32_t*)(dyn + p.o_chg);
+      uint32_t* nxt = (uint32_t*)(dyn + p.o_nxt);
+      auto row_of = [&](int e) -> uint32_t* {
+        return e < p.rows ? (uint32_t*)(dyn + p.o_row) + (size_t)e * W : G + (size_t)(k0 + e) * W;
+      };
+      auto gnt_of = [&](int e) -> uint32_t* {  // overflow: the forward walk's completion record is free
+        return e < p.rows ? (uint32_t*)(dyn + p.o_gnt) + (size_t)e * VW : a.bdone + (size_t)e * VW;
+      };
+      auto sux_of = [&](int s) -> uint32_t* {
+        return s < p.sux ? (uint32_t*)(dyn + p.o_sux) + (size_t)s * W : a.expn + (size_t)s * W;
+      };
+      // a row that its owner may be writing (bits only get set)
+      auto load_good = [&](int e, uint32_t(&v)[KW]) {
+        if (e < p.rows) {
+          Row::load_shared(s_row + (uint32_t)e * (uint32_t)(W * 4), W, v);
+        } else {
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        acc[i] = 0;
-        bits[i] = (w < W) ? bp[w] : 0u;
-      }
-      if (j == accept && o == start && lane == ((g.accept_item >> 5) & 31))
-        acc[g.accept_item >> 10] |= 1u << (g.accept_item & 31);
-      for (int ei = a.out_off[j]; ei < a.out_off[j + 1]; ++ei) {
-        const int e = a.out_idx[ei];
-        const int k2 = a.eidx[tri_index(a.rec.e_dst[e], o)];
-        if (k2 < 0 || !a.gnz[k2]) continue;
-        const uint32_t* G2 = G + (size_t)k2 * W;
-        const uint32_t* L = a.rec.e_lbl + (size_t)e * 8;
-        uint32_t lw8[8];
-        bool eps = true;
-        for (int lw = 0; lw < 8; ++lw) {
-          lw8[lw] = L[lw];
-          eps &= lw8[lw] == 0;
+          for (int i = 0; i < KW; ++i)
+            v[i] = li * KW + i < W ? *(volatile const uint32_t*)(G + (size_t)(k0 + e) * W + li * KW + i) : 0u;
         }
+      };
+      // in-row rules of this column: the gap self-loop and nullable completions
+      auto in_row = [&](uint32_t(&m)[KW], bool gp, int self_si) {
+        if (gp) {
+          Row::load(next_any, W, m);
+        } else {
 #pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          const int w = lane + 32 * i;
-          if (w < W) {
-            if (eps) {
-              acc[i] |= G2[w];
-            } else {
-              uint32_t m = 0;
-              for (int lw = 0; lw < 8; ++lw) {
-                uint32_t lm = lw8[lw];
-                while (lm) {
-                  const int bb = __ffs(lm) - 1;
-                  lm &= lm - 1;
-                  const int t = (lw << 5) + bb;
-                  if (t < g.T) m |= g.exp_term[(size_t)t * W + w];
-                }
-              }
-              acc[i] |= m & shr1_word(G2, w, W);
-            }
-          }
+          for (int i = 0; i < KW; ++i) m[i] = 0u;
         }
-      }
-      const uint32_t wfold = a.ws.esum[(size_t)k * 2];  // waited nonterminals, folded
-      // the most the nested rule can make good: items waiting on a
-      // nonterminal that completes from j somewhere after j
-      uint32_t want[KW];
+        if (self_si >= 0 && sfold[self_si]) {
+          uint32_t x[KW];
+          Row::load(sux_of(self_si), W, x);
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        want[i] = (w < W) ? (bits[i] & s_xall[w]) : 0u;
-      }
-      for (int sb = s0; sb < s1; sb += 32) {
-        bool open = false;
-#pragma unroll
-        for (int i = 0; i < KW; ++i) open |= (want[i] & ~acc[i]) != 0;
-        if (!__any_sync(0xffffffffu, open)) break;
-        const int si = sb + lane;
-        int k3 = -1;
-        if (si < s1 && si - s0 != self_si && (sfold[si - s0] & wfold) != 0) {
-          const int kk = a.eidx[tri_index(a.succ_idx[si], o)];
-          if (kk >= 0 && a.gnz[kk]) k3 = kk;
+          for (int i = 0; i < KW; ++i) m[i] |= x[i];
         }
-        unsigned act = __ballot_sync(0xffffffffu, k3 >= 0);
-        while (act) {
-          const int l = __ffs(act) - 1;
-          act &= act - 1;
-          const int kk = __shfl_sync(0xffffffffu, k3, l);
-          const uint32_t* ex = a.expn + (size_t)(sb + l - s0) * W;
-          const uint32_t* G3 = G + (size_t)kk * W;
-#pragma unroll
-          for (int i = 0; i < KW; ++i) {
-            const int w = lane + 32 * i;
-            if (w < W) {
-              const uint32_t xw = ex[w];
-              if (xw) acc[i] |= xw & shr1_word(G3, w, W);
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < KW; ++i) acc[i] &= bits[i];
-      good_in_row<KW>(acc, bits, inrow, W);
-      bool nz = false;
-      uint32_t* Gk = G + (size_t)k * W;
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        const int w = lane + 32 * i;
-        if (w < W) Gk[w] = acc[i];
-        nz |= acc[i] != 0;
-      }
-      nz = __any_sync(0xffffffffu, nz);
-      if (lane == 0) a.gnz[k] = nz ? 1 : 0;
-    }
-    __syncthreads();
-    PH_END(2, t_a);
-    // B. completions within the column, entries with complete items in
-    //    ascending origin order
-    for (long long k = k0; k < k1; ++k) {
-      const int o = org[k];
-      const uint32_t* cn = a.rec.cnt + (size_t)k * VW;
-      for (int v = tid; v < VW; v += nthr) {
-        s_cn[v] = cn[v];
-        s_bset[v] = 0;
-      }
+      };
+      // what completes from origin j at each column j2 (j2 = j included): the
+      // items waiting on it, and their union over the successors after j
+      PH_BEGIN(t_succ);
       if (tid == 0) {
-        uint32_t f = 0;
-        for (int v = 0; v < VW; ++v) f |= cn[v];
-        s_flag = f != 0;
+        s_self = -1;
+        s_next = 0;
+      }
+      for (int w = tid; w < W; w += nthr) s_xall[w] = 0;
+      for (int e = tid; e < ne; e += nthr) loc[org[k0 + e]] = (uint16_t)e;
+      for (int w = tid; w < ((ne + 31) >> 5); w += nthr) {
+        chg[w] = 0;
+        nxt[w] = 0;
+        open[w] = 0;
       }
       __syncthreads();
-      if (!s_flag) continue;  // no complete item here
-      // items waiting on a nonterminal completed at (j, o)
-      for (int w = tid; w < W; w += nthr) {
-        uint32_t acc = 0, m = tb.any_nt[w];
-        while (m) {
-          const int bb = __ffs(m) - 1;
-          m &= m - 1;
-          const int Bn = tb.item_next[(w << 5) + bb] - g.T;
-          if ((s_cn[Bn >> 5] >> (Bn & 31)) & 1u) acc |= 1u << bb;
-        }
-        s_expn[w] = acc;
-      }
-      __syncthreads();
-      PH_BEGIN(t_g);
-      // which of them some entry (o, o2 < o) of column o turns good at (j, o2):
-      // each warp ORs, over its entries of column o, the waiting items whose
-      // advance is good into registers (one operation per word); the items
-      // become nonterminals once, at the end
-      const int cb = col[o], ce = col[o + 1];
-      const bool self = ce > cb && org[ce - 1] == o;
-      const int nent = self ? ce - cb - 1 : ce - cb;
-      {
-        uint32_t ex[KW], acc[KW];
+      for (int si = s0 + warp; si < s1; si += kGoodWarps) {
+        const int j2 = a.succ_idx[si];
+        const uint32_t* cn = a.rec.cnt + (size_t)a.eidx[tri_index(j2, j)] * VW;
+        const uint32_t set = lane < VW ? cn[lane] : 0u;
+        const uint32_t f = __reduce_or_sync(0xffffffffu, set);  // folded (bit C mod 32): 0 = nothing completes
+        if (j2 == j && lane == 0) s_self = si - s0;
+        if (f) {
+          uint32_t ex[KW];
+          Row::waiting_on(set, exp_nt, W, VW, ex);
+          if (lane < LR) {
+            Row::store(sux_of(si - s0), W, ex);
+            if (j2 != j) {
 #pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          const int w = lane + 32 * i;
-          ex[i] = (w < W) ? s_expn[w] : 0u;
-          acc[i] = 0u;
-        }
-        for (int e = warp; e < nent; e += kGoodWarps) {
-          const int kp = cb + e;
-          const int kk = a.eidx[tri_index(j, org[kp])];
-          if (kk < 0 || !a.gnz[kk]) continue;
-          const uint32_t* P = a.ws.bits + (size_t)kp * W;
-          const uint32_t* GK = G + (size_t)kk * W;
-          uint32_t pv[KW], gv[KW];
-#pragma unroll
-          for (int i = 0; i < KW; ++i) {
-            const int w = lane + 32 * i;
-            pv[i] = ex[i] ? (P[w] & ex[i]) : 0u;
-            gv[i] = (w < W) ? GK[w] : 0u;
-          }
-#pragma unroll
-          for (int i = 0; i < KW; ++i) {
-            if (32 * i >= W) break;
-            // bit b of word w takes bit b + 1 of G (bit 0 of word w + 1 for b = 31)
-            uint32_t nxt = __shfl_down_sync(0xffffffffu, gv[i], 1);
-            const uint32_t wrap = (i + 1 < KW) ? __shfl_sync(0xffffffffu, gv[i + 1], 0) : 0u;
-            if (lane == 31) nxt = wrap;
-            acc[i] |= pv[i] & ((gv[i] >> 1) | (nxt << 31));
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          const int w = lane + 32 * i;
-          if (w < W && acc[i]) atomicOr(&s_items[w], acc[i]);
-        }
-      }
-      __syncthreads();
-      for (int w = tid; w < W; w += nthr) {
-        uint32_t m = s_items[w];
-        s_items[w] = 0;  // ready for the next entry
-        while (m) {
-          const int bb = __ffs(m) - 1;
-          m &= m - 1;
-          const int Bn = tb.item_next[(w << 5) + bb] - g.T;
-          const uint32_t bit = 1u << (Bn & 31);
-          if (!(s_bset[Bn >> 5] & bit)) atomicOr(&s_bset[Bn >> 5], bit);
-        }
-      }
-      __syncthreads();
-      PH_END(3, t_g);
-      // one warp: complete items with a good left side, the in-row closure,
-      // and the self-loop through the entry of column o with origin o
-      PH_BEGIN(t_w);
-      if (warp == 0) {
-        const uint32_t* bp = a.ws.bits + (size_t)k * W;
-        const uint32_t* E = self ? a.ws.bits + (size_t)(ce - 1) * W : nullptr;
-        uint32_t* Gk = G + (size_t)k * W;
-        uint32_t r[KW], bits[KW];
-#pragma unroll
-        for (int i = 0; i < KW; ++i) {
-          const int w = lane + 32 * i;
-          r[i] = (w < W) ? Gk[w] : 0u;
-          bits[i] = (w < W) ? bp[w] : 0u;
-        }
-        bool any_change = false;
-        for (int round = 0; round < 64 * kWMaxW; ++round) {
-          // the self entry's waiting items whose advance is good at (j, o)
-          if (self) {
-#pragma unroll
-            for (int i = 0; i < KW; ++i) {
-              if (32 * i >= W) break;
-              const int w = lane + 32 * i;
-              uint32_t nxt = __shfl_down_sync(0xffffffffu, r[i], 1);
-              const uint32_t wrap = (i + 1 < KW) ? __shfl_sync(0xffffffffu, r[i + 1], 0) : 0u;
-              if (lane == 31) nxt = wrap;
-              const uint32_t sh1 = (r[i] >> 1) | (nxt << 31);
-              uint32_t m = (w < W) ? (E[w] & s_expn[w] & sh1) : 0u;
-              while (m) {
-                const int bb = __ffs(m) - 1;
-                m &= m - 1;
-                const int Bn = tb.item_next[(w << 5) + bb] - g.T;
-                const uint32_t bit = 1u << (Bn & 31);
-                if (!(s_bset[Bn >> 5] & bit)) atomicOr(&s_bset[Bn >> 5], bit);
-              }
-            }
-            __syncwarp();
-          }
-          // complete items whose left side is turned good
-          bool ch = false;
-#pragma unroll
-          for (int i = 0; i < KW; ++i) {
-            const int w = lane + 32 * i;
-            uint32_t m = (w < W) ? (bits[i] & tb.complete[w] & ~r[i]) : 0u;
-            while (m) {
-              const int bb = __ffs(m) - 1;
-              m &= m - 1;
-              const int L2 = tb.item_lhs[(w << 5) + bb];
-              if ((s_bset[L2 >> 5] >> (L2 & 31)) & 1u) {
-                r[i] |= 1u << bb;
-                ch = true;
-              }
+              for (int i = 0; i < KW; ++i)
+                if (ex[i] & ~*(volatile uint32_t*)&s_xall[min(li * KW + i, kWMaxW - 1)])
+                  atomicOr(&s_xall[li * KW + i], ex[i]);
             }
           }
-          if (!__any_sync(0xffffffffu, ch)) break;
-          any_change = true;
-          good_in_row<KW>(r, bits, inrow, W);
-          if (!self) break;
         }
-        if (any_change) {
+        if (lane == 0) sfold[si - s0] = f;
+      }
+      // A. the rules that read later columns: out-edges, a chunk at a time
+      const int eb0 = a.out_off[j], eb1 = a.out_off[j + 1];
+      int chunk = eb0;
+      do {
+        const int nc = min(kGoodEdges, eb1 - chunk);
+        __syncthreads();
+        for (int q = warp; q < nc; q += kGoodWarps) {  // label masks of the chunk
+          const uint32_t* L = a.rec.e_lbl + (size_t)a.out_idx[chunk + q] * 8;
+          uint32_t m[KW];
+#pragma unroll
+          for (int i = 0; i < KW; ++i) m[i] = 0u;
+          int seen = 0;
+          for (int lw = 0; lw < 8; ++lw) {  // the lane groups share out the terminals
+            uint32_t lm = L[lw];
+            while (lm) {
+              const int t = (lw << 5) + __ffs(lm) - 1;
+              lm &= lm - 1;
+              if ((seen++ & (NG - 1)) != gi || t >= g.T) continue;
+              uint32_t x[KW];
+              Row::load(g.exp_term + (size_t)t * W, W, x);
+#pragma unroll
+              for (int i = 0; i < KW; ++i) m[i] |= x[i];
+            }
+          }
+          __syncwarp();
+          Row::join(m);
+          if (lane < LR) Row::store(lbl + (size_t)q * W, W, m);
+        }
+        __syncthreads();
+        PH_END(1, t_succ);
+        PH_BEGIN(t_a);
+        // this lane's edge of the chunk
+        int dst = -1;
+        bool eps = true;
+        if (lane < nc) {
+          const int e = a.out_idx[chunk + lane];
+          dst = a.rec.e_dst[e];
+          for (int lw = 0; lw < 8; ++lw) eps &= a.rec.e_lbl[(size_t)e * 8 + lw] == 0u;
+        }
+        const unsigned epsm = __ballot_sync(0xffffffffu, eps);
+        const bool first = chunk == eb0, last = chunk + nc >= eb1;
+        const int self_si = s_self;
+        uint32_t inrow[KW];  // in-row rules of this column: the gap self-loop and nullable completions
+        in_row(inrow, gap, self_si);
+        for (int e = warp; e < ne; e += kGoodWarps) {
+          const size_t k = (size_t)k0 + e;
+          const int o = org[k];
+          uint32_t* Gk = row_of(e);
+          uint32_t acc[KW], bits[KW];
+          // the lane groups take different edges and successors, and their
+          // parts are joined; `bits` is in every group
+          Row::load(bits_g + k * W, W, bits);
+          if (first) {
+#pragma unroll
+            for (int i = 0; i < KW; ++i) acc[i] = 0u;
+          } else {
+            Row::load(Gk, W, acc);
+          }
+          if (j == accept && o == start) {
+#pragma unroll
+            for (int i = 0; i < KW; ++i)
+              if (li * KW + i == (g.accept_item >> 5)) acc[i] |= 1u << (g.accept_item & 31);
+          }
+          int k2 = dst >= 0 ? a.eidx[tri_index(dst, o)] : -1;
+          if (k2 >= 0 && !a.gnz[k2]) k2 = -1;
+          const int na = compact(k2 >= 0, k2);
+          for (int t0 = 0; t0 < na; t0 += NG * U) {
+            uint32_t gv[U][KW];
+            int l[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int t = t0 + u * NG + gi;  // this group's edge: the t-th active one
+              l[u] = -1;
+              if (t < na) {
+                l[u] = cmp[t] & 31;
+                Row::load(G + (size_t)(cmp[t] >> 5) * W, W, gv[u]);
+              } else {
+#pragma unroll
+                for (int i = 0; i < KW; ++i) gv[u][i] = 0u;
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              uint32_t s[KW], m[KW];
+              Row::shift_down(gv[u], s);
+              const bool ep = l[u] >= 0 && ((epsm >> l[u]) & 1u);
+              Row::load(lbl + (size_t)(l[u] < 0 ? 0 : l[u]) * W, W, m);
+#pragma unroll
+              for (int i = 0; i < KW; ++i) acc[i] |= ep ? gv[u][i] : (s[i] & m[i]);
+            }
+          }
+          Row::join(acc);
+          if (last) {
+            const uint32_t wfold = a.rec.esum[k * 2];  // waited nonterminals, folded
+            // the most the nested rule can make good: items waiting on a
+            // nonterminal that completes from j somewhere after j
+            uint32_t want[KW];
+#pragma unroll
+            for (int i = 0; i < KW; ++i) want[i] = bits[i] & s_xall[min(li * KW + i, kWMaxW - 1)];
+            auto saturated = [&]() {
+              bool left = false;
+#pragma unroll
+              for (int i = 0; i < KW; ++i) left |= (want[i] & ~acc[i]) != 0;
+              return !__any_sync(0xffffffffu, left);
+            };
+            for (int sb = s0; sb < s1; sb += 32) {
+              if (saturated()) break;
+              const int si = sb + lane;
+              int k3 = -1;
+              if (si < s1 && si - s0 != self_si && (sfold[si - s0] & wfold) != 0) {
+                const int kk = a.eidx[tri_index(a.succ_idx[si], o)];
+                if (kk >= 0 && a.gnz[kk]) k3 = kk;
+              }
+              const int n3 = compact(k3 >= 0, k3);
+              for (int t0 = 0; t0 < n3; t0 += NG * U) {
+                uint32_t gv[U][KW], xv[U][KW];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                  const int t = t0 + u * NG + gi;
+                  if (t < n3) {
+                    Row::load(G + (size_t)(cmp[t] >> 5) * W, W, gv[u]);
+                    Row::load(sux_of(sb + (int)(cmp[t] & 31) - s0), W, xv[u]);
+                  } else {
+#pragma unroll
+                    for (int i = 0; i < KW; ++i) gv[u][i] = xv[u][i] = 0u;
+                  }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                  uint32_t s[KW];
+                  Row::shift_down(gv[u], s);
+#pragma unroll
+                  for (int i = 0; i < KW; ++i) acc[i] |= s[i] & xv[u][i];
+                }
+                Row::join(acc);
+                if (t0 + NG * U < n3 && saturated()) break;
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < KW; ++i) acc[i] &= bits[i];
+            good_in_row<S>(acc, bits, inrow);
+          }
           bool nz = false;
 #pragma unroll
-          for (int i = 0; i < KW; ++i) {
-            const int w = lane + 32 * i;
-            if (w < W) Gk[w] = r[i];
-            nz |= r[i] != 0;
+          for (int i = 0; i < KW; ++i) nz |= acc[i] != 0;
+          __syncwarp();
+          if (lane < LR) Row::store(Gk, W, acc);
+          if (last) {
+            nz = __any_sync(0xffffffffu, nz);
+            const uint32_t cn = lane < VW ? a.rec.cnt[k * VW + lane] : 0u;
+            const bool cpl = __any_sync(0xffffffffu, cn != 0);
+            if (lane < VW) gnt_of(e)[lane] = 0;
+            if (lane == 0) {
+              if (nz) atomicOr(&chg[e >> 5], 1u << (e & 31));
+              if (cpl) atomicOr(&open[e >> 5], 1u << (e & 31));
+            }
           }
-          nz = __any_sync(0xffffffffu, nz);
-          if (lane == 0 && nz) a.gnz[k] = 1;
+        }
+        PH_END(2, t_a);
+        chunk += nc;
+      } while (chunk < eb1);
+      __syncthreads();
+      // B. completions within the column, in rounds (see above)
+      PH_BEGIN(t_g);
+      for (int round = 0;; ++round) {
+        if (tid == 0) s_more = 0;
+        __syncthreads();
+        const int sel = s_self;
+        for (;;) {
+          int e = 0;
+          if (lane == 0) e = atomicAdd(&s_next, 1);
+          e = __shfl_sync(0xffffffffu, e, 0);
+          if (e >= ne) break;
+          if (!((open[e >> 5] >> (e & 31)) & 1u)) continue;
+          const size_t k = (size_t)k0 + e;
+          const int o = org[k];
+          uint32_t* gnt = gnt_of(e);
+          const uint32_t gn = lane < VW ? gnt[lane] : 0u;
+          uint32_t nt = lane < VW ? (a.rec.cnt[k * VW + lane] & ~gn) : 0u;  // completed, not known good
+          uint32_t found = 0, ex[KW];
+          bool have = false;
+          const int cb = col[o], ce = col[o + 1];
+          for (int c0 = cb; c0 < ce; c0 += 32) {
+            const int kp = c0 + lane;
+            int l2 = 0xFFFF;
+            if (kp < ce) l2 = loc[org[kp]];
+            const bool live = l2 != 0xFFFF && ((chg[l2 >> 5] >> (l2 & 31)) & 1u);
+            const int na = compact(live, l2);
+            if (na == 0) continue;
+            if (!have) {
+              Row::waiting_on(nt, exp_nt, W, VW, ex);
+              have = true;
+            }
+            uint32_t acc[KW];
+#pragma unroll
+            for (int i = 0; i < KW; ++i) acc[i] = 0u;
+            for (int t0 = 0; t0 < na; t0 += NG * U) {
+              uint32_t pv[U][KW];
+              int ee[U];
+#pragma unroll
+              for (int u = 0; u < U; ++u) {
+                const int t = t0 + u * NG + gi;
+                if (t < na) {
+                  ee[u] = (int)(cmp[t] >> 5);
+                  Row::load(bits_g + (size_t)(c0 + (int)(cmp[t] & 31)) * W, W, pv[u]);
+                } else {
+                  ee[u] = e;
+#pragma unroll
+                  for (int i = 0; i < KW; ++i) pv[u][i] = 0u;
+                }
+              }
+#pragma unroll
+              for (int u = 0; u < U; ++u) {
+                uint32_t gv[KW], s[KW];
+                load_good(ee[u], gv);
+                Row::shift_down(gv, s);
+#pragma unroll
+                for (int i = 0; i < KW; ++i) acc[i] |= pv[u][i] & s[i];
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < KW; ++i) acc[i] &= ex[i];
+            Row::join(acc);
+            bool any = false;
+#pragma unroll
+            for (int i = 0; i < KW; ++i) any |= acc[i] != 0;
+            if (!__any_sync(0xffffffffu, any)) continue;
+            const uint32_t nw = waited(acc) & nt;
+            found |= nw;
+            nt &= ~nw;
+            if (!__any_sync(0xffffffffu, nt != 0)) break;  // every completed nonterminal is good
+          }
+          if (!__any_sync(0xffffffffu, found != 0)) continue;
+          // complete items with a good left side, the in-row closure, and the
+          // loop through the entry of column o with origin o (which maps back
+          // to this row)
+          uint32_t r[KW], bits[KW], inrow[KW];
+          uint32_t* Gk = row_of(e);
+          Row::load(Gk, W, r);
+          Row::load(bits_g + k * W, W, bits);
+          in_row(inrow, gap, sel);
+          const bool self = ce > cb && org[ce - 1] == o;
+          uint32_t fresh = found;
+          bool changed = false;
+          for (int it = 0; it < 64 * kWMaxW; ++it) {
+            uint32_t cm[KW];
+            completes(fresh, cm);
+            bool ch = false;
+#pragma unroll
+            for (int i = 0; i < KW; ++i) {
+              const uint32_t add = bits[i] & cm[i] & ~r[i];
+              ch |= add != 0;
+              r[i] |= add;
+            }
+            if (!__any_sync(0xffffffffu, ch)) break;
+            changed = true;
+            good_in_row<S>(r, bits, inrow);
+            if (!self || !__any_sync(0xffffffffu, nt != 0)) break;
+            uint32_t s[KW], x[KW];
+            Row::shift_down(r, s);
+            Row::load(bits_g + (size_t)(ce - 1) * W, W, x);
+#pragma unroll
+            for (int i = 0; i < KW; ++i) x[i] &= ex[i] & s[i];
+            fresh = waited(x) & nt;
+            if (!__any_sync(0xffffffffu, fresh != 0)) break;
+            found |= fresh;
+            nt &= ~fresh;
+          }
+          if (lane < VW) gnt[lane] = gn | found;
+          if (!__any_sync(0xffffffffu, nt != 0) && lane == 0) atomicAnd(&open[e >> 5], ~(1u << (e & 31)));
+          if (changed) {
+            __syncwarp();
+            if (lane < LR) Row::store(Gk, W, r);
+            if (lane == 0) {
+              atomicOr(&nxt[e >> 5], 1u << (e & 31));
+              s_more = 1;
+            }
+          }
+        }
+        __syncthreads();
+        uint32_t* t = chg;
+        chg = nxt;
+        nxt = t;
+        const bool more = s_more != 0;
+        for (int w = tid; w < ((ne + 31) >> 5); w += nthr) nxt[w] = 0;
+        if (tid == 0) s_next = 0;
+        if (!more) break;
+        if (round > kGoodMaxRounds) {  // cannot happen; the checks would walk whole
+          if (tid == 0) meta[M_STATUS] = -1;
+          break;
+        }
+        __syncthreads();
+      }
+      PH_END(3, t_g);
+      // the column's masks to global memory
+      PH_BEGIN(t_w);
+      for (int e0 = warp * NG; e0 < ne; e0 += kGoodWarps * NG) {
+        const int e = e0 + gi;
+        bool nz = false;
+        if (e < ne) {
+          uint32_t v[KW];
+          Row::load(row_of(e), W, v);
+          Row::store(G + (size_t)(k0 + e) * W, W, v);
+#pragma unroll
+          for (int i = 0; i < KW; ++i) nz |= v[i] != 0;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, nz);
+        if (e < ne && li == 0) {
+          const unsigned group = LR == 32 ? 0xffffffffu : ((1u << LR) - 1u) << (gi * LR);
+          a.gnz[k0 + e] = (bal & group) ? 1 : 0;
+          loc[org[k0 + e]] = 0xFFFFu;
         }
       }
       __syncthreads();
       PH_END(4, t_w);
     }
-  }
-  __syncthreads();
+    __syncthreads();
   }
 }
-
 
 void launch_good(dim3 grid, cudaStream_t st, const DevGrammar& g, int B, const SeqPack& sp) {
-  const size_t dyn = gs_tables_bytes(g.D, g.W, g.adv_steps);
-  cudaFuncSetAttribute(k_good, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  k_good<<<grid, 32 * kGoodWarps, dyn, st>>>(g, B, sp);
+  const GoodPlan p = good_plan(g, sp.nmax);
+  with_row_shape(g.W, [&](auto s) {
+    auto* kernel = k_good<decltype(s)>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
+    kernel<<<grid, 32 * kGoodWarps, p.bytes, st>>>(g, B, sp, p);
+  });
 }
-
-int good_warps() { return kGoodWarps; }
 
 // measurement builds: this translation unit's phase counters
 int phase_read_good(unsigned long long* out16, int reset) {

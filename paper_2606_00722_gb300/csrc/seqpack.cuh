@@ -8,7 +8,8 @@ namespace epic {
 
 // Per-sequence forward chart and its tables.
 struct SeqArena {
-  WWs ws;          // the forward walk's workspace; org/bits/esum/col_off are the chart
+  WWs ws;          // the forward walk's workspace; org/bits/col_off are the chart
+  uint32_t* bdone; // [nmax][VW]
   SeqRec rec;
   uint32_t* good;      // [emax][W]
   int32_t* last_col;   // [nmax] last column holding origin u (-1: none)
@@ -21,9 +22,8 @@ struct SeqArena {
   int32_t* eidx;       // [nmax (nmax + 1) / 2] entry of (column j, origin o <= j), -1: none
   uint8_t* gnz;        // [emax] the entry has a good item
   int32_t* cursor;     // [2 (nmax + 1)] scratch of the good pass
-  int32_t* key_q;      // [kMaxQ] scratch of the block forward walk
-  uint32_t* bexpn;     // [nmax][W]
-  uint32_t* bnew;      // [nmax][VW]
+  int32_t* key_q;      // [kMaxQ] scratch of the forward walk
+  LexEntry* ent;       // [kMaxQ]
 };
 
 struct SeqPack {
@@ -35,12 +35,12 @@ struct SeqPack {
   __host__ __device__ size_t bytes() const {
     size_t nm = nmax;
     return r(nm * W * 4) + r(nm * VW * 4) + r((nm + 1) * 4) + 7 * r(kWMaxQ * 4) + r(kWMaxQ * 16) + r(kWMaxQ * 32) +
-           r(nm * 8) + r((size_t)emax * 4) + r((size_t)emax * 8) + r((size_t)emax * W * 4)  // WWs
+           r((size_t)emax * 4) + r((size_t)emax * 8) + r((size_t)emax * W * 4)  // WWs
            + r(nm) + 2 * r((size_t)edge_cap * 4) + r((size_t)edge_cap * 32) + 3 * r((size_t)n * 4) +
            r((size_t)emax * VW * 4) + r(32)                                                 // SeqRec
            + r((size_t)emax * W * 4) + r(nm * 4) + 3 * r((nm + 1) * 4) + r((size_t)edge_cap * 4) +
            r((size_t)emax * 4) + r(nm * W * 4) + r(nm * (nm + 1) / 2 * 4) + r((size_t)emax) + r(2 * (nm + 1) * 4) + r(kMaxQ * 4) +
-           r(nm * W * 4) + r(nm * VW * 4);
+           r(kMaxQ * 16);
   }
   __device__ SeqArena carve(long long b) const {
     SeqArena a;
@@ -52,7 +52,7 @@ struct SeqPack {
     };
     size_t nm = nmax;
     a.ws.stage = (uint32_t*)take(nm * W * 4);
-    a.ws.bdone = (uint32_t*)take(nm * VW * 4);
+    a.bdone = (uint32_t*)take(nm * VW * 4);
     a.ws.col_off = (int32_t*)take((nm + 1) * 4);
     a.ws.f_q = (int32_t*)take(kWMaxQ * 4);
     a.ws.f_c = (int32_t*)take(kWMaxQ * 4);
@@ -63,9 +63,8 @@ struct SeqPack {
     a.ws.key_q = (int32_t*)take(kWMaxQ * 4);
     a.ws.g_tail = (uint32_t*)take(kWMaxQ * 16);
     a.ws.g_lbl = (uint32_t*)take(kWMaxQ * 32);
-    a.ws.ssum = (uint32_t*)take(nm * 8);
     a.ws.org = (int32_t*)take((size_t)emax * 4);
-    a.ws.esum = (uint32_t*)take((size_t)emax * 8);
+    a.rec.esum = (uint32_t*)take((size_t)emax * 8);
     a.ws.bits = (uint32_t*)take((size_t)emax * W * 4);
     a.rec.col_gap = (uint8_t*)take(nm);
     a.rec.e_dst = (int32_t*)take((size_t)edge_cap * 4);
@@ -77,7 +76,6 @@ struct SeqPack {
     a.rec.cnt = (uint32_t*)take((size_t)emax * VW * 4);
     a.rec.meta = (int32_t*)take(32);
     a.rec.edge_cap = edge_cap;
-    a.rec.n_edges = 0;
     a.good = (uint32_t*)take((size_t)emax * W * 4);
     a.last_col = (int32_t*)take(nm * 4);
     a.in_off = (int32_t*)take((nm + 1) * 4);
@@ -90,8 +88,7 @@ struct SeqPack {
     a.gnz = (uint8_t*)take((size_t)emax);
     a.cursor = (int32_t*)take(2 * (nm + 1) * 4);
     a.key_q = (int32_t*)take(kMaxQ * 4);
-    a.bexpn = (uint32_t*)take(nm * W * 4);
-    a.bnew = (uint32_t*)take(nm * VW * 4);
+    a.ent = (LexEntry*)take(kMaxQ * 16);
     return a;
   }
 };

@@ -1,38 +1,47 @@
 // Warp-level Earley walk: one warp recognizes one partial output.
 //
-// Same graph and chart as the block-wide walk (walk.cuh / skeleton.cuh), with
-// every step done by one warp and no block barrier:
-//  - a chart row is W words, lane l holding words l, l+32, ...;
-//  - the closure of a column is a Gauss-Seidel sweep: completions from origin
-//    o' only advance items of origins <= o', so the highest dirty origin is
-//    closed first and its completions are pushed at once into lower rows;
-//  - completed and waited-on nonterminals are read off a row with ballots;
+// Same graph and chart as the CTA walk (walk.cuh / skeleton.cuh), with every
+// step done by one warp and no block barrier:
+//  - the open column's rows lie in the warp's global stage, which its SM's L1
+//    holds (the kernels leave almost all of the 256 KB to L1).  Staging them in
+//    shared memory instead cost 24 KB per warp, so that seven warps ran on an
+//    SM;
+//  - the closure of a column visits every origin once, from the highest down:
+//    completions from origin o only advance items of origins <= o, and the one
+//    entry of column o with origin o feeds row o itself (closed in registers);
+//  - a row takes a group of lanes (rows.cuh): entries are scattered 32 / LR at
+//    a time, with both the entries' and the destination rows' loads in flight,
+//    and a store only where a row changes;
 //  - the span step groups lexings by (source, end state, terminals after the
 //    first) chunk by chunk, lanes matching their keys against the groups made
 //    so far.
+// What bounds a walk is the chain of dependent L1 / L2 accesses of its visits;
+// many walks per SM hide it.
 #pragma once
 #include "device.cuh"
+#include "rows.cuh"
 
 namespace epic {
+
+// the steps of a column: calls where a file asks for them
+#ifndef EPIC_STEP
+#define EPIC_STEP
+#endif
 
 constexpr int kWarpsPerCta = 8;
 constexpr int kWCols = 4096;    // columns per walk (graph nodes)
 constexpr int kWMaxW = 256;
 constexpr int kWMaxVW = 32;
 constexpr int kWMaxQ = 1024;
-constexpr long long kWMaxSteps = 1ll << 24;  // closure iterations per column
 
 // index of (column j, origin o <= j) in a lower-triangular table
 __host__ __device__ __forceinline__ size_t tri_index(int j, int o) { return (size_t)j * (j + 1) / 2 + o; }
 
-struct WWs {  // per-warp global workspace
-  uint32_t* stage;   // [nmax][W]
-  uint32_t* bdone;   // [nmax][VW]
+struct WWs {  // per-walk global workspace
+  uint32_t* stage;   // [nmax][W] rows of the open column (zero when idle)
   int32_t* col_off;  // [nmax + 1]
   int32_t* org;      // [emax]
-  uint32_t* esum;    // [emax][2] folded summaries of each entry (see row_scan)
   uint32_t* bits;    // [emax][W]
-  uint32_t* ssum;    // [nmax][2] summaries of the stage rows (global staging)
   int32_t* f_q;      // [kWMaxQ]
   int32_t* f_c;      // [kWMaxQ]
   int32_t* g_src;    // [kWMaxQ]
@@ -44,10 +53,9 @@ struct WWs {  // per-warp global workspace
   uint32_t* g_lbl;   // [kWMaxQ][8]  first-terminal label set
 };
 
-// What a recording walk (a sequence's forward chart) writes besides the chart:
-// the graph's edges in creation order of their target, gap flags, where each
-// position's segment sits in the graph, and each entry's completed
-// nonterminals.
+// What a sequence's forward chart records besides the chart: the graph's edges
+// in creation order of their target, gap flags, where each position's segment
+// sits in the graph, and each entry's completed nonterminals and summaries.
 struct SeqRec {
   uint8_t* col_gap;    // [nmax]
   int32_t* e_dst;      // [edge_cap]
@@ -57,18 +65,17 @@ struct SeqRec {
   int32_t* pre_col;    // [n] fixed position -> column before its span (gap or BEGIN)
   int32_t* post_col;   // [n] fixed position -> column after its span (gap or END)
   uint32_t* cnt;       // [emax][VW] completed nonterminals of each entry
+  uint32_t* esum;      // [emax][2] folded summaries (bit B mod 32 of a waited-on nonterminal, a mod 32 of a terminal)
   int32_t* meta;       // [8]: ncols, nedges, start, accept, status, nent (low), -, -
   int edge_cap;
-  int n_edges;         // running count (kept by the walk)
 };
 
 struct WSh {  // per-warp shared memory
   uint32_t touched[kWCols / 32];
-  uint32_t dirty[kWCols / 32];
-  uint32_t vset[kWMaxVW], vdone[kWMaxVW], nt[kWMaxVW];
-  uint32_t vdone_tot[kWMaxVW];  // nonterminals newly completed from the origin being closed
-  uint32_t lbl[kWMaxW];
-  uint32_t expn[kWMaxW];
+  alignas(16) uint32_t lbl[kWMaxW];  // items that the arrivals' labels expect
+  alignas(16) uint32_t scr[kWMaxW];  // one row
+  uint32_t nt[kWMaxVW];
+  int32_t list[32];
 };
 
 __device__ __forceinline__ uint32_t wl_lane() { return threadIdx.x & 31; }
@@ -121,25 +128,13 @@ static __device__ unsigned long long g_phase[16];  // one per translation unit
 #define PH_END(i, v)
 #endif
 
-// SM = true keeps the rows of the column under construction in shared memory
-// (slot-mapped, rmax rows); SM = false keeps them in the per-warp global
-// stage.  KWv item words per lane: rows of up to 32 KWv words.  EXT = true
-// adds the base chart, the suffix mode and the recording of checks by region
-// (compiled out of whole-graph walks).
-template <bool SM, bool EXT = false, int KWv = (SM ? 1 : kWMaxW / 32)>
+// S: the row shape.  EXT = true adds the base chart and the suffix mode of
+// checks by region (compiled out of whole-graph walks).
+template <class S, bool EXT>
 class WarpWalker {
-  static constexpr int KW = KWv;  // item words per lane
-
  public:
-  // shared-memory staging (SM): rows [rmax][W], completed-NT sets [rmax][VW],
-  // slot of each origin (-1 = none) and origin of each slot
-  uint32_t* srow = nullptr;
-  uint32_t* sbdone = nullptr;
-  int16_t* slot_of = nullptr;
-  int32_t* slot_org = nullptr;
-  uint32_t* slot_sum = nullptr;  // [rmax][2]
-  int rmax = 0;
-  int nslots = 0;
+  static constexpr int KW = S::KW, LR = S::LR, NG = S::NG;
+  using Row = RowRegs<S>;
   const DevGrammar& g;
   const LexEntry* table;
   WWs ws;
@@ -151,23 +146,15 @@ class WarpWalker {
   // walk state (uniform across the warp, kept in registers)
   int ncols;
   long long nent;
-  int status;  // 0 ok, 1 overflow, 2 bad input
+  int status;  // 0 ok, 1 overflow
   int nf;
   int start_col;
-  uint32_t label_fold = 0;  // bit (a mod 32) of every terminal in sh.lbl
   // A read-only base chart (a sequence's forward chart) holds columns
-  // 0 .. base_cols-1 and entries 0 .. base_ent-1; this walk's own columns
-  // follow with ids from base_cols.
+  // 0 .. base_cols-1; this walk's own columns follow with ids from base_cols.
   int base_cols = 0;
-  long long base_ent = 0;
   const int32_t* b_col_off = nullptr;
   const int32_t* b_org = nullptr;
   const uint32_t* b_bits = nullptr;
-  const uint32_t* b_esum = nullptr;
-  // recording of the forward chart's graph (null when not recording)
-  SeqRec* rec = nullptr;
-  int cur_col = -1;
-  uint32_t cur_lbl8[8];      // label set of the arrivals being made (all zero = epsilon)
   bool col_labelled = false; // the open column has a labelled arrival (else only epsilon ones)
   // Checks by region: the span step about to run is the region's last and
   // the node after it is a gap resolved by the base chart's good masks.  An
@@ -183,410 +170,168 @@ class WarpWalker {
   }
 
   __device__ WarpWalker(const DevGrammar& g_, const LexEntry* t, WWs w, WSh& s, int nm, long long em, int voc)
-      : g(g_), table(t), ws(w), sh(s), nmax(nm), emax(em), vocab(voc), W(g_.W), VW(g_.VW) {}
-
-  __device__ void set_smem(uint32_t* rows, uint32_t* bd, int16_t* so, int32_t* sorg, uint32_t* ssum, int rm) {
-    slot_sum = ssum;
-    srow = rows;
-    sbdone = bd;
-    slot_of = so;
-    slot_org = sorg;
-    rmax = rm;
-    for (int i = wl_lane(); i < nmax; i += 32) slot_of[i] = -1;
-    nslots = 0;
+      : g(g_), table(t), ws(w), sh(s), nmax(nm), emax(em), vocab(voc), W(g_.W), VW(g_.VW) {
+    for (int i = wl_lane(); i < kWCols / 32; i += 32) sh.touched[i] = 0;
     __syncwarp();
-  }
-  // stage row of origin o (allocating a zeroed slot for a new origin); null on overflow
-  __device__ uint32_t* row_of(int o) {
-    if constexpr (!SM) {
-      return ws.stage + (size_t)o * W;
-    } else {
-      int sl = slot_of[o];
-      if (sl < 0) {
-        if (nslots >= rmax) {
-          status = 1;
-          return nullptr;
-        }
-        sl = nslots++;
-        for (int w = wl_lane(); w < W; w += 32) srow[sl * W + w] = 0;
-        for (int v = wl_lane(); v < VW; v += 32) sbdone[sl * VW + v] = 0;
-        if (wl_lane() == 0) {
-          slot_of[o] = (int16_t)sl;
-          slot_org[sl] = o;
-          slot_sum[sl * 2] = 0;
-          slot_sum[sl * 2 + 1] = 0;
-        }
-        __syncwarp();
-      }
-      return srow + sl * W;
-    }
-  }
-  // every slot of the open column goes back (also rows allocated but never
-  // touched, whose origin would otherwise keep a stale slot)
-  __device__ void release_slots() {
-    if constexpr (SM) {
-      for (int s2 = wl_lane(); s2 < nslots; s2 += 32) slot_of[slot_org[s2]] = -1;
-      nslots = 0;
-      __syncwarp();
-    }
-  }
-  __device__ uint32_t* bdone_of(int o) {
-    if constexpr (!SM) return ws.bdone + (size_t)o * VW;
-    else return sbdone + slot_of[o] * VW;
-  }
-  __device__ uint32_t* sum_of(int o) {
-    if constexpr (!SM) return ws.ssum + (size_t)o * 2;
-    else return slot_sum + slot_of[o] * 2;
   }
 
   // ------------------------------------------------------------ chart access
-  __device__ long long cbeg(int c) const {
-    if constexpr (!EXT) return ws.col_off[c];
-    return c < base_cols ? (long long)b_col_off[c] : base_ent + ws.col_off[c - base_cols];
+  // a column's entries: origins, rows, count
+  __device__ __forceinline__ int column(int c, const int32_t*& org, const uint32_t*& bits) const {
+    if (EXT && c < base_cols) {
+      const int b = b_col_off[c];
+      org = b_org + b;
+      bits = b_bits + (size_t)b * W;
+      return b_col_off[c + 1] - b;
+    }
+    const int oc = EXT ? c - base_cols : c, b = ws.col_off[oc];
+    org = ws.org + b;
+    bits = ws.bits + (size_t)b * W;
+    return ws.col_off[oc + 1] - b;
   }
-  __device__ long long cend(int c) const {
-    if constexpr (!EXT) return ws.col_off[c + 1];
-    return c < base_cols ? (long long)b_col_off[c + 1] : base_ent + ws.col_off[c - base_cols + 1];
-  }
-  __device__ int eorg(long long k) const {
-    if constexpr (!EXT) return ws.org[k];
-    return k < base_ent ? b_org[k] : ws.org[k - base_ent];
-  }
-  __device__ const uint32_t* ebits(long long k) const {
-    if constexpr (!EXT) return ws.bits + (size_t)k * W;
-    return k < base_ent ? b_bits + (size_t)k * W : ws.bits + (size_t)(k - base_ent) * W;
-  }
-  __device__ uint32_t esum(long long k, int which) const {
-    if constexpr (!EXT) return ws.esum[(size_t)k * 2 + which];
-    return k < base_ent ? b_esum[(size_t)k * 2 + which] : ws.esum[(size_t)(k - base_ent) * 2 + which];
+  __device__ bool column_empty(int c) const {
+    const int32_t* o;
+    const uint32_t* b;
+    return column(c, o, b) == 0;
   }
 
   // ------------------------------------------------------------ bitmaps
-  __device__ void bm_clear(uint32_t* bm, int nbits) {
-    for (int w = wl_lane(); w < ((nbits + 31) >> 5); w += 32) bm[w] = 0;
-    __syncwarp();
-  }
-  __device__ void bm_set(uint32_t* bm, int i) {
-    if (wl_lane() == 0) bm[i >> 5] |= 1u << (i & 31);
-    __syncwarp();
-  }
-  // highest set bit below nbits, or -1
-  __device__ int bm_highest(const uint32_t* bm, int nbits) {
-    int nw = (nbits + 31) >> 5;
-    for (int top = nw - 1; top >= 0; top -= 32) {
-      int w = top - (int)wl_lane();
-      uint32_t v = (w >= 0) ? bm[w] : 0u;
-      unsigned any = __ballot_sync(0xffffffffu, v != 0);
+  // highest touched origin below `top`, or -1
+  __device__ static int highest_below(const uint32_t* touched, int top) {
+    if (top <= 0) return -1;
+    const int t = top - 1;
+    for (int wtop = t >> 5; wtop >= 0; wtop -= 32) {
+      const int w = wtop - (int)wl_lane();
+      uint32_t v = (w >= 0) ? touched[w] : 0u;
+      if (w == (t >> 5)) v &= (t & 31) == 31 ? 0xffffffffu : ((2u << (t & 31)) - 1u);
+      const unsigned any = __ballot_sync(0xffffffffu, v != 0);
       if (any) {
-        int l = __ffs(any) - 1;  // lowest lane = highest word
-        uint32_t vv = __shfl_sync(0xffffffffu, v, l);
-        return ((top - l) << 5) + (31 - __clz(vv));
+        const int l = __ffs(any) - 1;
+        const uint32_t vv = __shfl_sync(0xffffffffu, v, l);
+        return ((wtop - l) << 5) + (31 - __clz(vv));
       }
     }
     return -1;
   }
-  // lowest set bit at or above `from`, below nbits, or -1
-  __device__ int bm_next(const uint32_t* bm, int from, int nbits) {
-    int nw = (nbits + 31) >> 5;
-    for (int base = from >> 5; base < nw; base += 32) {
-      int w = base + (int)wl_lane();
-      uint32_t v = (w < nw) ? bm[w] : 0u;
-      if (w == (from >> 5)) v &= ~0u << (from & 31);
+  // The touched origins below nbits in ascending order, up to 32 at a time
+  // (one bitmap word): f(count, first) with their list in sh.list.
+  template <class F>
+  __device__ __forceinline__ void for_touched(int nbits, F f) {
+    const int nw = (nbits + 31) >> 5, lane = wl_lane();
+    for (int w0 = 0; w0 < nw; w0 += 32) {
+      const uint32_t v = w0 + lane < nw ? sh.touched[w0 + lane] : 0u;
       unsigned any = __ballot_sync(0xffffffffu, v != 0);
-      if (any) {
-        int l = __ffs(any) - 1;
-        uint32_t vv = __shfl_sync(0xffffffffu, v, l);
-        return ((base + l) << 5) + (__ffs(vv) - 1);
+      while (any) {
+        const int l = __ffs(any) - 1;
+        any &= any - 1;
+        const uint32_t m = __shfl_sync(0xffffffffu, v, l);
+        if ((m >> lane) & 1u) sh.list[__popc(m & ((1u << lane) - 1u))] = ((w0 + l) << 5) + lane;
+        __syncwarp();
+        f(__popc(m));
+        __syncwarp();
       }
     }
-    return -1;
   }
+  __device__ __forceinline__ void touch(int o) { atomicOr(&sh.touched[o >> 5], 1u << (o & 31)); }
 
   // ------------------------------------------------------------ row ops
-  // row |= shift(row & M), until stable (item (p, d) -> (p, d+1)); the row is
-  // held in registers (lane l owns words l, l+32, ...) while it is iterated
-  __device__ void row_advance(uint32_t* row, const uint32_t* M) {
-    const int nw = (W + 31) >> 5;
-    const int lane = wl_lane();
-    uint32_t r[KW], m[KW];
-#pragma unroll
-    for (int i = 0; i < KW; ++i) {
-      int w = lane + 32 * i;
-      bool ok = i < nw && w < W;
-      r[i] = ok ? row[w] : 0u;
-      m[i] = ok ? M[w] : 0u;
-    }
-    bool any_change = false;
-    for (int it = 0; it < 64; ++it) {
-      bool ch = false;
-      uint32_t carry = 0;
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        if (i < nw) {
-          uint32_t v = r[i] & m[i];
-          uint32_t prev = __shfl_up_sync(0xffffffffu, v, 1);
-          if (lane == 0) prev = carry;
-          carry = __shfl_sync(0xffffffffu, v, 31);
-          uint32_t add = ((v << 1) | (prev >> 31)) & ~r[i];
-          ch |= add != 0;
-          r[i] |= add;
-        }
+  // What a column's visits read at every step, copied to registers once per
+  // column (the walker itself may lie in local memory when its steps are
+  // calls).
+  struct Hot {
+    int W, VW, V, steps, nullable, base_cols;
+    uint32_t *stage, *touched, *scr;
+    const uint32_t *adv, *complete, *exp_nt, *b_bits, *bits;
+    const int32_t *cpl_off, *b_off, *b_org, *off, *org;
+    const uint2* cpl;
+    __device__ __forceinline__ int column(int c, const int32_t*& o, const uint32_t*& x) const {
+      if (EXT && c < base_cols) {
+        const int b = b_off[c];
+        o = b_org + b;
+        x = b_bits + (size_t)b * W;
+        return b_off[c + 1] - b;
       }
-      if (!__any_sync(0xffffffffu, ch)) break;
-      any_change = true;
+      const int oc = EXT ? c - base_cols : c, b = off[oc];
+      o = org + b;
+      x = bits + (size_t)b * W;
+      return off[oc + 1] - b;
     }
-    if (any_change) {
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        int w = lane + 32 * i;
-        if (i < nw && w < W) row[w] = r[i];
-      }
-    }
-    __syncwarp();
-  }
-  // dst |= shift(src & M) (or src & M / src); marks origin o; returns nonzero
-  __device__ bool row_into(uint32_t* dst, const uint32_t* src, const uint32_t* M, bool shift) {
-    bool nz = false;
-    uint32_t carry = 0;
-    for (int base = 0; base < W; base += 32) {
-      int w = base + wl_lane();
-      uint32_t v = (w < W) ? (M ? (src[w] & M[w]) : src[w]) : 0u;
-      uint32_t add = v;
-      if (shift) {
-        uint32_t prev = __shfl_up_sync(0xffffffffu, v, 1);
-        if (wl_lane() == 0) prev = carry;
-        add = (v << 1) | (prev >> 31);
-        carry = __shfl_sync(0xffffffffu, v, 31);
-      }
-      if (w < W && add) {
-        uint32_t old = dst[w];
-        if ((old | add) != old) {
-          dst[w] = old | add;
-          nz = true;
-        }
-      }
-    }
-    __syncwarp();
-    return __any_sync(0xffffffffu, nz);
-  }
-  // nonterminal set of the items of `row` selected by mask (via lhs or next
-  // symbol), ORed into out (VW words in shared memory)
-  __device__ void row_nts(const uint32_t* row, const uint32_t* mask, bool by_lhs, uint32_t* out) {
-    for (int base = 0; base < W; base += 32) {
-      int w = base + wl_lane();
-      uint32_t m = (w < W) ? (row[w] & mask[w]) : 0u;
-      unsigned nzl = __ballot_sync(0xffffffffu, m != 0);
-      while (nzl) {
-        int s = __ffs(nzl) - 1;
-        nzl &= nzl - 1;
-        uint32_t mm = __shfl_sync(0xffffffffu, m, s);
-        if ((mm >> wl_lane()) & 1u) {
-          int item = ((base + s) << 5) + wl_lane();
-          int B = by_lhs ? g.item_lhs[item] : (g.item_next[item] - g.T);
-          atomicOr(&out[B >> 5], 1u << (B & 31));
-        }
-      }
-    }
-    __syncwarp();
+  };
+  __device__ __forceinline__ Hot hot() const {
+    Hot h;
+    h.W = W;
+    h.VW = VW;
+    h.V = g.V;
+    h.steps = g.adv_steps;
+    h.nullable = g.any_nullable;
+    h.base_cols = base_cols;
+    h.stage = ws.stage;
+    h.touched = sh.touched;
+    h.scr = sh.scr;
+    h.adv = g.adv_pow;
+    h.complete = g.complete;
+    h.exp_nt = g.exp_nt;
+    h.b_bits = b_bits;
+    h.bits = ws.bits;
+    h.cpl_off = g.cpl_off;
+    h.b_off = b_col_off;
+    h.b_org = b_org;
+    h.off = ws.col_off;
+    h.org = ws.org;
+    h.cpl = g.cpl;
+    return h;
   }
 
-  // One pass over a row: the nonterminals its items wait on (ORed into the
-  // exact set `vs`) and two folded 32-bit summaries -- bit (B mod 32) for a
-  // waited-on nonterminal B, bit (a mod 32) for an expected terminal a --
-  // used to skip chart entries that cannot take part in a completion or a
-  // scan (a superset filter, exact for up to 32 symbols).
-  __device__ void row_scan(const uint32_t* row, uint32_t* vs, uint32_t* sum2) {
-    uint32_t fnt = 0, ft = 0;
-    for (int base = 0; base < W; base += 32) {
-      int w = base + wl_lane();
-      uint32_t r = (w < W) ? row[w] : 0u;
-      uint32_t mn = (w < W) ? (r & g.any_nt[w]) : 0u;
-      uint32_t mt = (w < W) ? (r & g.any_term[w]) : 0u;
-      unsigned nzl = __ballot_sync(0xffffffffu, (mn | mt) != 0);
-      while (nzl) {
-        int s = __ffs(nzl) - 1;
-        nzl &= nzl - 1;
-        uint32_t a = __shfl_sync(0xffffffffu, mn, s);
-        uint32_t b = __shfl_sync(0xffffffffu, mt, s);
-        int item = ((base + s) << 5) + wl_lane();
-        if ((a >> wl_lane()) & 1u) {
-          int B = g.item_next[item] - g.T;
-          atomicOr(&vs[B >> 5], 1u << (B & 31));
-          fnt |= 1u << (B & 31);
-        }
-        if ((b >> wl_lane()) & 1u) ft |= 1u << (g.item_next[item] & 31);
-      }
-    }
-    for (int off = 16; off; off >>= 1) {
-      fnt |= __shfl_xor_sync(0xffffffffu, fnt, off);
-      ft |= __shfl_xor_sync(0xffffffffu, ft, off);
-    }
-    if (wl_lane() == 0) {
-      sum2[0] = fnt;
-      sum2[1] = ft;
-    }
-    __syncwarp();
-  }
-
-  // Scatter the entries of finished column `col` into the stage, one entry per
-  // lane: dst(org) |= shift(bits & M) (or bits & M, or bits).  Entries of one
-  // column have distinct origins, so lanes never share a destination row.
-  // `which` selects the summary filter (0: waited nonterminals, 1: expected
-  // terminals, -1: none) tested against `fold`.
-  __device__ void scatter(int col, const uint32_t* M, bool shift, int which, uint32_t fold, int skip_org = -1) {
-    const int lane = wl_lane();
-    const long long b = cbeg(col), e = skip_org >= 0 ? cend(col) - 1 : cend(col);
-    if (!SM && W > 16) {  // wide rows in the global stage: the lanes share each entry's words
-      for (long long base = b; base < e; base += 32) {
-        const long long k = base + lane;
-        const bool act = k < e && (which < 0 || (esum(k, which) & fold) != 0);
-        unsigned am = __ballot_sync(0xffffffffu, act);
-        const int my_org = act ? eorg(k) : -1;
-        while (am) {  // up to four entries at a time: their loads overlap
-          int ls[4];
-          int nl = 0;
-          while (am && nl < 4) {
-            ls[nl++] = __ffs(am) - 1;
-            am &= am - 1;
-          }
-          const uint32_t* src[4];
-          uint32_t* dst[4];
-          int o2[4];
-          uint32_t carry[4];
-          bool ch[4];
+  // Scatter entries of a column into the stage: row(origin) |= bits & m,
+  // shifted to the next item when SHIFT.  Entries of one column have distinct
+  // origins, so lane groups never share a destination row.
+  template <bool SHIFT>
+  __device__ static __forceinline__ void scatter(const Hot& h, const int32_t* org, const uint32_t* bits, int ne,
+                                                 const uint32_t (&m)[KW]) {
+    const int W = h.W;
+    constexpr int U = KW == 4 ? 4 : 2;  // steps in flight
+    const int lane = wl_lane(), li = Row::li(), gi = Row::gi();
+    const unsigned group = LR == 32 ? 0xffffffffu : ((1u << LR) - 1u) << (gi * LR);
+    for (int c0 = 0; c0 < ne; c0 += 32) {
+      const int o_t = c0 + lane < ne ? org[c0 + lane] : 0;
+      const int n = min(32, ne - c0);
+      for (int u0 = 0; u0 < n; u0 += U * NG) {
+        uint32_t v[U][KW], q[U][KW];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int l = i < nl ? ls[i] : ls[0];
-            o2[i] = __shfl_sync(0xffffffffu, my_org, l);
-            src[i] = ebits(base + l);
-            dst[i] = i < nl ? row_of(o2[i]) : nullptr;
-            carry[i] = 0;
-            ch[i] = false;
-          }
-          if (status) return;  // no shared-memory slot left
-          for (int w0 = 0; w0 < W; w0 += 32) {
-            const int w = w0 + lane;
-            const uint32_t m = (M && w < W) ? M[w] : 0xffffffffu;
-            uint32_t v[4];
+        for (int u = 0; u < U; ++u) {
+          const int t = u0 + u * NG + gi;
+          const int o2 = __shfl_sync(0xffffffffu, o_t, t & 31);
+          if (t < n) {
+            Row::load(bits + (size_t)(c0 + t) * W, W, v[u]);
+            Row::load(h.stage + (size_t)o2 * W, W, q[u]);
+          } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = (i < nl && w < W) ? (src[i][w] & m) : 0u;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              uint32_t add = v[i];
-              if (shift) {
-                uint32_t prev = __shfl_up_sync(0xffffffffu, v[i], 1);
-                if (lane == 0) prev = carry[i];
-                add = (v[i] << 1) | (prev >> 31);
-                carry[i] = __shfl_sync(0xffffffffu, v[i], 31);
-              }
-              if (i < nl && w < W && add) {
-                const uint32_t old = dst[i][w];
-                if ((old | add) != old) {
-                  dst[i][w] = old | add;
-                  ch[i] = true;
-                }
-              }
-            }
+            for (int i = 0; i < KW; ++i) v[u][i] = q[u][i] = 0u;
           }
+        }
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const bool any = __any_sync(0xffffffffu, ch[i]);
-            if (i < nl && any && lane == 0) {
-              sh.touched[o2[i] >> 5] |= 1u << (o2[i] & 31);
-              sh.dirty[o2[i] >> 5] |= 1u << (o2[i] & 31);
-            }
+        for (int u = 0; u < U; ++u) {
+#pragma unroll
+          for (int i = 0; i < KW; ++i) v[u][i] &= m[i];
+          if (SHIFT) Row::shift_up(v[u]);
+          uint32_t nw = 0;
+#pragma unroll
+          for (int i = 0; i < KW; ++i) {
+            nw |= v[u][i] & ~q[u][i];
+            q[u][i] |= v[u][i];
           }
-          __syncwarp();
-        }
-      }
-      return;
-    }
-    for (long long base = b; base < e; base += 32) {
-      long long k = base + lane;
-      bool act = k < e && (which < 0 || (esum(k, which) & fold) != 0);
-      unsigned am = __ballot_sync(0xffffffffu, act);
-      if (!am) continue;
-      int o2 = act ? eorg(k) : -1;
-      uint32_t* dst = nullptr;
-      if constexpr (SM) {
-        bool need = act && slot_of[o2] < 0;
-        unsigned nm = __ballot_sync(0xffffffffu, need);
-        int nneed = __popc(nm);
-        if (nslots + nneed > rmax) {
-          status = 1;
-          return;
-        }
-        if (need) {
-          int sl = nslots + __popc(nm & ((1u << lane) - 1u));
-          slot_of[o2] = (int16_t)sl;
-          slot_org[sl] = o2;
-          slot_sum[sl * 2] = 0;
-          slot_sum[sl * 2 + 1] = 0;
-          for (int w = 0; w < W; ++w) srow[sl * W + w] = 0;
-          for (int v = 0; v < VW; ++v) sbdone[sl * VW + v] = 0;
-        }
-        nslots += nneed;
-        __syncwarp();
-        if (act) dst = srow + slot_of[o2] * W;
-      } else {
-        if (act) dst = ws.stage + (size_t)o2 * W;
-      }
-      bool ch = false;
-      if (act) {
-        const uint32_t* src = ebits(k);
-        uint32_t carry = 0;
-        for (int w = 0; w < W; ++w) {
-          uint32_t v = M ? (src[w] & M[w]) : src[w];
-          uint32_t add = shift ? ((v << 1) | carry) : v;
-          carry = v >> 31;
-          if (add) {
-            uint32_t old = dst[w];
-            if ((old | add) != old) {
-              dst[w] = old | add;
-              ch = true;
+          const unsigned bal = __ballot_sync(0xffffffffu, nw != 0);
+          if (bal) {
+            const int o2 = __shfl_sync(0xffffffffu, o_t, (u0 + u * NG + gi) & 31);
+            if (bal & group) {
+              Row::store(h.stage + (size_t)o2 * W, W, q[u]);
+              if (li == 0) atomicOr(&h.touched[o2 >> 5], 1u << (o2 & 31));
             }
           }
         }
-        if (ch) {
-          atomicOr(&sh.touched[o2 >> 5], 1u << (o2 & 31));
-          atomicOr(&sh.dirty[o2 >> 5], 1u << (o2 & 31));
-        }
-      }
-      __syncwarp();
-    }
-  }
-
-  // row |= shift(items of E waiting on a member of the nonterminal set nts);
-  // returns whether row changed
-  __device__ bool row_into_waiting(uint32_t* row, const uint32_t* E, const uint32_t* nts) {
-    bool ch = false;
-    uint32_t carry = 0;
-    for (int base = 0; base < W; base += 32) {
-      const int w = base + wl_lane();
-      uint32_t x = 0;
-      if (w < W) {
-        uint32_t m = E[w] & g.any_nt[w];
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1;
-          const int B = g.item_next[(w << 5) + b] - g.T;
-          if ((nts[B >> 5] >> (B & 31)) & 1u) x |= 1u << b;
-        }
-      }
-      uint32_t prev = __shfl_up_sync(0xffffffffu, x, 1);
-      if (wl_lane() == 0) prev = carry;
-      carry = __shfl_sync(0xffffffffu, x, 31);
-      const uint32_t add = (x << 1) | (prev >> 31);
-      if (w < W && add) {
-        const uint32_t old = row[w];
-        if ((old | add) != old) {
-          row[w] = old | add;
-          ch = true;
-        }
       }
     }
     __syncwarp();
-    return __any_sync(0xffffffffu, ch);
   }
 
   // ------------------------------------------------------------ columns
@@ -595,44 +340,30 @@ class WarpWalker {
       status = 1;
       return -1;
     }
-    cur_col = ncols;
     return ncols;
   }
-  __device__ void arrive(int src, const uint32_t* M, bool shift) {
-    PH_BEGIN(t_arr);
-    arrive_inner(src, M, shift);
-    PH_END(1, t_arr);
-  }
-  __device__ void record_edge(int src, bool labelled) {
-    if (wl_lane() == 0) {
-      if (rec->n_edges >= rec->edge_cap) {
-        status = 1;
-      } else {
-        int e = rec->n_edges++;
-        rec->e_dst[e] = cur_col;
-        rec->e_src[e] = src;
-        for (int w = 0; w < 8; ++w) rec->e_lbl[(size_t)e * 8 + w] = labelled ? cur_lbl8[w] : 0u;
-      }
-    }
-    status = __shfl_sync(0xffffffffu, status, 0);
-    rec->n_edges = __shfl_sync(0xffffffffu, rec->n_edges, 0);
-  }
-  __device__ void arrive_inner(int src, const uint32_t* M, bool shift) {
+  __device__ EPIC_STEP void arrive(int src, bool shift) {
     col_labelled |= shift;
-    if constexpr (EXT)
-      if (rec) record_edge(src, shift);
-    if (shift)
-      scatter(src, M, true, 1, label_fold);
-    else
-      scatter(src, M, false, -1, 0u);
+    const Hot h = hot();
+    const int32_t* org;
+    const uint32_t* bits;
+    const int ne = h.column(src, org, bits);
+    uint32_t m[KW];
+    if (shift) {
+      Row::load(sh.lbl, W, m);
+      scatter<true>(h, org, bits, ne, m);
+    } else {
+#pragma unroll
+      for (int i = 0; i < KW; ++i) m[i] = 0xffffffffu;
+      scatter<false>(h, org, bits, ne, m);
+    }
   }
   __device__ void seed(int c) {
-    uint32_t* r = row_of(c);
-    if (!r) return;
-    if (wl_lane() == 0) r[g.start_item >> 5] |= 1u << (g.start_item & 31);
+    if (wl_lane() == 0) {
+      ws.stage[(size_t)c * W + (g.start_item >> 5)] |= 1u << (g.start_item & 31);
+      touch(c);
+    }
     __syncwarp();
-    bm_set(sh.touched, c);
-    bm_set(sh.dirty, c);
   }
 
   // Suffix mode (a check's nodes after its region): no predictions, and rows
@@ -650,238 +381,232 @@ class WarpWalker {
   const int32_t* b_eidx = nullptr;  // [(j (j + 1) / 2) + o] for o <= j
   __device__ long long find_base(int j, int o) const { return o > j ? -1 : (long long)b_eidx[tri_index(j, o)]; }
 
-  bool cur_gap = false;
-  __device__ void close_column(int c, bool gap) {
-    cur_gap = gap;
-    const uint32_t* P = gap ? g.gap_pred : g.pred;
-    // A node (not a gap) reached only by epsilon edges from finished columns:
-    // each row below c is a union of rows closed under completion and
-    // advance, and so is the union, so those rows only contribute their
-    // waited nonterminals (the predictions at c).
-    const bool eps_only = !gap && !col_labelled;
-    for (long long it = 0;; ++it) {
-      if (it > kWMaxSteps) {
-        status = 1;
-        return;
-      }
-      int o = bm_highest(sh.dirty, c + 1);
-      if (EXT && suffix_mode) {
-        if (o < 0) break;
-        if (o < base_cols) {  // resolved by the good masks at finish
-          if (wl_lane() == 0) sh.dirty[o >> 5] &= ~(1u << (o & 31));
-          __syncwarp();
-          continue;
-        }
-      }
-      if (o < 0) {
-        // predictions for origin c from the nonterminals waited on here
-        bool any = false;
-        for (int v = wl_lane(); v < VW; v += 32) any |= (sh.vset[v] & ~sh.vdone[v]) != 0;
-        if (!__any_sync(0xffffffffu, any)) break;
-        uint32_t* crow = row_of(c);
-        if (!crow) return;
-        for (int w = wl_lane(); w < W; w += 32) {
-          uint32_t acc = 0;
-          for (int v = 0; v < VW; ++v) {
-            uint32_t nw = sh.vset[v] & ~sh.vdone[v];
-            while (nw) {
-              int b = __ffs(nw) - 1;
-              nw &= nw - 1;
-              acc |= P[(size_t)((v << 5) + b) * W + w];
-            }
-          }
-          crow[w] |= acc;
-        }
-        __syncwarp();
-        for (int v = wl_lane(); v < VW; v += 32) sh.vdone[v] |= sh.vset[v];
-        __syncwarp();
-        bm_set(sh.touched, c);
-        bm_set(sh.dirty, c);
-        continue;
-      }
-      if (wl_lane() == 0) sh.dirty[o >> 5] &= ~(1u << (o & 31));
-      __syncwarp();
-      uint32_t* row = row_of(o);
-      if (eps_only && o < c) {
-        row_scan(row, sh.vset, sum_of(o));
-        continue;
-      }
-      if (o == c) {  // completions from c at c: the nullable / gap advance rules
-        PH_BEGIN(t_row);
-        row_advance(row, gap ? g.next_any : g.nullable_next);
-        PH_END(3, t_row);
-        row_scan(row, sh.vset, sum_of(o));
-        continue;
-      }
-      // Completions from o advance the items of column o; of those, only the
-      // entry with origin o itself (the last one: entries are stored by
-      // ascending origin) feeds row o again.  Close that loop first, then
-      // scatter everything completed from o once over the other entries.
-      const long long ke = cend(o);
-      const bool self = ke > cbeg(o) && eorg(ke - 1) == o;
-      uint32_t* bd = bdone_of(o);
-      for (int v = wl_lane(); v < VW; v += 32) sh.vdone_tot[v] = 0;
-      bool any_tot = false;
-      for (int round = 0; round < 64 * kWMaxW; ++round) {
-        PH_BEGIN(t_row);
-        row_advance(row, gap ? g.next_any : g.nullable_next);
-        PH_END(3, t_row);
-        PH_BEGIN(t_nts);
-        for (int v = wl_lane(); v < VW; v += 32) sh.nt[v] = 0;
-        __syncwarp();
-        row_nts(row, g.complete, true, sh.nt);
-        bool any = false;
-        for (int v = wl_lane(); v < VW; v += 32) {
-          const uint32_t d = sh.nt[v] & ~bd[v];
-          sh.nt[v] = d;
-          any |= d != 0;
-          bd[v] |= d;
-          sh.vdone_tot[v] |= d;
-        }
-        __syncwarp();
-        PH_END(4, t_nts);
-        any = __any_sync(0xffffffffu, any);
-        any_tot |= any;
-        if (!any || !self) break;
-        if (!row_into_waiting(row, ebits(ke - 1), sh.nt)) break;
-      }
-      row_scan(row, sh.vset, sum_of(o));
-      if (!any_tot) continue;
-      PH_BEGIN(t_expn);
-      // EXPN: items waiting on a nonterminal newly completed from o
-      expn_of_set(g, sh.vdone_tot, sh.expn);
-      __syncwarp();
-      PH_END(5, t_expn);
-      PH_BEGIN(t_part);
-      uint32_t fold = 0;
-      for (int v = 0; v < VW; ++v) fold |= sh.vdone_tot[v];
-      scatter(o, sh.expn, true, 0, fold, self ? o : -1);
-      if (status) return;
-      PH_END(6, t_part);
+  // Close row o (o below the open column) with its self-loop and scatter what
+  // it completes over the other entries of column o.  Every lane group holds a
+  // copy of the row.
+  __device__ static __forceinline__ void visit(const Hot& h, int o, int mode) {
+    const int W = h.W, VW = h.VW;
+    const int32_t* org;
+    const uint32_t* bits;
+    const int ne = h.column(o, org, bits);
+    uint32_t r[KW], r0[KW], e[KW], ex[KW], cs[KW];
+    Row::load(h.stage + (size_t)o * W, W, r);
+    const bool self = ne > 0 && org[ne - 1] == o;  // entries are stored by ascending origin
+    if (self) {
+      Row::load(bits + (size_t)(ne - 1) * W, W, e);
+    } else {
+#pragma unroll
+      for (int i = 0; i < KW; ++i) e[i] = 0u;
     }
+#pragma unroll
+    for (int i = 0; i < KW; ++i) {
+      r0[i] = r[i];
+      ex[i] = cs[i] = 0u;
+    }
+    uint32_t known = 0;  // lane v < VW: word v of the nonterminals completed from o
+    for (int round = 0; round < 64 * kWMaxW; ++round) {
+      Row::advance(r, h.adv, mode, h.steps, h.nullable, W);
+      uint32_t cm[KW];
+      Row::load(h.complete, W, cm);
+      bool fresh = false;
+#pragma unroll
+      for (int i = 0; i < KW; ++i) {
+        cm[i] &= r[i] & ~cs[i];
+        cs[i] |= cm[i];
+        fresh |= cm[i] != 0;
+      }
+      if (!__any_sync(0xffffffffu, fresh)) break;
+      if (wl_lane() < LR) Row::store(h.scr, W, cm);
+      __syncwarp();
+      const uint32_t nw = warp_ntset(h.scr, h.cpl_off, h.cpl, h.V, VW) & ~known;
+      __syncwarp();
+      if (!__any_sync(0xffffffffu, nw != 0)) break;
+      known |= nw;
+      uint32_t x[KW];
+      Row::waiting_on(nw, h.exp_nt, W, VW, x);
+      bool ch = false;
+#pragma unroll
+      for (int i = 0; i < KW; ++i) {
+        ex[i] |= x[i];
+        x[i] &= e[i];
+      }
+      Row::shift_up(x);
+#pragma unroll
+      for (int i = 0; i < KW; ++i) {
+        ch |= (x[i] & ~r[i]) != 0;
+        r[i] |= x[i];
+      }
+      if (!__any_sync(0xffffffffu, ch)) break;
+    }
+    bool ch = false;
+#pragma unroll
+    for (int i = 0; i < KW; ++i) ch |= r[i] != r0[i];
+    if (__any_sync(0xffffffffu, ch)) {
+      if (wl_lane() < LR) Row::store(h.stage + (size_t)o * W, W, r);
+      __syncwarp();
+    }
+    if (__any_sync(0xffffffffu, known != 0)) scatter<true>(h, org, bits, self ? ne - 1 : ne, ex);
   }
 
-  __device__ void finish_column(int c) {
-    PH_BEGIN(t_fin);
-    finish_inner(c);
-    PH_END(7, t_fin);
+  __device__ EPIC_STEP void close_column(int c, bool gap) {
+    const int mode = gap ? 1 : 0;
+    // Origins below c, each once, highest first.  A node (not a gap) reached
+    // only by epsilon edges from finished columns needs none of it: each row
+    // below c is a union of rows closed under completion and advance, and so
+    // is the union.  In suffix mode, base-chart origins are resolved by the
+    // good masks at finish.
+    if (gap || col_labelled) {
+      const Hot h = hot();
+      const int least = EXT && suffix_mode ? base_cols : 0;
+      int o = c;
+      while ((o = highest_below(h.touched, o)) >= least) visit(h, o, mode);
+    }
+    if (EXT && suffix_mode) return;
+    // predictions at c from the nonterminals waited on in any row (the
+    // prediction closures are closed under further predictions)
+    uint32_t uni[KW];
+#pragma unroll
+    for (int i = 0; i < KW; ++i) uni[i] = 0u;
+    for_touched(c + 1, [&](int cnt) {
+      for (int t = Row::gi(); t < cnt; t += NG) {
+        uint32_t v[KW];
+        Row::load(ws.stage + (size_t)sh.list[t] * W, W, v);
+#pragma unroll
+        for (int i = 0; i < KW; ++i) uni[i] |= v[i];
+      }
+    });
+    Row::join(uni);
+    if (wl_lane() < LR) Row::store(sh.scr, W, uni);
+    __syncwarp();
+    const uint32_t vs = warp_ntset(sh.scr, g.wait_off, g.wait, g.V, VW);
+    __syncwarp();
+    const bool any = __any_sync(0xffffffffu, vs != 0);
+    const bool seeded = (sh.touched[c >> 5] >> (c & 31)) & 1u;
+    if (!any && !seeded) return;
+    uint32_t r[KW], p[KW];
+    Row::load(ws.stage + (size_t)c * W, W, r);
+    Row::waiting_on(vs, gap ? g.gap_pred : g.pred, W, VW, p);
+#pragma unroll
+    for (int i = 0; i < KW; ++i) r[i] |= p[i];
+    // a seeded row (the walk's first column) is closed by the advance rule
+    if (seeded) Row::advance(r, g.adv_pow, mode, g.adv_steps, g.any_nullable, W);
+    if (wl_lane() < LR) Row::store(ws.stage + (size_t)c * W, W, r);
+    if (wl_lane() == 0) touch(c);
+    __syncwarp();
   }
-  __device__ void finish_inner(int c) {
+
+  // Move the open column's rows into the entry store (origins ascending).  A
+  // touched row is never empty.
+  __device__ EPIC_STEP void finish_column(int c) {
     const int oc = c - base_cols;  // own column index
+    const int gi = Row::gi(), li = Row::li();
     long long E = ws.col_off[oc];
-    int o = -1;
-    while ((o = bm_next(sh.touched, o + 1, c + 1)) >= 0) {
-      uint32_t* row = row_of(o);
-      bool nz = false;
-      for (int w = wl_lane(); w < W; w += 32) nz |= row[w] != 0;
-      nz = __any_sync(0xffffffffu, nz);
-      if (EXT && nz && suffix_mode && o < base_cols) {
-        long long kf = find_base(res_node, o);
+    for_touched(c + 1, [&](int cnt) {
+      // rows below the base chart in suffix mode come first (origins ascend):
+      // tested and dropped
+      int drop = 0;
+      if (EXT && suffix_mode) drop = __popc(__ballot_sync(0xffffffffu, wl_lane() < cnt && sh.list[wl_lane()] < base_cols));
+      const long long E0 = E;
+      const int keep = cnt - drop;
+      if (E0 + keep > emax)
+        status = 1;
+      else
+        E = E0 + keep;
+      for (int t0 = 0; t0 < cnt; t0 += NG) {
+        const int t = t0 + gi;
         bool hit = false;
-        if (kf >= 0)
-          for (int w = wl_lane(); w < W; w += 32) hit |= (row[w] & good[(size_t)kf * W + w]) != 0;
-        if (__any_sync(0xffffffffu, hit)) found = 1;
-        nz = false;  // not kept
-      }
-      if (EXT && nz && suffix_mode && o == region_start && res_node == accept_node &&
-          ((row[g.accept_item >> 5] >> (g.accept_item & 31)) & 1u))
-        found = 1;
-      if (nz) {
-        if (E >= emax) {
-          status = 1;
-        } else {
-          if (wl_lane() == 0) {
-            ws.org[E] = o;
-            uint32_t* sm = sum_of(o);
-            ws.esum[(size_t)E * 2] = sm[0];
-            ws.esum[(size_t)E * 2 + 1] = sm[1];
+        if (t < cnt) {
+          const int o = sh.list[t];
+          uint32_t* row = ws.stage + (size_t)o * W;
+          uint32_t v[KW];
+          Row::load(row, W, v);
+          if (t < drop) {
+            const long long kf = find_base(res_node, o);
+            if (kf >= 0) {
+              uint32_t gv[KW];
+              Row::load(good + (size_t)kf * W, W, gv);
+#pragma unroll
+              for (int i = 0; i < KW; ++i) hit |= (v[i] & gv[i]) != 0;
+            }
+          } else {
+            if (EXT && suffix_mode && o == region_start && res_node == accept_node) {
+#pragma unroll
+              for (int i = 0; i < KW; ++i)
+                hit |= li * KW + i == (g.accept_item >> 5) && ((v[i] >> (g.accept_item & 31)) & 1u);
+            }
+            if (!status) {
+              const long long k = E0 + t - drop;
+              if (li == 0) ws.org[k] = o;
+              Row::store(ws.bits + (size_t)k * W, W, v);
+            }
           }
-          uint32_t* dst = ws.bits + (size_t)E * W;
-          for (int w = wl_lane(); w < W; w += 32) dst[w] = row[w];
-          if (EXT && rec) {  // completed nonterminals of the entry
-            for (int v = wl_lane(); v < VW; v += 32) sh.nt[v] = 0;
-            __syncwarp();
-            row_nts(row, g.complete, true, sh.nt);
-            for (int v = wl_lane(); v < VW; v += 32) rec->cnt[(size_t)E * VW + v] = sh.nt[v];
-          }
-          ++E;
+#pragma unroll
+          for (int i = 0; i < KW; ++i) v[i] = 0u;
+          Row::store(row, W, v);
         }
+        if (EXT && suffix_mode && __any_sync(0xffffffffu, hit)) found = 1;
       }
-      if constexpr (!SM) {
-        for (int w = wl_lane(); w < W; w += 32) row[w] = 0;
-        for (int v = wl_lane(); v < VW; v += 32) ws.bdone[(size_t)o * VW + v] = 0;
-      }
-    }
-    release_slots();
-    bm_clear(sh.touched, c + 1);
-    for (int v = wl_lane(); v < VW; v += 32) {
-      sh.vset[v] = 0;
-      sh.vdone[v] = 0;
-    }
-    if (wl_lane() == 0) {
-      ws.col_off[oc + 1] = (int)E;
-      if (EXT && rec) rec->col_gap[c] = cur_gap ? 1 : 0;
-    }
+    });
+    for (int w = wl_lane(); w < ((c + 32) >> 5); w += 32) sh.touched[w] = 0;
+    if (wl_lane() == 0) ws.col_off[oc + 1] = (int)E;
     __syncwarp();
     nent = E;
     ncols = c + 1;
     col_labelled = false;
   }
-  __device__ bool column_empty(int c) { return cend(c) == cbeg(c); }
 
   // abandon the open column: zero its rows
   __device__ void cleanup() {
     col_labelled = false;
-    int o = -1;
-    while ((o = bm_next(sh.touched, o + 1, kWCols)) >= 0) {
-      if constexpr (!SM) {
-        for (int w = wl_lane(); w < W; w += 32) ws.stage[(size_t)o * W + w] = 0;
-        for (int v = wl_lane(); v < VW; v += 32) ws.bdone[(size_t)o * VW + v] = 0;
-      }
-    }
-    release_slots();
-    bm_clear(sh.touched, kWCols);
-    bm_clear(sh.dirty, kWCols);
-    for (int v = wl_lane(); v < VW; v += 32) {
-      sh.vset[v] = 0;
-      sh.vdone[v] = 0;
-    }
+    for_touched(kWCols, [&](int cnt) {
+      uint32_t z[KW];
+#pragma unroll
+      for (int i = 0; i < KW; ++i) z[i] = 0u;
+      for (int t = Row::gi(); t < cnt; t += NG) Row::store(ws.stage + (size_t)sh.list[t] * W, W, z);
+    });
+    for (int w = wl_lane(); w < kWCols / 32; w += 32) sh.touched[w] = 0;
     __syncwarp();
   }
 
   __device__ bool accepts(int c, int start) {
+    const int32_t* org;
+    const uint32_t* bits;
+    const int ne = column(c, org, bits);
     bool f = false;
-    for (long long k = cbeg(c) + wl_lane(); k < cend(c); k += 32)
-      if (eorg(k) == start && ((ebits(k)[g.accept_item >> 5] >> (g.accept_item & 31)) & 1u)) f = true;
+    for (int k = wl_lane(); k < ne; k += 32)
+      if (org[k] == start && ((bits[(size_t)k * W + (g.accept_item >> 5)] >> (g.accept_item & 31)) & 1u)) f = true;
     return __any_sync(0xffffffffu, f);
   }
 
   // ------------------------------------------------------------ labels
-  __device__ void label_set(const uint32_t* lbl8) {
-    label_fold = 0;
+  // sh.lbl = the items that expect a terminal of the set (the lane groups
+  // share out the terminals)
+  __device__ EPIC_STEP void label_set(const uint32_t* lbl8) {
+    uint32_t v[KW];
+#pragma unroll
+    for (int i = 0; i < KW; ++i) v[i] = 0u;
+    int seen = 0;
     for (int lw = 0; lw < 8; ++lw) {
-      label_fold |= lbl8[lw];
-      cur_lbl8[lw] = lbl8[lw];
-    }
-    for (int w = wl_lane(); w < W; w += 32) {
-      uint32_t acc = 0;
-      for (int lw = 0; lw < 8; ++lw) {
-        uint32_t m = lbl8[lw];
-        while (m) {
-          int b = __ffs(m) - 1;
-          m &= m - 1;
-          int a = (lw << 5) + b;
-          if (a < g.T) acc |= g.exp_term[(size_t)a * W + w];
-        }
+      uint32_t m = lbl8[lw];
+      while (m) {
+        const int a = (lw << 5) + __ffs(m) - 1;
+        m &= m - 1;
+        if ((seen++ & (NG - 1)) != Row::gi() || a >= g.T) continue;
+        uint32_t x[KW];
+        Row::load(g.exp_term + (size_t)a * W, W, x);
+#pragma unroll
+        for (int i = 0; i < KW; ++i) v[i] |= x[i];
       }
-      sh.lbl[w] = acc;
     }
+    __syncwarp();
+    Row::join(v);
+    if (wl_lane() < LR) Row::store(sh.lbl, W, v);
     __syncwarp();
   }
   __device__ void label_one(int a) {
-    label_fold = 1u << (a & 31);
-    for (int lw = 0; lw < 8; ++lw) cur_lbl8[lw] = (lw == (a >> 5)) ? (1u << (a & 31)) : 0u;
-    for (int w = wl_lane(); w < W; w += 32) sh.lbl[w] = g.exp_term[(size_t)a * W + w];
+    uint32_t v[KW];
+    Row::load(g.exp_term + (size_t)a * W, W, v);
+    if (wl_lane() < LR) Row::store(sh.lbl, W, v);
     __syncwarp();
   }
 
@@ -889,7 +614,7 @@ class WarpWalker {
   __device__ bool simple_column(int& c_out, int src, bool eps, bool gap) {
     int c = open_column();
     if (c < 0) return false;
-    arrive(src, eps ? nullptr : sh.lbl, !eps);
+    arrive(src, !eps);
     close_column(c, gap);
     finish_column(c);
     c_out = c;
@@ -906,7 +631,7 @@ class WarpWalker {
     return v;
   }
 
-  __device__ bool span_step(int tok) {
+  __device__ EPIC_STEP bool span_step(int tok) {
     if (g.lazy.stats && wl_lane() == 0) atomicAdd(&g.lazy.stats[0], (unsigned long long)nf);
     int ng = 0;
     PH_BEGIN(t_group);
@@ -1041,13 +766,13 @@ class WarpWalker {
         if (ws.g_end[gi] != best) continue;
         int len = ws.g_len[gi];
         if (len == 0) {
-          arrive(ws.g_src[gi], nullptr, false);
+          arrive(ws.g_src[gi], false);
         } else if (len == 1) {
           label_set(ws.g_lbl + gi * 8);
-          arrive(ws.g_src[gi], sh.lbl, true);
+          arrive(ws.g_src[gi], true);
         } else {
           label_one(tail_term(gi, len - 1));
-          arrive(ws.g_last[gi], sh.lbl, true);
+          arrive(ws.g_last[gi], true);
         }
       }
       bool defer = false;
@@ -1057,14 +782,7 @@ class WarpWalker {
           if (ws.key_q[tj] == ti && !eps_into_gap(ws.f_q[tj])) all_eps = false;
         defer = __all_sync(0xffffffffu, all_eps);
       }
-      if (defer) {
-        // rows as they arrived: only their summaries (scatter filters)
-        int o = -1;
-        while ((o = bm_next(sh.touched, o + 1, c + 1)) >= 0) row_scan(row_of(o), sh.vset, sum_of(o));
-        bm_clear(sh.dirty, c + 1);
-      } else {
-        close_column(c, false);
-      }
+      if (!defer) close_column(c, false);  // else: rows as they arrived
       finish_column(c);
       if (status) return false;
       if (wl_lane() == 0) ws.f_c[ti] = c;
@@ -1155,37 +873,40 @@ class WarpWalker {
     return r;
   }
 
-  // a gap node after the span in the frontier: a pending lexeme some byte
-  // can extend stays open (epsilon), one no byte can extend emits its terminal
+  // Arrivals of the frontier into the open column: by an epsilon edge, by the
+  // pending lexeme's terminal, or none (a dead end); frontier elements with
+  // the same column and the same edge arrive once.  At a gap a pending lexeme
+  // some byte can extend stays open (epsilon), one no byte can extend emits
+  // its terminal; at the END the pending lexeme is flushed.
+  __device__ void arrive_frontier(bool gap) {
+    for (int f = wl_lane(); f < nf; f += 32) {
+      const int q = ws.f_q[f], a = g.dfa_accept[q];
+      int kind = -2;
+      if (q == 0 || (gap && g.dfa_ext[q]) || (a >= 0 && g.skip[a]))
+        kind = -1;
+      else if (a >= 0)
+        kind = a;
+      ws.g_len[f] = kind;
+    }
+    __syncwarp();
+    for (int f = 0; f < nf; ++f) {
+      const int kind = ws.g_len[f], c = ws.f_c[f];
+      if (kind == -2) continue;
+      bool dup = false;
+      for (int h = wl_lane(); h < f; h += 32) dup |= ws.f_c[h] == c && ws.g_len[h] == kind;
+      if (__any_sync(0xffffffffu, dup)) continue;
+      if (kind >= 0) label_one(kind);
+      arrive(c, kind >= 0);
+    }
+  }
   __device__ int gap_from_frontier() {
     int c = open_column();
-    if (c < 0) return -1;
-    for (int f = 0; f < nf; ++f) {
-      int q = ws.f_q[f];
-      int a = g.dfa_accept[q];
-      if (q == 0 || g.dfa_ext[q] || (a >= 0 && g.skip[a])) {
-        arrive(ws.f_c[f], nullptr, false);
-      } else if (a >= 0) {
-        label_one(a);
-        arrive(ws.f_c[f], sh.lbl, true);
-      }
-    }
+    if (c >= 0) arrive_frontier(true);
     return c;
   }
-  // the END node: the pending lexeme is flushed
   __device__ int end_from_frontier() {
     int c = open_column();
-    if (c < 0) return -1;
-    for (int f = 0; f < nf; ++f) {
-      int q = ws.f_q[f];
-      int a = g.dfa_accept[q];
-      if (q == 0 || (a >= 0 && g.skip[a])) {
-        arrive(ws.f_c[f], nullptr, false);
-      } else if (a >= 0) {
-        label_one(a);
-        arrive(ws.f_c[f], sh.lbl, true);
-      }
-    }
+    if (c >= 0) arrive_frontier(false);
     return c;
   }
   // frontier of a span that starts at column src: q0 at the sequence start,
@@ -1206,16 +927,10 @@ class WarpWalker {
     }
     __syncwarp();
   }
-  __device__ void rec_range(int32_t* arr, int lo, int hi, int v) {
-    for (int p = lo + (int)wl_lane(); p < hi; p += 32) arr[p] = v;
-    __syncwarp();
-  }
-
   __device__ int run_inner(const int32_t* x, int n, int sp, int stok) {
     int i = 0;
     bool first = true;
     int prev_gap = -1;
-    int span_lo = -1, span_hi = -1;  // the last span, for post_col
     while (i < n) {
       int t0 = token_at(x, sp, stok, i);
       int j = i;
@@ -1234,10 +949,6 @@ class WarpWalker {
         close_column(c, true);
         finish_column(c);
         if (status) return -1;
-        if (EXT && rec) {
-          rec_range(rec->gap_col, i, j, c);
-          if (span_lo >= 0) rec_range(rec->post_col, span_lo, span_hi, c);
-        }
         prev_gap = c;
         if (column_empty(c)) return 0;
       } else {
@@ -1256,9 +967,6 @@ class WarpWalker {
           src = prev_gap;
         }
         frontier_from(src, first);
-        if (EXT && rec) rec_range(rec->pre_col, i, j, src);
-        span_lo = i;
-        span_hi = j;
         for (int p = i; p < j && nf > 0; ++p) {
           int tok = token_at(x, sp, stok, p);
           if (tok < 0 || tok >= vocab) return -2;
@@ -1271,17 +979,12 @@ class WarpWalker {
           close_column(c, false);
           finish_column(c);
           if (status) return -1;
-          if (EXT && rec) {
-            rec_range(rec->post_col, i, j, c);
-            if (wl_lane() == 0) rec->meta[3] = c;
-          }
           return accepts(c, start_col) ? 1 : 0;
         }
       }
       first = false;
       i = j;
     }
-    if (EXT && rec && wl_lane() == 0) rec->meta[3] = prev_gap;
     return accepts(prev_gap, start_col) ? 1 : 0;
   }
 };

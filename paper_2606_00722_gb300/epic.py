@@ -18,10 +18,10 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 # translation units, compiled in parallel and linked into one library
 _SRC = [os.path.join(_HERE, 'csrc', f) for f in
         ('epic.cu', 'kernels_walk.cu', 'kernels_select.cu', 'region_forward.cu', 'region_good.cu',
-         'region_check_sm.cu', 'region_check_global.cu', 'peak.cu', 'witness.cu', 'grammar.cpp')]
+         'region_check.cu', 'peak.cu', 'witness.cu', 'grammar.cpp')]
 _DEPS = _SRC + [os.path.join(_HERE, 'csrc', f) for f in
-                ('grammar.h', 'device.cuh', 'walk.cuh', 'cover.cuh', 'skeleton.cuh', 'warpwalk.cuh', 'packs.cuh',
-                 'seqpack.cuh', 'launch.h', 'region.cuh', 'region_check.cuh', 'gscols.cuh')] + \
+                ('grammar.h', 'device.cuh', 'walk.cuh', 'cover.cuh', 'warpwalk.cuh', 'packs.cuh',
+                 'seqpack.cuh', 'launch.h', 'region.cuh', 'gscols.cuh', 'rows.cuh', 'skeleton.cuh')] + \
     [os.path.join(_HERE, '..', 'include', 'epic.h'), os.path.join(_HERE, '..', 'include', 'epic_measure.h')]
 LIB_PATH = os.path.join(_HERE, '_build', 'libepic.so')
 ARCH_FLAGS = ['-gencode', 'arch=compute_103a,code=sm_103a']
