@@ -75,6 +75,8 @@ struct DevGrammar {
   const int32_t* wait_off;        // [V+1]
   const uint2* wait;
   int n_cpl, n_wait;
+  const int16_t* next_t;          // [32][W] nonterminal after the dot of item 32 w + b at [b][w], -1: none
+  const uint32_t* follow;         // [4][V][VW] completions that follow from one another (grammar.h)
   int any_nullable;               // some item's next symbol is a nullable nonterminal
 };
 

@@ -495,6 +495,13 @@ epic_status epic_grammar_create(const epic_grammar_desc* desc, epic_grammar** ou
   up(G.complete, &d.complete);
   up(G.pred, &d.pred);
   up(G.gap_pred, &d.gap_pred);
+  up(G.follow, &d.follow);
+  {
+    std::vector<int16_t> nt((size_t)32 * G.W, -1);
+    for (int i = 0; i < G.D; ++i)
+      if (G.item_next[i] >= G.T) nt[(size_t)(i & 31) * G.W + (i >> 5)] = (int16_t)(G.item_next[i] - G.T);
+    up(nt, &d.next_t);
+  }
   up(inext, &d.item_next);
   up(ilhs, &d.item_lhs);
   up(g->dfa.accept, &d.dfa_accept);

@@ -451,6 +451,34 @@ GrammarTables build_tables(int T, const std::vector<uint8_t>& skip, int V, int s
       }
     }
   }
+  // Completions that follow at one origin o and node c.  The items with origin
+  // o in column o are the predictions made there: dots at 0 and behind
+  // nullable prefixes, every dot at a gap.  So A's completion reaches the end
+  // of B -> alpha A beta if alpha is nullable (any alpha when o is a gap) and
+  // beta is (any beta when c is a gap, where items advance over everything).
+  // Nonterminals not predicted at o may be named too: no item of column o
+  // waits on them, and every link below a predicted one is predicted.
+  const int VW = (V + 31) / 32;
+  G.follow.assign((size_t)4 * V * VW, 0);
+  for (int kind = 0; kind < 4; ++kind) {
+    uint32_t* M = G.follow.data() + (size_t)kind * V * VW;
+    for (int A = 0; A < V; ++A) M[(size_t)A * VW + (A >> 5)] |= 1u << (A & 31);
+    for (int p = 0; p < G.aug; ++p) {
+      const int b = G.rhs_off[p], e = G.rhs_off[p + 1], B = G.lhs[p];
+      auto skips = [&](int lo, int hi) {
+        for (int i = lo; i < hi; ++i)
+          if (G.rhs[i] < T || !G.nullable[G.rhs[i] - T]) return false;
+        return true;
+      };
+      for (int i = b; i < e; ++i)
+        if (G.rhs[i] >= T && ((kind & 2) || skips(b, i)) && ((kind & 1) || skips(i + 1, e)))
+          M[(size_t)(G.rhs[i] - T) * VW + (B >> 5)] |= 1u << (B & 31);
+    }
+    for (int k = 0; k < V; ++k)  // transitive closure over k
+      for (int A = 0; A < V; ++A)
+        if ((M[(size_t)A * VW + (k >> 5)] >> (k & 31)) & 1u)
+          for (int w = 0; w < VW; ++w) M[(size_t)A * VW + w] |= M[(size_t)k * VW + w];
+  }
   return G;
 }
 

@@ -50,6 +50,11 @@ struct GrammarTables {
   std::vector<uint32_t> complete;       // [W] complete items (excluding S')
   std::vector<uint32_t> pred;           // [V][W] Earley prediction closure of B
   std::vector<uint32_t> gap_pred;       // [V][W] items predicted and fully advanced inside a gap
+  // completions that follow from one another at one origin o and node c
+  // (reflexive, transitive): bit B of row A of table 2 [o is a gap] + [c is a
+  // gap], [4][V][(V + 31) / 32] words -- completing A advances an item of B
+  // predicted at o over A and to its end
+  std::vector<uint32_t> follow;
   int accept_item = -1;                 // S' -> S .
   int start_item = -1;                  // S' -> . S
 };

@@ -35,6 +35,10 @@
 //    EXP_NT rows.  (Instruction issue, at 36 % of the active cycles with one
 //    word per lane and 32-word steps, was the bound: clike-512 spent about 70
 //    instructions per scattered entry.)
+//  - all nonterminals that complete at c from o through chains at the self
+//    entry (B -> A, or at gaps any production around A) follow from the
+//    directly completed ones by a table, so a visit is one pass instead of a
+//    round per link (2.7 on average for clike-512).
 // Predictions at c only feed row c (items predicted at c have origin c), and
 // the prediction closures are closed under further predictions, so they are
 // made once, after the lower origins are closed; completions from c at c are
@@ -101,7 +105,10 @@ struct GsPlan {
   uint32_t o_col;          // column offsets [nmax + 1]
   uint32_t o_slot;         // row slot of each origin [nmax] (uint16)
   uint32_t o_self;         // bit o: column o has an entry with origin o
+  uint32_t o_gap;          // bit o: column o is a gap
+  uint32_t o_fol;          // DevGrammar::follow; 0: read from global memory
   uint32_t o_exp;          // EXP_NT rows; 0: read from global memory
+  uint32_t o_next;         // DevGrammar::next_t (wide rows); 0: read from global memory
   uint32_t o_walk;         // span step tables; 0: in the global workspace
   uint32_t o_zero;         // a row of zeros, for origins without a slot
   uint32_t o_rows, o_done; // row slots, completed nonterminals per slot
@@ -129,11 +136,16 @@ inline GsPlan gs_plan(const DevGrammar& g, int nmax, size_t limit) {
   p.o_col = put((size_t)(nmax + 1) * 4);
   p.o_slot = put((size_t)nmax * 2);
   p.o_self = put((size_t)((nmax + 31) / 32) * 4);
+  p.o_gap = put((size_t)((nmax + 31) / 32) * 4);
   p.o_zero = put((size_t)g.W * 4);
   const size_t per_row = (size_t)(g.W + g.VW) * 4;
   const size_t least = 64 * per_row;  // rows that always come first
   const size_t walk = (size_t)g.Q * kGsWalkBytesPerState, ex = (size_t)g.V * g.W * 4;
   p.o_walk = o + r(walk) + least <= limit ? put(walk) : 0;
+  const size_t fol = (size_t)4 * g.V * g.VW * 4;
+  p.o_fol = fol <= 16 * 1024 && o + r(fol) + least <= limit ? put(fol) : 0;
+  const size_t nx = (size_t)64 * g.W;
+  p.o_next = g.W > 64 && o + r(nx) + least <= limit ? put(nx) : 0;
   p.o_exp = o + r(ex) + 2 * least <= limit ? put(ex) : 0;
   const size_t left = limit > o + 32 ? limit - o - 32 : 0;
   long long rows = (long long)(left / per_row);
@@ -164,7 +176,7 @@ class EarleyColsGS {
   WsDims dims;
   int W, VW, R;
   const BlockRec* rec = nullptr;
-  uint32_t *rows, *done, *selfb;
+  uint32_t *rows, *done, *selfb, *gapb;
   uint16_t* slot_of;
 
   // What the visits and scatters of a column read at every step, copied to
@@ -173,10 +185,11 @@ class EarleyColsGS {
   struct Hot {
     int W, VW, V, R, steps, nullable;
     uint32_t s_rows, s_zero;      // shared addresses: row slots, the zero row
-    const uint32_t *adv, *complete, *selfb, *exp_nt;
+    const uint32_t *adv, *complete, *selfb, *gapb, *exp_nt, *follow;
     uint32_t *scr, *rows, *done, *stage, *bdone;
     uint16_t* slot_of;
     const int32_t *c_off, *col, *org;
+    const int16_t* next_t;
     const uint2* c_lst;
     const uint32_t* bits;
     __device__ __forceinline__ uint32_t slot(int o) const { return *(const volatile uint16_t*)(slot_of + o); }
@@ -198,6 +211,9 @@ class EarleyColsGS {
     h.adv = tb.adv_pow;
     h.complete = tb.complete;
     h.selfb = (const uint32_t*)(m + plan.o_self);
+    h.gapb = (const uint32_t*)(m + plan.o_gap);
+    h.follow = plan.o_fol ? (const uint32_t*)(m + plan.o_fol) : g.follow;
+    h.next_t = plan.o_next ? (const int16_t*)(m + plan.o_next) : g.next_t;
     h.exp_nt = plan.o_exp ? (const uint32_t*)(m + plan.o_exp) : g.exp_nt;
     h.scr = (uint32_t*)(m + plan.o_scr) + (size_t)(threadIdx.x >> 5) * W;
     h.rows = (uint32_t*)(m + plan.o_rows);
@@ -219,6 +235,7 @@ class EarleyColsGS {
     ws.col_off = (int32_t*)(smem + p.o_col);
     slot_of = (uint16_t*)(smem + p.o_slot);
     selfb = (uint32_t*)(smem + p.o_self);
+    gapb = (uint32_t*)(smem + p.o_gap);
     rows = (uint32_t*)(smem + p.o_rows);
     done = (uint32_t*)(smem + p.o_done);
   }
@@ -248,6 +265,14 @@ class EarleyColsGS {
       uint32_t* ex = (uint32_t*)(smem + plan.o_exp);
       for (int i = threadIdx.x; i < g.V * W; i += blockDim.x) ex[i] = g.exp_nt[i];
     }
+    if (plan.o_next) {
+      int16_t* t = (int16_t*)(smem + plan.o_next);
+      for (int i = threadIdx.x; i < 32 * W; i += blockDim.x) t[i] = g.next_t[i];
+    }
+    if (plan.o_fol) {
+      uint32_t* f = (uint32_t*)(smem + plan.o_fol);
+      for (int i = threadIdx.x; i < 4 * g.V * VW; i += blockDim.x) f[i] = g.follow[i];
+    }
     for (int i = threadIdx.x; i < W; i += blockDim.x) ((uint32_t*)(smem + plan.o_zero))[i] = 0;
     for (int i = threadIdx.x; i < R * W; i += blockDim.x) rows[i] = 0;
     for (int i = threadIdx.x; i < R * VW; i += blockDim.x) done[i] = 0;
@@ -272,6 +297,7 @@ class EarleyColsGS {
     clear_bitmap(walk_sh().touched, kMaxCols);
     clear_bitmap(walk_sh().dirty, kMaxCols);
     clear_bitmap(selfb, dims.nmax);
+    clear_bitmap(gapb, dims.nmax);
     __syncthreads();
   }
 
@@ -481,48 +507,35 @@ class EarleyColsGS {
       for (int i = 0; i < KW; ++i) e[i] = 0u;
     }
 #pragma unroll
+    for (int i = 0; i < KW; ++i) r0[i] = r[i];
+    // what the row completes, and everything that follows from it through the
+    // self entry, at once (lane v < VW: word v)
+    uint32_t tot = 0;
+    Row::advance(r, h.adv, mode, h.steps, h.nullable, W);
+    uint32_t cm[KW];
+    Row::load(h.complete, W, cm);
+    bool any = false;
+#pragma unroll
     for (int i = 0; i < KW; ++i) {
-      r0[i] = r[i];
-      ex[i] = 0u;
+      cm[i] &= r[i];
+      any |= cm[i] != 0;
     }
-    uint32_t tot = 0;  // lane v < VW: word v of the nonterminals new in this visit
-    uint32_t cs[KW];   // complete items looked at
-#pragma unroll
-    for (int i = 0; i < KW; ++i) cs[i] = 0u;
-    for (int round = 0; round < 64 * kMaxW; ++round) {
-      Row::advance(r, h.adv, mode, h.steps, h.nullable, W);
-      uint32_t cm[KW];
-      Row::load(h.complete, W, cm);
-      bool fresh = false;
-#pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        cm[i] &= r[i] & ~cs[i];
-        cs[i] |= cm[i];
-        fresh |= cm[i] != 0;
-      }
-      if (!__any_sync(0xffffffffu, fresh)) break;
+    if (__any_sync(0xffffffffu, any)) {
       if (lane < LR) Row::store(h.scr, W, cm);
       __syncwarp();
-      const uint32_t nw = warp_ntset(h.scr, h.c_off, h.c_lst, h.V, VW) & ~known;
+      tot = warp_ntset(h.scr, h.c_off, h.c_lst, h.V, VW) & ~known;
       __syncwarp();
-      if (!__any_sync(0xffffffffu, nw != 0)) break;
-      known |= nw;
-      tot |= nw;
-      uint32_t x[KW];
-      Row::waiting_on(nw, h.exp_nt, W, VW, x);
-      bool ch = false;
+      if (__any_sync(0xffffffffu, tot != 0)) {
+        const int kind = 2 * (int)((h.gapb[o >> 5] >> (o & 31)) & 1u) + mode;
+        tot = warp_follow(tot, h.follow + (size_t)kind * h.V * VW, VW) & ~known;
+        Row::waiting_on(tot, h.exp_nt, h.next_t, h.scr, W, VW, ex);
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        ex[i] |= x[i];
-        x[i] &= e[i];  // the self entry's items waiting on a new nonterminal advance into r
-      }
-      Row::shift_up(x);
+        for (int i = 0; i < KW; ++i) e[i] &= ex[i];
+        Row::shift_up(e);
 #pragma unroll
-      for (int i = 0; i < KW; ++i) {
-        ch |= (x[i] & ~r[i]) != 0;
-        r[i] |= x[i];
+        for (int i = 0; i < KW; ++i) r[i] |= e[i];
+        Row::advance(r, h.adv, mode, h.steps, h.nullable, W);
       }
-      if (!__any_sync(0xffffffffu, ch)) break;
     }
     if (lane < LR) {
 #pragma unroll
@@ -599,7 +612,10 @@ class EarleyColsGS {
   // Closure of column c (gap: a node with a Sigma_lex* self-loop).
   __device__ __noinline__ void close_column(int c, bool gap) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = nwarps();
-    if (REC && threadIdx.x == 0) rec->col_gap[c] = gap ? 1 : 0;
+    if (threadIdx.x == 0) {
+      if (REC) rec->col_gap[c] = gap ? 1 : 0;
+      if (gap) gapb[c >> 5] |= 1u << (c & 31);
+    }
     const int mode = gap ? 1 : 0;  // the advance rule: next_any in a gap, nullable_next elsewhere
     // 1. origins below c.  A node (not a gap) reached only by epsilon edges
     //    from finished columns needs no sweep: each of its rows is a union of

@@ -172,7 +172,7 @@ struct RegionCheck {
         const uint32_t set = lane < w.VW ? a.rec.cnt[(size_t)kc * w.VW + lane] : 0u;
         if (!__any_sync(0xffffffffu, set != 0)) continue;
         uint32_t ex[S::KW];
-        RowRegs<S>::waiting_on(set, w.g.exp_nt, w.W, w.VW, ex);
+        RowRegs<S>::or_rows(set, w.g.exp_nt, w.W, w.VW, ex);
         w.col_labelled = true;  // new items to close, not a copy of a closed column
         const int32_t* org;
         const uint32_t* bits;

@@ -17,6 +17,10 @@ struct GoodPlan {
   uint32_t o_cpl_off, o_cpl;     // complete items by nonterminal
   uint32_t o_wait_off, o_wait;   // waiting items by nonterminal
   uint32_t o_exp;                // EXP_NT rows; 0: read from global memory
+  uint32_t o_next;               // DevGrammar::next_t (wide rows); 0: read from global memory
+  uint32_t o_fol;                // DevGrammar::follow; 0: read from global memory
+  uint32_t o_col;                // column offsets [nmax + 1]
+  uint32_t o_org;                // origins of the open column's entries (uint16)
   uint32_t o_scr;                // per-warp scratch, W words each
   uint32_t o_cmp;                // per-warp list of a batch's active lanes
   uint32_t o_lbl;                // label masks of a chunk of out-edges
@@ -24,7 +28,7 @@ struct GoodPlan {
   uint32_t o_chg, o_nxt, o_open; // bitmaps over the open column's entries
   uint32_t o_fold;               // folded completions of each successor
   uint32_t o_sux;                // items waiting on what completes at a successor; sux rows
-  uint32_t o_row, o_gnt;         // good masks and good nonterminals of the open column; rows rows
+  uint32_t o_row, o_gnt;         // good masks, and completed nonterminals not known good, of the open column; rows rows
   int sux, rows;
   uint32_t bytes;
 };
@@ -53,6 +57,11 @@ static GoodPlan good_plan(const DevGrammar& g, int nmax) {
   p.o_nxt = put(bm);
   p.o_open = put(bm);
   p.o_fold = put((size_t)nmax * 4);
+  p.o_col = put((size_t)(nmax + 1) * 4);
+  p.o_org = put((size_t)nmax * 2);
+  const size_t fol = (size_t)4 * g.V * g.VW * 4, nx = (size_t)64 * g.W;
+  p.o_fol = fol <= 16 * 1024 ? put(fol) : 0;
+  p.o_next = g.W > 64 ? put(nx) : 0;
   const size_t ex = (size_t)g.V * g.W * 4, per_row = (size_t)(2 * g.W + g.VW) * 4;
   p.o_exp = o + r(ex) + 64 * per_row <= limit ? put(ex) : 0;
   const size_t left = limit > o + 64 ? limit - o - 64 : 0;
@@ -152,7 +161,11 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
   uint16_t* loc = (uint16_t*)(dyn + p.o_loc);
   uint32_t* open = (uint32_t*)(dyn + p.o_open);
   uint32_t* sfold = (uint32_t*)(dyn + p.o_fold);
+  int32_t* col = (int32_t*)(dyn + p.o_col);
+  uint16_t* lorg = (uint16_t*)(dyn + p.o_org);
   const uint32_t* exp_nt = g.exp_nt;
+  const uint32_t* follow = g.follow;
+  const int16_t* next_t = g.next_t;
   __shared__ int s_self, s_more, s_next;
   __shared__ __align__(16) uint32_t s_xall[kWMaxW];
   // the grammar lists
@@ -167,6 +180,16 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
     uint32_t* ex = (uint32_t*)(dyn + p.o_exp);
     for (int i = tid; i < V * W; i += nthr) ex[i] = g.exp_nt[i];
     exp_nt = ex;
+  }
+  if (p.o_fol) {
+    uint32_t* f = (uint32_t*)(dyn + p.o_fol);
+    for (int i = tid; i < 4 * V * VW; i += nthr) f[i] = g.follow[i];
+    follow = f;
+  }
+  if (p.o_next) {
+    int16_t* t = (int16_t*)(dyn + p.o_next);
+    for (int i = tid; i < 32 * W; i += nthr) t[i] = g.next_t[i];
+    next_t = t;
   }
   for (int i = tid; i < sp.nmax; i += nthr) loc[i] = 0xFFFFu;
   __syncthreads();
@@ -217,7 +240,9 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
     int32_t* meta = a.rec.meta;
     if (meta[M_STATUS] != 1) continue;
     const int N = meta[M_NCOLS], NE = meta[M_NEDGES];
-    const int32_t* col = a.ws.col_off;
+    __syncthreads();  // the sequence before is done with the offsets
+    for (int j = tid; j <= N; j += nthr) col[j] = a.ws.col_off[j];
+    __syncthreads();
     const int32_t* org = a.ws.org;
     const uint32_t* bits_g = a.ws.bits;
     const int start = meta[M_START], accept = meta[M_ACCEPT];
@@ -308,7 +333,11 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         s_next = 0;
       }
       for (int w = tid; w < W; w += nthr) s_xall[w] = 0;
-      for (int e = tid; e < ne; e += nthr) loc[org[k0 + e]] = (uint16_t)e;
+      for (int e = tid; e < ne; e += nthr) {
+        const int o = org[k0 + e];
+        loc[o] = (uint16_t)e;
+        lorg[e] = (uint16_t)o;
+      }
       for (int w = tid; w < ((ne + 31) >> 5); w += nthr) {
         chg[w] = 0;
         nxt[w] = 0;
@@ -323,7 +352,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         if (j2 == j && lane == 0) s_self = si - s0;
         if (f) {
           uint32_t ex[KW];
-          Row::waiting_on(set, exp_nt, W, VW, ex);
+          Row::waiting_on(set, exp_nt, next_t, scr, W, VW, ex);
           if (lane < LR) {
             Row::store(sux_of(si - s0), W, ex);
             if (j2 != j) {
@@ -382,7 +411,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         in_row(inrow, gap, self_si);
         for (int e = warp; e < ne; e += kGoodWarps) {
           const size_t k = (size_t)k0 + e;
-          const int o = org[k];
+          const int o = lorg[e];
           uint32_t* Gk = row_of(e);
           uint32_t acc[KW], bits[KW];
           // the lane groups take different edges and successors, and their
@@ -487,7 +516,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
             nz = __any_sync(0xffffffffu, nz);
             const uint32_t cn = lane < VW ? a.rec.cnt[k * VW + lane] : 0u;
             const bool cpl = __any_sync(0xffffffffu, cn != 0);
-            if (lane < VW) gnt_of(e)[lane] = 0;
+            if (lane < VW) gnt_of(e)[lane] = cn;
             if (lane == 0) {
               if (nz) atomicOr(&chg[e >> 5], 1u << (e & 31));
               if (cpl) atomicOr(&open[e >> 5], 1u << (e & 31));
@@ -511,10 +540,9 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
           if (e >= ne) break;
           if (!((open[e >> 5] >> (e & 31)) & 1u)) continue;
           const size_t k = (size_t)k0 + e;
-          const int o = org[k];
+          const int o = lorg[e];
           uint32_t* gnt = gnt_of(e);
-          const uint32_t gn = lane < VW ? gnt[lane] : 0u;
-          uint32_t nt = lane < VW ? (a.rec.cnt[k * VW + lane] & ~gn) : 0u;  // completed, not known good
+          uint32_t nt = lane < VW ? gnt[lane] : 0u;  // completed, not known good
           uint32_t found = 0, ex[KW];
           bool have = false;
           const int cb = col[o], ce = col[o + 1];
@@ -526,7 +554,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
             const int na = compact(live, l2);
             if (na == 0) continue;
             if (!have) {
-              Row::waiting_on(nt, exp_nt, W, VW, ex);
+              Row::waiting_on(nt, exp_nt, next_t, scr, W, VW, ex);
               have = true;
             }
             uint32_t acc[KW];
@@ -569,42 +597,43 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
             if (!__any_sync(0xffffffffu, nt != 0)) break;  // every completed nonterminal is good
           }
           if (!__any_sync(0xffffffffu, found != 0)) continue;
-          // complete items with a good left side, the in-row closure, and the
-          // loop through the entry of column o with origin o (which maps back
-          // to this row)
-          uint32_t r[KW], bits[KW], inrow[KW];
+          // what completes here and leads to a good one through the entry of
+          // column o with origin o (which maps back to this row) is good too:
+          // one lane per nonterminal looks for a good one that follows from it
+          {
+            const uint32_t* fo = follow + (size_t)(2 * (a.rec.col_gap[o] != 0) + (gap ? 1 : 0)) * V * VW;
+            uint32_t more = 0;
+            if (lane < VW) scr[lane] = found;
+            __syncwarp();
+            for (int v = 0; v < VW; ++v) {
+              const uint32_t cand = __shfl_sync(0xffffffffu, nt, v);
+              bool hit = false;
+              if ((cand >> lane) & 1u)
+                for (int w = 0; w < VW && !hit; ++w) hit = (fo[(size_t)((v << 5) + lane) * VW + w] & scr[w]) != 0;
+              const uint32_t b2 = __ballot_sync(0xffffffffu, hit);
+              if (lane == v) more = b2;
+            }
+            __syncwarp();
+            found |= more;
+            nt &= ~more;
+          }
+          // complete items with a good left side, and the in-row closure
+          uint32_t r[KW], bits[KW], inrow[KW], cm[KW];
           uint32_t* Gk = row_of(e);
           Row::load(Gk, W, r);
           Row::load(bits_g + k * W, W, bits);
           in_row(inrow, gap, sel);
-          const bool self = ce > cb && org[ce - 1] == o;
-          uint32_t fresh = found;
+          completes(found, cm);
           bool changed = false;
-          for (int it = 0; it < 64 * kWMaxW; ++it) {
-            uint32_t cm[KW];
-            completes(fresh, cm);
-            bool ch = false;
 #pragma unroll
-            for (int i = 0; i < KW; ++i) {
-              const uint32_t add = bits[i] & cm[i] & ~r[i];
-              ch |= add != 0;
-              r[i] |= add;
-            }
-            if (!__any_sync(0xffffffffu, ch)) break;
-            changed = true;
-            good_in_row<S>(r, bits, inrow);
-            if (!self || !__any_sync(0xffffffffu, nt != 0)) break;
-            uint32_t s[KW], x[KW];
-            Row::shift_down(r, s);
-            Row::load(bits_g + (size_t)(ce - 1) * W, W, x);
-#pragma unroll
-            for (int i = 0; i < KW; ++i) x[i] &= ex[i] & s[i];
-            fresh = waited(x) & nt;
-            if (!__any_sync(0xffffffffu, fresh != 0)) break;
-            found |= fresh;
-            nt &= ~fresh;
+          for (int i = 0; i < KW; ++i) {
+            const uint32_t add = bits[i] & cm[i] & ~r[i];
+            changed |= add != 0;
+            r[i] |= add;
           }
-          if (lane < VW) gnt[lane] = gn | found;
+          changed = __any_sync(0xffffffffu, changed);
+          if (changed) good_in_row<S>(r, bits, inrow);
+          if (lane < VW) gnt[lane] = nt;
           if (!__any_sync(0xffffffffu, nt != 0) && lane == 0) atomicAnd(&open[e >> 5], ~(1u << (e & 31)));
           if (changed) {
             __syncwarp();
@@ -646,7 +675,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         if (e < ne && li == 0) {
           const unsigned group = LR == 32 ? 0xffffffffu : ((1u << LR) - 1u) << (gi * LR);
           a.gnz[k0 + e] = (bal & group) ? 1 : 0;
-          loc[org[k0 + e]] = 0xFFFFu;
+          loc[lorg[e]] = 0xFFFFu;
         }
       }
       __syncthreads();

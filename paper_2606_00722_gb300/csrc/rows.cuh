@@ -101,9 +101,48 @@ struct RowRegs {
       for (int i = 0; i < KW; ++i) v[i] |= __shfl_xor_sync(0xffffffffu, v[i], off);
   }
   // v = the items waiting on a nonterminal of the set (lane w < VW holds word
-  // w): the groups share out the EXP_NT rows, two in flight each
-  __device__ static __forceinline__ void waiting_on(uint32_t set, const uint32_t* exp_nt, int W, int VW,
-                                                    uint32_t (&v)[KW]) {
+  // w): ORs the set's EXP_NT rows, shared out among the lane groups, several in
+  // flight each.  Wide rows are too large to keep EXP_NT in shared memory, and
+  // a row from L2 costs about as much as testing 30 items: sets of more than
+  // kRowSetMax test every item's next symbol instead (next_t, lanes on
+  // consecutive words; scr: one row of shared scratch).  random-stress-1024
+  // grammar, 4 x 96: forward charts 60 -> 49 ms, good masks 67 -> 45 ms.  The
+  // warp walks keep or_rows: many of them share the rows in L1, and the item
+  // test took their checks from 37 to 50 ms.
+  static constexpr int kRowSetMax = 12;
+  __device__ static __forceinline__ void waiting_on(uint32_t set, const uint32_t* exp_nt, const int16_t* next_t,
+                                                    uint32_t* scr, int W, int VW, uint32_t (&v)[KW]) {
+    if constexpr (KW == 8) {
+      if (__reduce_add_sync(0xffffffffu, (unsigned)__popc(set)) > kRowSetMax) {
+        const int lane = threadIdx.x & 31;
+        if (lane < VW) scr[lane] = set;
+        __syncwarp();
+        uint32_t acc[KW];
+#pragma unroll
+        for (int i = 0; i < KW; ++i) acc[i] = 0u;
+        for (int b = 0; b < 32; ++b) {
+#pragma unroll
+          for (int i = 0; i < KW; ++i) {
+            const int w = lane + 32 * i;
+            const int s = w < W ? next_t[b * W + w] : -1;
+            if (s >= 0) acc[i] |= ((scr[s >> 5] >> (s & 31)) & 1u) << b;
+          }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < KW; ++i)
+          if (lane + 32 * i < W) scr[lane + 32 * i] = acc[i];
+        __syncwarp();
+        load(scr, W, v);
+        __syncwarp();
+        return;
+      }
+    }
+    or_rows(set, exp_nt, W, VW, v);
+  }
+  // v = the OR of the set's rows of table P ([V][W])
+  __device__ static __forceinline__ void or_rows(uint32_t set, const uint32_t* P, int W, int VW, uint32_t (&v)[KW]) {
+    constexpr int F = KW == 4 ? 4 : 2;
     uint32_t share = 0;
 #pragma unroll
     for (int b = 0; b < 32; b += S::NG) share |= 1u << b;
@@ -113,15 +152,21 @@ struct RowRegs {
     for (int w = 0; w < VW; ++w) {
       uint32_t m = __shfl_sync(0xffffffffu, set, w) & share;
       while (m) {
-        const int b0 = __ffs(m) - 1;
-        m &= m - 1;
-        const int b1 = m ? __ffs(m) - 1 : b0;
-        m &= m - 1;
-        uint32_t x[KW], y[KW];
-        load(exp_nt + (size_t)((w << 5) + b0) * W, W, x);
-        load(exp_nt + (size_t)((w << 5) + b1) * W, W, y);
+        uint32_t x[F][KW];
 #pragma unroll
-        for (int i = 0; i < KW; ++i) v[i] |= x[i] | y[i];
+        for (int u = 0; u < F; ++u) {
+          if (u == 0 || m) {
+            load(P + (size_t)((w << 5) + __ffs(m) - 1) * W, W, x[u]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < KW; ++i) x[u][i] = 0u;
+          }
+          m &= m - 1;
+        }
+#pragma unroll
+        for (int u = 0; u < F; ++u)
+#pragma unroll
+          for (int i = 0; i < KW; ++i) v[i] |= x[u][i];
       }
       __syncwarp();
     }
@@ -173,6 +218,25 @@ __device__ __forceinline__ uint32_t warp_ntset(const uint32_t* row, const int32_
     if (lane == v) mine = b;
   }
   return mine;
+}
+
+// Warp: every nonterminal whose completion follows from one of the set (lane
+// v < VW holds word v), by the rows of `follow` ([V][VW], transitively
+// closed: a nonterminal already reached adds nothing).
+__device__ __forceinline__ uint32_t warp_follow(uint32_t set, const uint32_t* follow, int VW) {
+  const int lane = threadIdx.x & 31;
+  uint32_t acc = 0;
+  for (int v = 0; v < VW; ++v) {
+    uint32_t m = __shfl_sync(0xffffffffu, set, v);
+    for (;;) {
+      m &= ~__shfl_sync(0xffffffffu, acc, v);
+      if (!m) break;
+      const int A = (v << 5) + __ffs(m) - 1;
+      m &= m - 1;
+      if (lane < VW) acc |= follow[(size_t)A * VW + lane];
+    }
+  }
+  return acc;
 }
 
 }  // namespace epic

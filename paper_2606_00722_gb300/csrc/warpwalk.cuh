@@ -423,7 +423,7 @@ class WarpWalker {
       if (!__any_sync(0xffffffffu, nw != 0)) break;
       known |= nw;
       uint32_t x[KW];
-      Row::waiting_on(nw, h.exp_nt, W, VW, x);
+      Row::or_rows(nw, h.exp_nt, W, VW, x);
       bool ch = false;
 #pragma unroll
       for (int i = 0; i < KW; ++i) {
@@ -485,7 +485,7 @@ class WarpWalker {
     if (!any && !seeded) return;
     uint32_t r[KW], p[KW];
     Row::load(ws.stage + (size_t)c * W, W, r);
-    Row::waiting_on(vs, gap ? g.gap_pred : g.pred, W, VW, p);
+    Row::or_rows(vs, gap ? g.gap_pred : g.pred, W, VW, p);
 #pragma unroll
     for (int i = 0; i < KW; ++i) r[i] |= p[i];
     // a seeded row (the walk's first column) is closed by the advance rule
