@@ -72,6 +72,10 @@ struct DevGrammar {
   // items with that left side, and the items waiting on it
   const int32_t* cpl_off;         // [V+1]
   const uint2* cpl;               // [n_cpl]
+  // the first four pairs of each nonterminal's complete items: words in
+  // bytes of .x of cpl4w (bit 0 of .y: there are more), masks in cpl4m
+  const uint2* cpl4w;             // [V]
+  const uint4* cpl4m;             // [V]
   const int32_t* wait_off;        // [V+1]
   const uint2* wait;
   int n_cpl, n_wait;

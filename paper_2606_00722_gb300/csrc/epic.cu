@@ -306,7 +306,7 @@ epic_status region_prepare(const epic_grammar* g, epic_lexer_table* t, const int
   }
   // 2. good masks
   mark(t, 1, st);
-  launch_good(B, st, dg, B, sp);
+  launch_good(B, st, dg, sp);
   mark(t, 2, st);
   return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
@@ -535,6 +535,21 @@ epic_status epic_grammar_create(const epic_grammar_desc* desc, epic_grammar** ou
     lists([&](int i) { return G.item_next[i] >= G.T ? G.item_next[i] - G.T : -1; }, woff, wl);
     d.n_cpl = (int)cl.size();
     d.n_wait = (int)wl.size();
+    std::vector<uint2> w4((size_t)G.V, uint2{0u, 0u});
+    std::vector<uint4> m4((size_t)G.V, uint4{0u, 0u, 0u, 0u});
+    for (int A = 0; A < G.V; ++A) {
+      uint32_t* m = &m4[(size_t)A].x;
+      for (int q = coff[A], j = 0; q < coff[A + 1]; ++q, ++j) {
+        if (j == 4) {
+          w4[(size_t)A].y = 1u;
+          break;
+        }
+        w4[(size_t)A].x |= cl[(size_t)q].x << (8 * j);
+        m[j] = cl[(size_t)q].y;
+      }
+    }
+    up(w4, &d.cpl4w);
+    up(m4, &d.cpl4m);
     up(coff, &d.cpl_off);
     up(cl, &d.cpl);
     up(woff, &d.wait_off);
@@ -819,7 +834,7 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   // (whole-graph walks of large grammars are far too long) or when there are
   // more checks than resident walks: the chart of x is then built once per
   // sequence instead of once per check.
-  bool region = g->dg.W > 32 || total > (long long)sm_count() * 2 * kWarpsPerCta;
+  bool region = g->dg.W > 32 || n >= 128 || total > (long long)sm_count() * 2 * kWarpsPerCta;
   if (const char* e = getenv("EPIC_REGION")) region = atoi(e) != 0;
   if (region) return validate_region(g, t, d_x, B, n, d_pos, k, d_cand, K, d_valid, st);
   epic_status s = ensure_wworkspace(t, total, n, st);
@@ -989,9 +1004,11 @@ epic_status epic_fallback_commit(const epic_grammar* g, const epic_lexer_table* 
     return EPIC_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const int nc = k * K;
-  // rounds of m tests per sequence, as many CTAs as two per SM (at most
-  // kMaxFallbackSpec tests per sequence, at least one)
-  int m = std::max(1, std::min(kMaxFallbackSpec, std::min(nc, (2 * sm_count()) / B)));
+  // rounds of m tests per sequence, one CTA per SM (at most kMaxFallbackSpec
+  // tests per sequence, at least one): tests after a round's first pass are
+  // spent, and a walk with an SM to itself has twice the warps (smiles 24 x 96,
+  // four commits a row: 42 ms with two CTAs per SM, 33 ms with one)
+  int m = std::max(1, std::min(kMaxFallbackSpec, std::min(nc, sm_count() / B)));
   epic_status s = ensure_workspace(t, std::min((long long)B * m, (long long)sm_count() * 2), n, st);
   if (s != EPIC_OK) return s;
   m = std::max(1, std::min(m, t->ctas / B));

@@ -52,12 +52,21 @@
 namespace epic {
 
 constexpr int kGsMaxWarps = 16;
-// Threads of a CTA walk: eight warps for narrow rows, so that two CTAs share
-// an SM with 128 registers a thread, four for tiny grammars, whose columns hold
-// too few origins for more.
-inline int gs_threads(int W) { return W <= 4 ? 128 : (W <= 16 ? 256 : 32 * kGsMaxWarps); }
-template <class S>
-constexpr int kGsThreads = S::LR == 4 ? 256 : 32 * kGsMaxWarps;
+// Threads of a CTA walk (128 registers each).  Sixteen warps; eight for narrow
+// rows when there are more walks than SMs, so that two CTAs share one (512
+// threads at 64 registers spilled: smiles-256 forward charts 95 ms against 68);
+// four for tiny grammars, whose columns hold too few origins for more.  With
+// one narrow walk per SM sixteen warps are the faster: smiles 48 x 144 exact
+// tests 20.5 -> 15.8 ms.
+inline int gs_sms() {
+  int dev = 0, n = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  return n > 0 ? n : 1;
+}
+inline int gs_threads(int W, long long walks, int sms) {
+  return W <= 4 ? 128 : (W <= 16 && walks > sms ? 256 : 32 * kGsMaxWarps);
+}
 constexpr long long kGsMaxSteps = 1ll << 22;  // origin visits per column and warp
 constexpr long long kGsMaxIdle = 1ll << 24;   // polls of an idle warp per column
 
@@ -100,7 +109,8 @@ __device__ inline void gs_stage_tables(const DevGrammar& g, unsigned char* smem,
 // Dynamic shared memory of the CTA walks (byte offsets): WalkSmem, the tables
 // above, then the pieces below; `rows` row slots take what is left.
 struct GsPlan {
-  uint32_t o_off, o_list;  // complete items by nonterminal (CSR over V)
+  uint32_t o_w4, o_m4;     // complete items by nonterminal (DevGrammar::cpl4w, cpl4m) ...
+  uint32_t o_off, o_list;  // ... and as lists (narrow rows: short lists, left early)
   uint32_t o_scr;          // per-warp scratch, W words each
   uint32_t o_col;          // column offsets [nmax + 1]
   uint32_t o_slot;         // row slot of each origin [nmax] (uint16)
@@ -130,8 +140,10 @@ inline GsPlan gs_plan(const DevGrammar& g, int nmax, size_t limit) {
     o += r(bytes);
     return (uint32_t)at;
   };
-  p.o_off = put((size_t)(g.V + 1) * 4);
-  p.o_list = put((size_t)g.n_cpl * 8);
+  p.o_w4 = put((size_t)g.V * 8);
+  p.o_m4 = put((size_t)g.V * 16);
+  p.o_off = g.W <= 16 ? put((size_t)(g.V + 1) * 4) : 0;
+  p.o_list = g.W <= 16 ? put((size_t)g.n_cpl * 8) : 0;
   p.o_scr = put((size_t)kGsMaxWarps * g.W * 4);
   p.o_col = put((size_t)(nmax + 1) * 4);
   p.o_slot = put((size_t)nmax * 2);
@@ -190,7 +202,8 @@ class EarleyColsGS {
     uint16_t* slot_of;
     const int32_t *c_off, *col, *org;
     const int16_t* next_t;
-    const uint2* c_lst;
+    const uint2 *c_lst, *w4;
+    const uint4* m4;
     const uint32_t* bits;
     __device__ __forceinline__ uint32_t slot(int o) const { return *(const volatile uint16_t*)(slot_of + o); }
     __device__ __forceinline__ uint32_t* done_of(uint32_t s, int o) const {
@@ -221,8 +234,10 @@ class EarleyColsGS {
     h.stage = ws.stage;
     h.bdone = ws.bdone;
     h.slot_of = (uint16_t*)(m + plan.o_slot);
-    h.c_off = (const int32_t*)(m + plan.o_off);
-    h.c_lst = (const uint2*)(m + plan.o_list);
+    h.w4 = (const uint2*)(m + plan.o_w4);
+    h.m4 = (const uint4*)(m + plan.o_m4);
+    h.c_off = plan.o_list ? (const int32_t*)(m + plan.o_off) : g.cpl_off;
+    h.c_lst = plan.o_list ? (const uint2*)(m + plan.o_list) : g.cpl;
     h.col = (const int32_t*)(m + plan.o_col);
     h.org = ws.org;
     h.bits = ws.bits;
@@ -257,10 +272,14 @@ class EarleyColsGS {
 
   // Block, once per kernel: the shared tables, empty slots, zero rows.
   __device__ void init(unsigned char* smem) {
-    int32_t* off = (int32_t*)(smem + plan.o_off);
-    for (int v = threadIdx.x; v <= g.V; v += blockDim.x) off[v] = g.cpl_off[v];
-    uint2* lst = (uint2*)(smem + plan.o_list);
-    for (int i = threadIdx.x; i < g.n_cpl; i += blockDim.x) lst[i] = g.cpl[i];
+    for (int v = threadIdx.x; v < g.V; v += blockDim.x) {
+      ((uint2*)(smem + plan.o_w4))[v] = g.cpl4w[v];
+      ((uint4*)(smem + plan.o_m4))[v] = g.cpl4m[v];
+    }
+    if (plan.o_list) {
+      for (int v = threadIdx.x; v <= g.V; v += blockDim.x) ((int32_t*)(smem + plan.o_off))[v] = g.cpl_off[v];
+      for (int i = threadIdx.x; i < g.n_cpl; i += blockDim.x) ((uint2*)(smem + plan.o_list))[i] = g.cpl[i];
+    }
     if (plan.o_exp) {
       uint32_t* ex = (uint32_t*)(smem + plan.o_exp);
       for (int i = threadIdx.x; i < g.V * W; i += blockDim.x) ex[i] = g.exp_nt[i];
@@ -477,6 +496,12 @@ class EarleyColsGS {
     return -1;
   }
 
+  // Warp: the nonterminals with a complete item in row (lane v < VW: word v).
+  __device__ static __forceinline__ uint32_t completed(const Hot& h, const uint32_t* row) {
+    if constexpr (LR == 4) return warp_ntset(row, h.c_off, h.c_lst, h.V, h.VW);
+    return warp_completed(row, h.w4, h.m4, h.c_off, h.c_lst, h.V, h.VW);
+  }
+
   // Warp: close row o with its self-loop and scatter the nonterminals that it
   // newly completes over the other entries of column o.
   __device__ static __forceinline__ void visit(const Hot& h, int o, int mode) {
@@ -523,7 +548,7 @@ class EarleyColsGS {
     if (__any_sync(0xffffffffu, any)) {
       if (lane < LR) Row::store(h.scr, W, cm);
       __syncwarp();
-      tot = warp_ntset(h.scr, h.c_off, h.c_lst, h.V, VW) & ~known;
+      tot = completed(h, h.scr) & ~known;
       __syncwarp();
       if (__any_sync(0xffffffffu, tot != 0)) {
         const int kind = 2 * (int)((h.gapb[o >> 5] >> (o & 31)) & 1u) + mode;
@@ -711,8 +736,8 @@ class EarleyColsGS {
   }
 
   // Move the rows of the open column into the entry store as column c
-  // (origins ascending), recording completed nonterminals and summaries.  A
-  // touched row is never empty.
+  // (origins ascending), recording completed nonterminals.  A touched row is
+  // never empty.
   __device__ __noinline__ void finish_column(int c) {
     PH_BEGIN(t_fi);
     const int warp = threadIdx.x >> 5, nw = nwarps();
@@ -771,32 +796,11 @@ class EarleyColsGS {
 
   __device__ bool column_empty(int c) const { return ws.col_off[c + 1] == ws.col_off[c]; }
 
-  // Warp: completed nonterminals and folded summaries of entry k, its row in
-  // memory.
+  // Warp: completed nonterminals of entry k, its row in memory.
   __device__ void record_entry(const uint32_t* row, size_t k) {
     const int lane = threadIdx.x & 31;
-    const uint32_t cn = warp_ntset(row, (const int32_t*)(gs_smem() + plan.o_off), (const uint2*)(gs_smem() + plan.o_list),
-                                   g.V, VW);
+    const uint32_t cn = completed(hot(), row);
     if (lane < VW) rec->cnt[k * VW + lane] = cn;
-    uint32_t fnt = 0, ft = 0;
-    for (int w = lane; w < W; w += 32) {
-      uint32_t m = row[w] & tb.next_any[w];
-      while (m) {
-        const int b = __ffs(m) - 1;
-        m &= m - 1;
-        const int s = tb.item_next[(w << 5) + b];
-        if (s >= g.T)
-          fnt |= 1u << ((s - g.T) & 31);
-        else
-          ft |= 1u << (s & 31);
-      }
-    }
-    fnt = __reduce_or_sync(0xffffffffu, fnt);
-    ft = __reduce_or_sync(0xffffffffu, ft);
-    if (lane == 0) {
-      rec->esum[k * 2] = fnt;
-      rec->esum[k * 2 + 1] = ft;
-    }
   }
 
   // After an aborted walk: return the rows of the open column to zero.

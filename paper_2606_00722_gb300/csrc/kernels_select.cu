@@ -28,7 +28,7 @@ struct SelFrame {
 // two answers when it asks for exactly these tests.  spec[b] = {cover,
 // exact}: 1 pass, 0 fail, -1 not available (overflow / bad input).
 template <class S>
-__global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1) k_select_spec(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table, int vocab,
+__global__ void __launch_bounds__(32 * kGsMaxWarps, 1) k_select_spec(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table, int vocab,
                                                           const int32_t* __restrict__ x, int B, int n,
                                                           const int32_t* __restrict__ pos, int k,
                                                           const int32_t* __restrict__ tok, int8_t* __restrict__ spec,
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1) k_select_sp
 }
 
 template <class S>
-__global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1) k_select(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table, int vocab,
+__global__ void __launch_bounds__(32 * kGsMaxWarps, 1) k_select(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table, int vocab,
                                                      const int32_t* __restrict__ x, int B, int n,
                                                      const int32_t* __restrict__ pos, int k,
                                                      const int32_t* __restrict__ tok, const float* __restrict__ conf,
@@ -389,7 +389,7 @@ __device__ int fallback_best(int b, const int32_t* xb, const int32_t* pos, int k
 // One round: job (b, s) tests the s-th candidate of sequence b's order.
 // res[(b m + s) 2] = candidate (-1: none), [+1] = 1 pass, 0 fail, -1 capacity.
 template <class S>
-__global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1) k_fallback_round(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table,
+__global__ void __launch_bounds__(32 * kGsMaxWarps, 1) k_fallback_round(GsPlan plan, DevGrammar g, const LexEntry* __restrict__ table,
                                                              int vocab, const int32_t* __restrict__ x, int B, int n,
                                                              const int32_t* __restrict__ pos, int k,
                                                              const int32_t* __restrict__ cand,
@@ -502,7 +502,7 @@ void launch_select_spec(dim3 grid, cudaStream_t st, const DevGrammar& g, const L
   const GsPlan p = gs_plan(g, wsp.dims.nmax, gs_limit(g.W));
   auto go = [&](auto* kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
-    kernel<<<grid, gs_threads(g.W), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, tok, spec, wsp);
+    kernel<<<grid, gs_threads(g.W, grid.x, gs_sms()), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, tok, spec, wsp);
   };
   with_row_shape(g.W, [&](auto s) { go(k_select_spec<decltype(s)>); });
 }
@@ -513,7 +513,7 @@ void launch_select(dim3 grid, cudaStream_t st, const DevGrammar& g, const LexEnt
   const GsPlan p = gs_plan(g, wsp.dims.nmax, gs_limit(g.W));
   auto go = [&](auto* kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
-    kernel<<<grid, gs_threads(g.W), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, tok, conf, selected, wsp, spec, stats);
+    kernel<<<grid, gs_threads(g.W, grid.x, gs_sms()), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, tok, conf, selected, wsp, spec, stats);
   };
   with_row_shape(g.W, [&](auto s) { go(k_select<decltype(s)>); });
 }
@@ -532,7 +532,7 @@ void launch_fallback_round(dim3 grid, cudaStream_t st, const DevGrammar& g, cons
   const GsPlan p = gs_plan(g, wsp.dims.nmax, gs_limit(g.W));
   auto go = [&](auto* kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
-    kernel<<<grid, gs_threads(g.W), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, cand, conf, K, m, rej, fb, res,
+    kernel<<<grid, gs_threads(g.W, grid.x, gs_sms()), p.bytes, st>>>(p, g, table, vocab, x, B, n, pos, k, cand, conf, K, m, rej, fb, res,
                                                 wsp, stats);
   };
   with_row_shape(g.W, [&](auto s) { go(k_fallback_round<decltype(s)>); });

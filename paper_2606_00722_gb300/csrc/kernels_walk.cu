@@ -27,11 +27,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta, 2) k_validate_warp(
   }
   WarpWalker<S, false> walk(g, table, ws, shm[warp], wp.nmax, wp.emax, vocab);
   unsigned long long n_checks = 0, n_valid = 0, n_ovf = 0, n_bad = 0, n_cols = 0, n_ent = 0;
-  for (;;) {
-    long long jb = 0;
-    if ((threadIdx.x & 31) == 0) jb = (long long)atomicAdd(counter, 1ull);
-    jb = __shfl_sync(0xffffffffu, jb, 0);
-    if (jb >= total) break;
+  for (long long jb = (long long)warp * gridDim.x + blockIdx.x; jb < total; jb = next_job(counter)) {
     long long b = jb / ((long long)k * K);
     long long j = (jb / K) % k;
     int r = walk.run(x + b * n, n, pos[b * k + j], cand[jb]);

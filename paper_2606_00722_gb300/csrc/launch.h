@@ -20,7 +20,7 @@ void launch_validate_warp(dim3 grid, dim3 block, cudaStream_t st, const DevGramm
 // checks by region
 void launch_forward_gs(dim3 grid, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
                        const int32_t* x, int B, int n, const SeqPack& sp, unsigned long long* stats);
-void launch_good(dim3 grid, cudaStream_t st, const DevGrammar& g, int B, const SeqPack& sp);
+void launch_good(int B, cudaStream_t st, const DevGrammar& g, const SeqPack& sp);
 void launch_check(dim3 grid, dim3 block, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
                   const int32_t* x, int n, const int32_t* pos, int k, const int32_t* cand, int K, long long total,
                   uint8_t* valid, const SeqPack& sp, const WPack& wp, int32_t* regs, unsigned long long* counter,

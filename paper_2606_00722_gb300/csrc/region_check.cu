@@ -242,11 +242,11 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta, 2) k_check(
   rs.act = rs.fmap + wp.nmax;
   rs.act_f = rs.act + wp.nmax;
   unsigned long long n_checks = 0, n_valid = 0, n_ovf = 0, n_bad = 0, n_cols = 0, n_ent = 0;
-  for (;;) {
-    long long jb = 0;
-    if (lane == 0) jb = (long long)atomicAdd(counter, 1ull);
-    jb = __shfl_sync(0xffffffffu, jb, 0);
-    if (jb >= total) break;
+  // The first checks go round the CTAs, then each warp takes the next one left.
+  // (Neighbouring checks cost alike and are issue-bound together: chunks of 16
+  // per CTA, for the sake of its L1, took the checks of code 8 x 96 from 6.5 to
+  // 12.7 ms.)
+  for (long long jb = (long long)warp * gridDim.x + blockIdx.x; jb < total; jb = next_job(counter)) {
     long long b = jb / ((long long)k * K);
     long long jj = (jb / K) % k;
     const int32_t* xb = x + b * n;

@@ -12,7 +12,7 @@ namespace epic {
 // origins of a column shared out among 16 warps, a CTA is the faster one there
 // too.)  Two CTAs share an SM when rows have at most 16 words.
 template <class S>
-__global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1)
+__global__ void __launch_bounds__(32 * kGsMaxWarps, 1)
     k_forward_gs(DevGrammar g, const LexEntry* __restrict__ table, int vocab, const int32_t* __restrict__ x, int B,
                  int n, SeqPack sp, GsPlan plan, unsigned long long* stats) {
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kGsThreads<S>, S::LR == 4 ? 2 : 1)
     sc.ent = a.ent;
     EarleyColsGS<true, S>::place_scratch(g, plan, dyn, sc);
     const BlockRec br{a.rec.col_gap, a.rec.e_dst,   a.rec.e_src,   a.rec.e_lbl,    a.rec.cnt,
-                      a.rec.esum,     a.rec.gap_col, a.rec.pre_col, a.rec.post_col, a.rec.edge_cap};
+                      a.rec.gap_col, a.rec.pre_col, a.rec.post_col, a.rec.edge_cap};
     WsDims d;
     d.nmax = sp.nmax;
     d.emax = sp.emax;
@@ -81,7 +81,7 @@ static void launch_forward_shape(dim3 grid, cudaStream_t st, const DevGrammar& g
                               const int32_t* x, int B, int n, const SeqPack& sp, unsigned long long* stats) {
   const GsPlan p = gs_plan(g, sp.nmax, gs_limit(g.W));
   cudaFuncSetAttribute(k_forward_gs<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
-  k_forward_gs<S><<<grid, gs_threads(g.W), p.bytes, st>>>(g, table, vocab, x, B, n, sp, p, stats);
+  k_forward_gs<S><<<grid, gs_threads(g.W, grid.x, gs_sms()), p.bytes, st>>>(g, table, vocab, x, B, n, sp, p, stats);
 }
 
 void launch_forward_gs(dim3 grid, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,

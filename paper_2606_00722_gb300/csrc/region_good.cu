@@ -7,7 +7,7 @@
 
 namespace epic {
 
-constexpr int kGoodWarps = 16;          // one CTA per sequence
+constexpr int kGoodWarps = 16;          // per CTA
 constexpr int kGoodEdges = 32;          // out-edges whose label masks are held at once
 constexpr int kGoodMaxRounds = 1 << 18; // in-column rounds (each makes at least one item good)
 
@@ -26,7 +26,7 @@ struct GoodPlan {
   uint32_t o_lbl;                // label masks of a chunk of out-edges
   uint32_t o_loc;                // entry of each origin in the open column (uint16), 0xFFFF none
   uint32_t o_chg, o_nxt, o_open; // bitmaps over the open column's entries
-  uint32_t o_fold;               // folded completions of each successor
+  uint32_t o_fold;               // per successor: something completes there
   uint32_t o_sux;                // items waiting on what completes at a successor; sux rows
   uint32_t o_row, o_gnt;         // good masks, and completed nonterminals not known good, of the open column; rows rows
   int sux, rows;
@@ -73,6 +73,60 @@ static GoodPlan good_plan(const DevGrammar& g, int nmax) {
   p.o_gnt = put((size_t)rows * g.VW * 4);
   p.bytes = (uint32_t)o;
   return p;
+}
+
+// ---- the CTAs of a cluster that share one sequence
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// barrier of the cluster's threads (of the CTA when it is alone)
+__device__ __forceinline__ void good_sync(int C) {
+  if (C == 1) {
+    __syncthreads();
+  } else {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+}
+// the address in CTA `rank` of the shared variable at addr here
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ uint4 peer_load4(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t peer_load(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void peer_store(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void peer_or(uint32_t addr, uint32_t v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// a row in global memory that another SM wrote in this kernel: past L1
+template <class S>
+__device__ __forceinline__ void load_row_l2(const uint32_t* p, int W, uint32_t (&v)[S::KW]) {
+  const int w0 = RowRegs<S>::li() * S::KW;
+#pragma unroll
+  for (int q = 0; q < S::KW; q += 4) {
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    if (w0 + q < W) x = __ldcg(reinterpret_cast<const uint4*>(p + w0 + q));
+    v[q] = x.x;
+    v[q + 1] = x.y;
+    v[q + 2] = x.z;
+    v[q + 3] = x.w;
+  }
 }
 
 // Row in registers (a copy in every lane group, or one per group):
@@ -136,18 +190,26 @@ __device__ inline void warp_prefix(int32_t* a, int n) {
 // one end node.  (One entry at a time in ascending origin order, with four
 // block barriers each, left the CTA at barriers for most of the pass.)
 //
+// A cluster of C CTAs shares a sequence when the sequences leave SMs idle: CTA r
+// takes the entries r, r + C, ... of a column and keeps their rows, which the
+// others read over distributed shared memory; successors are shared out the
+// same way, their masks then going through L2.  All barriers are the cluster's
+// and every CTA takes the same path to them.
+//
 // The open column's good masks, the items waiting on what completes at each
 // successor column and the grammar lists sit in shared memory; rows beyond
 // the slots stay in global memory.  What is left is bound by the loads of
 // other columns' rows (several in flight per warp) and the barriers per round.
-template <class S>
-__global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(DevGrammar g, int B, SeqPack sp, GoodPlan p) {
+template <class S, int PER_SM, bool CLUSTER>
+__global__ void __launch_bounds__(32 * kGoodWarps, PER_SM)
+    k_good(DevGrammar g, int B, SeqPack sp, GoodPlan p, int ctas) {
+  const int C = CLUSTER ? ctas : 1;  // CTAs per sequence
   extern __shared__ __align__(16) unsigned char dyn[];
   using Row = RowRegs<S>;
   constexpr int KW = S::KW, LR = S::LR, NG = S::NG;
   constexpr int U = KW == 4 ? 4 : 2;  // rows in flight per lane group
   const int li = Row::li(), gi = Row::gi();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nwarps = nthr >> 5;
   const int W = g.W, VW = g.VW, V = g.V;
   uint32_t* next_any = (uint32_t*)(dyn + p.o_masks);
   int32_t* c_off = (int32_t*)(dyn + p.o_cpl_off);
@@ -157,6 +219,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
   uint32_t* scr = (uint32_t*)(dyn + p.o_scr) + (size_t)warp * W;
   uint32_t* cmp = (uint32_t*)(dyn + p.o_cmp) + warp * 32;
   const uint32_t s_row = gs_saddr(dyn + p.o_row);
+  const int rank = C > 1 ? (int)cluster_rank() : 0;
   uint32_t* lbl = (uint32_t*)(dyn + p.o_lbl);
   uint16_t* loc = (uint16_t*)(dyn + p.o_loc);
   uint32_t* open = (uint32_t*)(dyn + p.o_open);
@@ -167,7 +230,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
   const uint32_t* follow = g.follow;
   const int16_t* next_t = g.next_t;
   __shared__ int s_self, s_more, s_next;
-  __shared__ __align__(16) uint32_t s_xall[kWMaxW];
+  __shared__ __align__(16) uint32_t s_xall[kWMaxW], s_xpart[kWMaxW];
   // the grammar lists
   for (int i = tid; i < W; i += nthr) next_any[i] = g.next_any[i];
   for (int i = tid; i <= V; i += nthr) {
@@ -234,7 +297,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
     Row::load(scr, W, c);
     __syncwarp();
   };
-  for (long long b = blockIdx.x; b < B; b += gridDim.x) {
+  for (long long b = blockIdx.x / C; b < B; b += gridDim.x / C) {
     PH_BEGIN(t_setup);
     SeqArena a = sp.carve(b);
     int32_t* meta = a.rec.meta;
@@ -246,42 +309,45 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
     const int32_t* org = a.ws.org;
     const uint32_t* bits_g = a.ws.bits;
     const int start = meta[M_START], accept = meta[M_ACCEPT];
-    int32_t* cur_o = a.cursor;          // [N + 1]
-    int32_t* cur_s = a.cursor + N + 1;  // [N + 1]
-    // edges by source and entries by origin (CSR), entry index by (column, origin)
-    for (int j = tid; j <= N; j += nthr) {
-      a.in_off[j] = 0;
-      a.out_off[j] = 0;
-      a.succ_off[j] = 0;
-    }
-    for (int u = tid; u < N; u += nthr) a.last_col[u] = -1;
-    const size_t ntri = (size_t)N * (N + 1) / 2;
-    for (size_t q = tid; q < ntri; q += nthr) a.eidx[q] = -1;
-    __syncthreads();
-    for (int e = tid; e < NE; e += nthr) {
-      atomicAdd(&a.in_off[a.rec.e_dst[e] + 1], 1);
-      atomicAdd(&a.out_off[a.rec.e_src[e] + 1], 1);
-    }
-    for (int j = warp; j < N; j += kGoodWarps)
-      for (long long k = col[j] + lane; k < col[j + 1]; k += 32) {
-        const int o = org[k];
-        a.eidx[tri_index(j, o)] = (int32_t)k;
-        a.gnz[k] = 0;
-        atomicAdd(&a.succ_off[o + 1], 1);
-        atomicMax(&a.last_col[o], j);
+    if (rank == 0) {  // the indexes, by the first CTA
+      int32_t* cur_o = a.cursor;          // [N + 1]
+      int32_t* cur_s = a.cursor + N + 1;  // [N + 1]
+      // edges by source and entries by origin (CSR), entry index by (column, origin)
+      for (int j = tid; j <= N; j += nthr) {
+        a.in_off[j] = 0;
+        a.out_off[j] = 0;
+        a.succ_off[j] = 0;
       }
-    __syncthreads();
-    if (warp < 3) warp_prefix(warp == 0 ? a.in_off : (warp == 1 ? a.out_off : a.succ_off), N);
-    __syncthreads();
-    for (int j = tid; j < N; j += nthr) {
-      cur_o[j] = a.out_off[j];
-      cur_s[j] = a.succ_off[j];
+      for (int u = tid; u < N; u += nthr) a.last_col[u] = -1;
+      const size_t ntri = (size_t)N * (N + 1) / 2;
+      for (size_t q = tid; q < ntri; q += nthr) a.eidx[q] = -1;
+      __syncthreads();
+      for (int e = tid; e < NE; e += nthr) {
+        atomicAdd(&a.in_off[a.rec.e_dst[e] + 1], 1);
+        atomicAdd(&a.out_off[a.rec.e_src[e] + 1], 1);
+      }
+      for (int j = warp; j < N; j += nwarps)
+        for (long long k = col[j] + lane; k < col[j + 1]; k += 32) {
+          const int o = org[k];
+          a.eidx[tri_index(j, o)] = (int32_t)k;
+          a.gnz[k] = 0;
+          atomicAdd(&a.succ_off[o + 1], 1);
+          atomicMax(&a.last_col[o], j);
+        }
+      __syncthreads();
+      if (warp < 3) warp_prefix(warp == 0 ? a.in_off : (warp == 1 ? a.out_off : a.succ_off), N);
+      __syncthreads();
+      for (int j = tid; j < N; j += nthr) {
+        cur_o[j] = a.out_off[j];
+        cur_s[j] = a.succ_off[j];
+      }
+      __syncthreads();
+      for (int e = tid; e < NE; e += nthr) a.out_idx[atomicAdd(&cur_o[a.rec.e_src[e]], 1)] = e;
+      for (int j = warp; j < N; j += nwarps)
+        for (long long k = col[j] + lane; k < col[j + 1]; k += 32) a.succ_idx[atomicAdd(&cur_s[org[k]], 1)] = j;
+      __syncthreads();
     }
-    __syncthreads();
-    for (int e = tid; e < NE; e += nthr) a.out_idx[atomicAdd(&cur_o[a.rec.e_src[e]], 1)] = e;
-    for (int j = warp; j < N; j += kGoodWarps)
-      for (long long k = col[j] + lane; k < col[j + 1]; k += 32) a.succ_idx[atomicAdd(&cur_s[org[k]], 1)] = j;
-    __syncthreads();
+    good_sync(C);
     PH_END(0, t_setup);
     uint32_t* G = a.good;
     for (int j = N - 1; j >= 0; --j) {
@@ -292,18 +358,48 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
       uint32_t* chg = (uint32_t*)(dyn + p.o_chg);
       uint32_t* nxt = (uint32_t*)(dyn + p.o_nxt);
       auto row_of = [&](int e) -> uint32_t* {
-        return e < p.rows ? (uint32_t*)(dyn + p.o_row) + (size_t)e * W : G + (size_t)(k0 + e) * W;
+        const int slot = e / C;  // rows of this CTA's entries (e % C == rank)
+        return slot < p.rows ? (uint32_t*)(dyn + p.o_row) + (size_t)slot * W : G + (size_t)(k0 + e) * W;
       };
       auto gnt_of = [&](int e) -> uint32_t* {  // overflow: the forward walk's completion record is free
-        return e < p.rows ? (uint32_t*)(dyn + p.o_gnt) + (size_t)e * VW : a.bdone + (size_t)e * VW;
+        const int slot = e / C;
+        return slot < p.rows ? (uint32_t*)(dyn + p.o_gnt) + (size_t)slot * VW : a.bdone + (size_t)e * VW;
       };
       auto sux_of = [&](int s) -> uint32_t* {
-        return s < p.sux ? (uint32_t*)(dyn + p.o_sux) + (size_t)s * W : a.expn + (size_t)s * W;
+        return C == 1 && s < p.sux ? (uint32_t*)(dyn + p.o_sux) + (size_t)s * W : a.expn + (size_t)s * W;
       };
+      auto load_sux = [&](int s, uint32_t(&v)[KW]) {
+        if (C == 1)
+          Row::load(sux_of(s), W, v);
+        else
+          load_row_l2<S>(sux_of(s), W, v);
+      };
+      auto load_later = [&](size_t k, uint32_t(&v)[KW]) {  // good mask of a later column's entry
+        if (C == 1)
+          Row::load(G + k * W, W, v);
+        else
+          load_row_l2<S>(G + k * W, W, v);
+      };
+      auto is_good = [&](int k) -> bool { return (C == 1 ? a.gnz[k] : __ldcg(a.gnz + k)) != 0; };
       // a row that its owner may be writing (bits only get set)
       auto load_good = [&](int e, uint32_t(&v)[KW]) {
-        if (e < p.rows) {
-          Row::load_shared(s_row + (uint32_t)e * (uint32_t)(W * 4), W, v);
+        const int slot = e / C;
+        if (slot < p.rows) {
+          const uint32_t at = s_row + (uint32_t)slot * (uint32_t)(W * 4);
+          if (C == 1) {
+            Row::load_shared(at, W, v);
+          } else {
+            const uint32_t far = peer_addr(at, (uint32_t)(e - slot * C)) + (uint32_t)(li * KW) * 4u;
+#pragma unroll
+            for (int q = 0; q < KW; q += 4) {
+              uint4 x = make_uint4(0u, 0u, 0u, 0u);
+              if (li * KW + q < W) x = peer_load4(far + 4u * q);
+              v[q] = x.x;
+              v[q + 1] = x.y;
+              v[q + 2] = x.z;
+              v[q + 3] = x.w;
+            }
+          }
         } else {
 #pragma unroll
           for (int i = 0; i < KW; ++i)
@@ -320,7 +416,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         }
         if (self_si >= 0 && sfold[self_si]) {
           uint32_t x[KW];
-          Row::load(sux_of(self_si), W, x);
+          load_sux(self_si, x);
 #pragma unroll
           for (int i = 0; i < KW; ++i) m[i] |= x[i];
         }
@@ -332,7 +428,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         s_self = -1;
         s_next = 0;
       }
-      for (int w = tid; w < W; w += nthr) s_xall[w] = 0;
+      for (int w = tid; w < W; w += nthr) s_xpart[w] = 0;
       for (int e = tid; e < ne; e += nthr) {
         const int o = org[k0 + e];
         loc[o] = (uint16_t)e;
@@ -344,12 +440,22 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         open[w] = 0;
       }
       __syncthreads();
-      for (int si = s0 + warp; si < s1; si += kGoodWarps) {
+      // s_self and sfold of every CTA may be written by the others from here on
+      if (C > 1) good_sync(C);
+      for (int si = s0 + warp * C + rank; si < s1; si += nwarps * C) {
         const int j2 = a.succ_idx[si];
         const uint32_t* cn = a.rec.cnt + (size_t)a.eidx[tri_index(j2, j)] * VW;
         const uint32_t set = lane < VW ? cn[lane] : 0u;
-        const uint32_t f = __reduce_or_sync(0xffffffffu, set);  // folded (bit C mod 32): 0 = nothing completes
-        if (j2 == j && lane == 0) s_self = si - s0;
+        const uint32_t f = __any_sync(0xffffffffu, set != 0) ? 1u : 0u;
+        if (lane < C) {
+          if (C == 1) {
+            sfold[si - s0] = f;
+            if (j2 == j) s_self = si - s0;
+          } else {
+            peer_store(peer_addr(gs_saddr(sfold + (si - s0)), lane), f);
+            if (j2 == j) peer_store(peer_addr(gs_saddr(&s_self), lane), (uint32_t)(si - s0));
+          }
+        }
         if (f) {
           uint32_t ex[KW];
           Row::waiting_on(set, exp_nt, next_t, scr, W, VW, ex);
@@ -358,12 +464,17 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
             if (j2 != j) {
 #pragma unroll
               for (int i = 0; i < KW; ++i)
-                if (ex[i] & ~*(volatile uint32_t*)&s_xall[min(li * KW + i, kWMaxW - 1)])
-                  atomicOr(&s_xall[li * KW + i], ex[i]);
+                if (ex[i] & ~*(volatile uint32_t*)&s_xpart[min(li * KW + i, kWMaxW - 1)])
+                  atomicOr(&s_xpart[li * KW + i], ex[i]);
             }
           }
         }
-        if (lane == 0) sfold[si - s0] = f;
+      }
+      good_sync(C);
+      for (int w = tid; w < W; w += nthr) {  // the CTAs' unions
+        uint32_t u = 0;
+        for (int r = 0; r < C; ++r) u |= C == 1 ? s_xpart[w] : peer_load(peer_addr(gs_saddr(s_xpart + w), r));
+        s_xall[w] = u;
       }
       // A. the rules that read later columns: out-edges, a chunk at a time
       const int eb0 = a.out_off[j], eb1 = a.out_off[j + 1];
@@ -371,7 +482,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
       do {
         const int nc = min(kGoodEdges, eb1 - chunk);
         __syncthreads();
-        for (int q = warp; q < nc; q += kGoodWarps) {  // label masks of the chunk
+        for (int q = warp; q < nc; q += nwarps) {  // label masks of the chunk
           const uint32_t* L = a.rec.e_lbl + (size_t)a.out_idx[chunk + q] * 8;
           uint32_t m[KW];
 #pragma unroll
@@ -409,7 +520,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         const int self_si = s_self;
         uint32_t inrow[KW];  // in-row rules of this column: the gap self-loop and nullable completions
         in_row(inrow, gap, self_si);
-        for (int e = warp; e < ne; e += kGoodWarps) {
+        for (int e = warp * C + rank; e < ne; e += nwarps * C) {
           const size_t k = (size_t)k0 + e;
           const int o = lorg[e];
           uint32_t* Gk = row_of(e);
@@ -429,7 +540,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
               if (li * KW + i == (g.accept_item >> 5)) acc[i] |= 1u << (g.accept_item & 31);
           }
           int k2 = dst >= 0 ? a.eidx[tri_index(dst, o)] : -1;
-          if (k2 >= 0 && !a.gnz[k2]) k2 = -1;
+          if (k2 >= 0 && !is_good(k2)) k2 = -1;
           const int na = compact(k2 >= 0, k2);
           for (int t0 = 0; t0 < na; t0 += NG * U) {
             uint32_t gv[U][KW];
@@ -440,7 +551,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
               l[u] = -1;
               if (t < na) {
                 l[u] = cmp[t] & 31;
-                Row::load(G + (size_t)(cmp[t] >> 5) * W, W, gv[u]);
+                load_later(cmp[t] >> 5, gv[u]);
               } else {
 #pragma unroll
                 for (int i = 0; i < KW; ++i) gv[u][i] = 0u;
@@ -458,7 +569,6 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
           }
           Row::join(acc);
           if (last) {
-            const uint32_t wfold = a.rec.esum[k * 2];  // waited nonterminals, folded
             // the most the nested rule can make good: items waiting on a
             // nonterminal that completes from j somewhere after j
             uint32_t want[KW];
@@ -474,9 +584,9 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
               if (saturated()) break;
               const int si = sb + lane;
               int k3 = -1;
-              if (si < s1 && si - s0 != self_si && (sfold[si - s0] & wfold) != 0) {
+              if (si < s1 && si - s0 != self_si && sfold[si - s0]) {
                 const int kk = a.eidx[tri_index(a.succ_idx[si], o)];
-                if (kk >= 0 && a.gnz[kk]) k3 = kk;
+                if (kk >= 0 && is_good(kk)) k3 = kk;
               }
               const int n3 = compact(k3 >= 0, k3);
               for (int t0 = 0; t0 < n3; t0 += NG * U) {
@@ -485,8 +595,8 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
                 for (int u = 0; u < U; ++u) {
                   const int t = t0 + u * NG + gi;
                   if (t < n3) {
-                    Row::load(G + (size_t)(cmp[t] >> 5) * W, W, gv[u]);
-                    Row::load(sux_of(sb + (int)(cmp[t] & 31) - s0), W, xv[u]);
+                    load_later(cmp[t] >> 5, gv[u]);
+                    load_sux(sb + (int)(cmp[t] & 31) - s0, xv[u]);
                   } else {
 #pragma unroll
                     for (int i = 0; i < KW; ++i) gv[u][i] = xv[u][i] = 0u;
@@ -518,7 +628,12 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
             const bool cpl = __any_sync(0xffffffffu, cn != 0);
             if (lane < VW) gnt_of(e)[lane] = cn;
             if (lane == 0) {
-              if (nz) atomicOr(&chg[e >> 5], 1u << (e & 31));
+              if (nz) {
+                if (C == 1)
+                  atomicOr(&chg[e >> 5], 1u << (e & 31));
+                else
+                  for (int r = 0; r < C; ++r) peer_or(peer_addr(gs_saddr(&chg[e >> 5]), r), 1u << (e & 31));
+              }
               if (cpl) atomicOr(&open[e >> 5], 1u << (e & 31));
             }
           }
@@ -526,17 +641,16 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         PH_END(2, t_a);
         chunk += nc;
       } while (chunk < eb1);
-      __syncthreads();
       // B. completions within the column, in rounds (see above)
       PH_BEGIN(t_g);
       for (int round = 0;; ++round) {
         if (tid == 0) s_more = 0;
-        __syncthreads();
+        good_sync(C);
         const int sel = s_self;
         for (;;) {
           int e = 0;
           if (lane == 0) e = atomicAdd(&s_next, 1);
-          e = __shfl_sync(0xffffffffu, e, 0);
+          e = __shfl_sync(0xffffffffu, e, 0) * C + rank;
           if (e >= ne) break;
           if (!((open[e >> 5] >> (e & 31)) & 1u)) continue;
           const size_t k = (size_t)k0 + e;
@@ -639,12 +753,19 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
             __syncwarp();
             if (lane < LR) Row::store(Gk, W, r);
             if (lane == 0) {
-              atomicOr(&nxt[e >> 5], 1u << (e & 31));
-              s_more = 1;
+              if (C == 1) {
+                atomicOr(&nxt[e >> 5], 1u << (e & 31));
+                s_more = 1;
+              } else {
+                for (int r = 0; r < C; ++r) {
+                  peer_or(peer_addr(gs_saddr(&nxt[e >> 5]), r), 1u << (e & 31));
+                  peer_store(peer_addr(gs_saddr(&s_more), r), 1u);
+                }
+              }
             }
           }
         }
-        __syncthreads();
+        good_sync(C);
         uint32_t* t = chg;
         chg = nxt;
         nxt = t;
@@ -661,8 +782,8 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
       PH_END(3, t_g);
       // the column's masks to global memory
       PH_BEGIN(t_w);
-      for (int e0 = warp * NG; e0 < ne; e0 += kGoodWarps * NG) {
-        const int e = e0 + gi;
+      for (int e0 = warp * NG; e0 * C < ne; e0 += nwarps * NG) {
+        const int e = (e0 + gi) * C + rank;
         bool nz = false;
         if (e < ne) {
           uint32_t v[KW];
@@ -675,22 +796,62 @@ __global__ void __launch_bounds__(32 * kGoodWarps, S::LR == 4 ? 2 : 1) k_good(De
         if (e < ne && li == 0) {
           const unsigned group = LR == 32 ? 0xffffffffu : ((1u << LR) - 1u) << (gi * LR);
           a.gnz[k0 + e] = (bal & group) ? 1 : 0;
-          loc[lorg[e]] = 0xFFFFu;
         }
       }
-      __syncthreads();
+      for (int e = tid; e < ne; e += nthr) loc[lorg[e]] = 0xFFFFu;
+      good_sync(C);  // masks written, and nobody reads this column's rows any more
       PH_END(4, t_w);
     }
     __syncthreads();
   }
+  if (C > 1) good_sync(C);  // no CTA ends while another may read its shared memory
 }
 
-void launch_good(dim3 grid, cudaStream_t st, const DevGrammar& g, int B, const SeqPack& sp) {
+// The CTAs that share a sequence: as many as leave every cluster its own SMs (a
+// seventh of the SMs is spared: clusters do not fill every group of SMs).
+// C-like 32 x 256: 67 ms alone, 33 ms with four; 400 nonterminals 4 x 96: 45 and
+// 18 ms with eight.  Narrow rows stay alone: their columns hold too little work
+// between the cluster's barriers (JSON 16 x 256: 4.0 ms alone, 6.8 ms with eight).
+static int good_cluster(int B, int W, int sms) {
+  int C = W <= 16 ? 1 : 8;
+  while (C > 1 && (long long)B * C * 8 > 7ll * sms) C >>= 1;
+  return C;
+}
+
+void launch_good(int B, cudaStream_t st, const DevGrammar& g, const SeqPack& sp) {
   const GoodPlan p = good_plan(g, sp.nmax);
-  with_row_shape(g.W, [&](auto s) {
-    auto* kernel = k_good<decltype(s)>;
+  const int sms = gs_sms(), C = good_cluster(B, g.W, sms);
+  auto go = [&](auto* kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.bytes);
-    kernel<<<grid, 32 * kGoodWarps, p.bytes, st>>>(g, B, sp, p);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(B * C));
+    cfg.blockDim = dim3(32 * kGoodWarps);
+    cfg.dynamicSmemBytes = p.bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, g, B, sp, p, C);
+  };
+  with_row_shape(g.W, [&](auto s) {
+    using S = decltype(s);
+    if constexpr (S::LR == 4) {
+      // more sequences than SMs: two CTAs per SM at 64 registers (molecules,
+      // 256 x 256: 52 ms; eight warps at 128 registers 60 ms)
+      if (B > sms)
+        go(k_good<S, 2, false>);
+      else
+        go(k_good<S, 1, false>);
+    } else {
+      if (C > 1)
+        go(k_good<S, 1, true>);
+      else
+        go(k_good<S, 1, false>);
+    }
   });
 }
 

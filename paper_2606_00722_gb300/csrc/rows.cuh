@@ -220,6 +220,29 @@ __device__ __forceinline__ uint32_t warp_ntset(const uint32_t* row, const int32_
   return mine;
 }
 
+// The same for the complete items, the first four pairs of a nonterminal's
+// list in one place: no loop unless its items lie in more than four words.
+__device__ __forceinline__ uint32_t warp_completed(const uint32_t* row, const uint2* w4, const uint4* m4,
+                                                   const int32_t* off, const uint2* lst, int V, int VW) {
+  const int lane = threadIdx.x & 31;
+  uint32_t mine = 0;
+  for (int v = 0; v < VW; ++v) {
+    const int A = (v << 5) + lane;
+    bool hit = false;
+    if (A < V) {
+      const uint2 w = w4[A];
+      const uint4 m = m4[A];
+      hit = ((row[w.x & 255u] & m.x) | (row[(w.x >> 8) & 255u] & m.y) | (row[(w.x >> 16) & 255u] & m.z) |
+             (row[w.x >> 24] & m.w)) != 0;
+      if (w.y && !hit)
+        for (int q = off[A] + 4, e = off[A + 1]; q < e && !hit; ++q) hit = (row[lst[q].x] & lst[q].y) != 0;
+    }
+    const uint32_t b = __ballot_sync(0xffffffffu, hit);
+    if (lane == v) mine = b;
+  }
+  return mine;
+}
+
 // Warp: every nonterminal whose completion follows from one of the set (lane
 // v < VW holds word v), by the rows of `follow` ([V][VW], transitively
 // closed: a nonterminal already reached adds nothing).

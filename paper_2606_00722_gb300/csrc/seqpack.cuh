@@ -35,7 +35,7 @@ struct SeqPack {
   __host__ __device__ size_t bytes() const {
     size_t nm = nmax;
     return r(nm * W * 4) + r(nm * VW * 4) + r((nm + 1) * 4) + 7 * r(kWMaxQ * 4) + r(kWMaxQ * 16) + r(kWMaxQ * 32) +
-           r((size_t)emax * 4) + r((size_t)emax * 8) + r((size_t)emax * W * 4)  // WWs
+           r((size_t)emax * 4) + r((size_t)emax * W * 4)  // WWs
            + r(nm) + 2 * r((size_t)edge_cap * 4) + r((size_t)edge_cap * 32) + 3 * r((size_t)n * 4) +
            r((size_t)emax * VW * 4) + r(32)                                                 // SeqRec
            + r((size_t)emax * W * 4) + r(nm * 4) + 3 * r((nm + 1) * 4) + r((size_t)edge_cap * 4) +
@@ -64,7 +64,6 @@ struct SeqPack {
     a.ws.g_tail = (uint32_t*)take(kWMaxQ * 16);
     a.ws.g_lbl = (uint32_t*)take(kWMaxQ * 32);
     a.ws.org = (int32_t*)take((size_t)emax * 4);
-    a.rec.esum = (uint32_t*)take((size_t)emax * 8);
     a.ws.bits = (uint32_t*)take((size_t)emax * W * 4);
     a.rec.col_gap = (uint8_t*)take(nm);
     a.rec.e_dst = (int32_t*)take((size_t)edge_cap * 4);

@@ -136,16 +136,13 @@ __device__ __forceinline__ void clear_bitmap(uint32_t* bm, int nbits) {
 // What a recording walk (a sequence's forward chart, for checks by region)
 // writes besides the chart: the graph's edges in target order with their
 // terminal sets (all zero: epsilon), gap flags, each entry's completed
-// nonterminals and folded summaries (bit B mod 32 of a waited-on nonterminal,
-// bit a mod 32 of an expected terminal), and the column before, at and after
-// each position's segment.
+// nonterminals, and the column before, at and after each position's segment.
 struct BlockRec {
   uint8_t* col_gap;   // [nmax]
   int32_t* e_dst;     // [edge_cap]
   int32_t* e_src;     // [edge_cap]
   uint32_t* e_lbl;    // [edge_cap][8]
   uint32_t* cnt;      // [emax][VW]
-  uint32_t* esum;     // [emax][2]
   int32_t* gap_col;   // [n]
   int32_t* pre_col;   // [n]
   int32_t* post_col;  // [n]

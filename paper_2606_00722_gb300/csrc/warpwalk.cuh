@@ -55,7 +55,7 @@ struct WWs {  // per-walk global workspace
 
 // What a sequence's forward chart records besides the chart: the graph's edges
 // in creation order of their target, gap flags, where each position's segment
-// sits in the graph, and each entry's completed nonterminals and summaries.
+// sits in the graph, and each entry's completed nonterminals.
 struct SeqRec {
   uint8_t* col_gap;    // [nmax]
   int32_t* e_dst;      // [edge_cap]
@@ -65,7 +65,6 @@ struct SeqRec {
   int32_t* pre_col;    // [n] fixed position -> column before its span (gap or BEGIN)
   int32_t* post_col;   // [n] fixed position -> column after its span (gap or END)
   uint32_t* cnt;       // [emax][VW] completed nonterminals of each entry
-  uint32_t* esum;      // [emax][2] folded summaries (bit B mod 32 of a waited-on nonterminal, a mod 32 of a terminal)
   int32_t* meta;       // [8]: ncols, nedges, start, accept, status, nent (low), -, -
   int edge_cap;
 };
@@ -79,6 +78,13 @@ struct WSh {  // per-warp shared memory
 };
 
 __device__ __forceinline__ uint32_t wl_lane() { return threadIdx.x & 31; }
+
+// Warp: the next job after the grid's first ones (one per warp).
+__device__ __forceinline__ long long next_job(unsigned long long* counter) {
+  long long j = 0;
+  if (wl_lane() == 0) j = (long long)atomicAdd(counter, 1ull) + (long long)gridDim.x * (blockDim.x >> 5);
+  return __shfl_sync(0xffffffffu, j, 0);
+}
 
 // Warp: out[w] = items waiting on a member of the nonterminal set nts
 // (VW words, readable by every lane), for the lane's words w.  A small set
@@ -243,7 +249,8 @@ class WarpWalker {
     uint32_t *stage, *touched, *scr;
     const uint32_t *adv, *complete, *exp_nt, *b_bits, *bits;
     const int32_t *cpl_off, *b_off, *b_org, *off, *org;
-    const uint2* cpl;
+    const uint2 *cpl, *w4;
+    const uint4* m4;
     __device__ __forceinline__ int column(int c, const int32_t*& o, const uint32_t*& x) const {
       if (EXT && c < base_cols) {
         const int b = b_off[c];
@@ -279,6 +286,8 @@ class WarpWalker {
     h.off = ws.col_off;
     h.org = ws.org;
     h.cpl = g.cpl;
+    h.w4 = g.cpl4w;
+    h.m4 = g.cpl4m;
     return h;
   }
 
@@ -418,7 +427,8 @@ class WarpWalker {
       if (!__any_sync(0xffffffffu, fresh)) break;
       if (wl_lane() < LR) Row::store(h.scr, W, cm);
       __syncwarp();
-      const uint32_t nw = warp_ntset(h.scr, h.cpl_off, h.cpl, h.V, VW) & ~known;
+      const uint32_t nw = (LR == 4 ? warp_ntset(h.scr, h.cpl_off, h.cpl, h.V, VW)
+                                   : warp_completed(h.scr, h.w4, h.m4, h.cpl_off, h.cpl, h.V, VW)) & ~known;
       __syncwarp();
       if (!__any_sync(0xffffffffu, nw != 0)) break;
       known |= nw;
