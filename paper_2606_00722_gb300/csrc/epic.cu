@@ -319,8 +319,9 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
   // per-warp workspace of the checks: own columns after the chart's
   WPack wp;
   wp.nmax = kWCols;
-  // own entries: the region's columns and the rows carried after it
-  wp.emax = std::max(8192ll, 64ll * n);
+  // own entries: the region's columns and the rows carried after it (narrow
+  // rows: as much as a whole walk, since a region can be most of a row)
+  wp.emax = std::max(8192ll, (dg.W <= 32 ? 256ll : 64ll) * n);
   if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) wp.emax = atoll(e);
   wp.W = dg.W;
   wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, wp.W);
@@ -362,6 +363,20 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
                k, d_cand, K, total, d_valid, sp, wp, t->d_regs, t->d_counter, t->d_stats);
   mark(t, 3, st);
   return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+}
+
+// Whole-graph walks with a CTA per check (`slots` of them at a time) or with a
+// warp per check?  A CTA walk ends several times sooner and fills an SM, so it
+// wins while every check has a slot at once: JSON 4 x 64, 128 checks: 1.7 ms
+// against 2.7 (by region 3.5); molecules 4 x 96, 128 checks: 7.0 against 21
+// (16); C-like rows cost one walk instead of the forward chart, good masks and
+// checks.  Longer narrow rows still gain with two rounds (256 checks: JSON
+// 4 x 150 8.8 ms against 15, by region 11; JSON 4 x 64 3.1 against 2.4).
+// Grammars of at most 4 item words have too little in a column for it (32 x 8
+// expression checks 0.83 ms against 0.78).
+bool cta_walks(long long total, int n, int W, long long slots) {
+  if (W <= 4) return false;
+  return total <= slots || (W <= 32 && n >= 96 && total <= 2 * slots);
 }
 
 WsPack pack_of(const epic_lexer_table* t) {
@@ -830,13 +845,35 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   if (total == 0) return EPIC_OK;
   if (!d_x || !d_pos || !d_cand || !d_valid || n == 0) return EPIC_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // Checks by region over a per-sequence chart when the item sets are wide
-  // (whole-graph walks of large grammars are far too long) or when there are
-  // more checks than resident walks: the chart of x is then built once per
-  // sequence instead of once per check.
-  bool region = g->dg.W > 32 || n >= 128 || total > (long long)sm_count() * 2 * kWarpsPerCta;
-  if (const char* e = getenv("EPIC_REGION")) region = atoi(e) != 0;
+  // Few checks walk their whole graphs, a CTA each.  Else checks by region over
+  // a per-sequence chart, built once per sequence instead of once per check:
+  // when the item sets are wide (whole-graph walks of large grammars are far
+  // too long), when there are more checks than resident walks, and on rows of
+  // at least 128 tokens (JSON 16 x 256, 1,024 checks: 20 ms against 25; 16 x
+  // 64: 4.9 against 3.3, and the lines cross in between).
+  bool few = cta_walks(total, n, g->dg.W, sm_count());
+  bool region = !few && (g->dg.W > 32 || n >= 128 || total > (long long)sm_count() * 2 * kWarpsPerCta);
+  if (const char* e = getenv("EPIC_REGION")) {
+    region = atoi(e) != 0;
+    few = few && !region;
+  }
   if (region) return validate_region(g, t, d_x, B, n, d_pos, k, d_cand, K, d_valid, st);
+  // Few checks: a CTA each.
+  if (few) {
+    const epic_status s = ensure_workspace(t, (int)std::min<long long>(total, sm_count()), n, st);
+    if (s != EPIC_OK) return s;
+    long long cap = t->dims.emax;
+    if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) cap = atoll(e);
+    t->last = st;
+    t->n_vkernels += 1;
+    t->nk = 1;
+    t->kname[0] = "k_validate_cta";
+    mark(t, 0, st);
+    launch_validate_cta((int)std::min<long long>(total, t->ctas), st, t->dgl, t->d_table, t->vocab, d_x, n, d_pos, k,
+                        d_cand, K, total, d_valid, pack_of(t), cap, 0, t->d_stats);
+    mark(t, 1, st);
+    return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+  }
   epic_status s = ensure_wworkspace(t, total, n, st);
   if (s != EPIC_OK) return s;
   t->last = st;
@@ -931,6 +968,27 @@ epic_status epic_validate_batch_noalloc(const epic_grammar* g, const epic_lexer_
   wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, W);
   long long fit = (long long)((kNoAllocBytes - 256) / wp.per_warp);
   if (fit < 1) return EPIC_ERR_CAPACITY;  // one walk's workspace does not fit the array
+  {
+    WsPack p;
+    p.base = base + 256;
+    p.dims.nmax = wp.nmax;
+    p.dims.emax = wp.emax;
+    p.W = W;
+    p.VW = g->dg.VW;
+    p.FW = 0;
+    p.per_cta = ws_bytes_per_cta(p.dims, W, p.VW, 0);
+    const long long ctas = std::min<long long>({total, (long long)((kNoAllocBytes - 256) / p.per_cta),
+                                                (long long)sm_count()});
+    // (the array holds fewer CTA walks than there are SMs: JSON 4 x 128, 71;
+    // 256 checks in four rounds of them 14 ms, a warp each 19 ms)
+    if (ctas >= 1 && (cta_walks(total, n, W, ctas) || (n >= 96 && W > 4 && total <= 4 * ctas))) {
+      t->last = st;
+      t->n_vkernels += 1;
+      launch_validate_cta((int)ctas, st, t->dgl, t->d_table, t->vocab, d_x, n, d_pos, k, d_cand, K, total, d_valid, p,
+                          wp.emax, 1, t->d_stats);
+      return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    }
+  }
   unsigned long long* counter = (unsigned long long*)base;
   // the kernel reads the table's lex entries and adds into its counters:
   // epic_get_stats and epic_lexer_table_destroy synchronize this stream

@@ -110,7 +110,8 @@ __device__ inline void gs_stage_tables(const DevGrammar& g, unsigned char* smem,
 // above, then the pieces below; `rows` row slots take what is left.
 struct GsPlan {
   uint32_t o_w4, o_m4;     // complete items by nonterminal (DevGrammar::cpl4w, cpl4m) ...
-  uint32_t o_off, o_list;  // ... and as lists (narrow rows: short lists, left early)
+  uint32_t o_off, o_list;  // ... and as lists
+  uint32_t o_woff, o_wait; // items waiting on each nonterminal, as lists; 0: read from global memory
   uint32_t o_scr;          // per-warp scratch, W words each
   uint32_t o_col;          // column offsets [nmax + 1]
   uint32_t o_slot;         // row slot of each origin [nmax] (uint16)
@@ -142,8 +143,11 @@ inline GsPlan gs_plan(const DevGrammar& g, int nmax, size_t limit) {
   };
   p.o_w4 = put((size_t)g.V * 8);
   p.o_m4 = put((size_t)g.V * 16);
-  p.o_off = g.W <= 16 ? put((size_t)(g.V + 1) * 4) : 0;
-  p.o_list = g.W <= 16 ? put((size_t)g.n_cpl * 8) : 0;
+  p.o_off = put((size_t)(g.V + 1) * 4);
+  p.o_list = put((size_t)g.n_cpl * 8);
+  const bool wait_in = (size_t)g.n_wait * 8 <= 12 * 1024;
+  p.o_woff = wait_in ? put((size_t)(g.V + 1) * 4) : 0;
+  p.o_wait = wait_in ? put((size_t)g.n_wait * 8) : 0;
   p.o_scr = put((size_t)kGsMaxWarps * g.W * 4);
   p.o_col = put((size_t)(nmax + 1) * 4);
   p.o_slot = put((size_t)nmax * 2);
@@ -236,8 +240,8 @@ class EarleyColsGS {
     h.slot_of = (uint16_t*)(m + plan.o_slot);
     h.w4 = (const uint2*)(m + plan.o_w4);
     h.m4 = (const uint4*)(m + plan.o_m4);
-    h.c_off = plan.o_list ? (const int32_t*)(m + plan.o_off) : g.cpl_off;
-    h.c_lst = plan.o_list ? (const uint2*)(m + plan.o_list) : g.cpl;
+    h.c_off = (const int32_t*)(m + plan.o_off);
+    h.c_lst = (const uint2*)(m + plan.o_list);
     h.col = (const int32_t*)(m + plan.o_col);
     h.org = ws.org;
     h.bits = ws.bits;
@@ -276,9 +280,11 @@ class EarleyColsGS {
       ((uint2*)(smem + plan.o_w4))[v] = g.cpl4w[v];
       ((uint4*)(smem + plan.o_m4))[v] = g.cpl4m[v];
     }
-    if (plan.o_list) {
-      for (int v = threadIdx.x; v <= g.V; v += blockDim.x) ((int32_t*)(smem + plan.o_off))[v] = g.cpl_off[v];
-      for (int i = threadIdx.x; i < g.n_cpl; i += blockDim.x) ((uint2*)(smem + plan.o_list))[i] = g.cpl[i];
+    for (int v = threadIdx.x; v <= g.V; v += blockDim.x) ((int32_t*)(smem + plan.o_off))[v] = g.cpl_off[v];
+    for (int i = threadIdx.x; i < g.n_cpl; i += blockDim.x) ((uint2*)(smem + plan.o_list))[i] = g.cpl[i];
+    if (plan.o_wait) {
+      for (int v = threadIdx.x; v <= g.V; v += blockDim.x) ((int32_t*)(smem + plan.o_woff))[v] = g.wait_off[v];
+      for (int i = threadIdx.x; i < g.n_wait; i += blockDim.x) ((uint2*)(smem + plan.o_wait))[i] = g.wait[i];
     }
     if (plan.o_exp) {
       uint32_t* ex = (uint32_t*)(smem + plan.o_exp);
@@ -679,12 +685,14 @@ class EarleyColsGS {
         if (acc[j] & an[j]) atomicOr(&walk_gs().uni[Row::li() * KW + j], acc[j] & an[j]);
     }
     __syncthreads();
+    const int32_t* w_off = plan.o_wait ? (const int32_t*)(gs_smem() + plan.o_woff) : g.wait_off;
+    const uint2* w_lst = plan.o_wait ? (const uint2*)(gs_smem() + plan.o_wait) : g.wait;
     for (int v = warp; v < VW; v += nw) {  // one warp per word of the set
       const int A = (v << 5) + lane;
       bool hit = false;
       if (A < g.V)
-        for (int q = g.wait_off[A], e = g.wait_off[A + 1]; q < e && !hit; ++q) {
-          const uint2 p = g.wait[q];
+        for (int q = w_off[A], e = w_off[A + 1]; q < e && !hit; ++q) {
+          const uint2 p = w_lst[q];
           hit = (walk_gs().uni[p.x] & p.y) != 0;
         }
       const uint32_t b = __ballot_sync(0xffffffffu, hit);
@@ -757,10 +765,11 @@ class EarleyColsGS {
       walk_gs().nslots = 0;
     }
     if constexpr (REC) {
+      const Hot h = hot();
       if (ok)
         for (int i = warp; i < nl; i += nw) {
           const int o = walk_sh().list[i];
-          record_entry(row_of(slot(o), o), (size_t)base + i);
+          record_entry(h, row_of(slot(o), o), (size_t)base + i);
         }
     }
     if (REC) __syncthreads();  // rows are cleared below, by other warps than read them here
@@ -797,9 +806,9 @@ class EarleyColsGS {
   __device__ bool column_empty(int c) const { return ws.col_off[c + 1] == ws.col_off[c]; }
 
   // Warp: completed nonterminals of entry k, its row in memory.
-  __device__ void record_entry(const uint32_t* row, size_t k) {
+  __device__ __forceinline__ void record_entry(const Hot& h, const uint32_t* row, size_t k) {
     const int lane = threadIdx.x & 31;
-    const uint32_t cn = completed(hot(), row);
+    const uint32_t cn = completed(h, row);
     if (lane < VW) rec->cnt[k * VW + lane] = cn;
   }
 

@@ -17,6 +17,12 @@ void launch_validate_warp(dim3 grid, dim3 block, cudaStream_t st, const DevGramm
                           long long total, uint8_t* valid, const WPack& wp, int zero_stage,
                           unsigned long long* counter, unsigned long long* stats);
 
+// whole-graph walks, one CTA per check
+void launch_validate_cta(int ctas, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
+                         const int32_t* x, int n, const int32_t* pos, int k, const int32_t* cand, int K,
+                         long long total, uint8_t* valid, const WsPack& wsp, long long cap, int zero_rows,
+                         unsigned long long* stats);
+
 // checks by region
 void launch_forward_gs(dim3 grid, cudaStream_t st, const DevGrammar& g, const LexEntry* table, int vocab,
                        const int32_t* x, int B, int n, const SeqPack& sp, unsigned long long* stats);

@@ -17,7 +17,7 @@ import numpy as np
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # translation units, compiled in parallel and linked into one library
 _SRC = [os.path.join(_HERE, 'csrc', f) for f in
-        ('epic.cu', 'kernels_walk.cu', 'kernels_select.cu', 'region_forward.cu', 'region_good.cu',
+        ('epic.cu', 'kernels_walk.cu', 'kernels_cta.cu', 'kernels_select.cu', 'region_forward.cu', 'region_good.cu',
          'region_check.cu', 'peak.cu', 'witness.cu', 'grammar.cpp')]
 _DEPS = _SRC + [os.path.join(_HERE, 'csrc', f) for f in
                 ('grammar.h', 'device.cuh', 'walk.cuh', 'cover.cuh', 'warpwalk.cuh', 'packs.cuh',
