@@ -386,24 +386,34 @@ class EarleyColsGS {
       const uint32_t s_t = okt ? h.slot(o_t) : kSlotNone;
       const uint32_t a_t = s_t < (uint32_t)R ? s_rows + s_t * (uint32_t)(W * 4) : s_zero;
       const int steps = min(LR, (ne - first * NG + stride * NG - 1) / (stride * NG) - c0);
+      const int last_t = 31 - __clz(__ballot_sync(0xffffffffu, okt));  // the lane of the chunk's last entry
       for (int u0 = 0; u0 < steps; u0 += U) {
         uint32_t v[U][KW];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int e = ((c0 + u0 + u) * stride + first) * NG + gi;
-          if (u0 + u < steps && e < ne) {
-            Row::load(bits + (size_t)e * W, W, v[u]);
-          } else {
+          if constexpr (LR == 4) {  // eight entries a step: columns often end within it
+            const int e = ((c0 + u0 + u) * stride + first) * NG + gi;
+            if (u0 + u < steps && e < ne) {
+              Row::load(bits + (size_t)e * W, W, v[u]);
+            } else {
 #pragma unroll
-            for (int i = 0; i < KW; ++i) v[u][i] = 0u;
+              for (int i = 0; i < KW; ++i) v[u][i] = 0u;
+            }
+          } else {  // past the end: the last entry again
+            Row::load_any(bits + (size_t)min(((c0 + min(u0 + u, steps - 1)) * stride + first) * NG + gi, ne - 1) * W, W,
+                          v[u]);
           }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int t = ((u0 + u) * NG + gi) & 31;
+          // (its lookup is in lane t of this chunk)
+          const int t = LR == 4 ? ((u0 + u) * NG + gi) & 31 : min(min(u0 + u, steps - 1) * NG + gi, last_t);
           const uint32_t addr = __shfl_sync(0xffffffffu, a_t, t);
           uint32_t q[KW];
-          Row::load_shared(addr, W, q);
+          if constexpr (LR == 4)
+            Row::load_shared(addr, W, q);
+          else
+            Row::load_shared_any(addr, W, q);
 #pragma unroll
           for (int i = 0; i < KW; ++i) v[u][i] &= m[i];
           if (SHIFT) Row::shift_up(v[u]);
@@ -465,6 +475,7 @@ class EarleyColsGS {
     } else {
 #pragma unroll
       for (int i = 0; i < KW; ++i) m[i] = 0xffffffffu;
+      Row::valid(m, h.W);
     }
     if (shift)
       scatter<true>(h, h.col[src], h.col[src + 1], m, warp, nw);

@@ -547,22 +547,17 @@ __global__ void __launch_bounds__(32 * kGoodWarps, PER_SM)
             int l[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-              const int t = t0 + u * NG + gi;  // this group's edge: the t-th active one
-              l[u] = -1;
-              if (t < na) {
-                l[u] = cmp[t] & 31;
-                load_later(cmp[t] >> 5, gv[u]);
-              } else {
-#pragma unroll
-                for (int i = 0; i < KW; ++i) gv[u][i] = 0u;
-              }
+              // this group's edge: the t-th active one (past the end: the last one again)
+              const uint32_t c = cmp[min(t0 + u * NG + gi, na - 1)];
+              l[u] = c & 31;
+              load_later(c >> 5, gv[u]);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
               uint32_t s[KW], m[KW];
               Row::shift_down(gv[u], s);
-              const bool ep = l[u] >= 0 && ((epsm >> l[u]) & 1u);
-              Row::load(lbl + (size_t)(l[u] < 0 ? 0 : l[u]) * W, W, m);
+              const bool ep = (epsm >> l[u]) & 1u;
+              Row::load(lbl + (size_t)l[u] * W, W, m);
 #pragma unroll
               for (int i = 0; i < KW; ++i) acc[i] |= ep ? gv[u][i] : (s[i] & m[i]);
             }
@@ -593,14 +588,9 @@ __global__ void __launch_bounds__(32 * kGoodWarps, PER_SM)
                 uint32_t gv[U][KW], xv[U][KW];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                  const int t = t0 + u * NG + gi;
-                  if (t < n3) {
-                    load_later(cmp[t] >> 5, gv[u]);
-                    load_sux(sb + (int)(cmp[t] & 31) - s0, xv[u]);
-                  } else {
-#pragma unroll
-                    for (int i = 0; i < KW; ++i) gv[u][i] = xv[u][i] = 0u;
-                  }
+                  const uint32_t c = cmp[min(t0 + u * NG + gi, n3 - 1)];
+                  load_later(c >> 5, gv[u]);
+                  load_sux(sb + (int)(c & 31) - s0, xv[u]);
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
@@ -679,15 +669,9 @@ __global__ void __launch_bounds__(32 * kGoodWarps, PER_SM)
               int ee[U];
 #pragma unroll
               for (int u = 0; u < U; ++u) {
-                const int t = t0 + u * NG + gi;
-                if (t < na) {
-                  ee[u] = (int)(cmp[t] >> 5);
-                  Row::load(bits_g + (size_t)(c0 + (int)(cmp[t] & 31)) * W, W, pv[u]);
-                } else {
-                  ee[u] = e;
-#pragma unroll
-                  for (int i = 0; i < KW; ++i) pv[u][i] = 0u;
-                }
+                const uint32_t c = cmp[min(t0 + u * NG + gi, na - 1)];
+                ee[u] = (int)(c >> 5);
+                Row::load(bits_g + (size_t)(c0 + (int)(c & 31)) * W, W, pv[u]);
               }
 #pragma unroll
               for (int u = 0; u < U; ++u) {

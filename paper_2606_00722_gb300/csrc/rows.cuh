@@ -61,6 +61,36 @@ struct RowRegs {
       v[q + 3] = x.w;
     }
   }
+  // The inner loops load without predicates: lanes beyond the row read its last
+  // words instead, and their masks are zero (valid()).
+  __device__ static __forceinline__ int word(int q, int W) {  // first word of this lane's piece q
+    return min(li() * KW + q, W - 4);
+  }
+  __device__ static __forceinline__ void load_any(const uint32_t* p, int W, uint32_t (&v)[KW]) {
+#pragma unroll
+    for (int q = 0; q < KW; q += 4) {
+      const uint4 x = *reinterpret_cast<const uint4*>(p + word(q, W));
+      v[q] = x.x;
+      v[q + 1] = x.y;
+      v[q + 2] = x.z;
+      v[q + 3] = x.w;
+    }
+  }
+  __device__ static __forceinline__ void load_shared_any(uint32_t addr, int W, uint32_t (&v)[KW]) {
+#pragma unroll
+    for (int q = 0; q < KW; q += 4) {
+      const uint4 x = gs_lds4(addr + (uint32_t)word(q, W) * 4u);
+      v[q] = x.x;
+      v[q + 1] = x.y;
+      v[q + 2] = x.z;
+      v[q + 3] = x.w;
+    }
+  }
+  __device__ static __forceinline__ void valid(uint32_t (&v)[KW], int W) {
+#pragma unroll
+    for (int q = 0; q < KW; q += 4)
+      if (li() * KW + q >= W) v[q] = v[q + 1] = v[q + 2] = v[q + 3] = 0u;
+  }
   __device__ static __forceinline__ void load_shared(uint32_t addr, int W, uint32_t (&v)[KW]) {
     const int w0 = li() * KW;
 #pragma unroll
@@ -153,15 +183,12 @@ struct RowRegs {
       uint32_t m = __shfl_sync(0xffffffffu, set, w) & share;
       while (m) {
         uint32_t x[F][KW];
+        int b = 0;
 #pragma unroll
-        for (int u = 0; u < F; ++u) {
-          if (u == 0 || m) {
-            load(P + (size_t)((w << 5) + __ffs(m) - 1) * W, W, x[u]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < KW; ++i) x[u][i] = 0u;
-          }
+        for (int u = 0; u < F; ++u) {  // the last one again when there are fewer
+          b = m ? __ffs(m) - 1 : b;
           m &= m - 1;
+          load_any(P + (size_t)((w << 5) + b) * W, W, x[u]);
         }
 #pragma unroll
         for (int u = 0; u < F; ++u)
@@ -170,6 +197,7 @@ struct RowRegs {
       }
       __syncwarp();
     }
+    valid(v, W);
     join(v);
   }
   // Closure of r under item i -> i + 1 for i in the advance mask (mode 0:

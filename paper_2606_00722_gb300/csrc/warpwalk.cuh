@@ -308,15 +308,10 @@ class WarpWalker {
         uint32_t v[U][KW], q[U][KW];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int t = u0 + u * NG + gi;
-          const int o2 = __shfl_sync(0xffffffffu, o_t, t & 31);
-          if (t < n) {
-            Row::load(bits + (size_t)(c0 + t) * W, W, v[u]);
-            Row::load(h.stage + (size_t)o2 * W, W, q[u]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < KW; ++i) v[u][i] = q[u][i] = 0u;
-          }
+          const int t = min(u0 + u * NG + gi, n - 1);  // past the end: the last entry again
+          const int o2 = __shfl_sync(0xffffffffu, o_t, t);
+          Row::load_any(bits + (size_t)(c0 + t) * W, W, v[u]);
+          Row::load_any(h.stage + (size_t)o2 * W, W, q[u]);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -331,7 +326,7 @@ class WarpWalker {
           }
           const unsigned bal = __ballot_sync(0xffffffffu, nw != 0);
           if (bal) {
-            const int o2 = __shfl_sync(0xffffffffu, o_t, (u0 + u * NG + gi) & 31);
+            const int o2 = __shfl_sync(0xffffffffu, o_t, min(u0 + u * NG + gi, n - 1));
             if (bal & group) {
               Row::store(h.stage + (size_t)o2 * W, W, q[u]);
               if (li == 0) atomicOr(&h.touched[o2 >> 5], 1u << (o2 & 31));
@@ -364,6 +359,7 @@ class WarpWalker {
     } else {
 #pragma unroll
       for (int i = 0; i < KW; ++i) m[i] = 0xffffffffu;
+      Row::valid(m, h.W);
       scatter<false>(h, org, bits, ne, m);
     }
   }
