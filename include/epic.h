@@ -154,11 +154,13 @@ epic_status epic_lexer_table_copy(const epic_lexer_table* t, int32_t first_token
  * EPIC_ERR_INVALID_ARG for sizes < 0 or NULL pointers with non-empty sizes.
  * Device-side: an unmasked position or an out-of-range token id yields 0 for
  * that check and counts in stats.bad_inputs.  Asynchronous.
- * Two strategies give identical results: one warp per check walking the
- * whole graph of x (+) (pos, tok); or, when item sets exceed 32 words or the
- * batch has more checks than resident walks, one forward chart of x per
- * sequence (with its graph and good-item masks) and one warp per check
- * walking only the candidate's region (stats.region_checks counts these).
+ * Three strategies give identical results: one CTA per check walking the
+ * whole graph of x (+) (pos, tok), for a check or two per SM; one warp per
+ * check doing so, for short rows; or one forward chart of x per sequence
+ * (with its graph and good-item masks) and one warp per check walking only
+ * the candidate's region, when item sets exceed 32 words, rows have 128
+ * tokens or more, or the batch has more checks than resident walks
+ * (stats.region_checks counts these).
  * The library's device workspaces grow on demand, each up to a share of the
  * GPU's memory (per-sequence charts 30 %, per-warp walks 25 %, block walks of
  * selection 25 %, never more than is free; EPIC_SEQ_WORKSPACE_MB,
