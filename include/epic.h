@@ -155,8 +155,8 @@ epic_status epic_lexer_table_copy(const epic_lexer_table* t, int32_t first_token
  * Device-side: an unmasked position or an out-of-range token id yields 0 for
  * that check and counts in stats.bad_inputs.  Asynchronous.
  * Three strategies give identical results: one CTA per check walking the
- * whole graph of x (+) (pos, tok), for a check or two per SM; one warp per
- * check doing so, for short rows; or one forward chart of x per sequence
+ * whole graph of x (+) (pos, tok), for a check or two per SM of a narrow
+ * grammar; one warp per check doing so, for short rows; or one forward chart of x per sequence
  * (with its graph and good-item masks) and one warp per check walking only
  * the candidate's region, when item sets exceed 32 words, rows have 128
  * tokens or more, or the batch has more checks than resident walks

@@ -369,8 +369,7 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
 // warp per check?  A CTA walk ends several times sooner and fills an SM, so it
 // wins while every check has a slot at once: JSON 4 x 64, 128 checks: 1.7 ms
 // against 2.7 (by region 3.5); molecules 4 x 96, 128 checks: 7.0 against 21
-// (16); C-like rows cost one walk instead of the forward chart, good masks and
-// checks.  Longer narrow rows still gain with two rounds (256 checks: JSON
+// (16).  Longer narrow rows still gain with two rounds (256 checks: JSON
 // 4 x 150 8.8 ms against 15, by region 11; JSON 4 x 64 3.1 against 2.4).
 // Grammars of at most 4 item words have too little in a column for it (32 x 8
 // expression checks 0.83 ms against 0.78).
@@ -845,13 +844,14 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   if (total == 0) return EPIC_OK;
   if (!d_x || !d_pos || !d_cand || !d_valid || n == 0) return EPIC_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // Few checks walk their whole graphs, a CTA each.  Else checks by region over
+  // Few checks of narrow item sets walk their whole graphs, a CTA each (wide
+  // item sets always go by region).  Else checks by region over
   // a per-sequence chart, built once per sequence instead of once per check:
   // when the item sets are wide (whole-graph walks of large grammars are far
   // too long), when there are more checks than resident walks, and on rows of
   // at least 128 tokens (JSON 16 x 256, 1,024 checks: 20 ms against 25; 16 x
   // 64: 4.9 against 3.3, and the lines cross in between).
-  bool few = cta_walks(total, n, g->dg.W, sm_count());
+  bool few = g->dg.W <= 32 && cta_walks(total, n, g->dg.W, sm_count());
   bool region = !few && (g->dg.W > 32 || n >= 128 || total > (long long)sm_count() * 2 * kWarpsPerCta);
   if (const char* e = getenv("EPIC_REGION")) {
     region = atoi(e) != 0;
