@@ -70,20 +70,16 @@ inline int gs_threads(int W, long long walks, int sms) {
 constexpr long long kGsMaxSteps = 1ll << 22;  // origin visits per column and warp
 constexpr long long kGsMaxIdle = 1ll << 24;   // polls of an idle warp per column
 
-// Grammar tables read by the per-item loops, staged in shared memory:
-// item -> next symbol (int16 [D]) and the W-word masks.
+// Grammar masks of W words, staged in shared memory.
 struct GsTables {
-  const int16_t* item_next;
   const uint32_t* complete;
   const uint32_t* any_nt;
-  const uint32_t* next_any;
-  const uint32_t* nullable_next;
   const uint32_t* adv_pow;  // [2][steps][W] (DevGrammar::adv_pow)
 };
 
-__host__ __device__ inline size_t gs_tables_bytes(int D, int W, int steps) {
+__host__ __device__ inline size_t gs_tables_bytes(int W, int steps) {
   auto r = [](size_t b) { return (b + 15) & ~(size_t)15; };
-  return r((size_t)D * 2) + 4 * r((size_t)W * 4) + r((size_t)2 * steps * W * 4);
+  return 2 * r((size_t)W * 4) + r((size_t)2 * steps * W * 4);
 }
 
 // Block: copy the tables into smem (gs_tables_bytes) and point t at them.
@@ -97,11 +93,8 @@ __device__ inline void gs_stage_tables(const DevGrammar& g, unsigned char* smem,
     p += (bytes + 15) & ~(size_t)15;
     return dst;
   };
-  t.item_next = (const int16_t*)put(g.item_next, (size_t)g.D * 2);
   t.complete = (const uint32_t*)put(g.complete, (size_t)g.W * 4);
   t.any_nt = (const uint32_t*)put(g.any_nt, (size_t)g.W * 4);
-  t.next_any = (const uint32_t*)put(g.next_any, (size_t)g.W * 4);
-  t.nullable_next = (const uint32_t*)put(g.nullable_next, (size_t)g.W * 4);
   t.adv_pow = (const uint32_t*)put(g.adv_pow, (size_t)2 * g.adv_steps * g.W * 4);
   __syncthreads();
 }
@@ -135,7 +128,7 @@ constexpr size_t kGsWalkBytesPerState = 7 * 4 + 16 + 32 + 16;  // WalkScratch pe
 inline GsPlan gs_plan(const DevGrammar& g, int nmax, size_t limit) {
   auto r = [](size_t b) { return (b + 15) & ~(size_t)15; };
   GsPlan p;
-  size_t o = kWalkSmemBytes + r(gs_tables_bytes(g.D, g.W, g.adv_steps));
+  size_t o = kWalkSmemBytes + r(gs_tables_bytes(g.W, g.adv_steps));
   auto put = [&](size_t bytes) {
     const size_t at = o;
     o += r(bytes);
