@@ -21,7 +21,7 @@ struct GoodPlan {
   uint32_t o_fol;                // DevGrammar::follow; 0: read from global memory
   uint32_t o_col;                // column offsets [nmax + 1]
   uint32_t o_org;                // origins of the open column's entries (uint16)
-  uint32_t o_scr;                // per-warp scratch, W words each
+  uint32_t o_scr;                // per-warp scratch, scr words each
   uint32_t o_cmp;                // per-warp list of a batch's active lanes
   uint32_t o_lbl;                // label masks of a chunk of out-edges
   uint32_t o_loc;                // entry of each origin in the open column (uint16), 0xFFFF none
@@ -30,6 +30,10 @@ struct GoodPlan {
   uint32_t o_sux;                // items waiting on what completes at a successor; sux rows
   uint32_t o_row, o_gnt;         // good masks, and completed nonterminals not known good, of the open column; rows rows
   int sux, rows;
+  // words of a warp's scratch: a row, or a nonterminal set.  Sets can be the
+  // longer of the two: nonterminals keep their declared numbers, rows hold the
+  // items that trimming leaves.
+  int scr;
   uint32_t bytes;
 };
 
@@ -48,7 +52,8 @@ static GoodPlan good_plan(const DevGrammar& g, int nmax) {
   p.o_cpl = put((size_t)g.n_cpl * 8);
   p.o_wait_off = put((size_t)(g.V + 1) * 4);
   p.o_wait = put((size_t)g.n_wait * 8);
-  p.o_scr = put((size_t)kGoodWarps * g.W * 4);
+  p.scr = g.W > g.VW ? g.W : (g.VW + 3) / 4 * 4;
+  p.o_scr = put((size_t)kGoodWarps * p.scr * 4);
   p.o_cmp = put((size_t)kGoodWarps * 32 * 4);
   p.o_lbl = put((size_t)kGoodEdges * g.W * 4);
   p.o_loc = put((size_t)nmax * 2);
@@ -216,7 +221,7 @@ __global__ void __launch_bounds__(32 * kGoodWarps, PER_SM)
   uint2* c_lst = (uint2*)(dyn + p.o_cpl);
   int32_t* w_off = (int32_t*)(dyn + p.o_wait_off);
   uint2* w_lst = (uint2*)(dyn + p.o_wait);
-  uint32_t* scr = (uint32_t*)(dyn + p.o_scr) + (size_t)warp * W;
+  uint32_t* scr = (uint32_t*)(dyn + p.o_scr) + (size_t)warp * p.scr;
   uint32_t* cmp = (uint32_t*)(dyn + p.o_cmp) + warp * 32;
   const uint32_t s_row = gs_saddr(dyn + p.o_row);
   const int rank = C > 1 ? (int)cluster_rank() : 0;

@@ -6,6 +6,7 @@ nullable symbols and on which of the two nodes is a gap.  The grammars here
 put W on both sides of every boundary and hold epsilon rules in every place of
 a production; every path (whole-graph walks, checks by region, selection, the
 rejection fallback) answers small batches bit for bit."""
+import dataclasses
 import os
 
 import numpy as np
@@ -37,6 +38,15 @@ def eps_grammar():
     b.rule('N', '', 'M', 'A N')
     b.rule('M', '', 'N M')
     return b.build('S', 'ab() ')
+
+
+def padded(spec, extra):
+    """The same language with `extra` nonterminals declared ahead of the others that no production uses."""
+    T = spec.T
+    shift = lambda s: s if s < T else s + extra
+    return dataclasses.replace(spec, nonterminals=['unused%d' % i for i in range(extra)] + list(spec.nonterminals),
+                               start=spec.start + extra,
+                               productions=[(lhs + extra, [shift(s) for s in rhs]) for lhs, rhs in spec.productions])
 
 
 def item_words(spec):
@@ -88,6 +98,23 @@ def test_rows_against_oracle(cuda, monkeypatch, name, path):
     assert st['overflow'] == 0
     O = oracle.Oracle(spec, vocab)
     np.testing.assert_array_equal(got, O.validate_batch(x, pos, cand, nthreads=NTHREADS))
+
+
+@pytest.mark.parametrize('name,extra,path', [('eps', 160, '1'), ('eps', 1000, '1'), ('eps', 1000, '0'),
+                                             ('random-40-130', 980, '1'), ('random-210-700', 800, '1')])
+def test_more_declared_nonterminals_than_items(cuda, monkeypatch, name, extra, path):
+    """Nonterminals keep their declared numbers and rows hold only the items
+    that trimming leaves, so a set of nonterminals can be longer than a row."""
+    monkeypatch.setenv('EPIC_REGION', path)
+    spec = GRAMMARS[name][0]()
+    n, rows, k, K = (18, 9, 5, 6) if name == 'eps' else (12, 4, 3, 4)
+    vocab, x, pos, cand, conf = random_rows(spec, 7, rows, n, k, K)
+    wide = padded(spec, extra)
+    ref = oracle.Oracle(wide, vocab).validate_batch(x, pos, cand, nthreads=NTHREADS)
+    np.testing.assert_array_equal(ref, oracle.Oracle(spec, vocab).validate_batch(x, pos, cand, nthreads=NTHREADS))
+    got, st = run_gpu(wide, vocab, x, pos, cand, cuda)
+    assert st['overflow'] == 0 and ref.any()
+    np.testing.assert_array_equal(got, ref)
 
 
 @pytest.mark.parametrize('name', sorted(GRAMMARS))
