@@ -37,11 +37,8 @@ class CoverCols {
   }
   __device__ void cleanup() {}
   __device__ int open_column() {
-    int c = walk_sh().ncols;
-    if (c >= dims.nmax || c >= kMaxCols) {
-      if (threadIdx.x == 0) walk_sh().status = kWalkOverflow;
-      return -1;
-    }
+    const int c = walk_sh().ncols;
+    if (c >= dims.nmax || c >= kMaxCols) return -1;  // (every thread sees this: no status needed)
     for (int w = threadIdx.x; w < FW; w += blockDim.x) ws.cov[(size_t)c * FW + w] = 0;
     if (threadIdx.x == 0) walk_sh().scratch_i[0] = c;
     __syncthreads();

@@ -320,13 +320,12 @@ class EarleyColsGS {
   }
 
   __device__ int ncols() const { return walk_sh().ncols; }
+  // The next column, or -1 when there is no room (known to every thread: the
+  // status is not written here, slower warps may still read it for the column
+  // before).
   __device__ int open_column() {
-    int c = walk_sh().ncols;
-    if (c >= dims.nmax || c >= kMaxCols) {
-      if (threadIdx.x == 0) walk_sh().status = kWalkOverflow;
-      return -1;
-    }
-    return c;
+    const int c = walk_sh().ncols;
+    return c < dims.nmax && c < kMaxCols ? c : -1;
   }
 
   // ------------------------------------------------------------ row slots
