@@ -162,11 +162,14 @@ epic_status epic_lexer_table_copy(const epic_lexer_table* t, int32_t first_token
  * tokens or more, or the batch has more checks than resident walks
  * (stats.region_checks counts these).
  * The library's device workspaces grow on demand, each up to a share of the
- * GPU's memory (per-sequence charts 30 %, per-warp walks 25 %, block walks of
- * selection 25 %, never more than is free; EPIC_SEQ_WORKSPACE_MB,
- * EPIC_WARP_WORKSPACE_MB and EPIC_WORKSPACE_MB override, in MiB).  Smaller
- * budgets run fewer walks at a time; a failed allocation returns
- * EPIC_ERR_OOM.  A sequence whose chart does not fit walks its checks whole.
+ * GPU's memory (per-sequence charts 30 %, per-warp walks 25 %, block walks --
+ * selection, the fallback and the CTA walks here -- 25 %, never more than is
+ * free; EPIC_SEQ_WORKSPACE_MB, EPIC_WARP_WORKSPACE_MB and EPIC_WORKSPACE_MB
+ * override, in MiB).  Smaller budgets run fewer walks at a time.  Item sets of
+ * at most 32 words fall back to a warp per check when the workspace of the
+ * other strategy is too small or cannot be had; else a failed allocation
+ * returns EPIC_ERR_OOM.  A sequence whose chart does not fit walks its checks
+ * whole.
  */
 epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t,
                                 const int32_t* d_x, int32_t B, int32_t n, const int32_t* d_pos,

@@ -146,6 +146,16 @@ epic_status upload(epic_grammar* g, const std::vector<T>& v, const T** out) {
   return EPIC_OK;
 }
 
+// Device memory for a workspace; false (and no error left behind for the next
+// call's check of its launches) when there is not enough.
+template <class T>
+bool device_alloc(T** p, size_t bytes) {
+  if (cudaMalloc((void**)p, bytes) == cudaSuccess) return true;
+  (void)cudaGetLastError();
+  *p = nullptr;
+  return false;
+}
+
 int sm_count() {
   int dev = 0, n = 0;
   cudaGetDevice(&dev);
@@ -154,8 +164,8 @@ int sm_count() {
 }
 
 // Default budget of one device workspace: a share of the GPU's memory, and no
-// more than is free now plus what the workspace already holds (it is freed
-// before it grows), less 1 GiB of headroom.  An environment variable (MiB)
+// more than it holds already plus what is free now less 1 GiB of headroom (so
+// a call that ran once finds the same room again).  An environment variable (MiB)
 // overrides.  The three workspaces (per-sequence charts 30 %, warp walks
 // 25 %, block walks 25 %) leave a fifth of the GPU to the caller.
 size_t workspace_budget(const char* env, double share, size_t held) {
@@ -163,30 +173,41 @@ size_t workspace_budget(const char* env, double share, size_t held) {
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return (size_t)4096 << 20;
   const size_t headroom = (size_t)1 << 30;
-  size_t avail = free_b + held > headroom ? free_b + held - headroom : 0;
-  return std::min((size_t)(share * (double)total_b), avail);
+  return std::min((size_t)(share * (double)total_b), held + (free_b > headroom ? free_b - headroom : 0));
 }
 
-// Block-walk workspace of selection and the fallback: every CTA gets room
-// for one whole chart of a row (4,096 columns, 640 n entries, as the
+// Block-walk workspace of selection, the fallback and few checks: every CTA
+// gets room for one whole chart of a row (4,096 columns, 640 n entries, as the
 // per-sequence forward charts; EPIC_ENTRIES_PER_CTA overrides), and as many
 // CTAs as asked run if their workspaces fit EPIC_WORKSPACE_MB (default a
 // quarter of the GPU), else fewer (the kernels loop over their sequences).
-epic_status ensure_workspace(epic_lexer_table* t, int want_ctas, int n, cudaStream_t st) {
+struct BlockPlan {
+  WsDims d;
+  size_t per;
+  int ctas;
+};
+BlockPlan plan_workspace(const epic_lexer_table* t, int want_ctas, int n) {
   const epic_grammar* g = t->g;
   int W = g->dg.W, VW = g->dg.VW, FW = g->dg.FW;
-  WsDims d;
+  BlockPlan p;
+  WsDims& d = p.d;
   d.nmax = kMaxCols;
   d.emax = std::max<long long>(4096, 640ll * std::max(1, n));
   if (const char* e = getenv("EPIC_ENTRIES_PER_CTA")) d.emax = std::max<long long>(64, atoll(e));
   const size_t budget = workspace_budget("EPIC_WORKSPACE_MB", 0.25, t->d_ws ? t->ws_bytes : 0);
-  size_t per = ws_bytes_per_cta(d, W, VW, FW);
-  while (per > budget && d.emax > 4096) {  // not even one CTA fits: smaller charts
+  p.per = ws_bytes_per_cta(d, W, VW, FW);
+  while (p.per > budget && d.emax > 4096) {  // not even one CTA fits: smaller charts
     d.emax = d.emax * 3 / 4;
-    per = ws_bytes_per_cta(d, W, VW, FW);
+    p.per = ws_bytes_per_cta(d, W, VW, FW);
   }
-  int ctas = (int)std::max<long long>(1, std::min<long long>(std::max(1, want_ctas), (long long)(budget / per)));
-  size_t need = per * (size_t)ctas;
+  p.ctas = (int)std::max<long long>(1, std::min<long long>(std::max(1, want_ctas), (long long)(budget / p.per)));
+  return p;
+}
+epic_status ensure_workspace(epic_lexer_table* t, int want_ctas, int n, cudaStream_t st) {
+  const BlockPlan p = plan_workspace(t, want_ctas, n);
+  const WsDims d = p.d;
+  const int ctas = p.ctas;
+  const size_t need = p.per * (size_t)ctas;
   if (t->d_ws && t->ws_bytes >= need && t->dims.nmax == d.nmax && t->dims.emax == d.emax) {
     t->ctas = ctas;
     return EPIC_OK;
@@ -196,16 +217,19 @@ epic_status ensure_workspace(epic_lexer_table* t, int want_ctas, int n, cudaStre
     cudaFree(t->d_ws);
     t->d_ws = nullptr;
   }
-  if (cudaMalloc(&t->d_ws, need) != cudaSuccess) {
-    t->d_ws = nullptr;
-    return EPIC_ERR_OOM;
-  }
+  if (!device_alloc(&t->d_ws, need)) return EPIC_ERR_OOM;
   // staging rows and bdone must start at zero; the rest is written before read
   if (cudaMemsetAsync(t->d_ws, 0, need, st) != cudaSuccess) return EPIC_ERR_CUDA;
   t->ws_bytes = need;
   t->dims = d;
   t->ctas = ctas;
   return EPIC_OK;
+}
+
+// Chart entries of a whole walk of validation.
+long long walk_entries(int n) {
+  if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) return atoll(e);
+  return 256ll * std::max(1, n);
 }
 
 // Warp-walk workspace: columns <= min(4096, 8 n + 256) per walk; entries
@@ -215,8 +239,7 @@ epic_status ensure_wworkspace(epic_lexer_table* t, long long checks, int n, cuda
   const epic_grammar* g = t->g;
   int W = g->dg.W;
   int nmax = std::min(kWCols, 8 * n + 256);
-  long long emax = 256ll * std::max(1, n);
-  if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) emax = atoll(e);
+  const long long emax = walk_entries(n);
   const size_t budget = workspace_budget("EPIC_WARP_WORKSPACE_MB", 0.25, t->d_wws ? t->wws_bytes : 0);
   size_t per = wbytes_per_warp(nmax, emax, W);
   long long warps = std::min<long long>(checks, (long long)sm_count() * 2 * kWarpsPerCta);
@@ -232,10 +255,7 @@ epic_status ensure_wworkspace(epic_lexer_table* t, long long checks, int n, cuda
     cudaFree(t->d_wws);
     t->d_wws = nullptr;
   }
-  if (cudaMalloc(&t->d_wws, need) != cudaSuccess) {
-    t->d_wws = nullptr;
-    return EPIC_ERR_OOM;
-  }
+  if (!device_alloc(&t->d_wws, need)) return EPIC_ERR_OOM;
   if (cudaMemsetAsync(t->d_wws, 0, need, st) != cudaSuccess) return EPIC_ERR_CUDA;
   t->wws_bytes = need;
   t->wnmax = nmax;
@@ -263,10 +283,7 @@ epic_status grow(epic_lexer_table* t, char** buf, size_t* have, size_t need) {
     *buf = nullptr;
     *have = 0;
   }
-  if (cudaMalloc(buf, need) != cudaSuccess) {
-    *buf = nullptr;
-    return EPIC_ERR_OOM;
-  }
+  if (!device_alloc(buf, need)) return EPIC_ERR_OOM;
   *have = need;
   return EPIC_OK;
 }
@@ -336,10 +353,7 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
       cudaFree(t->d_wws);
       t->d_wws = nullptr;
     }
-    if (cudaMalloc(&t->d_wws, wneed) != cudaSuccess) {
-      t->d_wws = nullptr;
-      return EPIC_ERR_OOM;
-    }
+    if (!device_alloc(&t->d_wws, wneed)) return EPIC_ERR_OOM;
     // the global stage starts at zero; walks return it zeroed
     if (cudaMemsetAsync(t->d_wws, 0, wneed, st) != cudaSuccess) return EPIC_ERR_CUDA;
     t->wws_bytes = wneed;
@@ -853,15 +867,31 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   // 64: 4.9 against 3.3, and the lines cross in between).
   bool few = g->dg.W <= 32 && cta_walks(total, n, g->dg.W, sm_count());
   bool region = !few && (g->dg.W > 32 || n >= 128 || total > (long long)sm_count() * 2 * kWarpsPerCta);
+  bool forced = false;
   if (const char* e = getenv("EPIC_REGION")) {
     region = atoi(e) != 0;
     few = few && !region;
+    forced = region;
   }
-  if (region) return validate_region(g, t, d_x, B, n, d_pos, k, d_cand, K, d_valid, st);
-  // Few checks: a CTA each.
+  if (region) {
+    const epic_status s = validate_region(g, t, d_x, B, n, d_pos, k, d_cand, K, d_valid, st);
+    // narrow item sets take this way for speed only: without memory for the
+    // charts, a warp walks each check (nothing was launched)
+    if (s != EPIC_ERR_OOM || g->dg.W > 32 || forced) return s;
+  }
+  // Few checks: a CTA each, where the block workspace holds a slot for each
+  // and charts as large as a warp's (a tight budget: a warp each).
+  const int slots = (int)std::min<long long>(total, sm_count());
   if (few) {
-    const epic_status s = ensure_workspace(t, (int)std::min<long long>(total, sm_count()), n, st);
-    if (s != EPIC_OK) return s;
+    const BlockPlan p = plan_workspace(t, slots, n);
+    few = p.ctas == slots && p.d.emax >= walk_entries(n);
+  }
+  if (few) {
+    const epic_status s = ensure_workspace(t, slots, n, st);
+    if (s != EPIC_OK && s != EPIC_ERR_OOM) return s;
+    few = s == EPIC_OK;
+  }
+  if (few) {
     long long cap = t->dims.emax;
     if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) cap = atoll(e);
     t->last = st;
@@ -1033,7 +1063,8 @@ epic_status epic_select_compatible_subset(const epic_grammar* g, const epic_lexe
       cudaFree(t->d_spec);
     }
     t->d_spec = nullptr;
-    if (cudaMalloc(&t->d_spec, (size_t)2 * B) != cudaSuccess) return EPIC_ERR_OOM;
+    t->spec_cap = 0;
+    if (!device_alloc(&t->d_spec, (size_t)2 * B)) return EPIC_ERR_OOM;
     t->spec_cap = B;
   }
   t->last = st;
