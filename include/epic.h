@@ -191,8 +191,11 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
  *     n > 128 (whole-graph walks of long rows of such grammars take
  *     seconds per check; use epic_validate_batch for them);
  *   - EPIC_ERR_CAPACITY when one walk's workspace, (8 n + 256) columns and
- *     256 n chart entries, does not fit in the array.
- * A check whose chart needs more than 256 n entries reports 2 (overflow).
+ *     256 n chart entries, does not fit in the array (counting rows of
+ *     ceil(items / 32) words and three words more per entry; rows are kept in
+ *     whole 16 bytes, and a walk that only this keeps out takes the entries
+ *     that fit, at least three quarters of 256 n).
+ * A check whose chart needs more than its entries reports 2 (overflow).
  * Fewer walks run at once than in epic_validate_batch, so it is slower on
  * large batches.
  *

@@ -996,8 +996,16 @@ epic_status epic_validate_batch_noalloc(const epic_grammar* g, const epic_lexer_
   wp.emax = 256ll * n;
   wp.W = W;
   wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, W);
-  long long fit = (long long)((kNoAllocBytes - 256) / wp.per_warp);
-  if (fit < 1) return EPIC_ERR_CAPACITY;  // one walk's workspace does not fit the array
+  if (wp.per_warp > kNoAllocBytes - 256) {
+    // One walk's workspace does not fit the array.  Rows are padded to four
+    // words: when the padding is what does not fit, the walk takes the entries
+    // that do (more than three quarters of 256 n: the padding is largest for
+    // one-word rows, 20 bytes an entry against 16).
+    if (wbytes_unpadded(wp.nmax, wp.emax, (g->dg.D + 31) / 32, g->dg.VW) > kNoAllocBytes - 256) return EPIC_ERR_CAPACITY;
+    wp.emax = (long long)((kNoAllocBytes - 1024 - wbytes_per_warp(wp.nmax, 0, W)) / (4 + 4 * (size_t)W));
+    wp.per_warp = wbytes_per_warp(wp.nmax, wp.emax, W);
+  }
+  const long long fit = (long long)((kNoAllocBytes - 256) / wp.per_warp);
   {
     WsPack p;
     p.base = base + 256;

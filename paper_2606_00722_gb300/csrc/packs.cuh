@@ -93,4 +93,11 @@ inline size_t wbytes_per_warp(int nmax, long long emax, int W) {
          r((size_t)emax * 4) + r((size_t)emax * W * 4);
 }
 
+// What the row limit of epic_validate_batch_noalloc is stated in: a walk with
+// rows of w words, not padded, and two words more per column and per entry.
+inline size_t wbytes_unpadded(int nmax, long long emax, int w, int VW) {
+  auto r = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  return wbytes_per_warp(nmax, emax, w) + r((size_t)nmax * VW * 4) + r((size_t)nmax * 8) + r((size_t)emax * 8);
+}
+
 }  // namespace epic

@@ -7,6 +7,8 @@ call reuses the library's one fixed scratch array.
 
 This file is collected last so that a run stopping at the first failure has
 already run every other test."""
+import types
+
 import numpy as np
 import pytest
 
@@ -73,6 +75,30 @@ def test_noalloc_rejects_long_rows_of_wide_grammars(cuda):
     assert e.value.status == 6  # EPIC_ERR_CAPACITY
     torch.cuda.synchronize()
     assert (valid.cpu().numpy() == 7).all()
+
+
+@pytest.mark.parametrize('n,accepted', [(10050, True), (10070, True), (10890, True), (10910, False)])
+def test_noalloc_row_limit_counts_unpadded_rows(cuda, n, accepted):
+    """Rows of nine words (kept in twelve): the longest row that the array
+    takes is 10,898 tokens, not the 10,060 at which 256 n padded entries end."""
+    import torch
+    import paper_2606_00722_gb300 as epic
+    w = make_workload('smiles-256', 42, batch=2, k=2, K=4)
+    x = np.full((2, n), -1, np.int32)
+    x[:, :w.n] = w.x
+    ref = _run(epic.validate_batch, types.SimpleNamespace(grammar=w.grammar, vocab=w.vocab, x=x, pos=w.pos, cand=w.cand), cuda)
+    g = epic.Grammar(w.grammar)
+    t = epic.LexTable(g, w.vocab)
+    dev = [torch.from_numpy(a).to(cuda) for a in (x, w.pos, w.cand)]
+    valid = torch.full(w.cand.shape, 7, dtype=torch.uint8, device=cuda)
+    if accepted:
+        epic.validate_batch_noalloc(g, t, *dev, valid)
+        assert (ref != 2).all()
+        np.testing.assert_array_equal(valid.cpu().numpy(), ref)
+    else:
+        with pytest.raises(epic.EpicError) as e:
+            epic.validate_batch_noalloc(g, t, *dev, valid)
+        assert e.value.status == 6  # EPIC_ERR_CAPACITY
 
 
 def test_noalloc_on_a_side_stream_then_stats(cuda):
