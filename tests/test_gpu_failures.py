@@ -12,18 +12,22 @@ import oracle
 from synth import make_workload
 
 from test_gpu_edges import run_gpu
+from test_gpu_scratch import validate
 
 pytestmark = pytest.mark.gpu
 NTHREADS = os.cpu_count() or 1
 
 
-def test_whole_walk_overflow_reports_two(cuda, monkeypatch):
-    """Whole-graph walks with room for 40 chart entries: checks whose chart
-    needs more report 2 and are counted; every other bit equals the oracle."""
+@pytest.mark.parametrize('k,K,kernel', [(3, 6, 'k_validate_cta'), (9, 18, 'k_validate_warp')])
+def test_whole_walk_overflow_reports_two(cuda, monkeypatch, k, K, kernel):
+    """Whole-graph walks, a CTA or a warp per check, with room for 40 chart
+    entries: checks whose chart needs more report 2 and are counted; every
+    other bit equals the oracle."""
     monkeypatch.setenv('EPIC_REGION', '0')
     monkeypatch.setenv('EPIC_ENTRIES_PER_WALK', '40')
-    w = make_workload('json-schema', 42, batch=2, k=3, K=6, n=64)
-    got, st = run_gpu(w.grammar, w.vocab, w.x, w.pos, w.cand, cuda)
+    w = make_workload('json-schema', 42, batch=2, k=k, K=K, n=64)
+    got, kernels, st = validate(w, cuda)
+    assert kernels == [kernel]
     ref = oracle.Oracle(w.grammar, w.vocab).validate_batch(w.x, w.pos, w.cand, nthreads=NTHREADS)
     ovf = got == 2
     assert ovf.any(), 'the tiny workspace should overflow some checks'
@@ -46,12 +50,10 @@ def test_region_chart_overflow_falls_back_to_whole_walks(cuda, monkeypatch):
     np.testing.assert_array_equal(got, ref)
 
 
-@pytest.mark.parametrize('forward_cta', ['0', '1'])
-def test_both_limits_at_once(cuda, monkeypatch, forward_cta):
-    """Forward charts and whole walks both too small (either forward kernel):
-    the checks report 2, none is silently answered."""
+def test_both_limits_at_once(cuda, monkeypatch):
+    """Forward charts and whole walks both too small: the checks report 2,
+    none is silently answered."""
     monkeypatch.setenv('EPIC_REGION', '1')
-    monkeypatch.setenv('EPIC_FORWARD_CTA', forward_cta)
     monkeypatch.setenv('EPIC_SEQ_ENTRIES', '200')
     monkeypatch.setenv('EPIC_ENTRIES_PER_WALK', '30')
     w = make_workload('json-schema', 44, batch=2, k=2, K=4, n=80)

@@ -107,6 +107,40 @@ def test_wide_grammars_by_region(cuda, name, seed, kw):
     np.testing.assert_array_equal(got, ref)
 
 
+@pytest.mark.parametrize('rows', [5, 30, 40, 80])
+def test_good_pass_clusters(cuda, rows):
+    """The CTAs that share a sequence's good pass (152 SMs): eight up to 16
+    rows, four up to 33, two up to 66, then one."""
+    w = make_workload('clike-512', 50, batch=rows, k=2, K=4, n=24)
+    got, st = run_gpu(w.grammar, w.vocab, w.x, w.pos, w.cand, cuda)
+    assert st['overflow'] == 0 and st['region_checks'] == w.cand.size
+    ref = oracle.Oracle(w.grammar, w.vocab).validate_batch(w.x, w.pos, w.cand, nthreads=NTHREADS)
+    np.testing.assert_array_equal(got, ref)
+
+
+def test_good_pass_more_entries_than_row_slots(cuda):
+    """One CTA per row and columns of more entries than its 65 row slots (216
+    item words): the rest of a column's masks are in global memory.  A sample
+    of the rows against the oracle; one completion of every row."""
+    import torch
+    import paper_2606_00722_gb300 as epic
+    w = make_workload('random-stress-1024', 51, batch=70, k=1, K=2, n=192)
+    g = epic.Grammar(w.grammar)
+    t = epic.LexTable(g, w.vocab)
+    x, pos, cand = (torch.from_numpy(a).to(cuda) for a in (w.x, w.pos, w.cand))
+    lens = torch.empty(70, dtype=torch.int32, device=cuda)
+    epic.extract_witness(g, t, x, torch.zeros((70, 32 * w.n), dtype=torch.int32, device=cuda), lens)
+    assert (lens.cpu().numpy() >= 0).all()
+    st = t.stats(reset=True)
+    assert st['entries'] > 66 * st['columns'], 'the mean column has more entries than slots'
+    valid = torch.full(w.cand.shape, 9, dtype=torch.uint8, device=cuda)
+    epic.validate_batch(g, t, x, pos, cand, valid)
+    assert t.stats()['overflow'] == 0
+    rows = np.random.default_rng(1).choice(70, 5, replace=False)
+    ref = oracle.Oracle(w.grammar, w.vocab).validate_batch(w.x[rows], w.pos[rows], w.cand[rows], nthreads=NTHREADS)
+    np.testing.assert_array_equal(valid.cpu().numpy()[rows], ref)
+
+
 def test_clike_full_length_row(cuda):
     """clike-512 at its full row length (512 tokens) on one row, 4 positions x
     8 candidates, by region (the default for its item width), against the

@@ -58,6 +58,26 @@ def test_noalloc_wide_items_short_rows_global_stage(cuda):
         np.testing.assert_array_equal(got, ref)
 
 
+@pytest.mark.parametrize('name,words,seed,kw', [
+    ('json-schema', 12, 44, dict(batch=4, k=6, K=8, n=48)),
+    ('clike-512', 64, 45, dict(batch=2, k=5, K=9, n=48)),
+    ('random-stress-1024', 216, 46, dict(batch=3, k=4, K=6, n=24)),
+])
+def test_noalloc_more_checks_than_cta_walks_fit(cuda, name, words, seed, kw):
+    """More checks of short rows than the array holds CTA walks (one per SM at
+    most, and 256 n entries each): a warp each, with rows in the global part
+    of the array, which holds the earlier calls' contents."""
+    import paper_2606_00722_gb300 as epic
+    slots = min(152, (128 << 20) // (256 * kw['n'] * 4 * (words + 1)))
+    assert kw['batch'] * kw['k'] * kw['K'] > slots and kw['n'] < 96
+    for s in (seed, seed + 1):
+        w = make_workload(name, s, **kw)
+        ref = _run(epic.validate_batch, w, cuda)
+        got = _run(epic.validate_batch_noalloc, w, cuda)
+        assert (ref != 2).all() and (got != 2).all()
+        np.testing.assert_array_equal(got, ref)
+
+
 def test_noalloc_rejects_long_rows_of_wide_grammars(cuda):
     """Wide item sets on rows longer than 128 tokens are refused with
     EPIC_ERR_CAPACITY before anything is enqueued (the output is untouched)."""
