@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(32 * kGsMaxWarps, 1)
     sc.g_last = a.ws.g_last;
     sc.f_q = a.ws.f_q;
     sc.f_c = a.ws.f_c;
-    sc.key_q = a.key_q;
+    sc.key_q = a.ws.key_q;
     sc.ent = a.ent;
     EarleyColsGS<true, S>::place_scratch(g, plan, dyn, sc);
     const BlockRec br{a.rec.col_gap, a.rec.e_dst,   a.rec.e_src,   a.rec.e_lbl,    a.rec.cnt,

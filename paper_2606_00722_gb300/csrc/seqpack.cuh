@@ -16,13 +16,12 @@ struct SeqArena {
   int32_t* in_off;     // [nmax + 1] edges are stored by target column
   int32_t* out_off;    // [nmax + 1]
   int32_t* out_idx;    // [edge_cap]
-  int32_t* succ_off;   // [nmax + 1] columns holding origin u, ascending
-  int32_t* succ_idx;   // [emax]
+  int32_t* succ_off;   // [nmax + 1] columns holding origin u ...
+  int32_t* succ_idx;   // [emax] ... in no order
   uint32_t* expn;      // [nmax][W] scratch of the good pass
   int32_t* eidx;       // [nmax (nmax + 1) / 2] entry of (column j, origin o <= j), -1: none
   uint8_t* gnz;        // [emax] the entry has a good item
   int32_t* cursor;     // [2 (nmax + 1)] scratch of the good pass
-  int32_t* key_q;      // [kMaxQ] scratch of the forward walk
   LexEntry* ent;       // [kMaxQ]
 };
 
@@ -39,7 +38,7 @@ struct SeqPack {
            + r(nm) + 2 * r((size_t)edge_cap * 4) + r((size_t)edge_cap * 32) + 3 * r((size_t)n * 4) +
            r((size_t)emax * VW * 4) + r(32)                                                 // SeqRec
            + r((size_t)emax * W * 4) + r(nm * 4) + 3 * r((nm + 1) * 4) + r((size_t)edge_cap * 4) +
-           r((size_t)emax * 4) + r(nm * W * 4) + r(nm * (nm + 1) / 2 * 4) + r((size_t)emax) + r(2 * (nm + 1) * 4) + r(kMaxQ * 4) +
+           r((size_t)emax * 4) + r(nm * W * 4) + r(nm * (nm + 1) / 2 * 4) + r((size_t)emax) + r(2 * (nm + 1) * 4) +
            r(kMaxQ * 16);
   }
   __device__ SeqArena carve(long long b) const {
@@ -86,7 +85,6 @@ struct SeqPack {
     a.eidx = (int32_t*)take(nm * (nm + 1) / 2 * 4);
     a.gnz = (uint8_t*)take((size_t)emax);
     a.cursor = (int32_t*)take(2 * (nm + 1) * 4);
-    a.key_q = (int32_t*)take(kMaxQ * 4);
     a.ent = (LexEntry*)take(kMaxQ * 16);
     return a;
   }

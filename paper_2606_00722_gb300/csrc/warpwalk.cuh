@@ -3,9 +3,9 @@
 // Same graph and chart as the CTA walk (walk.cuh / skeleton.cuh), with every
 // step done by one warp and no block barrier:
 //  - the open column's rows lie in the warp's global stage, which its SM's L1
-//    holds (the kernels leave almost all of the 256 KB to L1).  Staging them in
-//    shared memory instead cost 24 KB per warp, so that seven warps ran on an
-//    SM;
+//    holds (sixteen warps keep 42 KB of the 256 KB as shared memory, 2.6 KB
+//    each).  Staging the rows in shared memory instead cost 24 KB per warp, so
+//    that seven warps ran on an SM;
 //  - the closure of a column visits every origin once, from the highest down:
 //    completions from origin o only advance items of origins <= o, and the one
 //    entry of column o with origin o feeds row o itself (closed in registers);
@@ -31,7 +31,6 @@ namespace epic {
 constexpr int kWarpsPerCta = 8;
 constexpr int kWCols = 4096;    // columns per walk (graph nodes)
 constexpr int kWMaxW = 256;
-constexpr int kWMaxVW = 32;
 constexpr int kWMaxQ = 1024;
 
 // index of (column j, origin o <= j) in a lower-triangular table
@@ -73,7 +72,6 @@ struct WSh {  // per-warp shared memory
   uint32_t touched[kWCols / 32];
   alignas(16) uint32_t lbl[kWMaxW];  // items that the arrivals' labels expect
   alignas(16) uint32_t scr[kWMaxW];  // one row
-  uint32_t nt[kWMaxVW];
   int32_t list[32];
 };
 
