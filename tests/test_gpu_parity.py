@@ -44,7 +44,7 @@ CASES = [
     ('expr-tiny', 42, {}), ('expr-tiny', 43, {}), ('expr-tiny', 44, {}),
     ('json-schema', 42, dict(batch=4)), ('json-schema', 43, dict(batch=3, k=3)),
     ('smiles-256', 42, dict(batch=6, k=4)), ('smiles-256', 44, dict(batch=2, k=16, K=4)),
-    ('clike-512', 42, dict(batch=1, k=2, K=4)),
+    ('clike-512', 42, dict(batch=1, k=2, K=4)), ('clike-512', 42, dict(batch=2, k=4, K=4, n=160)),
 ]
 
 
@@ -63,16 +63,6 @@ def test_step_parity(cuda, name, seed, kw):
     np.testing.assert_array_equal(got['sel'], ref_sel)
     np.testing.assert_array_equal(got['x'], O.commit(w.x, w.pos, rtok, ref_sel))
     assert got['stats']['checks'] == w.cand.size
-
-
-@pytest.mark.parametrize('name,seed,kw', [('json-schema', 43, dict(batch=3, k=3)),
-                                          ('clike-512', 42, dict(batch=2, k=4, K=4, n=160))])
-def test_step_parity_descending_sweep(cuda, monkeypatch, name, seed, kw):
-    """The CTA walks (forward charts of wide grammars, selection's exact
-    tests) with the descending block sweep of the column closure instead of
-    the warp-parallel one: the same least fixpoint, so the same bits."""
-    monkeypatch.setenv('EPIC_GS_PARALLEL', '0')
-    test_step_parity(cuda, name, seed, kw)
 
 
 @pytest.mark.parametrize('name', ['expr-tiny', 'json-schema', 'smiles-256'])
