@@ -16,6 +16,7 @@ seeded batch of the same shape; there is no data-path collective.
 import argparse
 import json
 import os
+import re
 import subprocess
 import tempfile
 import sys
@@ -28,13 +29,18 @@ sys.path.insert(0, ROOT)
 
 # ncu summaries of the kernels' DRAM traffic (profiles/traffic_<kernel>_<workload>.txt): used only while the
 # kernel's sources hash to the value recorded with the counters
-KERNEL_SOURCES = {
-    'k_validate_warp': ['kernels_walk.cu', 'warpwalk.cuh', 'rows.cuh', 'device.cuh', 'packs.cuh'],
-    'k_forward_gs': ['region_forward.cu', 'gscols.cuh', 'rows.cuh', 'skeleton.cuh', 'walk.cuh', 'device.cuh',
-                     'seqpack.cuh'],
-    'k_good': ['region_good.cu', 'rows.cuh', 'device.cuh', 'seqpack.cuh'],
-    'k_check': ['region_check.cu', 'warpwalk.cuh', 'rows.cuh', 'device.cuh'],
+KERNEL_SOURCES = {  # the file of each kernel; what it includes counts too
+    'k_validate_cta': 'kernels_cta.cu',
+    'k_validate_warp': 'kernels_walk.cu',
+    'k_forward_gs': 'region_forward.cu',
+    'k_good': 'region_good.cu',
+    'k_check': 'region_check.cu',
 }
+
+
+# how epic_validate_batch took a batch, by the kernel that it spent most time in
+PATHS = {'k_forward_gs': 'region', 'k_good': 'region', 'k_check': 'region', 'k_validate_cta': 'walk, a CTA per check',
+         'k_validate_warp': 'walk, a warp per check'}
 
 
 def parse():
@@ -44,7 +50,8 @@ def parse():
     ap.add_argument('--warmup', type=int, default=3)
     # clike-512 (32 x 512, k 8, K 32) is the largest workload whose steps fit
     # a bench run of minutes; random-stress-1024 (64 x 1024, k 16, K 32) runs
-    # with --workload random-stress-1024 at several minutes per step
+    # with --workload random-stress-1024, but three steps of it (a warm-up, a
+    # timed and an end-to-end one) were not done after 15 minutes
     ap.add_argument('--workload', default='clike-512')
     ap.add_argument('--impl', default='epic', choices=['epic', 'reference'])
     ap.add_argument('--seed', type=int, default=42)
@@ -132,12 +139,26 @@ class Clocks:
                 'samples': len(sm)}
 
 
+def kernel_files(kernel):
+    """A kernel's source file and every project file that it includes, directly
+    or not, in the order of first inclusion."""
+    files, todo = [], [KERNEL_SOURCES[kernel]] if kernel in KERNEL_SOURCES else []
+    while todo:
+        f = todo.pop(0)
+        if f in files:
+            continue
+        files.append(f)
+        with open(os.path.join(ROOT, 'paper_2606_00722_gb300', 'csrc', f)) as fh:
+            todo += re.findall(r'^\s*#include "([^"]+)"', fh.read(), re.M)
+    return files
+
+
 def kernel_sha(kernel):
     """Hash of a kernel's source files (tells whether recorded counters still
     describe the current build)."""
     import hashlib
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES.get(kernel, []):
+    for f in kernel_files(kernel):
         with open(os.path.join(ROOT, 'paper_2606_00722_gb300', 'csrc', f), 'rb') as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -389,7 +410,6 @@ def main():
     step_ms = [a.elapsed_time(c) for a, b, c in ev]
     val_ms = [a.elapsed_time(b) for a, b, c in ev]
     st = t.stats()
-    region = st['region_checks'] > 0
     # kernels of the timed region: validate's own (one walk kernel, or the
     # forward chart, good masks and region checks) + pick + two selection
     # kernels + commit + the fallback's setup and two kernels per round
@@ -452,7 +472,7 @@ def main():
         work = 3.0 * cen['forward_pairs'] * cen['words']
         work_note = 'forward charts of x: %.0f (node, origin) pairs x %d words x 3 (oracle census, %s)' % (
             cen['forward_pairs'], cen['words'], cen['forward_sample'])
-    elif cen and dom == 'k_validate_warp' and 'checks_pairs' in cen:
+    elif cen and dom in ('k_validate_cta', 'k_validate_warp') and 'checks_pairs' in cen:
         work = 3.0 * cen['checks_pairs'] * cen['words']
         work_note = 'charts of every check: %.0f (node, origin) pairs x %d words x 3 (oracle census)' % (
             cen['checks_pairs'], cen['words'])
@@ -484,11 +504,11 @@ def main():
                        'parallelism': 'replicas' if world > 1 else 'single'},
             'step': 'validate, pick, select (Alg. 4), commit, rejection fallback (Alg. 1) with n_t = k',
             'workload_note': ('clike-512 is the default: the largest configuration whose bench run fits minutes '
-                              '(random-stress-1024 takes minutes per step)')
+                              '(three steps of random-stress-1024 were not done after 15 minutes)')
             if args.workload == 'clike-512' else None,
             'step_latency_us': ms * 1e3, 'validate_checks_per_s': total_checks / (vms / 1e3),
             'valid_fraction': st['valid'] / max(1, st['checks']), 'overflow': st['overflow'],
-            'gpu_launches': int(launches), 'validate_path': 'region' if region else 'walk',
+            'gpu_launches': int(launches), 'validate_path': PATHS.get(dom, dom),
             'commits': commit_sizes,
             'lex_table': {'kind': 'lazy memo (Alg. 2), %d entries' % args.lazy_lex if args.lazy_lex else 'dense',
                           'build_ms': table_ms,

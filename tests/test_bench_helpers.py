@@ -39,6 +39,15 @@ def test_recorded_traffic_needs_matching_sources(tmp_path, monkeypatch):
     assert bench.recorded_traffic('k_check', 'w') is None
 
 
+def test_kernel_sources_hold_what_they_include():
+    assert bench.kernel_files('no-such-kernel') == []
+    for k, f in bench.KERNEL_SOURCES.items():
+        files = bench.kernel_files(k)
+        assert files[0] == f and len(set(files)) == len(files)
+        assert {'launch.h', 'gscols.cuh', 'packs.cuh', 'seqpack.cuh', 'rows.cuh', 'walk.cuh', 'device.cuh'} <= set(files)
+    assert 'region.cuh' in bench.kernel_files('k_good') and 'warpwalk.cuh' in bench.kernel_files('k_check')
+
+
 def test_committed_traffic_records_are_well_formed():
     here = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     prof = os.path.join(here, 'profiles')
