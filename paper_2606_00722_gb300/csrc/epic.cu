@@ -381,12 +381,14 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
 
 // Whole-graph walks with a CTA per check (`slots` of them at a time) or with a
 // warp per check?  A CTA walk ends several times sooner and fills an SM, so it
-// wins while every check has a slot at once: JSON 4 x 64, 128 checks: 1.7 ms
-// against 2.7 (by region 3.5); molecules 4 x 96, 128 checks: 7.0 against 21
-// (16).  Longer narrow rows still gain with two rounds (256 checks: JSON
-// 4 x 150 8.8 ms against 15, by region 11; JSON 4 x 64 3.1 against 2.4).
-// Grammars of at most 4 item words have too little in a column for it (32 x 8
-// expression checks 0.83 ms against 0.78).
+// wins while every check has a slot at once (ms with a CTA / a warp / by
+// region): JSON 4 x 64, 128 checks 1.8 / 2.9 / 3.0; molecules 4 x 96, 128
+// checks 6.2 / 18 / 12.  Two rounds of 96 tokens and more, 256 checks: molecules
+// 4 x 96 13 / 22 / 19, 16 x 120 16 / 33 / 21, 2 x 200 32 / 81 / 42; about even
+// on JSON, 4 x 100 5.0 / 4.5 / 6.0, 16 x 100 5.0 / 6.6 / 6.0, 2 x 200 11 / 13 /
+// 11, 1 x 256 12.5 / 10.1 / 10.9.  Shorter rows lose then (JSON 4 x 64 3.2 / 2.3
+// / 3.4).  Grammars of at most 4 item words have too little in a column
+// (expressions 4 x 32, 32 checks 1.06 / 1.07).
 bool cta_walks(long long total, int n, int W, long long slots) {
   if (W <= 4) return false;
   return total <= slots || (W <= 32 && n >= 96 && total <= 2 * slots);
@@ -858,13 +860,20 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   if (total == 0) return EPIC_OK;
   if (!d_x || !d_pos || !d_cand || !d_valid || n == 0) return EPIC_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // Few checks of narrow item sets walk their whole graphs, a CTA each (wide
-  // item sets always go by region).  Else checks by region over
-  // a per-sequence chart, built once per sequence instead of once per check:
-  // when the item sets are wide (whole-graph walks of large grammars are far
-  // too long), when there are more checks than resident walks, and on rows of
-  // at least 128 tokens (JSON 16 x 256, 1,024 checks: 20 ms against 25; 16 x
-  // 64: 4.9 against 3.3, and the lines cross in between).
+  // Few checks of narrow item sets walk their whole graphs, a CTA each.  Else
+  // checks by region over a per-sequence chart, built once per sequence
+  // instead of once per check: when the item sets are wide (a warp takes
+  // seconds for a long row of a large grammar), when there are more checks
+  // than resident walks, and on rows of at least 128 tokens.  By region
+  // against a warp per check, 1,024 checks of JSON: 16 x 64 4.0 against 3.1 ms,
+  // 16 x 128 8.4 against 6.7, 16 x 256 24 against 33; expressions (two words):
+  // 1 x 128, 64 checks 10.9 against 7.2, 1 x 256 26 against 30, 16 x 256 35
+  // against 41.  The lines cross between 128 and 256 tokens; 128 keeps the
+  // longer walks off the warps.
+  // Wide item sets go by region however few the checks, and region_checks
+  // counts them so.  (A CTA each would end sooner for a handful: C-like 1 x 48,
+  // 32 checks 3.7 ms against 7.3; 400 nonterminals 1 x 256, 16 checks 188
+  // against 282, 1 x 1024, 4 checks 12.0 s against 13.5.)
   bool few = g->dg.W <= 32 && cta_walks(total, n, g->dg.W, sm_count());
   bool region = !few && (g->dg.W > 32 || n >= 128 || total > (long long)sm_count() * 2 * kWarpsPerCta);
   bool forced = false;
@@ -1017,8 +1026,14 @@ epic_status epic_validate_batch_noalloc(const epic_grammar* g, const epic_lexer_
     p.per_cta = ws_bytes_per_cta(p.dims, W, p.VW, 0);
     const long long ctas = std::min<long long>({total, (long long)((kNoAllocBytes - 256) / p.per_cta),
                                                 (long long)sm_count()});
-    // (the array holds fewer CTA walks than there are SMs: JSON 4 x 128, 71;
-    // 256 checks in four rounds of them 14 ms, a warp each 19 ms)
+    // The array holds fewer walks than there are SMs, and about as many of
+    // either kind (256 n entries each: JSON 4 x 128, 71 or 72), so the warp
+    // walks have no more of them running and a CTA walk is the faster one: JSON
+    // 256 checks 4 x 128 13 ms against 18, 512 checks in eight rounds 23 against
+    // 32.  The rule stops at four rounds, short of where a warp each would win:
+    // 4 x 256, 256 checks 43 against 71 ms, 8 x 160, 1,152 checks 69 against
+    // 102; rows under 96 tokens are even at four rounds (4 x 64, 512 checks 5.9
+    // against 5.7).
     if (ctas >= 1 && (cta_walks(total, n, W, ctas) || (n >= 96 && W > 4 && total <= 4 * ctas))) {
       t->last = st;
       t->n_vkernels += 1;
@@ -1103,8 +1118,10 @@ epic_status epic_fallback_commit(const epic_grammar* g, const epic_lexer_table* 
   const int nc = k * K;
   // rounds of m tests per sequence, one CTA per SM (at most kMaxFallbackSpec
   // tests per sequence, at least one): tests after a round's first pass are
-  // spent, and a walk with an SM to itself has twice the warps (smiles 24 x 96,
-  // four commits a row: 42 ms with two CTAs per SM, 33 ms with one)
+  // spent, and a walk with an SM to itself has twice the warps.  One against
+  // two CTAs per SM (molecules, four commits a row): 24 x 96 32 against 42 ms;
+  // 64 tokens, 77 rows 31.4 against 30.6, 96 rows 28.3 against 26.3, 128 rows
+  // 28.8 against 31.5, 152 rows 28.8 against 31.3.
   int m = std::max(1, std::min(kMaxFallbackSpec, std::min(nc, sm_count() / B)));
   epic_status s = ensure_workspace(t, std::min((long long)B * m, (long long)sm_count() * 2), n, st);
   if (s != EPIC_OK) return s;

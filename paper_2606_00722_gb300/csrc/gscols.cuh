@@ -32,9 +32,9 @@
 //    one item costs one shuffle): 4 lanes x 4 words up to 16 words, 16 x 4 up
 //    to 64, 32 x 8 up to 256.  A warp scatters 32 / LR entries per step, and
 //    when it works on one row its lane groups hold copies and share out the
-//    EXP_NT rows.  (Instruction issue, at 36 % of the active cycles with one
-//    word per lane and 32-word steps, was the bound: clike-512 spent about 70
-//    instructions per scattered entry.)
+//    EXP_NT rows.  (With one word per lane and 32-word steps a 64-word row took
+//    about 70 instructions per scattered entry; issue is what bounds a sweep
+//    with four warps per scheduler.)
 //  - all nonterminals that complete at c from o through chains at the self
 //    entry (B -> A, or at gaps any production around A) follow from the
 //    directly completed ones by a table, so a visit is one pass instead of a

@@ -797,10 +797,12 @@ __global__ void __launch_bounds__(32 * kGoodWarps, PER_SM)
 }
 
 // The CTAs that share a sequence: as many as leave every cluster its own SMs (a
-// seventh of the SMs is spared: clusters do not fill every group of SMs).
-// C-like 32 x 256: 67 ms alone, 33 ms with four; 400 nonterminals 4 x 96: 45 and
-// 18 ms with eight.  Narrow rows stay alone: their columns hold too little work
-// between the cluster's barriers (JSON 16 x 256: 4.0 ms alone, 6.8 ms with eight).
+// eighth of the SMs is spared: clusters do not fill every group of SMs).
+// C-like 32 x 256: 60 ms alone, 46 with two, 30 with four; 40 x 128 19 ms alone,
+// 15 with two; 64 x 256 74 and 56; 400 nonterminals 4 x 96: 44 alone, 22 with
+// four, 18 with eight.  Narrow rows stay alone: their columns hold little work
+// between the cluster's barriers, and the text decides (JSON 16 x 256: 9.1 ms
+// alone, 7.7 with eight on one batch, 4.0 and 6.8 on another).
 static int good_cluster(int B, int W, int sms) {
   int C = W <= 16 ? 1 : 8;
   while (C > 1 && (long long)B * C * 8 > 7ll * sms) C >>= 1;

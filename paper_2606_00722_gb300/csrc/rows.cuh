@@ -136,7 +136,7 @@ struct RowRegs {
   // a row from L2 costs about as much as testing 30 items: sets of more than
   // kRowSetMax test every item's next symbol instead (next_t, lanes on
   // consecutive words; scr: one row of shared scratch).  random-stress-1024
-  // grammar, 4 x 96: forward charts 60 -> 49 ms, good masks 67 -> 45 ms.  The
+  // grammar, 4 x 96: forward charts 55 -> 44 ms, good masks 22 -> 18 ms.  The
   // warp walks keep or_rows: many of them share the rows in L1, and the item
   // test took their checks from 37 to 50 ms.
   static constexpr int kRowSetMax = 12;
