@@ -203,8 +203,7 @@ BlockPlan plan_workspace(const epic_lexer_table* t, int want_ctas, int n) {
   p.ctas = (int)std::max<long long>(1, std::min<long long>(std::max(1, want_ctas), (long long)(budget / p.per)));
   return p;
 }
-epic_status ensure_workspace(epic_lexer_table* t, int want_ctas, int n, cudaStream_t st) {
-  const BlockPlan p = plan_workspace(t, want_ctas, n);
+epic_status ensure_workspace(epic_lexer_table* t, const BlockPlan& p, cudaStream_t st) {
   const WsDims d = p.d;
   const int ctas = p.ctas;
   const size_t need = p.per * (size_t)ctas;
@@ -894,11 +893,11 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   if (few) {
     const BlockPlan p = plan_workspace(t, slots, n);
     few = p.ctas == slots && p.d.emax >= walk_entries(n);
-  }
-  if (few) {
-    const epic_status s = ensure_workspace(t, slots, n, st);
-    if (s != EPIC_OK && s != EPIC_ERR_OOM) return s;
-    few = s == EPIC_OK;
+    if (few) {
+      const epic_status s = ensure_workspace(t, p, st);
+      if (s != EPIC_OK && s != EPIC_ERR_OOM) return s;
+      few = s == EPIC_OK;
+    }
   }
   if (few) {
     long long cap = t->dims.emax;
@@ -1078,7 +1077,7 @@ epic_status epic_select_compatible_subset(const epic_grammar* g, const epic_lexe
   if (!d_x || !d_pos || !d_tok || !d_conf || !d_selected || n == 0) return EPIC_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   int want = std::min(2 * B, sm_count() * 2);
-  epic_status s = ensure_workspace(t, want, n, st);
+  epic_status s = ensure_workspace(t, plan_workspace(t, want, n), st);
   if (s != EPIC_OK) return s;
   if (t->spec_cap < B) {
     if (t->d_spec) {
@@ -1123,7 +1122,8 @@ epic_status epic_fallback_commit(const epic_grammar* g, const epic_lexer_table* 
   // 64 tokens, 77 rows 31.4 against 30.6, 96 rows 28.3 against 26.3, 128 rows
   // 28.8 against 31.5, 152 rows 28.8 against 31.3.
   int m = std::max(1, std::min(kMaxFallbackSpec, std::min(nc, sm_count() / B)));
-  epic_status s = ensure_workspace(t, std::min((long long)B * m, (long long)sm_count() * 2), n, st);
+  epic_status s = ensure_workspace(
+      t, plan_workspace(t, (int)std::min((long long)B * m, (long long)sm_count() * 2), n), st);
   if (s != EPIC_OK) return s;
   m = std::max(1, std::min(m, t->ctas / B));
   auto r16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
