@@ -1,5 +1,5 @@
 // Host-side launchers of the kernels compiled in their own translation units
-// (kernels_walk.cu, region_*.cu, kernels_select.cu), so that the
+// (kernels_walk.cu, kernels_cta.cu, region_*.cu, kernels_select.cu), so that the
 // library's device code builds in parallel.  Each takes the launch shape and
 // stream followed by the kernel's own arguments.
 #pragma once

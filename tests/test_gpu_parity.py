@@ -114,6 +114,8 @@ def test_pick_golden(cuda, shape):
     ('expr-tiny', 42, {}, 8), ('expr-tiny', 45, dict(k=6, K=4), 6),
     ('json-schema', 43, dict(batch=3, k=6, K=6), 6), ('smiles-256', 44, dict(batch=3, k=6, K=5), 4),
     ('clike-512', 42, dict(batch=1, k=2, K=4, n=128), 2),
+    # one test of a row per round, and more rows than CTAs
+    ('smiles-256', 45, dict(batch=80, k=3, K=4, n=24), 3), ('expr-tiny', 46, dict(batch=310, k=3, K=3, n=16), 3),
 ])
 def test_decode_step_with_fallback(cuda, name, seed, kw, fill):
     """One whole step (validate, pick, select, commit, then Alg. 1's rejection
