@@ -20,7 +20,10 @@
  *     and counted in the statistics (epic_get_stats), never silently dropped.
  *   - The library owns the opaque objects and the device workspace they hold;
  *     a grammar or lexer table must not be destroyed while work that uses it
- *     is still in flight.  Calls that share one object must not overlap in
+ *     is still in flight.  Asynchronous calls may be captured in a CUDA graph
+ *     after a call of the same shape has made the workspaces; a captured
+ *     workspace is kept until the lexer table is destroyed, and the graph must
+ *     not be launched after that.  Calls that share one object must not overlap in
  *     time on different streams (they share its workspace).
  *   - There is no CPU fallback: when no CUDA device is usable the calls
  *     return EPIC_ERR_CUDA.

@@ -113,6 +113,9 @@ struct epic_lexer_table {
   long long wemax = 0;
   int wwarps = 0;
   cudaStream_t last = nullptr;
+  // workspaces that launches under stream capture were given: a graph may
+  // replay them, so they are kept until the table goes, also when replaced
+  std::vector<void*> in_graphs;
   // CUDA events around the kernels of the last epic_validate_batch call
   // (epic_last_kernel_times): kev[i] .. kev[i + 1] is kernel i
   cudaEvent_t kev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -154,6 +157,32 @@ bool device_alloc(T** p, size_t bytes) {
   (void)cudaGetLastError();
   *p = nullptr;
   return false;
+}
+
+// The workspaces in use now belong to a graph if `st` is being captured.
+// Called before a call's launches.
+epic_status note_capture(epic_lexer_table* t, cudaStream_t st) {
+  if (!st) return EPIC_OK;  // the legacy stream cannot be captured
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return EPIC_ERR_CUDA;
+  if (cap != cudaStreamCaptureStatusActive) return EPIC_OK;
+  try {
+    for (void* p : {(void*)t->d_ws, (void*)t->d_wws, (void*)t->d_spec, (void*)t->d_seq, (void*)t->d_regs, (void*)t->d_wit})
+      if (p && std::find(t->in_graphs.begin(), t->in_graphs.end(), p) == t->in_graphs.end()) t->in_graphs.push_back(p);
+  } catch (std::exception&) {
+    return EPIC_ERR_OOM;
+  }
+  return EPIC_OK;
+}
+
+// Give a workspace back (after the table's last stream), unless a graph holds it.
+template <class T>
+void release(epic_lexer_table* t, T** p) {
+  if (*p && std::find(t->in_graphs.begin(), t->in_graphs.end(), (void*)*p) == t->in_graphs.end()) {
+    cudaStreamSynchronize(t->last);
+    cudaFree(*p);
+  }
+  *p = nullptr;
 }
 
 int sm_count() {
@@ -211,11 +240,7 @@ epic_status ensure_workspace(epic_lexer_table* t, const BlockPlan& p, cudaStream
     t->ctas = ctas;
     return EPIC_OK;
   }
-  if (t->d_ws) {
-    cudaStreamSynchronize(t->last);
-    cudaFree(t->d_ws);
-    t->d_ws = nullptr;
-  }
+  release(t, &t->d_ws);
   if (!device_alloc(&t->d_ws, need)) return EPIC_ERR_OOM;
   // staging rows and bdone must start at zero; the rest is written before read
   if (cudaMemsetAsync(t->d_ws, 0, need, st) != cudaSuccess) return EPIC_ERR_CUDA;
@@ -249,11 +274,7 @@ epic_status ensure_wworkspace(epic_lexer_table* t, long long checks, int n, cuda
     t->wwarps = (int)std::min<long long>(warps, t->wws_bytes / per / kWarpsPerCta * kWarpsPerCta);
     return EPIC_OK;
   }
-  if (t->d_wws) {
-    cudaStreamSynchronize(t->last);
-    cudaFree(t->d_wws);
-    t->d_wws = nullptr;
-  }
+  release(t, &t->d_wws);
   if (!device_alloc(&t->d_wws, need)) return EPIC_ERR_OOM;
   if (cudaMemsetAsync(t->d_wws, 0, need, st) != cudaSuccess) return EPIC_ERR_CUDA;
   t->wws_bytes = need;
@@ -276,12 +297,8 @@ WPack wpack_of(const epic_lexer_table* t) {
 // Grow a device buffer owned by the table (synchronizing its last stream first).
 epic_status grow(epic_lexer_table* t, char** buf, size_t* have, size_t need) {
   if (*buf && *have >= need) return EPIC_OK;
-  if (*buf) {
-    cudaStreamSynchronize(t->last);
-    cudaFree(*buf);
-    *buf = nullptr;
-    *have = 0;
-  }
+  release(t, buf);
+  *have = 0;
   if (!device_alloc(buf, need)) return EPIC_ERR_OOM;
   *have = need;
   return EPIC_OK;
@@ -310,6 +327,8 @@ epic_status region_prepare(const epic_grammar* g, epic_lexer_table* t, const int
   epic_status s = grow(t, &t->d_seq, &t->seq_bytes, sp.per_seq * (size_t)B);
   if (s != EPIC_OK) return s;
   sp.base = t->d_seq;
+  s = note_capture(t, st);
+  if (s != EPIC_OK) return s;
   t->last = st;
   // 1. forward charts
   {
@@ -347,11 +366,7 @@ epic_status validate_region(const epic_grammar* g, epic_lexer_table* t, const in
   warps = std::max<long long>(1, std::min<long long>(warps, (long long)(wbudget / wp.per_warp)));
   size_t wneed = wp.per_warp * (size_t)warps;
   if (!t->d_wws || t->wws_bytes < wneed || t->wnmax != wp.nmax || t->wemax != wp.emax) {
-    if (t->d_wws) {
-      cudaStreamSynchronize(t->last);
-      cudaFree(t->d_wws);
-      t->d_wws = nullptr;
-    }
+    release(t, &t->d_wws);
     if (!device_alloc(&t->d_wws, wneed)) return EPIC_ERR_OOM;
     // the global stage starts at zero; walks return it zeroed
     if (cudaMemsetAsync(t->d_wws, 0, wneed, st) != cudaSuccess) return EPIC_ERR_CUDA;
@@ -815,13 +830,14 @@ epic_status epic_lexer_table_build_lazy(const epic_grammar* g, const int32_t* to
 void epic_lexer_table_destroy(epic_lexer_table* t) {
   if (!t) return;
   if (t->last) cudaStreamSynchronize(t->last);
+  release(t, &t->d_ws);
+  release(t, &t->d_wws);
+  release(t, &t->d_spec);
+  release(t, &t->d_seq);
+  release(t, &t->d_regs);
+  release(t, &t->d_wit);
+  for (void* p : t->in_graphs) cudaFree(p);
   cudaFree(t->d_table);
-  cudaFree(t->d_ws);
-  cudaFree(t->d_wws);
-  cudaFree(t->d_spec);
-  cudaFree(t->d_seq);
-  cudaFree(t->d_regs);
-  cudaFree(t->d_wit);
   cudaFree(t->d_fb);
   cudaFree(t->d_stats);
   cudaFree(t->d_counter);
@@ -902,6 +918,8 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
   if (few) {
     long long cap = t->dims.emax;
     if (const char* e = getenv("EPIC_ENTRIES_PER_WALK")) cap = atoll(e);
+    const epic_status sc = note_capture(t, st);
+    if (sc != EPIC_OK) return sc;
     t->last = st;
     t->n_vkernels += 1;
     t->nk = 1;
@@ -913,6 +931,7 @@ epic_status epic_validate_batch(const epic_grammar* g, const epic_lexer_table* t
     return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
   }
   epic_status s = ensure_wworkspace(t, total, n, st);
+  if (s == EPIC_OK) s = note_capture(t, st);
   if (s != EPIC_OK) return s;
   t->last = st;
   cudaMemsetAsync(t->d_counter, 0, 8, st);
@@ -1080,15 +1099,13 @@ epic_status epic_select_compatible_subset(const epic_grammar* g, const epic_lexe
   epic_status s = ensure_workspace(t, plan_workspace(t, want, n), st);
   if (s != EPIC_OK) return s;
   if (t->spec_cap < B) {
-    if (t->d_spec) {
-      cudaStreamSynchronize(t->last);
-      cudaFree(t->d_spec);
-    }
-    t->d_spec = nullptr;
+    release(t, &t->d_spec);
     t->spec_cap = 0;
     if (!device_alloc(&t->d_spec, (size_t)2 * B)) return EPIC_ERR_OOM;
     t->spec_cap = B;
   }
+  s = note_capture(t, st);
+  if (s != EPIC_OK) return s;
   t->last = st;
   mark_event(&t->sev[0], st);
   launch_select_spec(std::min(2 * B, t->ctas), st, t->dgl, t->d_table, t->vocab, d_x, B, n, d_pos, k, d_tok,
@@ -1169,6 +1186,7 @@ epic_status epic_extract_witness(const epic_grammar* g, const epic_lexer_table* 
   if (s != EPIC_OK) return s;
   const size_t per = witness_scratch_bytes(cap, t->dgl.D, t->dgl.W, t->dgl.VW);
   s = grow(t, &t->d_wit, &t->wit_bytes, per * (size_t)B);
+  if (s == EPIC_OK) s = note_capture(t, st);
   if (s != EPIC_OK) return s;
   launch_witness(B, st, t->dgl, sp, d_terms, cap, d_len, t->d_wit, t->d_stats);
   return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
